@@ -1,8 +1,10 @@
-"""Thin ctypes binding of libvispec.so: argument marshalling only.
+"""Thin binding of libvispec.so: argument marshalling only.
 
-Every step of the verification path runs in the library's CUDA kernels; torch is used here for
-device memory and streams.  There is no CPU fallback: if the shared object is missing or CUDA is
-unavailable the import of the library (``load()``) raises.
+The hot calls go through the native module ``_native`` (built beside the library; it reads device pointers and
+torch's current stream without ctypes), the rest and the raw C functions (``VerifyContext.lib``) through ctypes.
+Every step of the verification path runs in the library's CUDA kernels; torch is used here for device memory and
+streams.  There is no CPU fallback: if a shared object is missing or CUDA is unavailable the import of the library
+(``load()``) raises.
 """
 from __future__ import annotations
 
@@ -14,6 +16,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libvispec.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 VISPEC_OK = 0
 STATUS_NAMES = {
@@ -48,15 +51,17 @@ class VispecError(RuntimeError):
 
 
 _lib: Optional[ctypes.CDLL] = None
+_native = None
 
 
 def load() -> ctypes.CDLL:
     """dlopen the in-tree library.  Fails loudly when it has not been built."""
-    global _lib
+    global _lib, _native
     if _lib is None:
-        if not os.path.exists(LIB_PATH):
-            raise ImportError(f"{LIB_PATH} is missing: run `python -m paper_2509_15235_b200.build` "
-                              "(there is no fallback path)")
+        for path in (LIB_PATH, NATIVE_PATH):
+            if not os.path.exists(path):
+                raise ImportError(f"{path} is missing: run `python -m paper_2509_15235_b200.build` "
+                                  "(there is no fallback path)")
         lib = ctypes.CDLL(LIB_PATH)
         vp, ci, cf = ctypes.c_void_p, ctypes.c_int, ctypes.c_float
         lib.vispec_strerror.restype = ctypes.c_char_p
@@ -94,6 +99,8 @@ def load() -> ctypes.CDLL:
             fn = getattr(lib, name)
             fn.restype = ci
             fn.argtypes = argtypes
+        from . import _native as native
+        _native = native
         _lib = lib
     return _lib
 
@@ -124,11 +131,9 @@ def tree_verify_attn_static(q: torch.Tensor, k_cache: torch.Tensor, v_cache: tor
     """vispec_tree_verify_attn_static: the attention for callers that cannot allocate device memory
     (no context, no workspace; scratch is a fixed array inside the library).  One C call on torch's
     current stream; raises VispecError(VISPEC_E_WORKSPACE) when the problem exceeds the built-in scratch."""
-    B, N, Hq, D = q.shape
-    _, Hkv, S_max, _ = k_cache.shape
-    _check(load().vispec_tree_verify_attn_static(_ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(kv_len),
-                                                 _ptr(tree_mask), B, N, Hq, Hkv, D, S_max, ctypes.c_float(scale),
-                                                 _ptr(out), _ptr(lse), _ptr(status_word), _stream()),
+    if _native is None:
+        load()
+    _check(_native.tree_verify_attn_static(q, k_cache, v_cache, kv_len, tree_mask, scale, out, lse, status_word),
            "vispec_tree_verify_attn_static")
 
 
@@ -148,6 +153,7 @@ class VerifyContext:
         h = ctypes.c_void_p()
         _check(self.lib.vispec_ctx_create(ctypes.byref(h), ctypes.byref(self.shape), device), "vispec_ctx_create")
         self.handle = h
+        self._h = h.value or 0          # the handle as the native calls take it
         n = ctypes.c_size_t()
         _check(self.lib.vispec_workspace_bytes(self.handle, ctypes.byref(n)), "vispec_workspace_bytes")
         self.workspace = torch.empty(n.value, dtype=torch.uint8, device=self.device)
@@ -159,6 +165,7 @@ class VerifyContext:
         if getattr(self, "handle", None):
             self.lib.vispec_ctx_destroy(self.handle)
             self.handle = None
+            self._h = 0
 
     def __del__(self):
         try:
@@ -178,53 +185,42 @@ class VerifyContext:
     # -- hot calls --------------------------------------------------------------------------------
     def tree_mask_build(self, parents: torch.Tensor, tree_mask: torch.Tensor,
                         depth: Optional[torch.Tensor] = None) -> None:
-        B, N = parents.shape
-        _check(self.lib.vispec_tree_mask_build(self.handle, _ptr(parents), B, N, _ptr(tree_mask), _ptr(depth),
-                                               _stream()), "vispec_tree_mask_build")
+        _check(_native.tree_mask_build(self._h, parents, tree_mask, depth), "vispec_tree_mask_build")
 
     def tree_verify_attn(self, layer: int, q: torch.Tensor, kv_len: torch.Tensor, tree_mask: torch.Tensor,
                          scale: float, out: torch.Tensor, lse: Optional[torch.Tensor] = None,
                          positions: Optional[torch.Tensor] = None, k_cache: Optional[torch.Tensor] = None,
                          v_cache: Optional[torch.Tensor] = None) -> None:
-        B, N = q.shape[0], q.shape[1]
-        _check(self.lib.vispec_tree_verify_attn(self.handle, layer, _ptr(q), _ptr(k_cache), _ptr(v_cache),
-                                                _ptr(kv_len), _ptr(tree_mask), _ptr(positions), B, N,
-                                                ctypes.c_float(scale), _ptr(out), _ptr(lse), _stream()),
+        _check(_native.tree_verify_attn(self._h, layer, q, k_cache, v_cache, kv_len, tree_mask, positions, scale, out,
+                                        lse),
                "vispec_tree_verify_attn")
 
     def accept(self, draft_ids: torch.Tensor, target_ids: torch.Tensor, parents: torch.Tensor,
                path: torch.Tensor, accept_len: torch.Tensor, bonus: torch.Tensor) -> None:
-        B, N = parents.shape
-        _check(self.lib.vispec_accept(self.handle, _ptr(draft_ids), _ptr(target_ids), _ptr(parents), B, N,
-                                      _ptr(path), _ptr(accept_len), _ptr(bonus), _stream()), "vispec_accept")
+        _check(_native.accept(self._h, draft_ids, target_ids, parents, path, accept_len, bonus), "vispec_accept")
 
     def kv_compact(self, layer_begin: int, layer_end: int, path: torch.Tensor, accept_len: torch.Tensor,
                    kv_len: torch.Tensor, kv_len_out: Optional[torch.Tensor] = None) -> None:
-        B, N = path.shape
-        _check(self.lib.vispec_kv_compact(self.handle, layer_begin, layer_end, _ptr(path), _ptr(accept_len),
-                                          _ptr(kv_len), _ptr(kv_len_out), B, N, _stream()), "vispec_kv_compact")
+        _check(_native.kv_compact(self._h, layer_begin, layer_end, path, accept_len, kv_len, kv_len_out),
+               "vispec_kv_compact")
 
     def accept_commit(self, layer_begin: int, layer_end: int, draft_ids: torch.Tensor, target_ids: torch.Tensor,
                       parents: torch.Tensor, kv_len: torch.Tensor, path: torch.Tensor, accept_len: torch.Tensor,
                       bonus: torch.Tensor, kv_len_out: Optional[torch.Tensor] = None) -> None:
-        B, N = parents.shape
-        _check(self.lib.vispec_accept_commit(self.handle, layer_begin, layer_end, _ptr(draft_ids), _ptr(target_ids),
-                                             _ptr(parents), _ptr(kv_len), B, N, _ptr(path), _ptr(accept_len),
-                                             _ptr(bonus), _ptr(kv_len_out), _stream()), "vispec_accept_commit")
+        _check(_native.accept_commit(self._h, layer_begin, layer_end, draft_ids, target_ids, parents, kv_len, path,
+                                     accept_len, bonus, kv_len_out),
+               "vispec_accept_commit")
 
     def accept_sampled(self, draft_ids: torch.Tensor, parents: torch.Tensor, p_target: torch.Tensor,
                        p_draft: torch.Tensor, u_accept: torch.Tensor, u_bonus: torch.Tensor, path: torch.Tensor,
                        accept_len: torch.Tensor, bonus: torch.Tensor) -> None:
-        B, N, V = p_target.shape
-        _check(self.lib.vispec_accept_sampled(self.handle, _ptr(draft_ids), _ptr(parents), _ptr(p_target), _ptr(p_draft),
-                                              _ptr(u_accept), _ptr(u_bonus), B, N, V, _ptr(path), _ptr(accept_len),
-                                              _ptr(bonus), _stream()), "vispec_accept_sampled")
+        _check(_native.accept_sampled(self._h, draft_ids, parents, p_target, p_draft, u_accept, u_bonus, path,
+                                      accept_len, bonus),
+               "vispec_accept_sampled")
 
     def tree_rerank(self, cand_parent: torch.Tensor, cand_token: torch.Tensor, cand_score: torch.Tensor, K: int,
                     parents: torch.Tensor, draft_ids: torch.Tensor, selected: Optional[torch.Tensor]) -> None:
-        B, M = cand_parent.shape
-        _check(self.lib.vispec_tree_rerank(self.handle, _ptr(cand_parent), _ptr(cand_token), _ptr(cand_score), B, M, K,
-                                           _ptr(parents), _ptr(draft_ids), _ptr(selected), _stream()),
+        _check(_native.tree_rerank(self._h, cand_parent, cand_token, cand_score, K, parents, draft_ids, selected),
                "vispec_tree_rerank")
 
     def cache_register_paged(self, layer: int, k_pool: torch.Tensor, v_pool: torch.Tensor,
@@ -238,40 +234,31 @@ class VerifyContext:
     def tree_verify_attn_paged(self, layer: int, q: torch.Tensor, kv_len: torch.Tensor, block_table: torch.Tensor,
                                tree_mask: torch.Tensor, scale: float, out: torch.Tensor,
                                lse: Optional[torch.Tensor] = None) -> None:
-        B, N = q.shape[0], q.shape[1]
-        _check(self.lib.vispec_tree_verify_attn_paged(self.handle, layer, _ptr(q), _ptr(kv_len), _ptr(block_table),
-                                                      block_table.shape[1], _ptr(tree_mask), B, N, ctypes.c_float(scale),
-                                                      _ptr(out), _ptr(lse), _stream()), "vispec_tree_verify_attn_paged")
+        _check(_native.tree_verify_attn_paged(self._h, layer, q, kv_len, block_table, tree_mask, scale, out, lse),
+               "vispec_tree_verify_attn_paged")
 
     def kv_compact_paged(self, layer_begin: int, layer_end: int, path: torch.Tensor, accept_len: torch.Tensor,
                          kv_len: torch.Tensor, block_table: torch.Tensor, kv_len_out: Optional[torch.Tensor]) -> None:
-        B, N = path.shape
-        _check(self.lib.vispec_kv_compact_paged(self.handle, layer_begin, layer_end, _ptr(path), _ptr(accept_len),
-                                                _ptr(kv_len), _ptr(block_table), block_table.shape[1], _ptr(kv_len_out),
-                                                B, N, _stream()), "vispec_kv_compact_paged")
+        _check(_native.kv_compact_paged(self._h, layer_begin, layer_end, path, accept_len, kv_len, block_table,
+                                        kv_len_out),
+               "vispec_kv_compact_paged")
 
     def accept_commit_paged(self, layer_begin: int, layer_end: int, draft_ids: torch.Tensor, target_ids: torch.Tensor,
                             parents: torch.Tensor, kv_len: torch.Tensor, block_table: torch.Tensor, path: torch.Tensor,
                             accept_len: torch.Tensor, bonus: torch.Tensor, kv_len_out: Optional[torch.Tensor]) -> None:
-        B, N = parents.shape
-        _check(self.lib.vispec_accept_commit_paged(self.handle, layer_begin, layer_end, _ptr(draft_ids), _ptr(target_ids),
-                                                   _ptr(parents), _ptr(kv_len), _ptr(block_table), block_table.shape[1],
-                                                   B, N, _ptr(path), _ptr(accept_len), _ptr(bonus), _ptr(kv_len_out),
-                                                   _stream()), "vispec_accept_commit_paged")
+        _check(_native.accept_commit_paged(self._h, layer_begin, layer_end, draft_ids, target_ids, parents, kv_len,
+                                           block_table, path, accept_len, bonus, kv_len_out),
+               "vispec_accept_commit_paged")
 
     def rope_tree_rows_paged(self, layer: int, q: torch.Tensor, k_new: torch.Tensor, v_new: torch.Tensor,
                              positions: torch.Tensor, kv_len: torch.Tensor, block_table: torch.Tensor,
                              theta: float) -> None:
-        B, N = positions.shape
-        _check(self.lib.vispec_rope_tree_rows_paged(self.handle, layer, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(positions),
-                                                    _ptr(kv_len), _ptr(block_table), block_table.shape[1], B, N,
-                                                    ctypes.c_float(theta), _stream()), "vispec_rope_tree_rows_paged")
+        _check(_native.rope_tree_rows_paged(self._h, layer, q, k_new, v_new, positions, kv_len, block_table, theta),
+               "vispec_rope_tree_rows_paged")
 
     def rope_tree_rows(self, layer: int, q: torch.Tensor, k_new: torch.Tensor, v_new: torch.Tensor,
                        positions: torch.Tensor, kv_len: torch.Tensor, theta: float) -> None:
-        B, N = positions.shape
-        _check(self.lib.vispec_rope_tree_rows(self.handle, layer, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(positions),
-                                              _ptr(kv_len), B, N, ctypes.c_float(theta), _stream()),
+        _check(_native.rope_tree_rows(self._h, layer, q, k_new, v_new, positions, kv_len, theta),
                "vispec_rope_tree_rows")
 
     def rope_table_build(self, positions: torch.Tensor, theta: float, table: Optional[torch.Tensor] = None) -> torch.Tensor:
@@ -281,17 +268,15 @@ class VerifyContext:
             n = ctypes.c_size_t()
             _check(self.lib.vispec_rope_table_bytes(self.handle, B, N, ctypes.byref(n)), "vispec_rope_table_bytes")
             table = torch.empty(max(n.value, 16), dtype=torch.uint8, device=self.device)
-        _check(self.lib.vispec_rope_table_build(self.handle, _ptr(positions), B, N, ctypes.c_float(theta), _ptr(table),
-                                                _stream()), "vispec_rope_table_build")
+        _check(_native.rope_table_build(self._h, positions, theta, table), "vispec_rope_table_build")
         return table
 
     def tree_verify_attn_rope(self, layer: int, q: torch.Tensor, k_new: torch.Tensor, v_new: torch.Tensor,
                               rope_table: torch.Tensor, kv_len: torch.Tensor, tree_mask: torch.Tensor, scale: float,
                               out: torch.Tensor, lse: Optional[torch.Tensor] = None) -> None:
-        B, N = q.shape[0], q.shape[1]
-        _check(self.lib.vispec_tree_verify_attn_rope(self.handle, layer, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(rope_table),
-                                                     _ptr(kv_len), _ptr(tree_mask), B, N, ctypes.c_float(scale), _ptr(out),
-                                                     _ptr(lse), _stream()), "vispec_tree_verify_attn_rope")
+        _check(_native.tree_verify_attn_rope(self._h, layer, q, k_new, v_new, rope_table, kv_len, tree_mask, scale, out,
+                                             lse),
+               "vispec_tree_verify_attn_rope")
 
     def stream_probe(self, layer: int, kv_len: torch.Tensor, N: int) -> None:
         _check(self.lib.vispec_stream_probe(self.handle, layer, _ptr(kv_len), kv_len.shape[0], N, _stream()),
