@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 
+#include "launch.cuh"
 #include "vispec_internal.h"
 
 namespace vispec {
@@ -126,9 +127,6 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 __device__ __forceinline__ void mbar_arrive_peer(uint32_t peer_bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_bar) : "memory");
 }
-// Programmatic dependent launch: let the next kernel in the stream be scheduled / wait for the previous one.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // One tcgen05.mma (cta_group::1, kind::f16) with the A operand in TMEM and B described in shared memory.
 // The 64-bit descriptor is passed as 32-bit halves: the high half is constant, the low half carries the address.
 __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi,
@@ -506,24 +504,6 @@ attn_tc5_merge_kernel(const Tc5Params p) {
 
     if (FINE) merge_row_c4<ROWS>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
     else merge_row_cols<ROWS>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
-}
-
-// Launch with programmatic stream serialisation and, when cluster > 0, thread-block clusters of that size.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 1;
-    if (cluster > 0) {
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-        cfg.numAttrs = 2;
-    }
-    cfg.attrs = attr;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 }  // namespace tc5

@@ -1,7 +1,15 @@
 // Integer kernels of the verification step: ancestor mask, greedy acceptance, KV commit.
 // All three are latency-bound (a few KB of traffic); each is a single launch.
+//
+// What bounds them is the chain launch -> first load -> dependent load -> store, so (a) every kernel is launched with
+// programmatic stream serialisation (its blocks are resident and past their set-up when the predecessor ends; every
+// read and write comes after griddepcontrol.wait), and (b) loads that do not depend on one another go out together.
+// Only a kernel that has waited for its predecessor lets its successor in early (tree_mask_kernel, rope_rows_kernel,
+// rope_table_kernel): an attention call that follows reads kv_len and committed rows before its own wait.  The commits
+// never do: what follows them starts when they have ended.
 #include <cuda_bf16.h>
 
+#include "launch.cuh"
 #include "vispec_internal.h"
 
 namespace vispec {
@@ -20,6 +28,8 @@ tree_mask_kernel(const int32_t* __restrict__ parents, int N, uint64_t* __restric
                  int32_t* __restrict__ depth, int* status) {
     __shared__ int32_t par[VISPEC_MAX_TREE_NODES];
     const int b = blockIdx.x, i = threadIdx.x;
+    pdl_wait();
+    pdl_launch_dependents();
     if (i < N) par[i] = parents[(size_t)b * N + i];
     __syncthreads();
     if (i >= N) return;
@@ -50,8 +60,7 @@ tree_mask_kernel(const int32_t* __restrict__ parents, int N, uint64_t* __restric
 cudaError_t launch_tree_mask(const int32_t* parents, int B, int N, uint64_t* mask, int32_t* depth,
                              int* status, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    tree_mask_kernel<<<B, 128, 0, st>>>(parents, N, mask, depth, status);
-    return cudaGetLastError();
+    return launch_pdl(tree_mask_kernel, dim3(B), dim3(128), 0, st, 0, parents, N, mask, depth, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -67,6 +76,9 @@ cudaError_t launch_tree_mask(const int32_t* parents, int B, int N, uint64_t* mas
 __device__ int accept_warp(const int32_t* __restrict__ draft_row, const int32_t* par, const int32_t* tgt, int N,
                            int32_t* path_out, int32_t* bonus_out, int* status) {
     const int lane = threadIdx.x & 31;
+    int32_t mine[4];                             // the lane's drafted tokens, fetched ahead of the validity vote
+#pragma unroll
+    for (int w = 0; w < 4; ++w) mine[w] = w * 32 + lane < N ? draft_row[w * 32 + lane] : 0;
     // validity of the whole tree (every link must point to an earlier node)
     bool tree_ok = true;
     for (int i = lane; i < N; i += 32) tree_ok &= (i == 0) ? (par[0] == -1) : (par[i] >= 0 && par[i] < i);
@@ -77,7 +89,7 @@ __device__ int accept_warp(const int32_t* __restrict__ draft_row, const int32_t*
     for (int w = 0; w < 4; ++w) {
         const int i = w * 32 + lane;
         bool m = false;
-        if (tree_ok && i < N) m = (i == 0) || (draft_row[i] == tgt[par[i]]);
+        if (tree_ok && i < N) m = (i == 0) || (mine[w] == tgt[par[i]]);
         matched[w] = __ballot_sync(0xffffffffu, m);
     }
     int best_key = -1;
@@ -118,6 +130,7 @@ accept_kernel(const int32_t* __restrict__ draft, const int32_t* __restrict__ tar
     __shared__ int32_t tgt[VISPEC_MAX_TREE_NODES];
     const int b = blockIdx.x, lane = threadIdx.x;
     const size_t base = (size_t)b * N;
+    pdl_wait();
     for (int i = lane; i < N; i += 32) { par[i] = parents[base + i]; tgt[i] = target[base + i]; }
     __syncwarp();
     const int len = accept_warp(draft + base, par, tgt, N, path + base, bonus + b, status);
@@ -128,8 +141,7 @@ cudaError_t launch_accept(const int32_t* draft, const int32_t* target, const int
                           int N, int32_t* path, int32_t* accept_len, int32_t* bonus, int* status,
                           cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    accept_kernel<<<B, 32, 0, st>>>(draft, target, parents, N, path, accept_len, bonus, status);
-    return cudaGetLastError();
+    return launch_pdl(accept_kernel, dim3(B), dim3(32), 0, st, 0, draft, target, parents, N, path, accept_len, bonus, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -165,7 +177,10 @@ kv_compact_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, const i
     __shared__ uint4 stage[2][kCompactRows][16];   // up to 256 B per row (D = 128)
     __shared__ int32_t src_row[kCompactRows];
     const int layer = layer_begin + blockIdx.z, b = blockIdx.y, h = blockIdx.x;
+    pdl_wait();
     const int S = kv_len[b], L = accept_len[b];
+    // the first pass's entry, fetched beside the two lengths (path rows are N long whatever the length says)
+    int first = threadIdx.x < kCompactRows && (int)threadIdx.x < N ? path[(size_t)b * N + threadIdx.x] : -1;
     const bool ok = (L >= 1 && L <= N && S >= 0 && S + N <= S_max);
     if (!ok) {
         if (threadIdx.x == 0) record_status(status, VISPEC_E_RANGE);
@@ -187,7 +202,7 @@ kv_compact_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, const i
     for (int k0 = 0; k0 < L; k0 += kCompactRows) {
         if (threadIdx.x < kCompactRows) {
             const int k = k0 + threadIdx.x;
-            int s = (k < L) ? path[(size_t)b * N + k] : -1;
+            int s = (k < L) ? (k0 == 0 ? first : path[(size_t)b * N + k]) : -1;
             if (k < L && (s < k || s >= N)) { s = -1; bad = true; }
             src_row[threadIdx.x] = (s == k) ? -1 : s;   // -1: nothing to move
         }
@@ -218,10 +233,8 @@ cudaError_t launch_kv_compact(void* const* cache_ptrs, int layer_begin, int laye
                               int num_blocks, int token_major) {
     if (B == 0 || layer_end <= layer_begin) return cudaSuccess;
     dim3 grid(Hkv, B, layer_end - layer_begin);
-    kv_compact_kernel<<<grid, 256, 0, st>>>(cache_ptrs, layer_begin, path, accept_len, kv_len, kv_len_out,
-                                            N, Hkv, D, S_max, status, block_table, table_stride, page_rows, num_blocks,
-                                            token_major);
-    return cudaGetLastError();
+    return launch_pdl(kv_compact_kernel, grid, dim3(256), 0, st, 0, cache_ptrs, layer_begin, path, accept_len, kv_len,
+                      kv_len_out, N, Hkv, D, S_max, status, block_table, table_stride, page_rows, num_blocks, token_major);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -244,6 +257,8 @@ accept_commit_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, cons
     __shared__ int32_t s_len, s_bonus;
     const int layer = layer_begin + blockIdx.z, b = blockIdx.y, h = blockIdx.x;
     const size_t rb = (size_t)b * N;
+    pdl_wait();
+    const int S = kv_len[b];
     for (int i = threadIdx.x; i < N; i += 256) { par[i] = parents[rb + i]; tgt[i] = target[rb + i]; }
     __syncthreads();
     const bool writer = (blockIdx.x == 0 && blockIdx.z == 0);
@@ -252,7 +267,7 @@ accept_commit_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, cons
         if (threadIdx.x == 0) s_len = len;
     }
     __syncthreads();
-    const int S = kv_len[b], L = s_len;
+    const int L = s_len;
     if (writer) {
         for (int i = threadIdx.x; i < N; i += 256) path[rb + i] = spath[i];
         if (threadIdx.x == 0) { accept_len[b] = L; bonus[b] = s_bonus; }
@@ -300,9 +315,8 @@ cudaError_t launch_accept_commit(void* const* cache_ptrs, int layer_begin, int l
     if (B == 0 || layer_end <= layer_begin) return cudaSuccess;
     dim3 grid(Hkv, B, layer_end - layer_begin);
     const RowMap rows = {block_table, table_stride, page_rows, num_blocks, token_major};
-    accept_commit_kernel<<<grid, 256, 0, st>>>(cache_ptrs, layer_begin, draft, target, parents, kv_len, path,
-                                               accept_len, bonus, kv_len_out, N, Hkv, D, S_max, status, rows);
-    return cudaGetLastError();
+    return launch_pdl(accept_commit_kernel, grid, dim3(256), 0, st, 0, cache_ptrs, layer_begin, draft, target, parents, kv_len,
+                      path, accept_len, bonus, kv_len_out, N, Hkv, D, S_max, status, rows);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -338,8 +352,8 @@ rope_rows_kernel(__nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict_
     // the next kernel in: an attention call that follows reads kv_len and committed cache rows before its own wait,
     // and must not do so while the kernel two places back (a commit, say) is still running.  Its prologue still
     // overlaps these blocks; this kernel writes only q and slots at or above kv_len.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_launch_dependents();
     const int i = blockIdx.x, b = blockIdx.y, half = D / 2;
     const int S = kv_len[b];
     if (S < 0 || S + N > S_max) {
@@ -394,6 +408,8 @@ namespace {
 __global__ void rope_table_kernel(const int32_t* __restrict__ positions, double log2_theta, int N, int D,
                                   double2* __restrict__ tab64, float2* __restrict__ tab32) {
     const int i = blockIdx.x, b = blockIdx.y, j = threadIdx.x;
+    pdl_wait();
+    pdl_launch_dependents();
     if (j >= D / 2) return;
     const double ang = (double)positions[(size_t)b * N + i] * exp2(-2.0 * (double)j / (double)D * log2_theta);
     double s_, c_;
@@ -408,8 +424,7 @@ cudaError_t launch_rope_table(const int32_t* positions, int B, int N, int D, flo
     if (B * N == 0) return cudaSuccess;
     double2* t64 = (double2*)table;
     float2* t32 = (float2*)(t64 + (size_t)B * N * (D / 2));
-    rope_table_kernel<<<dim3(N, B), D / 2, 0, st>>>(positions, log2((double)theta), N, D, t64, t32);
-    return cudaGetLastError();
+    return launch_pdl(rope_table_kernel, dim3(N, B), dim3(D / 2), 0, st, 0, positions, log2((double)theta), N, D, t64, t32);
 }
 
 namespace {
@@ -440,88 +455,99 @@ cudaError_t launch_rope_rows(void* q, const void* k_new, const void* v_new, cons
                              const void* angle_table) {
     if (B == 0) return cudaSuccess;
     const RowMap rmap = {block_table, table_stride, page_rows, num_blocks, token_major};
-    cudaLaunchConfig_t cfg = {};
     const int rows_per_block = 128 / (D / 16);
-    cfg.gridDim = dim3(N, B, (Hq + 2 * Hkv + rows_per_block - 1) / rows_per_block);
-    cfg.blockDim = dim3(128);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rope_rows_kernel, (__nv_bfloat16*)q, (const __nv_bfloat16*)k_new,
-                              (const __nv_bfloat16*)v_new, positions, kv_len, (__nv_bfloat16*)k_cache,
-                              (__nv_bfloat16*)v_cache, angle_table ? 0.0 : log2((double)theta), N, Hq, Hkv, D, S_max, status,
-                              rmap, (__nv_bfloat16*)(q_out ? q_out : q), (const double2*)angle_table);
+    return launch_pdl(rope_rows_kernel, dim3(N, B, (Hq + 2 * Hkv + rows_per_block - 1) / rows_per_block), dim3(128), 0, st, 0,
+                      (__nv_bfloat16*)q, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, positions, kv_len,
+                      (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, angle_table ? 0.0 : log2((double)theta), N, Hq, Hkv, D,
+                      S_max, status, rmap, (__nv_bfloat16*)(q_out ? q_out : q), (const double2*)angle_table);
 }
 
 // ------------------------------------------------------------------------------------------------
 // Tree rerank (App. A: 30 draft tokens kept from a depth-3, width-8 expansion; the tree is EAGLE-2's, which
-// keeps the candidates of highest cumulative log-probability).  One block per sequence.  Scores become
-// order-preserving 32-bit keys (NaN lowest); a candidate's rank is the number of candidates ahead of it
-// (higher key, or equal key and lower index), counted against the keys in shared memory: M^2 compares,
-// 18 K for the paper's 136 candidates.  Kept candidates are numbered in candidate order, which keeps
-// parents ahead of children.
+// keeps the candidates of highest cumulative log-probability).  One block per sequence, one or two candidates per
+// thread, everything a thread needs of them fetched at once.  Scores become order-preserving 32-bit keys (NaN lowest).
+// The K-th largest key is found bit by bit from the top: a bit stays set if at least K keys reach the value so far, one
+// barrier with a count per bit; the keys above it are kept, and of those equal to it the lowest indices.  Kept
+// candidates are numbered in candidate order, which keeps parents ahead of children.
+// 32 counts of M keys instead of M^2 compares; at 136 candidates it is the load, 32 short barriers and the store.
+// Rerank + mask build, us per pass, M^2 compares -> this: 136 candidates 4.5 -> 3.7, 1020 43.4 -> 7.2, 1808 136 -> 12.2.
 // ------------------------------------------------------------------------------------------------
 constexpr int kRerankMaxM = 2048;
 
-__global__ void __launch_bounds__(256)
+template <int IT>      // candidates per thread
+__global__ void __launch_bounds__(1024)
 tree_rerank_kernel(const int32_t* __restrict__ cand_parent, const int32_t* __restrict__ cand_token,
                    const float* __restrict__ cand_score, int M, int K, int32_t* __restrict__ parents,
                    int32_t* __restrict__ draft_ids, int32_t* __restrict__ selected, int* status) {
-    __shared__ uint32_t key[kRerankMaxM];
     __shared__ int16_t node[kRerankMaxM];        // node number of a kept candidate, 0 if dropped
-    __shared__ int warp_cnt[8];
-    __shared__ int sh_bad;
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int32_t* cp = cand_parent + (size_t)b * M;
-    if (tid == 0) sh_bad = 0;
-    for (int i = tid; i < M; i += 256) {
-        const float s = cand_score[(size_t)b * M + i];
-        const uint32_t u = __float_as_uint(s);
-        // ascending float order -> ascending unsigned order; -0 and +0 made equal; NaN below everything
-        uint32_t k = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-        if (s == 0.0f) k = 0x80000000u;
-        if (s != s) k = 0u;
-        key[i] = k;
-    }
-    __syncthreads();
-    // pass over the candidates in chunks of 256 (in index order) so that the node numbers can be handed out
-    // by a block-wide prefix count
-    int base = 0;
-    for (int i0 = 0; i0 < M; i0 += 256) {
-        const int i = i0 + tid;
-        bool keep = false;
-        if (i < M) {
-            const uint32_t ki = key[i];
-            int ahead = 0;
-            for (int j = 0; j < M; ++j) {
-                const uint32_t kj = key[j];
-                ahead += (kj > ki) || (kj == ki && j < i);
-            }
-            keep = ahead < K;
-            const int pr = cp[i];
-            if (pr < -1 || pr >= i) sh_bad = 1;
+    __shared__ int warp_cnt[2][32];              // per warp: keys equal to the K-th largest / kept candidates
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+    const unsigned below = (1u << lane) - 1;
+    pdl_wait();
+    pdl_launch_dependents();
+    // candidates tid and tid + nt: index order is (pass, thread)
+    uint32_t key[IT];
+    int pr[IT], tok[IT];
+    bool there[IT], bad = false;
+#pragma unroll
+    for (int t = 0; t < IT; ++t) {
+        const int i = tid + t * nt;
+        there[t] = i < M;
+        key[t] = 0u; pr[t] = -1; tok[t] = 0;
+        if (there[t]) {
+            const float s = cand_score[(size_t)b * M + i];
+            pr[t] = cand_parent[(size_t)b * M + i];
+            tok[t] = cand_token[(size_t)b * M + i];
+            const uint32_t u = __float_as_uint(s);
+            // ascending float order -> ascending unsigned order; -0 and +0 made equal; NaN below everything
+            key[t] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+            if (s == 0.0f) key[t] = 0x80000000u;
+            if (s != s) key[t] = 0u;
+            bad |= pr[t] < -1 || pr[t] >= i;
         }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) warp_cnt[w] = __popc(m);
-        __syncthreads();
-        int before = base + __popc(m & ((1u << lane) - 1));
-        for (int x = 0; x < w; ++x) before += warp_cnt[x];
-        int total = 0;
-        for (int x = 0; x < 8; ++x) total += warp_cnt[x];
-        if (i < M) node[i] = keep ? (int16_t)(before + 1) : (int16_t)0;
-        base += total;
-        __syncthreads();
     }
-    // a kept candidate whose parent was dropped breaks the tree
-    for (int i = tid; i < M; i += 256) {
-        const int pr = cp[i];
-        if (node[i] && pr >= 0 && pr < i && !node[pr]) sh_bad = 1;
+    // the largest T that at least K keys reach: the K-th largest key
+    uint32_t T = 0;
+    for (int bit = 31; bit >= 0 && K > 0; --bit) {
+        const uint32_t cand = T | (1u << bit);
+        int n = __syncthreads_count(key[0] >= cand);           // (cand > 0: a slot without a candidate never counts)
+        if (IT > 1) n += __syncthreads_count(key[IT - 1] >= cand);
+        if (n >= K) T = cand;
+    }
+    int above = __syncthreads_count(there[0] && key[0] > T);
+    if (IT > 1) above += __syncthreads_count(there[IT - 1] && key[IT - 1] > T);
+    int eq_base = 0, kept_base = 0;
+    bool keep[IT];
+    int number[IT];
+#pragma unroll
+    for (int t = 0; t < IT; ++t) {
+        const bool eq = there[t] && key[t] == T;
+        const unsigned em = __ballot_sync(0xffffffffu, eq);
+        if (lane == 0) warp_cnt[0][w] = __popc(em);
+        __syncthreads();
+        int eq_before = eq_base + __popc(em & below);
+        for (int x = 0; x < nw; ++x) { const int c = warp_cnt[0][x]; eq_before += x < w ? c : 0; eq_base += c; }
+        keep[t] = K > 0 && there[t] && (key[t] > T || (eq && eq_before < K - above));
+        const unsigned km = __ballot_sync(0xffffffffu, keep[t]);
+        if (lane == 0) warp_cnt[1][w] = __popc(km);
+        __syncthreads();
+        int before = kept_base + __popc(km & below);
+        for (int x = 0; x < nw; ++x) { const int c = warp_cnt[1][x]; before += x < w ? c : 0; kept_base += c; }
+        number[t] = keep[t] ? before + 1 : 0;
+        if (there[t]) node[tid + t * nt] = (int16_t)number[t];
     }
     __syncthreads();
-    const bool bad = sh_bad != 0;
+    // a kept candidate whose parent was dropped breaks the tree
+    int parent_node[IT];
+#pragma unroll
+    for (int t = 0; t < IT; ++t) {
+        parent_node[t] = 0;
+        if (keep[t] && pr[t] >= 0 && pr[t] < tid + t * nt) {
+            parent_node[t] = node[pr[t]];
+            bad |= parent_node[t] == 0;
+        }
+    }
+    bad = __syncthreads_or(bad);
     int32_t* po = parents + (size_t)b * (K + 1);
     int32_t* io = draft_ids + (size_t)b * (K + 1);
     if (tid == 0) {
@@ -529,13 +555,13 @@ tree_rerank_kernel(const int32_t* __restrict__ cand_parent, const int32_t* __res
         io[0] = 0;
         if (bad) record_status(status, VISPEC_E_BAD_TREE);
     }
-    for (int i = tid; i < M; i += 256) {
-        const int n = node[i];
-        if (!n) continue;
-        selected[(size_t)b * K + n - 1] = i;
-        io[n] = cand_token[(size_t)b * M + i];
-        const int pr = cp[i];
-        po[n] = bad ? -1 : (pr == -1 ? 0 : (int)node[pr]);
+#pragma unroll
+    for (int t = 0; t < IT; ++t) {
+        if (!keep[t]) continue;
+        const int n = number[t];
+        selected[(size_t)b * K + n - 1] = tid + t * nt;
+        io[n] = tok[t];
+        po[n] = bad ? -1 : parent_node[t];
     }
 }
 
@@ -543,8 +569,13 @@ cudaError_t launch_tree_rerank(const int32_t* cand_parent, const int32_t* cand_t
                                int M, int K, int32_t* parents, int32_t* draft_ids, int32_t* selected, int* status,
                                cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    tree_rerank_kernel<<<B, 256, 0, st>>>(cand_parent, cand_token, cand_score, M, K, parents, draft_ids, selected, status);
-    return cudaGetLastError();
+    // one thread per candidate up to a block's 1024, two beyond
+    const int threads = M > 1024 ? 1024 : (M + 31) / 32 * 32;
+    if (M > 1024)
+        return launch_pdl(tree_rerank_kernel<2>, dim3(B), dim3(threads), 0, st, 0, cand_parent, cand_token, cand_score, M, K,
+                          parents, draft_ids, selected, status);
+    return launch_pdl(tree_rerank_kernel<1>, dim3(B), dim3(threads), 0, st, 0, cand_parent, cand_token, cand_score, M, K,
+                      parents, draft_ids, selected, status);
 }
 
 }  // namespace vispec
