@@ -1,6 +1,7 @@
 // C ABI of libvispec: context management, argument validation, dispatch to the kernels.
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include <nvtx3/nvToolsExt.h>
@@ -55,6 +56,19 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 
+// Kernel attributes and occupancy answers are a device's, not a context's: found once (context creation goes through
+// here with the device current; a failed attempt is made again).
+bool init_device(int device) {
+    static std::mutex mu;
+    static bool done[64];
+    std::lock_guard<std::mutex> lock(mu);
+    if (device < 64 && done[device]) return true;
+    const bool ok = init_attn_generic() == cudaSuccess && init_attn_tc5() == cudaSuccess && init_stream_probe() == cudaSuccess &&
+                    init_accept_sampled(device) == cudaSuccess;
+    if (device < 64) done[device] = ok;
+    return ok;
+}
+
 }  // namespace
 
 extern "C" {
@@ -96,9 +110,7 @@ int vispec_ctx_create(vispec_ctx** out, const vispec_shape* s, int device) {
     ok = ok && cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_cache_ptrs, sizeof(void*) * 2 * s->layers) == cudaSuccess;
     ok = ok && cudaMemset(c->d_cache_ptrs, 0, sizeof(void*) * 2 * s->layers) == cudaSuccess;
-    ok = ok && init_attn_generic() == cudaSuccess;
-    ok = ok && init_attn_tc5() == cudaSuccess;
-    ok = ok && init_stream_probe() == cudaSuccess;
+    ok = ok && init_device(device);
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) { vispec_ctx_destroy(c); return VISPEC_E_CUDA; }
     c->h_k.assign(s->layers, nullptr);

@@ -67,6 +67,7 @@ cudaError_t launch_rope_rows(void* q, const void* k_new, const void* v_new, cons
 // (q_out: where the rotated q rows go, q itself when null; angle_table: the fp64 half of a vispec_rope_table_build
 // table to take cosines and sines from instead of forming them from positions and theta)
 
+cudaError_t init_accept_sampled(int device);   // with that device current
 cudaError_t launch_accept_sampled(const int32_t* draft_ids, const int32_t* parents, const float* p, const float* p_hat,
                                   const float* u_accept, const float* u_bonus, int B, int N, int V, int32_t* path,
                                   int32_t* accept_len, int32_t* bonus, int* status, cudaStream_t st);
