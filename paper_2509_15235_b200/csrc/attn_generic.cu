@@ -1,8 +1,8 @@
 // Generic split-KV tree-verification attention (Eq. 1 restricted to prefix + ancestors) on
 // warp-level tensor-core instructions (mma.sync m16n8k16, bf16 in, fp32 accumulate).
 //
-// It serves every supported shape (D = 64 or 128, any G, N <= 128) and is the path for shapes the
-// TMA/tcgen05 kernel does not take.  Work unit: (sequence b, kv head, block of 64 query rows,
+// It serves every supported shape (D = 64 or 128, any G, N <= 128) and is the path for calls the
+// TMA/tcgen05 kernel does not take (more than 32 sequences, a scale that is not positive).  Work unit: (sequence b, kv head, block of 64 query rows,
 // KV split).  Query rows of one kv head are ordered node-major: row r = i * G + g  (node i, group
 // member g, query head kvh*G + g), so all G heads and all N nodes of a head group share each K/V tile.
 // Tiles of 64 cached tokens stream through a 2-stage cp.async ring; scores are masked with the node's

@@ -1,4 +1,4 @@
-// Tree-verification attention for sm_100a (D = 128): TMA-staged K/V tiles, tcgen05 tensor-core products
+// Tree-verification attention for sm_100a (D = 128 and 64): TMA-staged K/V tiles, tcgen05 tensor-core products
 // with fp32 accumulators in TMEM, fp32 online softmax (Eq. 1 restricted to prefix + ancestors), work split
 // over the SMs.
 //
@@ -83,13 +83,14 @@ constexpr int SMEM_Q = SMEM_V + NSV * STAGE_BYTES;             // Q tile, 128 ro
                                                                // segments it is the PAIR exchange [32 col4][64 rows] float4
 constexpr int SMEM_XM = SMEM_Q + STAGE_BYTES;                  // 512 floats: tile maxima / row statistics exchanged between threads
 constexpr int SMEM_BAR = SMEM_XM + 2048;
-constexpr int BAR_BYTES = 256;
+constexpr int BAR_BYTES = 352;
 constexpr int SMEM_SCHED = SMEM_BAR + BAR_BYTES;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t COL_S = 0, COL_O = 256, COL_P = 384;
 
-enum { B_KFULL = 0, B_KEMPTY = B_KFULL + NSK, B_VFULL = B_KEMPTY + NSK, B_VEMPTY = B_VFULL + NSV,
-       B_SFULL = B_VEMPTY + NSV, B_SFREE = B_SFULL + 2, B_PFULL = B_SFREE + 2, B_PVDONE = B_PFULL + 2,
+constexpr int kMaxRing = 2 * NSK;              // stages of a ring at head size 64: half the bytes each, twice as many
+enum { B_KFULL = 0, B_KEMPTY = B_KFULL + kMaxRing, B_VFULL = B_KEMPTY + kMaxRing, B_VEMPTY = B_VFULL + kMaxRing,
+       B_SFULL = B_VEMPTY + kMaxRing, B_SFREE = B_SFULL + 2, B_PFULL = B_SFREE + 2, B_PVDONE = B_PFULL + 2,
        B_QFULL = B_PVDONE + 2, B_PAIRX = B_QFULL + 1, B_XCH = B_PAIRX + 4, B_XFREE = B_XCH + 1,
        B_SEGSYNC = B_XFREE + 1,
        B_ROWS = B_SEGSYNC + 1,      // fused rotary embedding: every rank of the cluster has put its share of the tree rows into the cache
@@ -340,12 +341,18 @@ __device__ __forceinline__ float exp2_fma(float x) {
 
 // PAGED instantiations carry the paged producer; the others are compiled without it (its call sites cost the
 // contiguous kernels registers they do not have to spare).
-template <bool PAIR, bool CL, bool PAGED, bool ROPE = false>
+template <bool PAIR, bool CL, bool PAGED, bool ROPE = false, int HD = 128>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map, const Tc5Params p,
                 const std::conditional_t<ROPE, RopeArgs, PagedArgs> pa) {
     static_assert(!(ROPE && PAGED), "the fused rotary embedding serves contiguous caches");
     static_assert(!ROPE || CL, "the fused rotary embedding exists in the cluster form only (the even split goes through the rotation kernel)");
+    static_assert(HD == 128 || (HD == 64 && !PAGED && !ROPE), "head size 64: plain calls on contiguous caches");
+    // A stage holds NH halves of 64 d-columns.  At head size 64 the rings have twice the stages, so that the bytes in flight
+    // per SM stay the same; the scores cost half the product, the softmax is unchanged, O has half the columns.
+    // Against the mma.sync kernel and its merge that served head size 64 before (us per layer, mask and commit aside): 38 -> 17
+    // at 8 sequences x 4 heads x 67 nodes on 3325 tokens, 86 -> 51 at 6 x 16 heads (4 kv) x 128 nodes on 2300-4096.
+    constexpr int D = HD, NH = HD / 64, STAGE_BYTES = NH * HALF_BYTES, NSK = kMaxRing / NH, NSV = kMaxRing / NH;
     constexpr int ROWS = PAIR ? 64 : 128;      // distinct query rows per CTA
     constexpr int NC = PAIR ? 32 : 64;         // tokens of a step one softmax thread handles (two threads per row)
     // The V ring can have a producer of its own, the spare warp (its lane 0; paged: all of it).  With at most 64 rows per
@@ -396,11 +403,11 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    pdl_launch_dependents();
     if (!p.early) {                                          // nothing is read before the preceding kernel has ended
         pdl_wait();
         if (warp == 3 && lane < p.B) kv_first = p.kv_len[lane];
     }
+    pdl_launch_dependents();
     if (warp == 3) sched_build(sched, p, lane, kv_first);
     tc_fence_before();
     __syncthreads();
@@ -468,14 +475,14 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     if (!mbar_wait(bar(B_KEMPTY + sk), ((it / NSK) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     mbar_expect_tx(bar(B_KFULL + sk), STAGE_BYTES);
                     tma_load_3d(base + SMEM_K + sk * STAGE_BYTES, &k_map, bar(B_KFULL + sk), 0, tok, bh, pol);
-                    tma_load_3d(base + SMEM_K + sk * STAGE_BYTES + HALF_BYTES, &k_map, bar(B_KFULL + sk), 64, tok, bh, pol);
+                    if constexpr (NH == 2) tma_load_3d(base + SMEM_K + sk * STAGE_BYTES + HALF_BYTES, &k_map, bar(B_KFULL + sk), 64, tok, bh, pol);
                     ++nk;
                     if constexpr (!SPLIT_V) {
                         const int sv = it % NSV;
                         if (!mbar_wait(bar(B_VEMPTY + sv), ((it / NSV) & 1) ^ 1, abort_flag)) { ok = false; break; }
                         mbar_expect_tx(bar(B_VFULL + sv), STAGE_BYTES);
                         tma_load_3d(base + SMEM_V + sv * STAGE_BYTES, &v_map, bar(B_VFULL + sv), 0, tok, bh, pol);
-                        tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
+                        if constexpr (NH == 2) tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
                         ++nv;
                     }
                 }
@@ -533,7 +540,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     if (!mbar_wait(bar(B_VEMPTY + sv), ((it / NSV) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     mbar_expect_tx(bar(B_VFULL + sv), STAGE_BYTES);
                     tma_load_3d(base + SMEM_V + sv * STAGE_BYTES, &v_map, bar(B_VFULL + sv), 0, tok, bh, pol);
-                    tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
+                    if constexpr (NH == 2) tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
                 }
             }
             if (*abort_flag) {
@@ -576,7 +583,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     } else if (warp == 2) {
         // ================= issuer of the PV products =================
         if (lane == 0 && active) {
-            constexpr uint32_t IDESC_O = instr_desc(1);            // B = V stage, MN-major
+            constexpr uint32_t IDESC_O = instr_desc(1, D);           // B = V stage, MN-major
             constexpr uint32_t DESC_HI = desc_hi(1024);
             bool ok = true;
             int u = 0;
@@ -631,7 +638,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         }
 
         // Q of a segment -> shared memory, rows in the swizzled K-major layout of a K stage (PAIR: rows 64-127
-        // repeat rows 0-63).  Thread t moves 16-byte chunk t%16 of rows t/16, t/16 + 16, ...
+        // repeat rows 0-63).  Thread t moves 16-byte chunk t%16 of rows t/16, t/16 + 16, ... (head size 64: t%8 of t/8, t/8 + 32, ...)
         auto load_q = [&](const Seg& sg, int seg) -> bool {
             if (PAIR && seg > 0) {
                 // the tile doubles as the exchange area of the previous segment's epilogue
@@ -647,12 +654,13 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 mbar_arrive(bar(B_QFULL));
                 return true;
             }
-            constexpr int ITEMS = ROWS * 16 / kSmx;
-            const int qc = st & 15;
+            constexpr int QC = D / 8, QR = kSmx / QC;             // 16-byte chunks per row; rows per pass
+            constexpr int ITEMS = ROWS / QR;
+            const int qc = st % QC;
             uint4 v[ITEMS];
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
-                const int row = sg.mblock * ROWS + (st >> 4) + 16 * k;
+                const int row = sg.mblock * ROWS + st / QC + QR * k;
                 v[k] = make_uint4(0, 0, 0, 0);
                 if (row < rows_total) {
                     const int node = row / G, head = sg.kvh * G + row % G;
@@ -661,7 +669,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             }
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
-                const int r = (st >> 4) + 16 * k;
+                const int r = st / QC + QR * k;
                 unsigned char* dst = sm + SMEM_Q + (qc >> 3) * HALF_BYTES + r * 128 + (((qc & 7) ^ (r & 7)) << 4);
                 *reinterpret_cast<uint4*>(dst) = v[k];
                 if (PAIR) *reinterpret_cast<uint4*>(dst + 64 * 128) = v[k];
@@ -785,13 +793,13 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                         if (!mbar_wait_warp(bar(B_PVDONE + (bs ^ 1)), ((it - 1) >> 1) & 1, abort_flag)) { ok = false; break; }
                         tc_fence_after();
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
+                        for (int c = 0; c < NH; ++c) {
                             uint32_t o[32];
-                            tmem_ld32(lane_addr + COL_O + ch * 64 + c * 32, o);
+                            tmem_ld32(lane_addr + COL_O + ch * (D / 2) + c * 32, o);
                             tmem_wait_ld();
 #pragma unroll
                             for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                            tmem_st32(lane_addr + COL_O + ch * 64 + c * 32, o);
+                            tmem_st32(lane_addr + COL_O + ch * (D / 2) + c * 32, o);
                         }
                     }
                     // P[bs] is free once the PV product of step it-2 has completed: as a rule it has, long ago, and one test
@@ -838,7 +846,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
 #pragma unroll
                             for (int c = 0; c < 8; ++c) {
                                 *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
-                                *reinterpret_cast<uint4*>(vrow + HALF_BYTES + c * 16) = make_uint4(0, 0, 0, 0);
+                                if (NH == 2) *reinterpret_cast<uint4*>(vrow + HALF_BYTES + c * 16) = make_uint4(0, 0, 0, 0);
                             }
                         }
                         fence_async_smem();
@@ -851,7 +859,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 if (!ok) break;
 
                 // ---- segment epilogue: wait for the last product, add up the row statistics, (PAIR) merge the two
-                // halves, write out.  A thread owns columns [64 ch, 64 ch + 64) of its lane's accumulator row. ----
+                // halves, write out.  A thread owns columns [D/2 ch, D/2 ch + D/2) of its lane's accumulator row. ----
                 if (sg.n > 0) ok = mbar_wait_warp(bar(B_PVDONE + ((it - 1) & 1)), ((it - 1) >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
@@ -867,13 +875,13 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                         // hand the raw accumulator to the lane that owns the row (the Q tile is idle: every S product
                         // of the segment has completed); the statistics are in place already
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
+                        for (int c = 0; c < NH; ++c) {
                             uint32_t o[32];
-                            tmem_ld32(lane_addr + COL_O + ch * 64 + c * 32, o);
+                            tmem_ld32(lane_addr + COL_O + ch * (D / 2) + c * 32, o);
                             tmem_wait_ld();
 #pragma unroll
                             for (int c4 = 0; c4 < 8; ++c4)
-                                xch[(ch * 16 + c * 8 + c4) * 64 + lrow] = make_float4(__uint_as_float(o[4 * c4]), __uint_as_float(o[4 * c4 + 1]),
+                                xch[(ch * (D / 8) + c * 8 + c4) * 64 + lrow] = make_float4(__uint_as_float(o[4 * c4]), __uint_as_float(o[4 * c4 + 1]),
                                                                                      __uint_as_float(o[4 * c4 + 2]), __uint_as_float(o[4 * c4 + 3]));
                         }
                         tc_fence_before();
@@ -891,17 +899,17 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 }
                 // O is only defined once a product has run (an empty cluster part never ran one): select, never
                 // multiply, where the weight is zero
-                float4* pbuf = reinterpret_cast<float4*>(sm + SMEM_K);                       // cluster form: [32 col4][ROWS]
-                float2* pst = reinterpret_cast<float2*>(sm + SMEM_K + 32 * ROWS * 16);       //               [ROWS] (m, l)
+                float4* pbuf = reinterpret_cast<float4*>(sm + SMEM_K);                       // cluster form: [D/4 col4][ROWS]
+                float2* pst = reinterpret_cast<float2*>(sm + SMEM_K + (D / 4) * ROWS * 16);  //               [ROWS] (m, l)
                 if (half == 0) {
                     const bool final_out = !CL && sg.slot < 0;
                     const float inv = final_out ? (l_all > 0.f ? 1.f / l_all : 0.f) : 1.f;
-                    __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * D + ch * 64;
-                    float4* prow = (CL ? pbuf : p.part_o + (size_t)(final_out ? 0 : sg.slot) * 32 * ROWS) + (size_t)ch * 16 * ROWS + lrow;
+                    __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * D + ch * (D / 2);
+                    float4* prow = (CL ? pbuf : p.part_o + (size_t)(final_out ? 0 : sg.slot) * (D / 4) * ROWS) + (size_t)ch * (D / 8) * ROWS + lrow;
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
+                    for (int c = 0; c < NH; ++c) {
                         uint32_t o[32];
-                        tmem_ld32(lane_addr + COL_O + ch * 64 + c * 32, o);
+                        tmem_ld32(lane_addr + COL_O + ch * (D / 2) + c * 32, o);
                         tmem_wait_ld();
                         float v[32];
 #pragma unroll
@@ -910,7 +918,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                             if (w_other > 0.f) {
 #pragma unroll
                                 for (int c4 = 0; c4 < 8; ++c4) {
-                                    const float4 w = xch[(ch * 16 + c * 8 + c4) * 64 + lrow];
+                                    const float4 w = xch[(ch * (D / 8) + c * 8 + c4) * 64 + lrow];
                                     v[4 * c4] += w.x * w_other; v[4 * c4 + 1] += w.y * w_other;
                                     v[4 * c4 + 2] += w.z * w_other; v[4 * c4 + 3] += w.w * w_other;
                                 }
@@ -968,7 +976,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     if (*seg_flag) {
                         __threadfence();
                         const MergeArgs ma = {p.part_o, p.part_ml, p.out, p.lse, p.Hq, G, N, rows_total};
-                        merge_unit<ROWS>(ma, T, geff, ub, c0, c1, sg.b, sg.kvh, sg.mblock, st, kSmx);
+                        merge_unit<ROWS, D>(ma, T, geff, ub, c0, c1, sg.b, sg.kvh, sg.mblock, st, kSmx);
                     }
                 }
 
@@ -996,11 +1004,11 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         const int rp = (ROWS + ck - 1) / ck;
         const int row0 = cr * rp;
         const int nrows = min(rp, ROWS - row0);
-        const uint32_t pbuf_a = base + SMEM_K, pst_a = base + SMEM_K + 32 * ROWS * 16;
+        const uint32_t pbuf_a = base + SMEM_K, pst_a = base + SMEM_K + (D / 4) * ROWS * 16;
         // IT items (row, column quad) at a time per thread, all loads of all KM pieces issued before the first use
         auto merge_items = [&](auto km_tag, auto it_tag) {
             constexpr int KM = decltype(km_tag)::value, IT = decltype(it_tag)::value;
-            for (int item0 = tid - 128; item0 < nrows * 32; item0 += kSmx * IT) {
+            for (int item0 = tid - 128; item0 < nrows * (D / 4); item0 += kSmx * IT) {
                 float2 ml[IT][KM];
                 float4 pv[IT][KM];
                 int c4s[IT], grows[IT];
@@ -1009,7 +1017,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     const int item = item0 + e * kSmx;
                     const int c4 = item / nrows, lr = row0 + (item - c4 * nrows);
                     c4s[e] = c4;
-                    grows[e] = (item < nrows * 32) ? cl_seg.mblock * ROWS + lr : rows_total;
+                    grows[e] = (item < nrows * (D / 4)) ? cl_seg.mblock * ROWS + lr : rows_total;
 #pragma unroll
                     for (int j = 0; j < KM; ++j) {
                         ml[e][j] = make_float2(-INFINITY, 0.f);
@@ -1067,7 +1075,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
 }  // namespace
 
 
-static size_t tc5_partial_bytes(int grid, int rows) { return (size_t)2 * grid * rows * (D * 4 + 8); }
+static size_t tc5_partial_bytes(int grid, int rows, int D) { return (size_t)2 * grid * rows * (D * 4 + 8); }
 
 namespace {
 
@@ -1182,12 +1190,13 @@ static int tc5_cluster_size(const AttnArgs& a, bool pair, int n_mblocks, double*
     // has given the length it expects (VISPEC_OPT_KV_LEN_HINT).
     const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
     const double steps = (double)((slots + STEP - 1) / STEP), T = steps * units;
+    const double hbm = a.D / 128.0;        // a step's bytes follow the head size, its softmax does not
     const double n_c = (double)units * best, per_c = (double)(((slots + STEP - 1) / STEP + best - 1) / best);
-    const double est_c = 11.0 + per_c * fmax(1.2, n_c * 0.0125 / n_mblocks);
+    const double est_c = 11.0 + per_c * fmax(1.2, n_c * 0.0125 * hbm / n_mblocks);
     const double n_e = fmin((double)a.sm_count, fmax(1.0, T / 2.0));
     // (merge: 0.25 per piece of a unit; from four pieces on the fine-grained merge kernel, 1 + 0.055 per piece)
     const double pieces = n_e / units;
-    const double est_e = 14.0 + (T / n_e) * fmax(1.2, n_e * 0.00973 / n_mblocks) + (pieces >= 4.0 ? 1.0 + 0.055 * pieces : 0.25 * pieces);
+    const double est_e = 14.0 + (T / n_e) * fmax(1.2, n_e * 0.00973 * hbm / n_mblocks) + (pieces >= 4.0 ? 1.0 + 0.055 * pieces : 0.25 * pieces);
     // (units of several row blocks per kv head in small clusters: measured over the sweep, the even split's steps come
     // out dearer than the estimate there - 54.8 against 52.6 us on qwen3b_S8192_N60_B8, 96.1 against 92.4 on
     // qwen3b_S16384_N128_B4 - so the clusters get a tenth of tolerance)
@@ -1217,7 +1226,7 @@ static Tc5Layout tc5_layout(const AttnArgs& a) {
     const int steps = (slots + STEP - 1) / STEP;
     auto est = [&](const Tc5Layout& l, double step_us) {
         const double n_c = (double)a.B * a.Hkv * l.n_mblocks * l.ck;
-        return 11.0 + (double)((steps + l.ck - 1) / l.ck) * fmax(step_us, n_c * 0.0125 / l.n_mblocks);
+        return 11.0 + (double)((steps + l.ck - 1) / l.ck) * fmax(step_us, n_c * 0.0125 * (a.D / 128.0) / l.n_mblocks);
     };
     if (full.ck > 0) return est(half, 0.95) < 0.95 * est(full, full.n_mblocks > 1 ? 1.7 : 1.45) ? half : full;
     // 128-row blocks would go as an even split (its estimate: est_full); small clusters of 64-row blocks, whose fixed
@@ -1226,22 +1235,25 @@ static Tc5Layout tc5_layout(const AttnArgs& a) {
 }
 
 bool attn_tc5_supports(const AttnArgs& a) {
-    if (!(a.D == 128 && a.k_map && a.v_map && a.B > 0 && a.B <= kMaxB)) return false;
+    if (!((a.D == 128 || a.D == 64) && a.k_map && a.v_map && a.B > 0 && a.B <= kMaxB)) return false;
+    if (a.D == 64 && (a.rope_table || a.page_rows)) return false;
     const int rows_total = (a.Hq / a.Hkv) * a.N;
     const int rows = rows_total <= 64 ? 64 : 128;
     const long long n_mblocks = (rows_total + 63) / 64;          // the most either layout makes
     const long long t_max = (long long)a.B * a.Hkv * n_mblocks * ((a.S_max + STEP - 1) / STEP);
     if (t_max * a.sm_count >= (1ll << 31)) return false;
     if (!(a.scale > 0.f)) return false;       // the kernel takes the maximum before scaling
-    return kCounterBytes + tc5_partial_bytes(a.sm_count, rows) <= a.ws_bytes;
+    return kCounterBytes + tc5_partial_bytes(a.sm_count, rows, a.D) <= a.ws_bytes;
 }
 
 cudaError_t init_attn_tc5() {
     cudaError_t e = cudaSuccess;
-    const void* kernels[8] = {(const void*)attn_tc5_kernel<true, false, false>, (const void*)attn_tc5_kernel<false, false, false>,
-                              (const void*)attn_tc5_kernel<true, true, false>, (const void*)attn_tc5_kernel<false, true, false>,
-                              (const void*)attn_tc5_kernel<true, false, true>, (const void*)attn_tc5_kernel<false, false, true>,
-                              (const void*)attn_tc5_kernel<true, true, true>, (const void*)attn_tc5_kernel<false, true, true>};
+    const void* kernels[12] = {(const void*)attn_tc5_kernel<true, false, false>, (const void*)attn_tc5_kernel<false, false, false>,
+                               (const void*)attn_tc5_kernel<true, true, false>, (const void*)attn_tc5_kernel<false, true, false>,
+                               (const void*)attn_tc5_kernel<true, false, true>, (const void*)attn_tc5_kernel<false, false, true>,
+                               (const void*)attn_tc5_kernel<true, true, true>, (const void*)attn_tc5_kernel<false, true, true>,
+                               (const void*)attn_tc5_kernel<true, false, false, false, 64>, (const void*)attn_tc5_kernel<false, false, false, false, 64>,
+                               (const void*)attn_tc5_kernel<true, true, false, false, 64>, (const void*)attn_tc5_kernel<false, true, false, false, 64>};
     for (const void* k : kernels) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_ALLOC);
         if (e != cudaSuccess) return e;
@@ -1254,8 +1266,10 @@ cudaError_t init_attn_tc5() {
     for (int k = 1; k <= 8; ++k) { g_max_clusters[0][k] = query_max_clusters(false, k); g_max_clusters[1][k] = query_max_clusters(true, k); }
     if (getenv("VISPEC_DEBUG")) for (int k = 1; k <= 8; ++k) fprintf(stderr, "vispec: cluster size %d: %d (rows > 64) / %d (rows <= 64) co-resident clusters\n", k, g_max_clusters[0][k], g_max_clusters[1][k]);
     // The merge blocks must be able to join an SM that an attention CTA has configured for maximum shared memory.
-    const void* merge_kernels[4] = {(const void*)attn_tc5_merge_kernel<64>, (const void*)attn_tc5_merge_kernel<128>,
-                                    (const void*)attn_tc5_merge_kernel<64, true>, (const void*)attn_tc5_merge_kernel<128, true>};
+    const void* merge_kernels[8] = {(const void*)attn_tc5_merge_kernel<64>, (const void*)attn_tc5_merge_kernel<128>,
+                                    (const void*)attn_tc5_merge_kernel<64, true>, (const void*)attn_tc5_merge_kernel<128, true>,
+                                    (const void*)attn_tc5_merge_kernel<64, false, 64>, (const void*)attn_tc5_merge_kernel<128, false, 64>,
+                                    (const void*)attn_tc5_merge_kernel<64, true, 64>, (const void*)attn_tc5_merge_kernel<128, true, 64>};
     for (const void* k : merge_kernels) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
@@ -1279,7 +1293,7 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     p.out = (__nv_bfloat16*)a.out; p.lse = a.lse;
     unsigned char* ws = (unsigned char*)a.ws + kCounterBytes;
     p.part_o = (float4*)ws;
-    p.part_ml = (float2*)(ws + (size_t)2 * grid * rows * D * 4);
+    p.part_ml = (float2*)(ws + (size_t)2 * grid * rows * a.D * 4);
     p.B = a.B; p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.S_max = a.S_max; p.n_mblocks = n_mblocks;
     p.grid_attn = grid; p.min_steps = 2; p.early = a.early_prefetch ? 1 : 0; p.step = STEP;
     p.scale_log2 = a.scale * 1.4426950408889634f;
@@ -1289,7 +1303,7 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     // even split, at most 64 rows per unit: the arrival counters at the head of the workspace serve the in-kernel
     // merge (measured: 68.8 against 70.3 us per layer on llava13b_b4; with 128 rows it lost, 65.9 against 60.5 us on
     // qwen3b_S32768_N16_B8, so those, a grid with more units than counters, and split form 3 get the merge kernel)
-    const bool own_merge = pair && ck == 0 && a.tc5_path != 3 && (size_t)units * sizeof(int) <= kCounterBytes;
+    const bool own_merge = pair && ck == 0 && a.tc5_path != 3 && !a.no_counters && (size_t)units * sizeof(int) <= kCounterBytes;
     const PagedArgs pa = {a.block_table, a.table_stride, a.page_rows, a.num_blocks, a.Hkv, a.N, a.token_major, a.status,
                           own_merge ? (int*)a.ws : nullptr};
     auto launch_attn = [&](auto kernel, int cluster) {
@@ -1310,25 +1324,27 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
         ++*n_launches;
         return cudaSuccess;
     }
-    if (ck > 0) {
-        // cluster form: the CTAs of a unit merge their partials through distributed shared memory; one launch
-        err = paged ? (pair ? launch_attn(attn_tc5_kernel<true, true, true>, ck) : launch_attn(attn_tc5_kernel<false, true, true>, ck))
-                    : (pair ? launch_attn(attn_tc5_kernel<true, true, false>, ck) : launch_attn(attn_tc5_kernel<false, true, false>, ck));
-        if (err != cudaSuccess) return err;
-        ++*n_launches;
-        return cudaSuccess;
-    }
-    err = paged ? (pair ? launch_attn(attn_tc5_kernel<true, false, true>, 0) : launch_attn(attn_tc5_kernel<false, false, true>, 0))
-                : (pair ? launch_attn(attn_tc5_kernel<true, false, false>, 0) : launch_attn(attn_tc5_kernel<false, false, false>, 0));
+    // one launch in the cluster form (the CTAs of a unit merge their partials through distributed shared memory)
+    auto launch_form = [&](auto cl) {
+        constexpr bool CL = decltype(cl)::value;
+        if (a.D == 64) return pair ? launch_attn(attn_tc5_kernel<true, CL, false, false, 64>, ck) : launch_attn(attn_tc5_kernel<false, CL, false, false, 64>, ck);
+        if (paged) return pair ? launch_attn(attn_tc5_kernel<true, CL, true>, ck) : launch_attn(attn_tc5_kernel<false, CL, true>, ck);
+        return pair ? launch_attn(attn_tc5_kernel<true, CL, false>, ck) : launch_attn(attn_tc5_kernel<false, CL, false>, ck);
+    };
+    err = ck > 0 ? launch_form(std::true_type{}) : launch_form(std::false_type{});
     if (err != cudaSuccess) return err;
     ++*n_launches;
-    if (own_merge) return cudaSuccess;
-    if (grid >= 4 * units)        // units cut into many pieces: the fine-grained merge
-        err = pair ? launch_pdl(attn_tc5_merge_kernel<64, true>, dim3(units, 16), dim3(128), 0, st, 0, p)
-                   : launch_pdl(attn_tc5_merge_kernel<128, true>, dim3(units, 32), dim3(128), 0, st, 0, p);
-    else
-        err = pair ? launch_pdl(attn_tc5_merge_kernel<64>, dim3(units, 4), dim3(128), 0, st, 0, p)
-                   : launch_pdl(attn_tc5_merge_kernel<128>, dim3(units, 8), dim3(128), 0, st, 0, p);
+    if (ck > 0 || own_merge) return cudaSuccess;
+    // the merge: fine-grained where units are cut into many pieces
+    auto launch_merge = [&](auto hd) {
+        constexpr int HD = decltype(hd)::value;
+        if (grid >= 4 * units)
+            return pair ? launch_pdl(attn_tc5_merge_kernel<64, true, HD>, dim3(units, HD / 8), dim3(128), 0, st, 0, p)
+                        : launch_pdl(attn_tc5_merge_kernel<128, true, HD>, dim3(units, HD / 4), dim3(128), 0, st, 0, p);
+        return pair ? launch_pdl(attn_tc5_merge_kernel<64, false, HD>, dim3(units, HD / 32), dim3(128), 0, st, 0, p)
+                    : launch_pdl(attn_tc5_merge_kernel<128, false, HD>, dim3(units, HD / 16), dim3(128), 0, st, 0, p);
+    };
+    err = a.D == 64 ? launch_merge(std::integral_constant<int, 64>{}) : launch_merge(std::integral_constant<int, 128>{});
     if (err != cudaSuccess) return err;
     ++*n_launches;
     return cudaSuccess;

@@ -10,7 +10,7 @@
 namespace vispec {
 namespace tc5 {
 
-constexpr int D = 128;
+constexpr int D = 128;                         // head size of the paged and fused-rotary forms; the plain one also takes 64
 constexpr int kMaxB = 32;                      // sequences per call these kernels take
 constexpr float kRescaleGap = 8.0f;            // log2 units
 constexpr long long kWaitCycles = 1500000000LL;   // ~0.8 s at 1.9 GHz
@@ -194,9 +194,9 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo_bytes) {
 __host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo_bytes) {
     return (sbo_bytes >> 4) | (1u << 14) | (2u << 29);
 }
-// Instruction descriptor, kind::f16: D fp32, A and B bf16, A K-major, M = 128, N = 128; b_mn = 1 if B is MN-major.
-__host__ __device__ constexpr uint32_t instr_desc(int b_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+// Instruction descriptor, kind::f16: D fp32, A and B bf16, A K-major, M = 128, N = n; b_mn = 1 if B is MN-major.
+__host__ __device__ constexpr uint32_t instr_desc(int b_mn, int n = 128) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn << 16) | (((uint32_t)n >> 3) << 17) | ((128u >> 4) << 24);
 }
 // 128-bit shifts on (lo, hi) pairs; any shift count >= 0.
 __device__ __forceinline__ void shr128(uint64_t lo, uint64_t hi, int s, uint64_t& rlo, uint64_t& rhi) {
@@ -218,7 +218,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 struct Tc5Params {
     const __nv_bfloat16* q; const int32_t* kv_len; const uint64_t* mask;
     __nv_bfloat16* out; float* lse;
-    float4* part_o;            // [slot][32 col4][ROWS]: column-of-4 major, so that a warp's 32 rows are contiguous
+    float4* part_o;            // [slot][D/4 col4][ROWS]: column-of-4 major, so that a warp's 32 rows are contiguous
     float2* part_ml;           // [slot][ROWS]: (m in log2 units or -inf, l)
     int B, N, Hq, Hkv, S_max, n_mblocks;
     int grid_attn;             // CTAs of the attention kernel (the merge kernel needs it for the schedule)
@@ -327,7 +327,7 @@ struct SegIter {
 
 // One (row, 16 output columns) of a unit: the partials of CTAs c0..c1 (slot 2c if the unit starts CTA c's range,
 // else 2c + 1) folded into the final output.  Shared by the merge kernel and by the attention kernel's own merge.
-template <int ROWS>
+template <int ROWS, int HD>
 __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o, const float2* __restrict__ part_ml,
                                                __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int geff,
                                                int ub, int c0, int c1, int b, int node, int head, int Hq, int N,
@@ -351,7 +351,7 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
             if (c <= c1) {
                 const int slot = slot_of(c);
                 ml[j] = __ldcg(&part_ml[(size_t)slot * ROWS + lrow]);
-                const float4* src = part_o + ((size_t)slot * 32 + cw * 4) * ROWS + lrow;
+                const float4* src = part_o + ((size_t)slot * (HD / 4) + cw * 4) * ROWS + lrow;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) v[j][k] = __ldcg(src + (size_t)k * ROWS);
             }
@@ -376,7 +376,7 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
         m_all = m_new;
     }
     const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
-    __nv_bfloat16* orow = out + (((size_t)b * N + node) * Hq + head) * D + cw * 16;
+    __nv_bfloat16* orow = out + (((size_t)b * N + node) * Hq + head) * HD + cw * 16;
 #pragma unroll
     for (int k = 0; k < 2; ++k)
         *reinterpret_cast<uint4*>(orow + k * 8) =
@@ -389,7 +389,7 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
 // One (row, 4 output columns) of a unit, the merge kernel's piece: sixteen segments at a time with every load issued
 // before the first use (a unit cut over many CTAs - few sequences, long caches - is merged from dozens of partials,
 // and a round of loads is a memory round trip).
-template <int ROWS>
+template <int ROWS, int HD>
 __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, const float2* __restrict__ part_ml,
                                              __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int geff,
                                              int ub, int c0, int c1, int b, int node, int head, int Hq, int N,
@@ -408,7 +408,7 @@ __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, 
             if (c <= c1) {
                 const int slot = slot_of(c);
                 ml[j] = __ldcg(&part_ml[(size_t)slot * ROWS + lrow]);
-                v[j] = __ldcg(part_o + ((size_t)slot * 32 + c4) * ROWS + lrow);
+                v[j] = __ldcg(part_o + ((size_t)slot * (HD / 4) + c4) * ROWS + lrow);
             }
         }
         float m_new = m_all;
@@ -427,7 +427,7 @@ __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, 
         m_all = m_new;
     }
     const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
-    *reinterpret_cast<uint2*>(out + (((size_t)b * N + node) * Hq + head) * D + c4 * 4) =
+    *reinterpret_cast<uint2*>(out + (((size_t)b * N + node) * Hq + head) * HD + c4 * 4) =
         make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
     if (lse && c4 == 0)
         lse[((size_t)b * Hq + head) * N + node] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
@@ -436,14 +436,14 @@ __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, 
 // The whole unit, by the softmax threads of the CTA that delivered the unit's last partial (thread st of nthreads).
 // Not inlined: its accumulators stay out of the attention kernel's register budget.
 struct MergeArgs { const float4* part_o; const float2* part_ml; __nv_bfloat16* out; float* lse; int Hq, G, N, rows_total; };
-template <int ROWS>
+template <int ROWS, int HD>
 __device__ __noinline__ void merge_unit(const MergeArgs m, int T, int geff, int ub, int c0, int c1, int b, int kvh,
                                         int mblock, int st, int nthreads) {
-    for (int item = st; item < ROWS * 8; item += nthreads) {
+    for (int item = st; item < ROWS * (HD / 16); item += nthreads) {
         const int cw = item / ROWS, lrow = item - cw * ROWS;
         const int row = mblock * ROWS + lrow;
         if (row >= m.rows_total) continue;
-        merge_row_cols<ROWS>(m.part_o, m.part_ml, m.out, m.lse, T, geff, ub, c0, c1, b, row / m.G, kvh * m.G + row % m.G,
+        merge_row_cols<ROWS, HD>(m.part_o, m.part_ml, m.out, m.lse, T, geff, ub, c0, c1, b, row / m.G, kvh * m.G + row % m.G,
                              m.Hq, m.N, lrow, cw);
     }
 }
@@ -464,14 +464,14 @@ struct PagedArgs { const int32_t* block_table; int table_stride, page_rows, num_
                    int* unit_counters; };   // even split: arrivals per unit (all zero between calls); nullptr: a merge kernel follows
 
 // Merge of the partials of every unit that more than one CTA worked on, 4 warps per block, lane <-> row.  Two
-// shapes: grid (unit, 2 * group of 32 rows + half of the columns), a warp sums 16 output columns over the unit's
-// segments four at a time - for units cut into a few pieces; FINE: grid (unit, 8 * group of 32 rows + eighth of the
-// columns), a warp sums 4 output columns sixteen segments at a time - for units cut over many CTAs (few sequences, long
+// shapes (figures of head size 128): grid (unit, 2 * group of 32 rows + half of the columns), a warp sums 16 output
+// columns over the unit's segments four at a time - for units cut into a few pieces; FINE: grid (unit, 8 * group of 32
+// rows + eighth of the columns), a warp sums 4 output columns sixteen segments at a time - for units cut over many CTAs (few sequences, long
 // caches), where the rounds of loads are what the merge takes: qwen3b_S32768_N16_B1 (2 units over 148 CTAs) 42.7 ->
 // 29.1 us per layer, qwen3b_S32768_N60_B1 34.8 -> 31.8; with many units of two partials the coarse shape is 3 % faster.
 // The blocks are small so that they fit beside a resident attention CTA: they are launched early
 // (programmatic dependent launch) and must not keep the next layer's attention CTAs off the SMs.
-template <int ROWS, bool FINE = false>
+template <int ROWS, bool FINE = false, int HD = 128>
 __global__ void __launch_bounds__(128)
 attn_tc5_merge_kernel(const Tc5Params p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -496,14 +496,15 @@ attn_tc5_merge_kernel(const Tc5Params p) {
     if (c0 == c1) return;                              // one CTA had the whole unit and wrote the output itself
     const int G = p.Hq / p.Hkv, N = p.N;
     const int kvh = uib / p.n_mblocks, mblock = uib - kvh * p.n_mblocks;
-    const int lrow = (FINE ? blockIdx.y >> 3 : blockIdx.y >> 1) * 32 + lane;
-    const int cw = FINE ? (blockIdx.y & 7) * 4 + warp : (blockIdx.y & 1) * 4 + warp;    // which 4 (FINE) or 16 output columns
+    constexpr int CB = FINE ? HD / 16 : HD / 64;       // blocks per group of 32 rows
+    const int lrow = (blockIdx.y / CB) * 32 + lane;
+    const int cw = (blockIdx.y % CB) * 4 + warp;       // which 4 (FINE) or 16 output columns
     const int row = mblock * ROWS + lrow;
     if (row >= G * N) return;
     const int node = row / G, head = kvh * G + row % G;
 
-    if (FINE) merge_row_c4<ROWS>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
-    else merge_row_cols<ROWS>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
+    if (FINE) merge_row_c4<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
+    else merge_row_cols<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
 }
 
 }  // namespace tc5

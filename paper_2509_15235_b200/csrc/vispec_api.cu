@@ -56,6 +56,10 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 
+}  // namespace
+
+namespace vispec {
+
 // Kernel attributes and occupancy answers are a device's, not a context's: found once (context creation goes through
 // here with the device current; a failed attempt is made again).
 bool init_device(int device) {
@@ -69,7 +73,21 @@ bool init_device(int device) {
     return ok;
 }
 
-}  // namespace
+// 3-D view (d, slot, sequence*head) of a [B,Hkv,S_max,D] bf16 cache; one box = 64 d-columns (128 bytes, the swizzle
+// span) x 128 slots.  Slots past S_max read as zero.
+bool encode_cache_map(CUtensorMap* map, const void* cache, int D, int S_max, long long heads) {
+    EncodeTiledFn enc = get_encode_fn();
+    if (!enc) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)S_max, (cuuint64_t)heads};
+    const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)S_max * D * 2};
+    const cuuint32_t box[3] = {64, 128, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(cache), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace vispec
 
 extern "C" {
 
@@ -174,24 +192,9 @@ int vispec_cache_register(vispec_ctx* c, int layer, void* k_cache, void* v_cache
     if (layer < 0 || layer >= c->shape.layers) return VISPEC_E_RANGE;
     if (!aligned(k_cache, 128) || !aligned(v_cache, 128)) return VISPEC_E_ALIGN;
     const vispec_shape& s = c->shape;
-    if (s.D == 128) {
-        // 3-D view (d, slot, sequence*head) of a [B,Hkv,S_max,D] bf16 cache; one box = 64 d-columns
-        // (128 bytes, the swizzle span) x 128 slots.  Slots past S_max read as zero.
-        EncodeTiledFn enc = get_encode_fn();
-        if (!enc) return VISPEC_E_CUDA;
-        const cuuint64_t dims[3] = {(cuuint64_t)s.D, (cuuint64_t)s.S_max, (cuuint64_t)s.B_max * s.Hkv};
-        const cuuint64_t strides[2] = {(cuuint64_t)s.D * 2, (cuuint64_t)s.S_max * s.D * 2};
-        const cuuint32_t box[3] = {64, 128, 1};
-        const cuuint32_t estr[3] = {1, 1, 1};
-        void* ptrs[2] = {k_cache, v_cache};
-        CUtensorMap* maps[2] = {&c->k_map[layer], &c->v_map[layer]};
-        for (int t = 0; t < 2; ++t) {
-            CUresult r = enc(maps[t], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, ptrs[t], dims, strides, box, estr,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return VISPEC_E_CUDA;
-        }
-    }
+    const long long heads = (long long)s.B_max * s.Hkv;
+    if (!encode_cache_map(&c->k_map[layer], k_cache, s.D, s.S_max, heads) || !encode_cache_map(&c->v_map[layer], v_cache, s.D, s.S_max, heads))
+        return VISPEC_E_CUDA;
     void* pair[2] = {k_cache, v_cache};
     if (cudaMemcpy(c->d_cache_ptrs + 2 * layer, pair, sizeof(pair), cudaMemcpyHostToDevice) != cudaSuccess)
         return VISPEC_E_CUDA;

@@ -15,7 +15,7 @@ struct vispec_ctx {
     int* d_status = nullptr;        // device status word (first asynchronous error wins)
     void** d_cache_ptrs = nullptr;  // device table [layers][2]: k_cache, v_cache
     std::vector<void*> h_k, h_v;    // host copy of the registered pointers
-    std::vector<CUtensorMap> k_map, v_map;  // TMA descriptors per layer (D == 128 only)
+    std::vector<CUtensorMap> k_map, v_map;  // TMA descriptors per layer
     std::vector<int> page_rows, num_blocks; // per layer: slots per pool block (0 = contiguous cache), pool blocks
     std::vector<int> token_major;           // per layer: pool is [block][slot][head][D] instead of [block][head][slot][D]
     void* ws = nullptr;             // caller-owned workspace
@@ -91,15 +91,20 @@ struct AttnArgs {
     // fused rotary embedding (TMA + tcgen05 kernel, contiguous caches): rope_table non-null turns it on
     const void* rope_table; const void* k_new; const void* v_new;
     const CUtensorMap* k_map; const CUtensorMap* v_map;
+    bool no_counters;      // the arrival counters at the head of the workspace may not be relied on: merge with a kernel of its own
     // paged cache (page_rows != 0): pool blocks of page_rows slots, block_table [B][table_stride]; S_max is then
     // table_stride * page_rows
     const int32_t* block_table; int table_stride, page_rows, num_blocks, token_major;
 };
+// Everything that is set once per device (kernel attributes, occupancy answers), with that device current.
+bool init_device(int device);
+// TMA descriptor of a contiguous cache [heads][S_max][D] (heads = sequences * kv heads).
+bool encode_cache_map(CUtensorMap* map, const void* cache, int D, int S_max, long long heads);
 // Generic split-KV kernel on warp-level tensor-core instructions (any supported shape).
 cudaError_t init_attn_generic();   // once per device, with that device current
 cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st, int* n_launches);
 
-// TMA + tcgen05 kernel (D = 128), work split evenly over the SMs, followed by its merge kernel.
+// TMA + tcgen05 kernel, work split evenly over the SMs, followed by its merge kernel.
 bool attn_tc5_supports(const AttnArgs& a);
 cudaError_t init_attn_tc5();           // once per device, with that device current
 cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches);

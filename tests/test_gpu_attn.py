@@ -71,6 +71,25 @@ def test_shapes_span_tiles_tails_and_group_sizes(gu, Hq, Hkv, D, N, S, S_max, sp
     _check(gu, q, k, v, kv_len, mask, 1 / math.sqrt(D), split_form=split_form)
 
 
+# Head size 64 on the tensor-core kernel: one node on an empty cache, a full and a just overfull 64-row block, a row block
+# of 128 with a ragged rest, more steps than the rings have stages (6), a tree that straddles two steps.
+@pytest.mark.parametrize("Hq,Hkv,N,S,S_max", [
+    (4, 4, 1, 0, 64), (4, 4, 64, 127, 256), (5, 1, 13, 640, 700), (16, 4, 127, 2049, 2304), (8, 2, 33, 1000, 1152),
+    (2, 2, 128, 64, 192),
+])
+@pytest.mark.parametrize("split_form", [0, 1, 2, 3])
+def test_head_size_64_edges(gu, Hq, Hkv, N, S, S_max, split_form):
+    rng = np.random.Generator(np.random.Philox(Hq * 1000 + N + 64))
+    B, D = 3, 64
+    q = synth.normal_bf16((B, N, Hq, D), 5 + N)
+    k = synth.normal_bf16((B, Hkv, S_max, D), 6 + N)
+    v = synth.normal_bf16((B, Hkv, S_max, D), 7 + N)
+    kv_len = np.array([S, S // 3, max(0, S - 1)], dtype=np.int32)
+    parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
+    mask, _, _ = oracle.tree_mask(parents)
+    _check(gu, q, k, v, kv_len, mask, 1 / math.sqrt(D), split_form=split_form)
+
+
 def test_arbitrary_mask_bits_all_ones_and_zero_rows(gu):
     B, N, Hq, Hkv, D, S_max = 2, 20, 4, 2, 128, 256
     q = synth.normal_bf16((B, N, Hq, D), 21); k = synth.normal_bf16((B, Hkv, S_max, D), 22)
