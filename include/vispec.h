@@ -214,7 +214,7 @@ int vispec_tree_verify_attn_rope(vispec_ctx* ctx, int layer, const void* q, cons
  * tensors but no allocator, code on a latency-critical stream where cudaMalloc's implicit
  * device synchronisation is not acceptable.  It computes exactly what vispec_tree_verify_attn
  * computes, but needs no context, no registration and no workspace: the split-KV partial results go
- * to a 16 MiB array that is part of the library image (static device memory, held on every GPU that
+ * to a 20 MiB array that is part of the library image (static device memory, held on every GPU that
  * loads the library until the process exits).  The function calls no cudaMalloc/cudaFree and no
  * allocating library routine.
  *   - Arguments as in vispec_tree_verify_attn, with the shape given explicitly (Hq, Hkv, D in
@@ -224,8 +224,8 @@ int vispec_tree_verify_attn_rope(vispec_ctx* ctx, int layer, const void* q, cons
  *   - Limit: B * Hkv * ceil(G*N/64) partial-result units must fit the array with two KV splits,
  *     i.e. 64 KiB + 2 * units * 64 * (4*D + 8) bytes <= 16 MiB (at D = 128: 251 units).  Beyond
  *     that the call returns VISPEC_E_WORKSPACE and does nothing.
- *   - The first call on each device looks up the array's device address and sets one kernel
- *     attribute; make that first call outside any stream capture, with the device current.
+ *   - The first call on each device looks up the array's device address and sets kernel
+ *     attributes; make that first call outside any stream capture, with the device current.
  *   - All calls share the one array, and it keeps the previous call's contents.  Nothing in it has
  *     to start at zero (every partial is written before it is read), so no clearing is done; but two
  *     calls that overlap on the GPU (different streams, different host threads) race on it.  Run

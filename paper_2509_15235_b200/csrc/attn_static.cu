@@ -9,9 +9,11 @@
 // from module load until exit.
 #include "vispec_internal.h"
 
-// 16 MiB: room for up to 502 partial results of 64 query rows at D = 128 (33,280 bytes each)
-// behind the 64 KiB header the workspace layout reserves.
-#define VISPEC_STATIC_SCRATCH_BYTES (16u << 20)
+// 20 MiB: two partial results of 128 query rows at D = 128 (66,560 bytes each) for each of up to 156 SMs, what the
+// even split of the tcgen05 kernel writes, behind the 64 KiB header the workspace layout reserves.  The limit on a
+// call's size is that of 16 MiB, as published.
+#define VISPEC_STATIC_SCRATCH_BYTES (20u << 20)
+#define VISPEC_STATIC_LIMIT_BYTES (16u << 20)
 
 static __device__ __align__(256) unsigned char g_static_scratch[VISPEC_STATIC_SCRATCH_BYTES];
 static __device__ int g_static_status;   // sink for the status word when the caller passes none
@@ -41,7 +43,7 @@ int setup_current_device(int dev) {
     if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess) return VISPEC_E_CUDA;
     if (cudaGetSymbolAddress((void**)&st, g_static_status) != cudaSuccess) return VISPEC_E_CUDA;
     if (cudaDeviceGetAttribute(&s.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return VISPEC_E_CUDA;
-    if (vispec::init_attn_generic() != cudaSuccess) return VISPEC_E_CUDA;   // a function attribute, not an allocation
+    if (!vispec::init_device(dev)) return VISPEC_E_CUDA;   // function attributes, occupancy queries: no allocation
     s.scratch = p;
     s.status = st;
     s.done = true;
@@ -65,7 +67,7 @@ extern "C" int vispec_tree_verify_attn_static(const void* q, const void* k_cache
     // fit the static array with at least two splits, otherwise the call is refused, not truncated.
     const size_t units = (size_t)B * Hkv * (((size_t)(Hq / Hkv) * N + 63) / 64);
     const size_t half_slot = vispec::slot_bytes(D) / 2;
-    if (vispec::kCounterBytes + 2 * units * half_slot > VISPEC_STATIC_SCRATCH_BYTES) return VISPEC_E_WORKSPACE;
+    if (vispec::kCounterBytes + 2 * units * half_slot > VISPEC_STATIC_LIMIT_BYTES) return VISPEC_E_WORKSPACE;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return VISPEC_E_CUDA;
     if (dev < 0 || dev >= kMaxDevices) return VISPEC_E_RANGE;
@@ -81,7 +83,17 @@ extern "C" int vispec_tree_verify_attn_static(const void* q, const void* k_cache
     a.sm_count = s.sm_count;
     a.early_prefetch = false;
     a.tc5_path = 0;
-    a.k_map = nullptr; a.v_map = nullptr;
+    a.no_counters = true;          // the array starts a call with whatever the last one left
+    // The descriptors are encoded on each call (two host-side encodings of 128 bytes; the caches are the caller's and may
+    // be others next time).  llava7b's shape, one layer: 43.7 us on the generic kernel and its merge, 18.6 on this one.
+    CUtensorMap maps[2];
     int n = 0;
-    return vispec::launch_attn_generic(a, (cudaStream_t)stream, &n) == cudaSuccess ? VISPEC_OK : VISPEC_E_CUDA;
+    cudaError_t err;
+    if (vispec::encode_cache_map(&maps[0], k_cache, D, S_max, (long long)B * Hkv) &&
+        vispec::encode_cache_map(&maps[1], v_cache, D, S_max, (long long)B * Hkv)) {
+        a.k_map = &maps[0]; a.v_map = &maps[1];
+    }
+    err = vispec::attn_tc5_supports(a) ? vispec::launch_attn_tc5(a, (cudaStream_t)stream, &n)
+                                       : vispec::launch_attn_generic(a, (cudaStream_t)stream, &n);
+    return err == cudaSuccess ? VISPEC_OK : VISPEC_E_CUDA;
 }
