@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvispec.so")
 NATIVE_SRC = os.path.join(CSRC, "binding_native.cpp")
 NATIVE = os.path.join(HERE, "_native.so")
-SOURCES = ["vispec_api.cu", "tree_kernels.cu", "attn_generic.cu", "attn_tc5.cu", "attn_static.cu", "accept_sampled.cu"]
+SOURCES = ["vispec_api.cu", "tree_kernels.cu", "attn_generic.cu", "attn_tc5.cu", "attn_tc5_wide.cu", "attn_static.cu", "accept_sampled.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math", "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
 

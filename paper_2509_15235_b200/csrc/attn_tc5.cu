@@ -71,8 +71,6 @@ using namespace tc5;
 
 namespace {
 
-constexpr int STEP = 128;                      // tokens per pipeline step = rows of one K or V stage
-constexpr int HALF_BYTES = STEP * 128;         // one d-half (64 columns) of a stage: 128 rows x 128 B
 constexpr int STAGE_BYTES = 2 * HALF_BYTES;    // 32 KB
 constexpr int NSK = 3, NSV = 3;
 constexpr int kThreads = 384;                  // 12 warps: producer, two issuers, one spare, eight softmax
@@ -97,96 +95,16 @@ enum { B_KFULL = 0, B_KEMPTY = B_KFULL + kMaxRing, B_VFULL = B_KEMPTY + kMaxRing
        B_COUNT = B_ROWS + 1 };
 static_assert(B_COUNT * 8 + 20 <= BAR_BYTES, "barrier block too small");
 
+// the rings' geometry, for the paged producer
+struct Ring128 {
+    static constexpr int NSK = 3, NSV = 3, STAGE = STAGE_BYTES, OFF_K = SMEM_K, OFF_V = SMEM_V;
+    static constexpr int KFULL = B_KFULL, KEMPTY = B_KEMPTY, VFULL = B_VFULL, VEMPTY = B_VEMPTY;
+};
+
 constexpr int SMEM_TABRING = SMEM_SCHED + ((int)sizeof(Sched) + 15) / 16 * 16;   // 8 steps x 8 block numbers (paged cache)
 constexpr int SMEM_TOTAL = SMEM_TABRING + 256;
 constexpr int SMEM_ALLOC = SMEM_TOTAL;                         // the base must come out 1024-byte aligned (checked)
 static_assert(SMEM_ALLOC <= 232448, "over the 227 KB a CTA may have");
-
-
-
-
-
-
-// ---- producer of a paged segment ---------------------------------------------------------------------
-// Paged cache: a step's 128 slots are 128 / page_rows pool blocks, each its own box.  Run by the whole producer
-// warp: lane j owns block j of every step - its table entry and its four copies (two d-halves of K and of V) -
-// so that one instruction issues the copies of all the step's blocks; lane 0 alone waits for the free stage and
-// posts the expected byte count.  The block numbers travel from the table to a small ring in shared memory by
-// asynchronous 4-byte copies issued six steps ahead of their use: a plain load held in a register that long would
-// share a scoreboard with the waits and copies in between and stall them for its whole latency.  Blocks that start
-// at or past kv_len + N are not fetched: their table entries need not exist, and the rows they would fill are
-// masked like any slot past the end.  Not inlined, so that it stays out of the kernel's register budget, and
-// everything by value, so that the caller's counters stay in registers.  Returns steps issued in full | K-only
-// step << 28 | a wait gave up << 29 | has waited for the preceding kernel << 30 (the same in every lane).
-constexpr int kTabRing = 4, kTabAhead = 3;     // steps held in a ring / steps a copy is issued ahead (two rings of
-                                               // 128 bytes: the K producer's and, where V has its own warp, the V producer's)
-__device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensorMap* k_map, const CUtensorMap* v_map,
-                                               int b, int kvh, int st0, int n, int S, uint32_t base, uint32_t bars,
-                                               uint32_t ring, volatile int* abort_flag, uint64_t pol, int it,
-                                               bool waited, int lane, int which /* 0: K and V, 1: K only, 2: V only */) {
-    auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
-    const int nsub = STEP / p.page_rows;
-    const uint32_t sub_bytes = (uint32_t)p.page_rows * 128u;
-    const int32_t* trow = p.block_table + (size_t)b * p.table_stride;
-    const int total = S + p.N;
-    const bool mine = lane < nsub;
-    auto issue = [&](int t) {                  // one group per step and lane, empty where there is nothing to fetch
-        const int blk = (st0 + t) * nsub + lane;
-        if (mine && t < n && blk * p.page_rows < total)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ring + 4u * (uint32_t)((t % kTabRing) * 8 + lane)), "l"(trow + blk) : "memory");
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    for (int t = 0; t < kTabAhead; ++t) issue(t);
-    uint32_t fail = 0;
-    int t = 0;
-    for (; t < n; ++t, ++it) {
-        issue(t + kTabAhead);
-        asm volatile("cp.async.wait_group %0;" ::"n"(kTabAhead) : "memory");     // this lane's entry of step t has landed
-        const int tok = (st0 + t) * STEP;
-        if (!waited && tok + STEP > S) { pdl_wait(); waited = true; }   // the tree's rows come from the preceding kernel
-        const bool load = mine && tok + lane * p.page_rows < total;
-        int c1 = 0, c2 = -p.page_rows;                                   // a box outside the pool: reads as zeros
-        if (load) {
-            int e;
-            asm volatile("ld.shared.s32 %0, [%1];" : "=r"(e) : "r"(ring + 4u * (uint32_t)((t % kTabRing) * 8 + lane)) : "memory");
-            if (e >= 0 && e < p.num_blocks) {
-                c1 = p.token_major ? kvh : 0;
-                c2 = p.token_major ? e * p.page_rows : e * p.Hkv + kvh;
-            } else if (p.status) {
-                atomicCAS(p.status, 0, VISPEC_E_RANGE);
-            }
-        }
-        const uint32_t tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, load)) * sub_bytes * 2u;
-        const int sk = it % NSK, sv = it % NSV;
-        bool w = true;
-        if (which != 2) {
-            if (lane == 0) {
-                w = mbar_wait(bar(B_KEMPTY + sk), ((it / NSK) & 1) ^ 1, abort_flag);
-                if (w) mbar_expect_tx(bar(B_KFULL + sk), tx);
-            }
-            w = __shfl_sync(0xffffffffu, w, 0);                          // the byte count is posted before any lane copies
-            if (!w) { fail = 2u << 28; break; }
-            if (load) {
-                tma_load_3d(base + SMEM_K + sk * STAGE_BYTES + lane * sub_bytes, k_map, bar(B_KFULL + sk), 0, c1, c2, pol);
-                tma_load_3d(base + SMEM_K + sk * STAGE_BYTES + HALF_BYTES + lane * sub_bytes, k_map, bar(B_KFULL + sk), 64, c1, c2, pol);
-            }
-        }
-        if (which != 1) {
-            if (lane == 0) {
-                w = mbar_wait(bar(B_VEMPTY + sv), ((it / NSV) & 1) ^ 1, abort_flag);
-                if (w) mbar_expect_tx(bar(B_VFULL + sv), tx);
-            }
-            w = __shfl_sync(0xffffffffu, w, 0);
-            if (!w) { fail = (which == 2 ? 2u : 3u) << 28; break; }      // (V only: nothing of this step was issued)
-            if (load) {
-                tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + lane * sub_bytes, v_map, bar(B_VFULL + sv), 0, c1, c2, pol);
-                tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES + lane * sub_bytes, v_map, bar(B_VFULL + sv), 64, c1, c2, pol);
-            }
-        }
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");                     // nothing of this segment stays in flight
-    return (uint32_t)t | fail | (waited ? 1u << 30 : 0u);
-}
 
 // ---- fused rotary embedding ---------------------------------------------------------------------------
 // Eight pairs (x = element j of the lower half, y = element j + D/2) rotated by their angles: fp64 with one rounding
@@ -422,7 +340,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     // unit's steps (an empty part still takes part in the exchange).  Otherwise: equal ranges of the line of
     // all steps.
     const int T = sched.base[p.B];
-    const int geff = CL ? (int)gridDim.x : (T > 0 ? sched_ctas(T, sched.units, (int)gridDim.x, p.min_steps) : 0);
+    const int geff = CL ? (int)gridDim.x : (T > 0 ? sched_ctas(T, sched.units, (int)gridDim.x, p.min_steps, sched_round_steps(p)) : 0);
     const bool active = cta < geff;
     const int lo = (!CL && active) ? cta_lo(cta, T, geff) : 0, hi = (!CL && active) ? cta_lo(cta + 1, T, geff) : 0;
     const uint32_t tmem = *tmem_slot;
@@ -454,7 +372,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             Seg sg;
             if constexpr (PAGED) {
                 while (ok && si.next(sg)) {
-                    const uint32_t r = produce_paged(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING, abort_flag, pol, it, waited, lane, split_v ? 1 : 0);
+                    const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING, abort_flag, pol, it, waited, lane, split_v ? 1 : 0);
                     const int done = (int)(r & 0x0fffffffu);
                     it += done; nv += split_v ? 0 : done; nk += done + (int)((r >> 28) & 1u);
                     ok = !((r >> 29) & 1u);
@@ -510,7 +428,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 SegIter si = make_iter();
                 Seg sg;
                 while (ok && si.next(sg)) {
-                    const uint32_t r = produce_paged(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING + 128, abort_flag, pol, it, waited, lane, 2);
+                    const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING + 128, abort_flag, pol, it, waited, lane, 2);
                     it += (int)(r & 0x0fffffffu);
                     ok = !((r >> 29) & 1u);
                     waited = (r >> 30) & 1u;
@@ -622,20 +540,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         pdl_wait();                                           // q, tree_mask and every output come after the preceding kernel
 
         // rejected sequences (kv_len < 0 or kv_len + N > S_max): zero output, -inf lse, status word
-        {
-            bool any_bad = false;
-            for (int b = 0; b < p.B; ++b) {
-                const int S = sched.len[b];
-                if (S >= 0 && S + N <= p.S_max) continue;
-                any_bad = true;
-                const int vecs = N * p.Hq * (D / 8);
-                uint4* o = reinterpret_cast<uint4*>(p.out + (size_t)b * N * p.Hq * D);
-                for (int i = cta * kSmx + st; i < vecs; i += (int)gridDim.x * kSmx) o[i] = make_uint4(0, 0, 0, 0);
-                if (p.lse)
-                    for (int i = cta * kSmx + st; i < N * p.Hq; i += (int)gridDim.x * kSmx) p.lse[(size_t)b * p.Hq * N + i] = -INFINITY;
-            }
-            if (any_bad && cta == 0 && st == 0) atomicCAS(p.status, 0, (int)VISPEC_E_RANGE);
-        }
+        zero_rejected<D>(p, sched, cta, st);
 
         // Q of a segment -> shared memory, rows in the swizzled K-major layout of a K stage (PAIR: rows 64-127
         // repeat rows 0-63).  Thread t moves 16-byte chunk t%16 of rows t/16, t/16 + 16, ... (head size 64: t%8 of t/8, t/8 + 32, ...)
@@ -1001,59 +906,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(TMEM_COLS) : "memory");
         }
         if (warp >= 4 && !*abort_flag) {
-        const int rp = (ROWS + ck - 1) / ck;
-        const int row0 = cr * rp;
-        const int nrows = min(rp, ROWS - row0);
-        const uint32_t pbuf_a = base + SMEM_K, pst_a = base + SMEM_K + (D / 4) * ROWS * 16;
-        // IT items (row, column quad) at a time per thread, all loads of all KM pieces issued before the first use
-        auto merge_items = [&](auto km_tag, auto it_tag) {
-            constexpr int KM = decltype(km_tag)::value, IT = decltype(it_tag)::value;
-            for (int item0 = tid - 128; item0 < nrows * (D / 4); item0 += kSmx * IT) {
-                float2 ml[IT][KM];
-                float4 pv[IT][KM];
-                int c4s[IT], grows[IT];
-#pragma unroll
-                for (int e = 0; e < IT; ++e) {
-                    const int item = item0 + e * kSmx;
-                    const int c4 = item / nrows, lr = row0 + (item - c4 * nrows);
-                    c4s[e] = c4;
-                    grows[e] = (item < nrows * (D / 4)) ? cl_seg.mblock * ROWS + lr : rows_total;
-#pragma unroll
-                    for (int j = 0; j < KM; ++j) {
-                        ml[e][j] = make_float2(-INFINITY, 0.f);
-                        pv[e][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (j < ck && grows[e] < rows_total) {
-                            ml[e][j] = dsmem_ld2(dsmem_addr(pst_a + lr * 8, (uint32_t)j));
-                            pv[e][j] = dsmem_ld4(dsmem_addr(pbuf_a + (c4 * ROWS + lr) * 16, (uint32_t)j));
-                        }
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < IT; ++e) {
-                    if (grows[e] >= rows_total) continue;
-                    float mm = -INFINITY;
-#pragma unroll
-                    for (int j = 0; j < KM; ++j) mm = fmaxf(mm, ml[e][j].x);
-                    const float m_fin = (mm == -INFINITY) ? 0.f : mm;
-                    float ll = 0.f;
-                    float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < KM; ++j) {
-                        const float w = exp2f(ml[e][j].x - m_fin);          // 0 for an empty or absent part
-                        ll += ml[e][j].y * w;
-                        a4.x += w * pv[e][j].x; a4.y += w * pv[e][j].y; a4.z += w * pv[e][j].z; a4.w += w * pv[e][j].w;
-                    }
-                    const float inv2 = ll > 0.f ? 1.f / ll : 0.f;
-                    const int nd = grows[e] / G, hd = cl_seg.kvh * G + grows[e] % G;
-                    *reinterpret_cast<uint2*>(p.out + (((size_t)cl_seg.b * N + nd) * p.Hq + hd) * D + c4s[e] * 4) =
-                        make_uint2(pack_bf16(a4.x * inv2, a4.y * inv2), pack_bf16(a4.z * inv2, a4.w * inv2));
-                    if (c4s[e] == 0 && p.lse)
-                        p.lse[((size_t)cl_seg.b * p.Hq + hd) * N + nd] = ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
-                }
-            }
-        };
-        if (ck <= 4) merge_items(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
-        else merge_items(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
+        cluster_merge<ROWS, D>(p, cl_seg, ck, cr, base + SMEM_K, base + SMEM_K + (D / 4) * ROWS * 16, tid - 128);
         }
     }
 
@@ -1108,7 +961,7 @@ stream_probe_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_cons
     if (!p.early) pdl_wait();
     __syncthreads();
     const int T = sched.base[p.B];
-    const int geff = T > 0 ? sched_ctas(T, sched.units, (int)gridDim.x, p.min_steps) : 0;
+    const int geff = T > 0 ? sched_ctas(T, sched.units, (int)gridDim.x, p.min_steps, sched_round_steps(p)) : 0;
     const int cta = blockIdx.x;
     if (cta < geff && lane == 0) {
         const int lo = cta_lo(cta, T, geff), hi = cta_lo(cta + 1, T, geff);
@@ -1277,11 +1130,44 @@ cudaError_t init_attn_tc5() {
     return cudaSuccess;
 }
 
-bool attn_tc5_uses_clusters(const AttnArgs& a) { return tc5_layout(a).ck > 0; }
+// Would units of 256 rows in two tiles (attn_tc5_wide.cu) serve the call better?  Both kernels are estimated the way
+// tc5_cluster_size does it, here with what its comparison of two forms of one kernel can leave out: an even split of
+// several row blocks per kv head uses a multiple of the units, and where there are more units than CTAs every further
+// segment of a CTA costs 11 us (Q tile, pipeline start, epilogue).  Measured, one-tile / two-tile kernel, us per layer
+// (16 query and 2 kv heads unless said otherwise): 8 x 128 nodes on 32768 tokens 345 / 273, on 4096 50.5 / 48.4; 1 x 128 on
+// 32768 47.6 / 44.0; 28 / 4 heads: 4 x 128 on 8192 90.8 / 80.9, 8 x 128 on 1000 47.9 / 36.7; 16 / 4 heads of size 64:
+// 6 x 128 on 3000 37.6 / 28.5.  Short ranges go the other way (4 x 60 on 8192 31.1 / 33.7, 28 / 4 heads 3 x 128 on 300
+// 18.8 / 21.1): the two-tile kernel's first step and epilogue are longer.
+static bool tc5_prefers_wide(const AttnArgs& a, const Tc5Layout& lay, const WidePlan& wide, double extra_us = 0.0) {
+    if (wide.est_us > 1e29 || lay.rows * lay.n_mblocks <= 128) return false;
+    const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
+    const int steps = (slots + STEP - 1) / STEP, units = a.B * a.Hkv * lay.n_mblocks;
+    const double hbm = a.D / 128.0, step_us = lay.pair ? 0.95 : a.D == 64 ? 1.08 : 1.2;
+    double est;
+    if (lay.ck > 0) {
+        est = (lay.pair ? 8.0 : 11.0) + (double)((steps + lay.ck - 1) / lay.ck) * fmax(step_us, (double)units * lay.ck * 0.0125 * hbm / lay.n_mblocks);
+    } else {
+        const double T = (double)steps * units;
+        const double n = units <= a.sm_count ? (double)(a.sm_count / units * units) : fmin((double)a.sm_count, fmax(1.0, T / 2.0));
+        est = 14.0 + (T / n) * fmax(step_us, n * 0.00973 * hbm / lay.n_mblocks) + 0.25 * n / units + (units > n ? 11.0 * units / n : 0.0);
+    }
+    return wide.est_us + extra_us < 0.97 * est;
+}
+
+// (the fused rotary embedding exists in the cluster form of the one-tile kernel; a call that goes elsewhere pays 3 us for
+// the rotation kernel, 2 of which the fused form would have cost too)
+bool attn_tc5_uses_clusters(const AttnArgs& a) {
+    const Tc5Layout lay = tc5_layout(a);
+    AttnArgs plain = a;
+    plain.rope_table = nullptr;
+    return lay.ck > 0 && !tc5_prefers_wide(a, lay, attn_tc5_wide_plan(plain), 1.0);
+}
 
 cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches) {
     *n_launches = 0;
     const Tc5Layout lay = tc5_layout(a);
+    const WidePlan wide = attn_tc5_wide_plan(a);
+    if (tc5_prefers_wide(a, lay, wide)) return launch_attn_tc5_wide(a, wide, st, n_launches);
     const bool pair = lay.pair;
     const int rows = lay.rows, n_mblocks = lay.n_mblocks, ck = lay.ck;
     const int units = a.B * a.Hkv * n_mblocks;

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_bf16.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "launch.cuh"
 #include "vispec_internal.h"
@@ -161,6 +162,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -227,6 +236,7 @@ struct Tc5Params {
     float scale_log2;
     int* status;
     int step;                  // cached tokens per pipeline step (rows of one K or V stage)
+    int lock;                  // even split by groups of n_mblocks CTAs: CTA c works for group c / n_mblocks on row block c % n_mblocks
 };
 
 // The schedule every CTA (and the merge kernel) derives from kv_len.
@@ -241,7 +251,7 @@ struct Sched {
 // Built by one full warp.  Reads kv_len only.
 static __device__ void sched_build(Sched& s, const Tc5Params& p, int lane, int kv_first) {   // kv_first: kv_len[lane], fetched by the caller
 
-    const int upb = p.Hkv * p.n_mblocks;        // units per sequence
+    const int upb = p.lock ? p.Hkv : p.Hkv * p.n_mblocks;        // units (lock: kv heads) per sequence
     int carry = 0;
     for (int b0 = 0; b0 < p.B; b0 += 32) {
         const int b = b0 + lane;
@@ -272,12 +282,19 @@ static __device__ void sched_build(Sched& s, const Tc5Params& p, int lane, int k
     if (lane == 0) s.units = live * upb;
 }
 // Number of CTAs that get work: every CTA at least min_steps steps; a multiple of the unit count when
-// the units are fewer than the CTAs (equally long units then never share a CTA).
-__device__ __forceinline__ int sched_ctas(int T, int units, int grid, int min_steps) {
+// the units are fewer than the CTAs (equally long units then never share a CTA) - unless the CTAs left out cost more
+// steps than a second segment's Q tile and epilogue in every CTA (round_steps).  Unaligned ranges put the row blocks of a
+// kv head, where they are units of their own, at different places of the cache, which is then read once per row block
+// (qwen3b_S32768_N128_B8 345 -> 417 us): those are always aligned.
+__device__ __forceinline__ int sched_round_steps(const Tc5Params& p) { return p.lock || p.n_mblocks == 1 ? 3 : 1 << 30; }
+__device__ __forceinline__ int sched_ctas(int T, int units, int grid, int min_steps, int round_steps) {
     int g = T / min_steps;
     g = g < 1 ? 1 : g;
     g = g < grid ? g : grid;
-    if (units <= g) g = (g / units) * units;
+    if (units <= g) {
+        const int r = (g / units) * units;
+        if (r != g && (T + r - 1) / r - (T + g - 1) / g <= round_steps) g = r;
+    }
     return g;
 }
 // (T * grid < 2^31 is checked on the host, so 32-bit arithmetic suffices)
@@ -331,8 +348,8 @@ template <int ROWS, int HD>
 __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o, const float2* __restrict__ part_ml,
                                                __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int geff,
                                                int ub, int c0, int c1, int b, int node, int head, int Hq, int N,
-                                               int lrow, int cw) {
-    auto slot_of = [&](int c) { return cta_lo(c, T, geff) >= ub ? 2 * c : 2 * c + 1; };
+                                               int lrow, int cw, int smul = 1, int sadd = 0) {
+    auto slot_of = [&](int c) { return (cta_lo(c, T, geff) >= ub ? 2 * c : 2 * c + 1) * smul + sadd; };
     // Segments are taken four at a time with every load of a group issued before the first use, so that a
     // group costs one memory round trip; groups are folded with the usual running-maximum rescale.
     float m_all = -INFINITY, l_all = 0.f;
@@ -393,8 +410,8 @@ template <int ROWS, int HD>
 __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, const float2* __restrict__ part_ml,
                                              __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int geff,
                                              int ub, int c0, int c1, int b, int node, int head, int Hq, int N,
-                                             int lrow, int c4) {
-    auto slot_of = [&](int c) { return cta_lo(c, T, geff) >= ub ? 2 * c : 2 * c + 1; };
+                                             int lrow, int c4, int smul = 1, int sadd = 0) {
+    auto slot_of = [&](int c) { return (cta_lo(c, T, geff) >= ub ? 2 * c : 2 * c + 1) * smul + sadd; };
     float m_all = -INFINITY, l_all = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int cb = c0; cb <= c1; cb += 16) {
@@ -463,6 +480,167 @@ struct RopeArgs {
 struct PagedArgs { const int32_t* block_table; int table_stride, page_rows, num_blocks, Hkv, N, token_major; int* status;
                    int* unit_counters; };   // even split: arrivals per unit (all zero between calls); nullptr: a merge kernel follows
 
+// ---- producer of a paged segment ---------------------------------------------------------------------
+// Paged cache: a step's 128 slots are 128 / page_rows pool blocks, each its own box.  Run by the whole producer
+// warp: lane j owns block j of every step - its table entry and its four copies (two d-halves of K and of V) -
+// so that one instruction issues the copies of all the step's blocks; lane 0 alone waits for the free stage and
+// posts the expected byte count.  The block numbers travel from the table to a small ring in shared memory by
+// asynchronous 4-byte copies issued six steps ahead of their use: a plain load held in a register that long would
+// share a scoreboard with the waits and copies in between and stall them for its whole latency.  Blocks that start
+// at or past kv_len + N are not fetched: their table entries need not exist, and the rows they would fill are
+// masked like any slot past the end.  Not inlined, so that it stays out of the kernel's register budget, and
+// everything by value, so that the caller's counters stay in registers.  Returns steps issued in full | K-only
+// step << 28 | a wait gave up << 29 | has waited for the preceding kernel << 30 (the same in every lane).
+constexpr int STEP = 128;                      // tokens per pipeline step = rows of one K or V stage
+constexpr int HALF_BYTES = STEP * 128;         // one d-half (64 columns) of a stage: 128 rows x 128 B
+constexpr int kTabRing = 4, kTabAhead = 3;     // steps held in a ring / steps a copy is issued ahead (two rings of
+                                               // 128 bytes: the K producer's and, where V has its own warp, the V producer's)
+template <class R>   // ring geometry: stages, bytes, offsets in shared memory, barrier indices
+__device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensorMap* k_map, const CUtensorMap* v_map,
+                                               int b, int kvh, int st0, int n, int S, uint32_t base, uint32_t bars,
+                                               uint32_t ring, volatile int* abort_flag, uint64_t pol, int it,
+                                               bool waited, int lane, int which /* 0: K and V, 1: K only, 2: V only */) {
+    auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
+    const int nsub = STEP / p.page_rows;
+    const uint32_t sub_bytes = (uint32_t)p.page_rows * 128u;
+    const int32_t* trow = p.block_table + (size_t)b * p.table_stride;
+    const int total = S + p.N;
+    const bool mine = lane < nsub;
+    auto issue = [&](int t) {                  // one group per step and lane, empty where there is nothing to fetch
+        const int blk = (st0 + t) * nsub + lane;
+        if (mine && t < n && blk * p.page_rows < total)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ring + 4u * (uint32_t)((t % kTabRing) * 8 + lane)), "l"(trow + blk) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int t = 0; t < kTabAhead; ++t) issue(t);
+    uint32_t fail = 0;
+    int t = 0;
+    for (; t < n; ++t, ++it) {
+        issue(t + kTabAhead);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kTabAhead) : "memory");     // this lane's entry of step t has landed
+        const int tok = (st0 + t) * STEP;
+        if (!waited && tok + STEP > S) { pdl_wait(); waited = true; }   // the tree's rows come from the preceding kernel
+        const bool load = mine && tok + lane * p.page_rows < total;
+        int c1 = 0, c2 = -p.page_rows;                                   // a box outside the pool: reads as zeros
+        if (load) {
+            int e;
+            asm volatile("ld.shared.s32 %0, [%1];" : "=r"(e) : "r"(ring + 4u * (uint32_t)((t % kTabRing) * 8 + lane)) : "memory");
+            if (e >= 0 && e < p.num_blocks) {
+                c1 = p.token_major ? kvh : 0;
+                c2 = p.token_major ? e * p.page_rows : e * p.Hkv + kvh;
+            } else if (p.status) {
+                atomicCAS(p.status, 0, VISPEC_E_RANGE);
+            }
+        }
+        const uint32_t tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, load)) * sub_bytes * 2u;
+        const int sk = it % R::NSK, sv = it % R::NSV;
+        bool w = true;
+        if (which != 2) {
+            if (lane == 0) {
+                w = mbar_wait(bar(R::KEMPTY + sk), ((it / R::NSK) & 1) ^ 1, abort_flag);
+                if (w) mbar_expect_tx(bar(R::KFULL + sk), tx);
+            }
+            w = __shfl_sync(0xffffffffu, w, 0);                          // the byte count is posted before any lane copies
+            if (!w) { fail = 2u << 28; break; }
+            if (load) {
+                tma_load_3d(base + R::OFF_K + sk * R::STAGE + lane * sub_bytes, k_map, bar(R::KFULL + sk), 0, c1, c2, pol);
+                tma_load_3d(base + R::OFF_K + sk * R::STAGE + HALF_BYTES + lane * sub_bytes, k_map, bar(R::KFULL + sk), 64, c1, c2, pol);
+            }
+        }
+        if (which != 1) {
+            if (lane == 0) {
+                w = mbar_wait(bar(R::VEMPTY + sv), ((it / R::NSV) & 1) ^ 1, abort_flag);
+                if (w) mbar_expect_tx(bar(R::VFULL + sv), tx);
+            }
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (!w) { fail = (which == 2 ? 2u : 3u) << 28; break; }      // (V only: nothing of this step was issued)
+            if (load) {
+                tma_load_3d(base + R::OFF_V + sv * R::STAGE + lane * sub_bytes, v_map, bar(R::VFULL + sv), 0, c1, c2, pol);
+                tma_load_3d(base + R::OFF_V + sv * R::STAGE + HALF_BYTES + lane * sub_bytes, v_map, bar(R::VFULL + sv), 64, c1, c2, pol);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");                     // nothing of this segment stays in flight
+    return (uint32_t)t | fail | (waited ? 1u << 30 : 0u);
+}
+
+// Rejected sequences (kv_len < 0 or kv_len + N > S_max): zero output, -inf lse, status word.  By the NT softmax threads.
+template <int HD, int NT = 256>
+__device__ __forceinline__ void zero_rejected(const Tc5Params& p, const Sched& sched, int cta, int st) {
+    const int N = p.N;
+    bool any_bad = false;
+    for (int b = 0; b < p.B; ++b) {
+        const int S = sched.len[b];
+        if (S >= 0 && S + N <= p.S_max) continue;
+        any_bad = true;
+        const int vecs = N * p.Hq * (HD / 8);
+        uint4* o = reinterpret_cast<uint4*>(p.out + (size_t)b * N * p.Hq * HD);
+        for (int i = cta * NT + st; i < vecs; i += (int)gridDim.x * NT) o[i] = make_uint4(0, 0, 0, 0);
+        if (p.lse)
+            for (int i = cta * NT + st; i < N * p.Hq; i += (int)gridDim.x * NT) p.lse[(size_t)b * p.Hq * N + i] = -INFINITY;
+    }
+    if (any_bad && cta == 0 && st == 0) atomicCAS(p.status, 0, (int)VISPEC_E_RANGE);
+}
+
+// Cluster form: rank cr of ck merges its rows of the unit's partials, parked by every rank at pbuf_a ([HD/4 col4][ROWS]
+// float4) and pst_a ([ROWS] (m, l)) of its own shared memory, and writes them out.  By the NT softmax threads (st).
+template <int ROWS, int HD, int NT = 256>
+__device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st) {
+    const int N = p.N, G = p.Hq / p.Hkv, rows_total = G * N;
+    const int rp = (ROWS + ck - 1) / ck;
+    const int row0 = cr * rp;
+    const int nrows = min(rp, ROWS - row0);
+    // IT items (row, column quad) at a time per thread, all loads of all KM pieces issued before the first use
+    auto merge_items = [&](auto km_tag, auto it_tag) {
+        constexpr int KM = decltype(km_tag)::value, IT = decltype(it_tag)::value;
+        for (int item0 = st; item0 < nrows * (HD / 4); item0 += NT * IT) {
+            float2 ml[IT][KM];
+            float4 pv[IT][KM];
+            int c4s[IT], grows[IT];
+#pragma unroll
+            for (int e = 0; e < IT; ++e) {
+                const int item = item0 + e * NT;
+                const int c4 = item / nrows, lr = row0 + (item - c4 * nrows);
+                c4s[e] = c4;
+                grows[e] = (item < nrows * (HD / 4)) ? sg.mblock * ROWS + lr : rows_total;
+#pragma unroll
+                for (int j = 0; j < KM; ++j) {
+                    ml[e][j] = make_float2(-INFINITY, 0.f);
+                    pv[e][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (j < ck && grows[e] < rows_total) {
+                        ml[e][j] = dsmem_ld2(dsmem_addr(pst_a + lr * 8, (uint32_t)j));
+                        pv[e][j] = dsmem_ld4(dsmem_addr(pbuf_a + (c4 * ROWS + lr) * 16, (uint32_t)j));
+                    }
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < IT; ++e) {
+                if (grows[e] >= rows_total) continue;
+                float mm = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < KM; ++j) mm = fmaxf(mm, ml[e][j].x);
+                const float m_fin = (mm == -INFINITY) ? 0.f : mm;
+                float ll = 0.f;
+                float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < KM; ++j) {
+                    const float w = exp2f(ml[e][j].x - m_fin);          // 0 for an empty or absent part
+                    ll += ml[e][j].y * w;
+                    a4.x += w * pv[e][j].x; a4.y += w * pv[e][j].y; a4.z += w * pv[e][j].z; a4.w += w * pv[e][j].w;
+                }
+                const float inv2 = ll > 0.f ? 1.f / ll : 0.f;
+                const int nd = grows[e] / G, hd = sg.kvh * G + grows[e] % G;
+                *reinterpret_cast<uint2*>(p.out + (((size_t)sg.b * N + nd) * p.Hq + hd) * HD + c4s[e] * 4) =
+                    make_uint2(pack_bf16(a4.x * inv2, a4.y * inv2), pack_bf16(a4.z * inv2, a4.w * inv2));
+                if (c4s[e] == 0 && p.lse)
+                    p.lse[((size_t)sg.b * p.Hq + hd) * N + nd] = ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
+            }
+        }
+    };
+    if (ck <= 4) merge_items(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
+    else merge_items(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
+}
+
 // Merge of the partials of every unit that more than one CTA worked on, 4 warps per block, lane <-> row.  Two
 // shapes (figures of head size 128): grid (unit, 2 * group of 32 rows + half of the columns), a warp sums 16 output
 // columns over the unit's segments four at a time - for units cut into a few pieces; FINE: grid (unit, 8 * group of 32
@@ -478,20 +656,21 @@ attn_tc5_merge_kernel(const Tc5Params p) {
     pdl_launch_dependents();
     // The schedule, recomputed per thread from kv_len (which the attention kernel does not write) without
     // shared memory: beside a resident attention CTA an SM has no shared memory to spare.
-    const int upb = p.Hkv * p.n_mblocks;
+    constexpr bool LOCK = ROWS == 256;                 // (p.lock, known at compile time)
+    const int upb = p.Hkv * p.n_mblocks, spb = LOCK ? p.Hkv : upb;      // units / units of the schedule per sequence
     const int unit = blockIdx.x, b = unit / upb, uib = unit - b * upb;
     int T = 0, live = 0, base_b = 0, steps = 0;
     for (int bb = 0; bb < p.B; ++bb) {
         const int S = p.kv_len[bb];
         const int st = (S >= 0 && S + p.N <= p.S_max) ? (S + p.N + p.step - 1) / p.step : 0;
         if (bb == b) { base_b = T; steps = st; }
-        T += st * upb;
-        live += st > 0 ? upb : 0;
+        T += st * spb;
+        live += st > 0 ? spb : 0;
     }
     pdl_wait();                                        // the partials are complete
     if (steps == 0) return;
-    const int geff = sched_ctas(T, live, p.grid_attn, p.min_steps);
-    const int ub = base_b + uib * steps, ue = ub + steps;
+    const int geff = sched_ctas(T, live, LOCK ? p.grid_attn / p.n_mblocks : p.grid_attn, p.min_steps, sched_round_steps(p));
+    const int ub = base_b + (LOCK ? uib / p.n_mblocks : uib) * steps, ue = ub + steps;
     const int c0 = cta_of(ub, T, geff), c1 = cta_of(ue - 1, T, geff);
     if (c0 == c1) return;                              // one CTA had the whole unit and wrote the output itself
     const int G = p.Hq / p.Hkv, N = p.N;
@@ -503,8 +682,9 @@ attn_tc5_merge_kernel(const Tc5Params p) {
     if (row >= G * N) return;
     const int node = row / G, head = kvh * G + row % G;
 
-    if (FINE) merge_row_c4<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
-    else merge_row_cols<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw);
+    const int smul = LOCK ? p.n_mblocks : 1, sadd = LOCK ? mblock : 0;
+    if (FINE) merge_row_c4<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
+    else merge_row_cols<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
 }
 
 }  // namespace tc5

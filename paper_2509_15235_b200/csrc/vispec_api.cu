@@ -67,7 +67,7 @@ bool init_device(int device) {
     static bool done[64];
     std::lock_guard<std::mutex> lock(mu);
     if (device < 64 && done[device]) return true;
-    const bool ok = init_attn_generic() == cudaSuccess && init_attn_tc5() == cudaSuccess && init_stream_probe() == cudaSuccess &&
+    const bool ok = init_attn_generic() == cudaSuccess && init_attn_tc5() == cudaSuccess && init_attn_tc5_wide() == cudaSuccess && init_stream_probe() == cudaSuccess &&
                     init_accept_sampled(device) == cudaSuccess;
     if (device < 64) done[device] = ok;
     return ok;

@@ -109,6 +109,11 @@ bool attn_tc5_supports(const AttnArgs& a);
 cudaError_t init_attn_tc5();           // once per device, with that device current
 cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches);
 bool attn_tc5_uses_clusters(const AttnArgs& a);   // the call would run in the cluster form (one launch, short calls)
+// The same with 256 query rows per unit (attn_tc5_wide.cu); est_us is 1e30 where it does not serve the call.
+struct WidePlan { int ck, grid; double est_us; };   // cluster size (0: even split in lock-step groups), CTAs, estimate
+cudaError_t init_attn_tc5_wide();
+WidePlan attn_tc5_wide_plan(const AttnArgs& a);
+cudaError_t launch_attn_tc5_wide(const AttnArgs& a, const WidePlan& w, cudaStream_t st, int* n_launches);
 // The bounded wait of the attention kernels on a barrier that never completes (failure-detection self-test).
 cudaError_t launch_bounded_wait_selftest(long long limit, int* status, int* counters, cudaStream_t st);
 // positions[b][i] == kv_len[b] + popcount(mask row i) - 1, else status VISPEC_E_POSITIONS.

@@ -90,6 +90,30 @@ def test_head_size_64_edges(gu, Hq, Hkv, N, S, S_max, split_form):
     _check(gu, q, k, v, kv_len, mask, 1 / math.sqrt(D), split_form=split_form)
 
 
+# Units of 256 query rows in two tiles, which the host chooses by the capacity (40000 slots: mostly NaN here): an empty cache
+# and several steps; a second block whose second tile has 36 rows; a third block with 4 rows in its second tile; 136 rows,
+# 8 of them in the second tile; head size 64; clusters of three CTAs and of one; more kv heads than groups of CTAs (several segments per CTA).
+@pytest.mark.parametrize("Hq,Hkv,D,N,kv_len,S_max,split_form", [
+    (16, 2, 128, 128, [0, 700], 40000, 0), (28, 4, 128, 60, [1, 1000], 40000, 0), (16, 2, 128, 128, [700, 0, 64, 333, 5], 20000, 2),
+    (28, 4, 128, 92, [515, 127], 40000, 0), (8, 1, 128, 17, [250, 40], 40000, 0), (16, 4, 64, 100, [3000, 64], 40000, 0),
+    (16, 4, 64, 128, [172, 1, 100, 172, 30, 128, 77, 0, 172, 129], 300, 2), (28, 4, 128, 128, [172, 1, 100, 172, 30, 128, 77, 0, 172, 129], 300, 0),
+])
+def test_two_tile_units(gu, Hq, Hkv, D, N, kv_len, S_max, split_form):
+    B, used = len(kv_len), max(kv_len) + N
+    rng = np.random.Generator(np.random.Philox(Hq * 1000 + N + D))
+    q = synth.normal_bf16((B, N, Hq, D), 15 + N)
+    k = np.full((B, Hkv, S_max, D), 0x7FC0, dtype=np.uint16)
+    v = np.full((B, Hkv, S_max, D), 0x7FC0, dtype=np.uint16)
+    k[:, :, :used] = synth.normal_bf16((B, Hkv, used, D), 16 + N)
+    v[:, :, :used] = synth.normal_bf16((B, Hkv, used, D), 17 + N)
+    for b in range(B):
+        k[b, :, kv_len[b] + N:] = 0x7FC0
+        v[b, :, kv_len[b] + N:] = 0x7FC0
+    parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
+    mask, _, _ = oracle.tree_mask(parents)
+    _check(gu, q, k, v, np.array(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=split_form)
+
+
 def test_arbitrary_mask_bits_all_ones_and_zero_rows(gu):
     B, N, Hq, Hkv, D, S_max = 2, 20, 4, 2, 128, 256
     q = synth.normal_bf16((B, N, Hq, D), 21); k = synth.normal_bf16((B, Hkv, S_max, D), 22)

@@ -95,6 +95,22 @@ def test_paged_attention_equals_contiguous_and_oracle(page_rows, split_form, tok
     assert st == 0 and np.array_equal(out, ref) and np.array_equal(lse, ref_lse)
 
 
+@pytest.mark.parametrize("page_rows", [16, 64, 128])
+def test_paged_attention_two_tile_units(page_rows):
+    """Units of 256 rows, which the host chooses by the table's capacity (40960 slots, of which few are in use)."""
+    q, k, v, kv_len, mask, rng = _case(2, 60, 28, 4, [1000, 70], 1152, 700 + page_rows)
+    scale = 1 / math.sqrt(128)
+    pools, table = _page((k, v), page_rows, rng)
+    wide = np.full((2, 40960 // page_rows), 2 ** 30, dtype=np.int32)
+    for b in range(2):
+        used = -(-(int(kv_len[b]) + 60) // page_rows)
+        wide[b, :used] = table[b, :used]
+    out, lse, status = _run_paged(q, pools, wide, kv_len, mask, scale)
+    want, want_lse = oracle.tree_attn(q, k, v, kv_len, mask, scale)
+    assert status == 0 and not np.isnan(out).any()
+    assert np.abs(out - want).max() <= TOL and np.abs(lse - want_lse).max() <= LSE_TOL
+
+
 @pytest.mark.parametrize("B,N,Hq,Hkv,S_list,S_max,page_rows,token_major", [
     (2, 128, 8, 1, [200, 77], 384, 32, False),       # largest tree: 1024 query rows per kv head, two mask words
     (2, 1, 4, 2, [129, 0], 256, 16, True),           # a single node (plain decode step); an empty prefix
