@@ -1053,69 +1053,69 @@ static int query_max_clusters(bool pair, int k) {
     return n;
 }
 
-// Cluster size for the cluster form, or 0 when the even split with partials in global memory serves better:
-// one cluster per unit, all clusters co-resident.  `pair`: units of at most 64 rows in the duplicated-row layout,
-// n_mblocks of them per kv head.  *est_us: the estimate of the form it returns.
-static int tc5_cluster_size(const AttnArgs& a, bool pair, int n_mblocks, double* est_us = nullptr, bool clusters_if_possible = false) {
+// Estimates in microseconds per call, fitted to measurements over the long-response shapes (16 query and 2 kv heads, 2048 to
+// 32768 tokens, 16 to 128 nodes, 1 to 8 sequences) and the 7B and 13B ones: a fixed part, then the steps of the busiest
+// CTA, each at the rate its softmax warps reach (a little slower the more SMs are at work) or at its share of HBM (64 KB
+// per step over 7 TB/s; the row blocks of a kv head read the same tiles, so one in n_mblocks comes from HBM; a
+// step's bytes follow the head size, its softmax does not).  The host knows only the capacity S_max, not kv_len: the
+// estimate is for full caches unless the caller has given the length it expects (VISPEC_OPT_KV_LEN_HINT).
+static double tc5_step_us(const AttnArgs& a, bool pair, int n_mblocks, double ctas) {
+    const double busy = ctas / a.sm_count, compute = pair ? 0.8 + 0.25 * busy : 1.05 + 0.15 * busy;
+    return fmax(a.D == 64 ? 0.9 * compute : compute, ctas * 0.0093 * (a.D / 128.0) / n_mblocks);
+}
+static int tc5_steps(const AttnArgs& a) {
+    const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
+    return (slots + STEP - 1) / STEP;
+}
+static double tc5_cluster_us(const AttnArgs& a, bool pair, int n_mblocks, int k) {
+    return (pair ? 6.9 : 9.6) + (double)((tc5_steps(a) + k - 1) / k) * tc5_step_us(a, pair, n_mblocks, (double)a.B * a.Hkv * n_mblocks * k);
+}
+// (even split: the CTAs as sched_ctas counts them; partials of 128 rows cost 34 ns per CTA, written and merged, those of 64
+// rows go in the fixed part; where there are more units than CTAs every further segment of a CTA costs a Q tile, a
+// pipeline start and an epilogue)
+static double tc5_even_us(const AttnArgs& a, bool pair, int n_mblocks) {
     const int units = a.B * a.Hkv * n_mblocks;
-    if (est_us) *est_us = 1e30;
-    if (a.tc5_path == 1 || a.tc5_path == 3) return 0;
+    const double T = (double)tc5_steps(a) * units;
+    double n = fmin((double)a.sm_count, fmax(1.0, floor(T / 2.0)));
+    if (units <= n) {
+        const double r = floor(n / units) * units;
+        if (n_mblocks > 1 || ceil(T / r) - ceil(T / n) <= 3.0) n = r;
+    }
+    return (pair ? 9.5 : 10.4 + 0.034 * n) + ceil(T / n) * tc5_step_us(a, pair, n_mblocks, n) + (units > n && n_mblocks > 1 ? 11.0 * units / n : 0.0);
+}
+
+// Cluster size of the cluster form: one cluster per unit, as large as all clusters fit at once (0: they do not).
+static int tc5_max_cluster(const AttnArgs& a, bool pair, int n_mblocks) {
+    const int units = a.B * a.Hkv * n_mblocks;
     int best = 0;
     for (int k = 1; k <= 8; ++k)
         if (units * k <= a.sm_count && g_max_clusters[pair][k] >= units) best = k;
-    if (best == 0) return 0;
-    if (a.tc5_path == 2 || clusters_if_possible) return best;
-    // Both forms, estimated in microseconds from what was measured over the workloads (the long-response sweep
-    // cells, the 7B and 13B shapes): a fixed part (11 for the cluster form, 14 for the even split with its partials
-    // and second phase), the steps of the busiest CTA at 1.2 per step or at the HBM share of that many CTAs (64 KB
-    // per step at 5.2 TB/s over the cluster form's CTAs, 6.6 TB/s over the even split's; the row blocks of one kv
-    // head read the same tiles, so only one in n_mblocks comes from HBM), and 0.25 per partial a unit is merged
-    // from.  The host knows only the capacity S_max, not kv_len: the estimate is for full caches unless the caller
-    // has given the length it expects (VISPEC_OPT_KV_LEN_HINT).
-    const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
-    const double steps = (double)((slots + STEP - 1) / STEP), T = steps * units;
-    const double hbm = a.D / 128.0;        // a step's bytes follow the head size, its softmax does not
-    const double n_c = (double)units * best, per_c = (double)(((slots + STEP - 1) / STEP + best - 1) / best);
-    const double est_c = 11.0 + per_c * fmax(1.2, n_c * 0.0125 * hbm / n_mblocks);
-    const double n_e = fmin((double)a.sm_count, fmax(1.0, T / 2.0));
-    // (merge: 0.25 per piece of a unit; from four pieces on the fine-grained merge kernel, 1 + 0.055 per piece)
-    const double pieces = n_e / units;
-    const double est_e = 14.0 + (T / n_e) * fmax(1.2, n_e * 0.00973 * hbm / n_mblocks) + (pieces >= 4.0 ? 1.0 + 0.055 * pieces : 0.25 * pieces);
-    // (units of several row blocks per kv head in small clusters: measured over the sweep, the even split's steps come
-    // out dearer than the estimate there - 54.8 against 52.6 us on qwen3b_S8192_N60_B8, 96.1 against 92.4 on
-    // qwen3b_S16384_N128_B4 - so the clusters get a tenth of tolerance)
-    const double tol = (n_mblocks > 1 && best <= 4) ? 1.1 : 1.0;
-    if (est_us) *est_us = est_c <= tol * est_e ? est_c : est_e;
-    return est_c <= tol * est_e ? best : 0;
+    return best;
 }
 
-// Row layout of a call.  At most 64 query rows per kv head: one unit of 64 rows, rows duplicated over the two lane
+// Row layout and form of a call.  At most 64 query rows per kv head: one unit of 64 rows, rows duplicated over the two lane
 // halves.  More: blocks of 128 rows, lane = row - unless that leaves most of the GPU idle (few sequences and kv
 // heads, rows just over 64: one cluster of at most 8 CTAs per unit is all the cluster form can use): then blocks of 64
 // rows in the duplicated layout make twice the units, and a step of such a unit costs its softmax threads half the
-// columns (measured per step and CTA: 0.9 against 1.4-1.8 us), at the price of every K/V tile crossing from L2 twice as
-// often and half of each product computed for nothing.  Taken when both layouts would run as clusters and the
-// estimate (steps of the busiest CTA at those rates) says a twentieth less or better.
-struct Tc5Layout { bool pair; int rows, n_mblocks, ck; };
+// columns, at the price of every K/V tile crossing from L2 twice as often and half of each product computed for nothing.
+// (As an even split the smaller blocks gain nothing.)  The best estimate decides, a form that options ask for first.
+struct Tc5Layout { bool pair; int rows, n_mblocks, ck; double est_us; };
 static Tc5Layout tc5_layout(const AttnArgs& a) {
     const int rows_total = (a.Hq / a.Hkv) * a.N;
-    Tc5Layout full = {rows_total <= 64, rows_total <= 64 ? 64 : 128, rows_total <= 64 ? 1 : (rows_total + 127) / 128, 0};
-    double est_full = 0.0;
-    full.ck = tc5_cluster_size(a, full.pair, full.n_mblocks, &est_full);
-    if (full.pair || a.tc5_path != 0) return full;
-    Tc5Layout half = {true, 64, (rows_total + 63) / 64, 0};
-    half.ck = tc5_cluster_size(a, true, half.n_mblocks, nullptr, true);     // (clusters or nothing: the even split gains nothing from smaller blocks)
-    if (half.ck == 0) return full;
-    const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
-    const int steps = (slots + STEP - 1) / STEP;
-    auto est = [&](const Tc5Layout& l, double step_us) {
-        const double n_c = (double)a.B * a.Hkv * l.n_mblocks * l.ck;
-        return 11.0 + (double)((steps + l.ck - 1) / l.ck) * fmax(step_us, n_c * 0.0125 * (a.D / 128.0) / l.n_mblocks);
-    };
-    if (full.ck > 0) return est(half, 0.95) < 0.95 * est(full, full.n_mblocks > 1 ? 1.7 : 1.45) ? half : full;
-    // 128-row blocks would go as an even split (its estimate: est_full); small clusters of 64-row blocks, whose fixed
-    // part measures 8 rather than 11 us, against that
-    return est(half, 0.95) - 3.0 < 0.95 * est_full ? half : full;
+    const bool small = rows_total <= 64;
+    const int nmb = small ? 1 : (rows_total + 127) / 128, k = tc5_max_cluster(a, small, nmb);
+    const bool want_even = a.tc5_path == 1 || a.tc5_path == 3, want_clusters = a.tc5_path == 2;
+    Tc5Layout best = {small, small ? 64 : 128, nmb, 0, tc5_even_us(a, small, nmb)};
+    if (k > 0 && !want_even) {
+        const double us = tc5_cluster_us(a, small, nmb, k);
+        if (want_clusters || us <= best.est_us) { best.ck = k; best.est_us = us; }
+    }
+    if (!small && a.tc5_path == 0) {
+        const int nmb64 = (rows_total + 63) / 64, k64 = tc5_max_cluster(a, true, nmb64);
+        const double us = k64 > 0 ? tc5_cluster_us(a, true, nmb64, k64) : 1e30;
+        if (us < best.est_us) best = {true, 64, nmb64, k64, us};
+    }
+    return best;
 }
 
 bool attn_tc5_supports(const AttnArgs& a) {
@@ -1149,40 +1149,18 @@ cudaError_t init_attn_tc5() {
     }
     for (int k = 1; k <= 8; ++k) { g_max_clusters[0][k] = query_max_clusters(false, k); g_max_clusters[1][k] = query_max_clusters(true, k); }
     if (getenv("VISPEC_DEBUG")) for (int k = 1; k <= 8; ++k) fprintf(stderr, "vispec: cluster size %d: %d (rows > 64) / %d (rows <= 64) co-resident clusters\n", k, g_max_clusters[0][k], g_max_clusters[1][k]);
-    // The merge blocks must be able to join an SM that an attention CTA has configured for maximum shared memory.
-    const void* merge_kernels[8] = {(const void*)attn_tc5_merge_kernel<64>, (const void*)attn_tc5_merge_kernel<128>,
-                                    (const void*)attn_tc5_merge_kernel<64, true>, (const void*)attn_tc5_merge_kernel<128, true>,
-                                    (const void*)attn_tc5_merge_kernel<64, false, 64>, (const void*)attn_tc5_merge_kernel<128, false, 64>,
-                                    (const void*)attn_tc5_merge_kernel<64, true, 64>, (const void*)attn_tc5_merge_kernel<128, true, 64>};
-    for (const void* k : merge_kernels) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-    }
+    for (cudaError_t m : {init_merge<64, 128>(), init_merge<128, 128>(), init_merge<64, 64>(), init_merge<128, 64>()})
+        if (m != cudaSuccess) return m;
     return cudaSuccess;
 }
 
-// Would units of 256 rows in two tiles (attn_tc5_wide.cu) serve the call better?  Both kernels are estimated the way
-// tc5_cluster_size does it, here with what its comparison of two forms of one kernel can leave out: an even split of
-// several row blocks per kv head uses a multiple of the units, and where there are more units than CTAs every further
-// segment of a CTA costs 11 us (Q tile, pipeline start, epilogue).  Measured, one-tile / two-tile kernel, us per layer
-// (16 query and 2 kv heads unless said otherwise): 8 x 128 nodes on 32768 tokens 345 / 273, on 4096 50.5 / 48.4; 1 x 128 on
-// 32768 47.6 / 44.0; 28 / 4 heads: 4 x 128 on 8192 90.8 / 80.9, 8 x 128 on 1000 47.9 / 36.7; 16 / 4 heads of size 64:
-// 6 x 128 on 3000 37.6 / 28.5.  Short ranges go the other way (4 x 60 on 8192 31.1 / 33.7, 28 / 4 heads 3 x 128 on 300
-// 18.8 / 21.1): the two-tile kernel's first step and epilogue are longer.
+// Would units of 256 rows in two tiles (attn_tc5_wide.cu) serve the call better?  Measured, one-tile / two-tile kernel, us
+// per layer (16 query and 2 kv heads unless said otherwise): 8 x 128 nodes
+// on 32768 tokens 345 / 273, on 4096 47.4 / 45.7, on 2048 30.2 / 31.8; 8 x 60 on 16384 88.5 / 80.6; 28 / 4 heads: 8 x 60 on 8192
+// 89.5 / 81.1, 8 x 128 on 1000 43.8 / 36.7, 3 x 128 on 300 16.6 / 20.9; 16 / 4 heads of size 64: 6 x 128 on 3000 34.3 /
+// 27.9, 4 x 100 on 4096 25.0 / 26.0.  The two-tile kernel's steps are cheaper, its first step and its epilogue longer.
 static bool tc5_prefers_wide(const AttnArgs& a, const Tc5Layout& lay, const WidePlan& wide, double extra_us = 0.0) {
-    if (wide.est_us > 1e29 || lay.rows * lay.n_mblocks <= 128) return false;
-    const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
-    const int steps = (slots + STEP - 1) / STEP, units = a.B * a.Hkv * lay.n_mblocks;
-    const double hbm = a.D / 128.0, step_us = lay.pair ? 0.95 : a.D == 64 ? 1.08 : 1.2;
-    double est;
-    if (lay.ck > 0) {
-        est = (lay.pair ? 8.0 : 11.0) + (double)((steps + lay.ck - 1) / lay.ck) * fmax(step_us, (double)units * lay.ck * 0.0125 * hbm / lay.n_mblocks);
-    } else {
-        const double T = (double)steps * units;
-        const double n = units <= a.sm_count ? (double)(a.sm_count / units * units) : fmin((double)a.sm_count, fmax(1.0, T / 2.0));
-        est = 14.0 + (T / n) * fmax(step_us, n * 0.00973 * hbm / lay.n_mblocks) + 0.25 * n / units + (units > n ? 11.0 * units / n : 0.0);
-    }
-    return wide.est_us + extra_us < 0.97 * est;
+    return wide.est_us < 1e29 && wide.est_us + extra_us < 0.98 * lay.est_us;
 }
 
 // (the fused rotary embedding exists in the cluster form of the one-tile kernel; a call that goes elsewhere pays 3 us for
@@ -1252,16 +1230,8 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     if (err != cudaSuccess) return err;
     ++*n_launches;
     if (ck > 0 || own_merge) return cudaSuccess;
-    // the merge: fine-grained where units are cut into many pieces
-    auto launch_merge = [&](auto hd) {
-        constexpr int HD = decltype(hd)::value;
-        if (grid >= 4 * units)
-            return pair ? launch_pdl(attn_tc5_merge_kernel<64, true, HD>, dim3(units, HD / 8), dim3(128), 0, st, 0, p)
-                        : launch_pdl(attn_tc5_merge_kernel<128, true, HD>, dim3(units, HD / 4), dim3(128), 0, st, 0, p);
-        return pair ? launch_pdl(attn_tc5_merge_kernel<64, false, HD>, dim3(units, HD / 32), dim3(128), 0, st, 0, p)
-                    : launch_pdl(attn_tc5_merge_kernel<128, false, HD>, dim3(units, HD / 16), dim3(128), 0, st, 0, p);
-    };
-    err = a.D == 64 ? launch_merge(std::integral_constant<int, 64>{}) : launch_merge(std::integral_constant<int, 128>{});
+    err = a.D == 64 ? (pair ? launch_merge<64, 64>(p, units, grid, st) : launch_merge<128, 64>(p, units, grid, st))
+                    : (pair ? launch_merge<64, 128>(p, units, grid, st) : launch_merge<128, 128>(p, units, grid, st));
     if (err != cudaSuccess) return err;
     ++*n_launches;
     return cudaSuccess;

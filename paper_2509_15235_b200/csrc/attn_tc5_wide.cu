@@ -523,12 +523,8 @@ cudaError_t init_attn_tc5_wide() {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_ALLOC);
         if (e != cudaSuccess) return e;
     }
-    const void* merge_kernels[4] = {(const void*)attn_tc5_merge_kernel<256, false, 128>, (const void*)attn_tc5_merge_kernel<256, true, 128>,
-                                    (const void*)attn_tc5_merge_kernel<256, false, 64>, (const void*)attn_tc5_merge_kernel<256, true, 64>};
-    for (const void* k : merge_kernels) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-    }
+    for (cudaError_t m : {init_merge<256, 128>(), init_merge<256, 64>()})
+        if (m != cudaSuccess) return m;
     for (int k = 1; k <= 8; ++k) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(k * 64); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = SMEM_ALLOC;
@@ -550,7 +546,7 @@ WidePlan attn_tc5_wide_plan(const AttnArgs& a) {
     if (rows_total <= 128 || a.rope_table || nmb > a.sm_count) return w;
     const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
     const double steps = (double)((slots + STEP - 1) / STEP), hbm = a.D / 128.0;
-    const double step_us = a.D == 64 ? 1.6 : 2.15;              // a 128-token step of both tiles
+    // (fixed part and time of a 128-token step of both tiles, fitted like the one-tile kernel's estimates in attn_tc5.cu)
     if (a.tc5_path != 1 && a.tc5_path != 3) {
         int best = 0;
         for (int k = 1; k <= 8; ++k)
@@ -558,7 +554,7 @@ WidePlan attn_tc5_wide_plan(const AttnArgs& a) {
         if (best) {
             const double per = (double)(((int)steps + best - 1) / best);
             w.ck = best; w.grid = units * best;
-            w.est_us = 15.0 + per * fmax(step_us, (double)units * best * 0.0125 * hbm / nmb);
+            w.est_us = (a.D == 64 ? 13.5 : 16.0) + per * fmax(a.D == 64 ? 1.65 : 1.8, (double)units * best * 0.0093 * hbm / nmb);
             if (a.tc5_path == 2) return w;
         }
     }
@@ -566,10 +562,14 @@ WidePlan attn_tc5_wide_plan(const AttnArgs& a) {
     const long long t_max = (long long)a.B * a.Hkv * (long long)((a.S_max + STEP - 1) / STEP);
     const int groups = (int)(t_max < groups_max ? t_max : groups_max);
     if (kCounterBytes + (size_t)2 * groups * nmb * kRows * (a.D * 4 + 8) > a.ws_bytes) return w;
-    const double T = steps * a.B * a.Hkv, n_g = fmin((double)groups, fmax(1.0, T / 2.0)), pieces = n_g / ((double)a.B * a.Hkv);
-    // (a range is half a step longer than the average, for its remainder; heads beyond one per group cost a segment)
-    const double est = 14.0 + (T / n_g + 0.5) * fmax(step_us, n_g * 0.00973 * hbm) + (pieces >= 4.0 ? 0.055 * pieces : 0.0) +
-                       (pieces < 1.0 ? 11.0 / pieces : 0.0);
+    const int heads = a.B * a.Hkv;
+    const double T = steps * heads;
+    double n = fmin((double)groups, fmax(1.0, floor(T / 2.0)));
+    if (heads <= n) {                          // as sched_ctas counts the groups
+        const double r = floor(n / heads) * heads;
+        if (ceil(T / r) - ceil(T / n) <= 3.0) n = r;
+    }
+    const double est = (a.D == 64 ? 13.7 : 15.5) + ceil(T / n) * fmax(a.D == 64 ? 1.6 : 2.0, n * 0.0093 * hbm) + (heads > n ? 11.0 * heads / n : 0.0);
     if (est < w.est_us) { w.ck = 0; w.grid = groups * nmb; w.est_us = est; }
     return w;
 }
@@ -598,10 +598,7 @@ cudaError_t launch_attn_tc5_wide(const AttnArgs& a, const WidePlan& w, cudaStrea
     if (err != cudaSuccess) return err;
     ++*n_launches;
     if (w.ck > 0) return cudaSuccess;
-    const bool fine = w.grid >= 4 * units;
-    auto merge = [&](auto kernel, int cb) { return launch_pdl(kernel, dim3(units, kRows / 32 * cb), dim3(128), 0, st, 0, p); };
-    if (a.D == 64) err = fine ? merge(attn_tc5_merge_kernel<256, true, 64>, 4) : merge(attn_tc5_merge_kernel<256, false, 64>, 1);
-    else err = fine ? merge(attn_tc5_merge_kernel<256, true, 128>, 8) : merge(attn_tc5_merge_kernel<256, false, 128>, 2);
+    err = a.D == 64 ? launch_merge<256, 64>(p, units, w.grid, st) : launch_merge<256, 128>(p, units, w.grid, st);
     if (err != cudaSuccess) return err;
     ++*n_launches;
     return cudaSuccess;

@@ -409,26 +409,29 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
         lse[((size_t)b * Hq + head) * N + node] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
 }
 
-// One (row, 4 output columns) of a unit, the merge kernel's piece: sixteen segments at a time with every load issued
-// before the first use (a unit cut over many CTAs - few sequences, long caches - is merged from dozens of partials,
-// and a round of loads is a memory round trip).
-template <int ROWS, int HD>
+// One (row, 4 output columns) of a unit, the merge kernel's fine piece, by Q lanes of a warp (lanes 32/Q apart): lane part
+// `part` takes the segments c0 + part, c0 + part + Q, ..., U at a time with every load issued before the first use (a
+// unit cut over many CTAs - few sequences, long caches - is merged from dozens of partials, and a round of loads is a memory
+// round trip); the Q sums meet by shuffles.  All lanes of the warp take part; those of a row that does not exist pass
+// row_ok = false.
+template <int ROWS, int HD, int Q>
 __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, const float2* __restrict__ part_ml,
                                              __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int geff,
                                              int ub, int c0, int c1, int b, int node, int head, int Hq, int N,
-                                             int lrow, int c4, int smul = 1, int sadd = 0) {
+                                             int lrow, int c4, int part, bool row_ok, int smul, int sadd) {
+    constexpr int U = Q == 1 ? 16 : 10;
     auto slot_of = [&](int c) { return (cta_lo(c, T, geff) >= ub ? 2 * c : 2 * c + 1) * smul + sadd; };
     float m_all = -INFINITY, l_all = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int cb = c0; cb <= c1; cb += 16) {
-        float2 ml[16];
-        float4 v[16];
+    for (int cb = c0; cb <= c1; cb += Q * U) {
+        float2 ml[U];
+        float4 v[U];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int c = cb + j;
+        for (int j = 0; j < U; ++j) {
+            const int c = cb + part + j * Q;
             ml[j] = make_float2(-INFINITY, 0.f);
             v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c <= c1) {
+            if (c <= c1 && row_ok) {
                 const int slot = slot_of(c);
                 ml[j] = __ldcg(&part_ml[(size_t)slot * ROWS + lrow]);
                 v[j] = __ldcg(part_o + ((size_t)slot * (HD / 4) + c4) * ROWS + lrow);
@@ -436,19 +439,32 @@ __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, 
         }
         float m_new = m_all;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) m_new = fmaxf(m_new, ml[j].x);
+        for (int j = 0; j < U; ++j) m_new = fmaxf(m_new, ml[j].x);
         const float m_fin = (m_new == -INFINITY) ? 0.f : m_new;
         const float a = exp2f(m_all - m_fin);                 // 0 while nothing has been accumulated
         l_all *= a;
         acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
+        for (int j = 0; j < U; ++j) {
             const float w = exp2f(ml[j].x - m_fin);           // 0 for a segment that saw nothing (or is absent)
             l_all += ml[j].y * w;
             acc.x += w * v[j].x; acc.y += w * v[j].y; acc.z += w * v[j].z; acc.w += w * v[j].w;
         }
         m_all = m_new;
     }
+#pragma unroll
+    for (int o = 32 / Q; o < 32; o <<= 1) {
+        const float m_o = __shfl_xor_sync(0xffffffffu, m_all, o), m_new = fmaxf(m_all, m_o);
+        const float m_fin = (m_new == -INFINITY) ? 0.f : m_new;
+        const float a = exp2f(m_all - m_fin);
+        // (both sides scale by their own weight before the exchange, so the sum is the same in all of them)
+        l_all *= a; acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a;
+        l_all += __shfl_xor_sync(0xffffffffu, l_all, o);
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+        m_all = m_new;
+    }
+    if (!row_ok || part != 0) return;
     const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
     *reinterpret_cast<uint2*>(out + (((size_t)b * N + node) * Hq + head) * HD + c4 * 4) =
         make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
@@ -647,15 +663,15 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
     else merge_items(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
 }
 
-// Merge of the partials of every unit that more than one CTA worked on, 4 warps per block, lane <-> row.  Two
-// shapes (figures of head size 128): grid (unit, 2 * group of 32 rows + half of the columns), a warp sums 16 output
-// columns over the unit's segments four at a time - for units cut into a few pieces; FINE: grid (unit, 8 * group of 32
-// rows + eighth of the columns), a warp sums 4 output columns sixteen segments at a time - for units cut over many CTAs (few sequences, long
-// caches), where the rounds of loads are what the merge takes: qwen3b_S32768_N16_B1 (2 units over 148 CTAs) 42.7 ->
-// 29.1 us per layer, qwen3b_S32768_N60_B1 34.8 -> 31.8; with many units of two partials the coarse shape is 3 % faster.
-// The blocks are small so that they fit beside a resident attention CTA: they are launched early
-// (programmatic dependent launch) and must not keep the next layer's attention CTAs off the SMs.
-template <int ROWS, bool FINE = false, int HD = 128>
+// Merge of the partials of every unit that more than one CTA worked on, 4 warps per block.  Q = 0, coarse: grid (unit, group
+// of 32 rows x group of 64 columns), lane <-> row, a warp sums 16 output columns over the unit's segments four at a time -
+// for units cut into a few pieces.  Q = 1, 2, 4, 8, fine: grid (unit, group of 32/Q rows x group of 16 columns), Q lanes share
+// a row, a warp sums 4 output columns - for units cut over many CTAs (few sequences, long caches), where the rounds of
+// loads are what the merge takes: qwen3b_S32768_N16_B1 (2 units over 148 CTAs, 74 partials each) 42.7 us per layer coarse,
+// 28.1 with Q = 1, MERGE_FIG with Q = 8; with many units of two partials the coarse shape is 3 % faster.
+// The blocks are small: they are launched early (programmatic dependent launch) and must not keep the next layer's
+// attention CTAs off the SMs.
+template <int ROWS, int Q, int HD>
 __global__ void __launch_bounds__(128)
 attn_tc5_merge_kernel(const Tc5Params p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -681,16 +697,48 @@ attn_tc5_merge_kernel(const Tc5Params p) {
     if (c0 == c1) return;                              // one CTA had the whole unit and wrote the output itself
     const int G = p.Hq / p.Hkv, N = p.N;
     const int kvh = uib / p.n_mblocks, mblock = uib - kvh * p.n_mblocks;
-    constexpr int CB = FINE ? HD / 16 : HD / 64;       // blocks per group of 32 rows
-    const int lrow = (blockIdx.y / CB) * 32 + lane;
-    const int cw = (blockIdx.y % CB) * 4 + warp;       // which 4 (FINE) or 16 output columns
+    constexpr int CB = Q > 0 ? HD / 16 : HD / 64, RW = Q > 0 ? 32 / Q : 32;     // blocks and rows per group of rows
+    const int lrow = (blockIdx.y / CB) * RW + lane % RW;
+    const int cw = (blockIdx.y % CB) * 4 + warp;       // which 4 (fine) or 16 output columns
     const int row = mblock * ROWS + lrow;
-    if (row >= G * N) return;
-    const int node = row / G, head = kvh * G + row % G;
+    const bool row_ok = row < G * N;
+    const int node = row_ok ? row / G : 0, head = kvh * G + (row_ok ? row % G : 0);
 
     const int smul = LOCK ? p.n_mblocks : 1, sadd = LOCK ? mblock : 0;
-    if (FINE) merge_row_c4<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
-    else merge_row_cols<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
+    if constexpr (Q > 0)
+        merge_row_c4<ROWS, HD, Q>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, lane / RW, row_ok, smul, sadd);
+    else if (row_ok)
+        merge_row_cols<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
+}
+
+// Host side: the merge of `units` units written by `ctas` CTAs; as many lanes share a row as keep the grid within what
+// starts at once beside the next call's CTAs (8 units of 128 rows: 512 blocks with Q = 2; 1024 with Q = 4 took 3 us more).
+constexpr int kMergeBlocks = 512;
+template <int ROWS, int HD>
+cudaError_t launch_merge(const Tc5Params& p, int units, int ctas, cudaStream_t st) {
+    auto go = [&](auto q) {
+        constexpr int Q = decltype(q)::value;
+        constexpr int GY = Q > 0 ? ROWS * Q / 32 * (HD / 16) : ROWS / 32 * (HD / 64);
+        return launch_pdl(attn_tc5_merge_kernel<ROWS, Q, HD>, dim3(units, GY), dim3(128), 0, st, 0, p);
+    };
+    const long long blocks = (long long)units * (ROWS / 32) * (HD / 16);       // at Q = 1
+    if (ctas < 4 * units || blocks > 2 * kMergeBlocks) return go(std::integral_constant<int, 0>{});
+    if (blocks * 8 <= kMergeBlocks) return go(std::integral_constant<int, 8>{});
+    if (blocks * 4 <= kMergeBlocks) return go(std::integral_constant<int, 4>{});
+    if (blocks * 2 <= kMergeBlocks) return go(std::integral_constant<int, 2>{});
+    return go(std::integral_constant<int, 1>{});
+}
+// Per-device set-up of those kernels: the merge blocks must be able to join an SM that an attention CTA has configured
+// for maximum shared memory.
+template <int ROWS, int HD>
+cudaError_t init_merge() {
+    const void* kernels[5] = {(const void*)attn_tc5_merge_kernel<ROWS, 0, HD>, (const void*)attn_tc5_merge_kernel<ROWS, 1, HD>,
+                              (const void*)attn_tc5_merge_kernel<ROWS, 2, HD>, (const void*)attn_tc5_merge_kernel<ROWS, 4, HD>, (const void*)attn_tc5_merge_kernel<ROWS, 8, HD>};
+    for (const void* k : kernels) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace tc5
