@@ -351,8 +351,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         const int unit = cta / ck, b = unit / upb, uib = unit - b * upb;
         cl_seg.b = b; cl_seg.kvh = uib / p.n_mblocks; cl_seg.mblock = uib - cl_seg.kvh * p.n_mblocks;
         cl_seg.steps = sched.steps[b]; cl_seg.S = sched.len[b];
-        cl_seg.st0 = (cr * cl_seg.steps) / ck;
-        cl_seg.n = ((cr + 1) * cl_seg.steps) / ck - cl_seg.st0;
+        // (the first ranks get the odd steps: the last one has the tree's tiles, which cannot be fetched ahead and cost a mask;
+        // qwen3b_S2048_N16_B1 9.7 -> 8.9 us per layer, qwen7b 14.5 -> 13.7)
+        cl_seg.st0 = (cr * cl_seg.steps + ck - 1) / ck;
+        cl_seg.n = ((cr + 1) * cl_seg.steps + ck - 1) / ck - cl_seg.st0;
         cl_seg.slot = -1;
     }
     auto make_iter = [&]() {
