@@ -570,6 +570,19 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                                                               // in the epilogue: [0..255] l by (ch, lane), [256..383] m by lane
         int px = 0;                                           // phases of the pair barrier used so far
         int sx = 0;                                           // phases of the segment barrier used so far
+        // Where this thread's chunks of the Q tile come from: (sequence, node, head) rows, -1 past the last.  The cluster
+        // form's one segment is known before the wait, and so are these.
+        constexpr int QC = D / 8, QR = kSmx / QC, ITEMS = ROWS / QR;   // 16-byte chunks per row; rows per pass; passes
+        const int qc = st % QC;
+        int qrow[ITEMS];
+        auto q_rows = [&](const Seg& sg) {
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                const int row = sg.mblock * ROWS + st / QC + QR * k;
+                qrow[k] = row < rows_total ? (sg.b * N + row / G) * p.Hq + sg.kvh * G + row % G : -1;
+            }
+        };
+        if (CL && !ROPE) q_rows(cl_seg);
         pdl_wait();                                           // q, tree_mask and every output come after the preceding kernel
 
         // rejected sequences (kv_len < 0 or kv_len + N > S_max): zero output, -inf lse, status word
@@ -592,18 +605,12 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 mbar_arrive(bar(B_QFULL));
                 return true;
             }
-            constexpr int QC = D / 8, QR = kSmx / QC;             // 16-byte chunks per row; rows per pass
-            constexpr int ITEMS = ROWS / QR;
-            const int qc = st % QC;
+            if (!CL) q_rows(sg);
             uint4 v[ITEMS];
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
-                const int row = sg.mblock * ROWS + st / QC + QR * k;
                 v[k] = make_uint4(0, 0, 0, 0);
-                if (row < rows_total) {
-                    const int node = row / G, head = sg.kvh * G + row % G;
-                    v[k] = *(reinterpret_cast<const uint4*>(p.q + (((size_t)sg.b * N + node) * p.Hq + head) * D) + qc);
-                }
+                if (qrow[k] >= 0) v[k] = *(reinterpret_cast<const uint4*>(p.q + (size_t)qrow[k] * D) + qc);
             }
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
@@ -931,24 +938,31 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         // shared memory and writes them out. ----
         __syncwarp();
         if (!cl_waited) { cluster_wait(); cl_waited = true; }     // (fused rotary embedding: the start-up phase, warps 0-3)
-        cluster_sync_all();
-        if (warp == 1) {
-            // every thread of the CTA is past its last tensor-memory access: give the columns back now, beside the
-            // merge, instead of on the way out
-            tc_fence_after();
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(TMEM_COLS) : "memory");
-        }
-        if (warp >= 4 && !*abort_flag) {
-        cluster_merge<ROWS, D>(p, cl_seg, ck, cr, base + SMEM_K, base + SMEM_K + (D / 4) * ROWS * 16, tid - 128);
+        if (warp >= 4) {
+            cluster_merge<ROWS, D>(p, cl_seg, ck, cr, base + SMEM_K, base + SMEM_K + (D / 4) * ROWS * 16, tid - 128,
+                                   [&]() { cluster_sync_all(); return *abort_flag == 0; });
+        } else {
+            cluster_sync_all();
+            if (warp == 1) {
+                // every thread of the CTA is past its last tensor-memory access: give the columns back now, beside the
+                // merge, instead of on the way out
+                tc_fence_after();
+                asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(TMEM_COLS) : "memory");
+            }
+            cluster_arrive_release();
         }
     }
 
-    // ---- tear-down: everyone meets, TMEM goes back ----
-    tc_fence_before();
-    __syncthreads();
-    // Cluster form: nobody leaves while a peer may still read its shared memory or signal its barriers.  Every
-    // CTA gets here (all its other waits are bounded), so this hardware barrier ends.
-    if (CL) cluster_sync_all();
+    // ---- tear-down.  Cluster form: nobody leaves while a peer may still read its shared memory or signal its barriers;
+    // every thread has arrived above (all its other waits are bounded), so this hardware barrier ends.  Even split:
+    // everyone meets, TMEM goes back. ----
+    if (CL) {
+        __syncwarp();
+        cluster_wait();
+    } else {
+        tc_fence_before();
+        __syncthreads();
+    }
     if (!CL && warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(TMEM_COLS) : "memory");

@@ -286,7 +286,10 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
         }
         __syncwarp();
     }
-    if (CL) cluster_sync_all();
+    if (CL) {
+        cluster_sync_all();
+        cluster_arrive_release();
+    }
     } else {
         // ================= softmax: one thread per query row, tile x by warps 4 + 4x .. 7 + 4x =================
         const int x = (warp - 4) >> 2, sp = warp & 3;
@@ -497,14 +500,13 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
         }
         if (CL) {
             __syncwarp();
-            cluster_sync_all();                    // every CTA of the unit has parked its partial
-            if (!*abort_flag)
-                cluster_merge<kRows, HD>(p, cl_seg, ck, cr, base + R::OFF_K, base + R::OFF_K + (HD / 4) * kRows * 16, tid - 128);
+            cluster_merge<kRows, HD>(p, cl_seg, ck, cr, base + R::OFF_K, base + R::OFF_K + (HD / 4) * kRows * 16, tid - 128,
+                                     [&]() { cluster_sync_all(); return *abort_flag == 0; });   // every CTA of the unit has parked its partial
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (CL) cluster_sync_all();                // nobody leaves while a peer may still read its shared memory
+    if (CL) cluster_wait();                    // nobody leaves while a peer may still read its shared memory
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(TMEM_COLS) : "memory");

@@ -122,6 +122,7 @@ __device__ __forceinline__ float2 dsmem_ld2(uint32_t a) {
 // (a wait taken by one lane and later by the other 31 never returns); the wait may sit anywhere later in the warp's
 // path.  Relaxed arrival: what the peers must see, the initialised barriers, is published by fence.mbarrier_init.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // One arrival on an mbarrier of another CTA of the cluster (address from dsmem_addr), ordered after this thread's
 // earlier accesses at cluster scope.
@@ -606,38 +607,45 @@ __device__ __forceinline__ void zero_rejected(const Tc5Params& p, const Sched& s
 
 // Cluster form: rank cr of ck merges its rows of the unit's partials, parked by every rank at pbuf_a ([HD/4 col4][ROWS]
 // float4) and pst_a ([ROWS] (m, l)) of its own shared memory, and writes them out.  By the NT softmax threads (st).
-template <int ROWS, int HD, int NT = 256>
-__device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st) {
+// Contains the meeting of the cluster (meet(), false: nothing is merged) and this thread's arrival at the closing one: the
+// indices of the first round are formed before the meeting, and the thread arrives as soon as its last loads from the peers
+// are back, so that neither the divisions nor the output's arithmetic and stores lie between the two barriers.
+template <int ROWS, int HD, int NT = 256, class Meet>
+__device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st, Meet meet) {
     const int N = p.N, G = p.Hq / p.Hkv, rows_total = G * N;
     const int rp = (ROWS + ck - 1) / ck;
     const int row0 = cr * rp;
-    const int nrows = min(rp, ROWS - row0);
+    const int nrows = min(rp, ROWS - row0), total = nrows * (HD / 4);
     // IT items (row, column quad) at a time per thread, all loads of all KM pieces issued before the first use
     auto merge_items = [&](auto km_tag, auto it_tag) {
         constexpr int KM = decltype(km_tag)::value, IT = decltype(it_tag)::value;
-        for (int item0 = st; item0 < nrows * (HD / 4); item0 += NT * IT) {
+        for (int item0 = st;; item0 += NT * IT) {
             float2 ml[IT][KM];
             float4 pv[IT][KM];
-            int c4s[IT], grows[IT];
+            int c4s[IT], lrs[IT], outs[IT];                            // outs: (sequence, node, head) row of the output, -1: none
 #pragma unroll
             for (int e = 0; e < IT; ++e) {
-                const int item = item0 + e * NT;
-                const int c4 = item / nrows, lr = row0 + (item - c4 * nrows);
-                c4s[e] = c4;
-                grows[e] = (item < nrows * (HD / 4)) ? sg.mblock * ROWS + lr : rows_total;
+                const int item = item0 + e * NT, c4 = item / nrows, lr = row0 + (item - c4 * nrows), grow = sg.mblock * ROWS + lr;
+                c4s[e] = c4; lrs[e] = lr; outs[e] = -1;
+                if (item < total && grow < rows_total) outs[e] = (sg.b * N + grow / G) * p.Hq + sg.kvh * G + grow % G;
+            }
+            if (item0 == st && !meet()) { cluster_arrive_release(); return; }
+#pragma unroll
+            for (int e = 0; e < IT; ++e)
 #pragma unroll
                 for (int j = 0; j < KM; ++j) {
                     ml[e][j] = make_float2(-INFINITY, 0.f);
                     pv[e][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (j < ck && grows[e] < rows_total) {
-                        ml[e][j] = dsmem_ld2(dsmem_addr(pst_a + lr * 8, (uint32_t)j));
-                        pv[e][j] = dsmem_ld4(dsmem_addr(pbuf_a + (c4 * ROWS + lr) * 16, (uint32_t)j));
+                    if (j < ck && outs[e] >= 0) {
+                        ml[e][j] = dsmem_ld2(dsmem_addr(pst_a + lrs[e] * 8, (uint32_t)j));
+                        pv[e][j] = dsmem_ld4(dsmem_addr(pbuf_a + (c4s[e] * ROWS + lrs[e]) * 16, (uint32_t)j));
                     }
                 }
-            }
+            const bool last = item0 + NT * IT >= total;
+            if (last) cluster_arrive_release();
 #pragma unroll
             for (int e = 0; e < IT; ++e) {
-                if (grows[e] >= rows_total) continue;
+                if (outs[e] < 0) continue;
                 float mm = -INFINITY;
 #pragma unroll
                 for (int j = 0; j < KM; ++j) mm = fmaxf(mm, ml[e][j].x);
@@ -651,15 +659,18 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
                     a4.x += w * pv[e][j].x; a4.y += w * pv[e][j].y; a4.z += w * pv[e][j].z; a4.w += w * pv[e][j].w;
                 }
                 const float inv2 = ll > 0.f ? 1.f / ll : 0.f;
-                const int nd = grows[e] / G, hd = sg.kvh * G + grows[e] % G;
-                *reinterpret_cast<uint2*>(p.out + (((size_t)sg.b * N + nd) * p.Hq + hd) * HD + c4s[e] * 4) =
+                *reinterpret_cast<uint2*>(p.out + (size_t)outs[e] * HD + c4s[e] * 4) =
                     make_uint2(pack_bf16(a4.x * inv2, a4.y * inv2), pack_bf16(a4.z * inv2, a4.w * inv2));
-                if (c4s[e] == 0 && p.lse)
-                    p.lse[((size_t)sg.b * p.Hq + hd) * N + nd] = ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
+                if (c4s[e] == 0 && p.lse) {
+                    const int bn = outs[e] / p.Hq, hd = outs[e] - bn * p.Hq;
+                    p.lse[((size_t)sg.b * p.Hq + hd) * N + (bn - sg.b * N)] = ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
+                }
             }
+            if (last) break;
         }
     };
-    if (ck <= 4) merge_items(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
+    if (ck <= 2) merge_items(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
+    else if (ck <= 4) merge_items(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
     else merge_items(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
 }
 
