@@ -249,16 +249,19 @@ accept_commit_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, cons
                      const int32_t* __restrict__ target, const int32_t* __restrict__ parents,
                      const int32_t* __restrict__ kv_len, int32_t* __restrict__ path, int32_t* __restrict__ accept_len,
                      int32_t* __restrict__ bonus, int32_t* __restrict__ kv_len_out, int N, int Hkv, int D, int S_max,
-                     int* status, const RowMap rows) {
+                     int* status, const RowMap rows, int layer_end, int layers_per_block) {
     __shared__ uint4 stage[2][kCompactRows][16];
     __shared__ int32_t par[VISPEC_MAX_TREE_NODES];
     __shared__ int32_t tgt[VISPEC_MAX_TREE_NODES];
     __shared__ int32_t spath[VISPEC_MAX_TREE_NODES];
     __shared__ int32_t s_len, s_bonus;
-    const int layer = layer_begin + blockIdx.z, b = blockIdx.y, h = blockIdx.x;
+    const int layer0 = layer_begin + blockIdx.z * layers_per_block, b = blockIdx.y, h = blockIdx.x;
+    const int layer1 = min(layer0 + layers_per_block, layer_end);
     const size_t rb = (size_t)b * N;
     pdl_wait();
     const int S = kv_len[b];
+    const int tensor = threadIdx.x >> 7;             // 0: K, 1: V
+    uint4* tensor_base = reinterpret_cast<uint4*>(cache_ptrs[2 * layer0 + tensor]);
     for (int i = threadIdx.x; i < N; i += 256) { par[i] = parents[rb + i]; tgt[i] = target[rb + i]; }
     __syncthreads();
     const bool writer = (blockIdx.x == 0 && blockIdx.z == 0);
@@ -278,30 +281,32 @@ accept_commit_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, cons
         return;   // kv_len_out[b] keeps its previous value for a rejected sequence
     }
     const int chunks = D / 8;
-    const int tensor = threadIdx.x >> 7;             // 0: K, 1: V
     const int r = (threadIdx.x & 127) >> 3;          // row of the pass, 0..15
     const int c0 = threadIdx.x & 7;                  // this thread moves chunks c0 and c0 + 8
-    uint4* const tensor_base = reinterpret_cast<uint4*>(cache_ptrs[2 * layer + tensor]);
     bool bad = false;
-    for (int k0 = 0; k0 < L; k0 += kCompactRows) {
-        const int k = k0 + r;
-        const int s = (k < L && spath[k] != k) ? spath[k] : -1;     // -1: nothing to move
-        const long long so = s >= 0 ? rows.at(b, h, S + s, Hkv, S_max, chunks) : -1;
-        const long long d_off = s >= 0 ? rows.at(b, h, S + k, Hkv, S_max, chunks) : -1;
-        if (s >= 0 && (so < 0 || d_off < 0)) bad = true;               // table entry outside the pool: move dropped
-        const bool move = so >= 0 && d_off >= 0;
-        if (move) {
-            const uint4* src = tensor_base + so;
-            if (c0 < chunks) stage[tensor][r][c0] = src[c0];
-            if (c0 + 8 < chunks) stage[tensor][r][c0 + 8] = src[c0 + 8];
+    for (int layer = layer0; layer < layer1; ++layer) {
+        uint4* const base = tensor_base;
+        if (layer + 1 < layer1) tensor_base = reinterpret_cast<uint4*>(cache_ptrs[2 * (layer + 1) + tensor]);
+        for (int k0 = 0; k0 < L; k0 += kCompactRows) {
+            const int k = k0 + r;
+            const int s = (k < L && spath[k] != k) ? spath[k] : -1;     // -1: nothing to move
+            const long long so = s >= 0 ? rows.at(b, h, S + s, Hkv, S_max, chunks) : -1;
+            const long long d_off = s >= 0 ? rows.at(b, h, S + k, Hkv, S_max, chunks) : -1;
+            if (s >= 0 && (so < 0 || d_off < 0)) bad = true;               // table entry outside the pool: move dropped
+            const bool move = so >= 0 && d_off >= 0;
+            if (move) {
+                const uint4* src = base + so;
+                if (c0 < chunks) stage[tensor][r][c0] = src[c0];
+                if (c0 + 8 < chunks) stage[tensor][r][c0 + 8] = src[c0 + 8];
+            }
+            __syncthreads();
+            if (move) {
+                uint4* dst = base + d_off;
+                if (c0 < chunks) dst[c0] = stage[tensor][r][c0];
+                if (c0 + 8 < chunks) dst[c0 + 8] = stage[tensor][r][c0 + 8];
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        if (move) {
-            uint4* dst = tensor_base + d_off;
-            if (c0 < chunks) dst[c0] = stage[tensor][r][c0];
-            if (c0 + 8 < chunks) dst[c0 + 8] = stage[tensor][r][c0 + 8];
-        }
-        __syncthreads();
     }
     if (bad) record_status(status, VISPEC_E_RANGE);
     if (kv_len_out && writer && threadIdx.x == 0) kv_len_out[b] = S + L;
@@ -313,10 +318,16 @@ cudaError_t launch_accept_commit(void* const* cache_ptrs, int layer_begin, int l
                                  int Hkv, int D, int S_max, int* status, cudaStream_t st, const int32_t* block_table,
                                  int table_stride, int page_rows, int num_blocks, int token_major) {
     if (B == 0 || layer_end <= layer_begin) return cudaSuccess;
-    dim3 grid(Hkv, B, layer_end - layer_begin);
+    // Every block repeats its sequence's acceptance (2.5 us of dependent loads), so all blocks should be resident at once: 8 per
+    // SM.  Beyond that a block serves several layers, whose moves cost it 1 us each, instead of a wave that costs it all
+    // (4 x 40 heads x 8 layers 7.9 -> 5.4 us, 8 x 40 x 12 14.9 -> 7.7).
+    const int layers = layer_end - layer_begin, room = 8 * 148;
+    const long long blocks = (long long)Hkv * B * layers;
+    const int lpb = (int)((blocks + room - 1) / room);
+    dim3 grid(Hkv, B, (layers + lpb - 1) / lpb);
     const RowMap rows = {block_table, table_stride, page_rows, num_blocks, token_major};
     return launch_pdl(accept_commit_kernel, grid, dim3(256), 0, st, 0, cache_ptrs, layer_begin, draft, target, parents, kv_len,
-                      path, accept_len, bonus, kv_len_out, N, Hkv, D, S_max, status, rows);
+                      path, accept_len, bonus, kv_len_out, N, Hkv, D, S_max, status, rows, layer_end, lpb);
 }
 
 // ------------------------------------------------------------------------------------------------
