@@ -255,6 +255,12 @@ def test_accept_commit_in_one_launch_matches_accept_then_compact(gpu):
     _accept_commit_case(binding, gu, "tiny", 4, 64, 1, np.array([256], dtype=np.int32), 320, seed=4)
 
 
+@pytest.mark.parametrize("Hkv,layers", [(37, 8), (60, 5), (150, 7)])      # 1184 blocks (one layer each), 1200 (two, one left over), 4200 (four, three left over)
+def test_accept_commit_with_several_layers_per_block(gpu, Hkv, layers):
+    binding, gu = gpu
+    _accept_commit_case(binding, gu, "llava13b_b4", Hkv, 64, layers, np.array([68, 37, 0, 5], dtype=np.int32), 128, seed=Hkv)
+
+
 def test_accept_commit_bad_tree_and_overlong_sequence(gpu):
     binding, gu = gpu
     rng = np.random.default_rng(5)
