@@ -239,23 +239,12 @@ __device__ __noinline__ void rope_prologue(unsigned char* sm, const __nv_bfloat1
     }
 }
 
-// The softmax's exponentials are what the special-function pipe (16 lanes per SM) spends a step on; one in
-// 2 * kPolyEvery of them is formed on the FMA pipe instead.  Timed in one call, none / 1 in 6 / 1 in 8 / 1 in 16:
-// llava7b 17.33 / 17.12 / 17.15 / 17.24 us per layer, qwen7b 16.5 / 16.2 / 16.2 / 16.3, qwen3b_S8192_N60_B4 32.1 / 31.3 /
-// 31.3 / 31.8; 1 in 4 and 1 in 2 were slower again (issue slots).
+// The softmax's exponentials are what the special-function pipe (16 lanes per SM) spends a step on; one in eight of them is
+// formed on the FMA pipe instead: in the duplicated-row layout two neighbouring columns of every sixteen by one packed
+// evaluation, with 128 rows one column of every eight (packed there: 517.6 against 507.1 us per pass on qwen3b_S8192_N60_B4).
+// None / 1 in 16 / 1 in 8, us per pass: llava7b 559.6 / 558.4 / 550.3, qwen3b_S8192_N60_B4 532.1 / 526.1 / 507.1, qwen7b fused
+// 455.3 / 454.8 / 451.8; 1 in 6 moves nothing, 1 in 4 and 1 in 2 are slower (issue slots).
 constexpr int kPolyEvery = 4;
-// 2^x on the FMA pipe (x <= 120; anything at or below -126 comes out as a denormal, which the flush-to-zero arithmetic that
-// follows reads as 0): nearest integer by the 1.5 * 2^23 trick, cubic on the remainder in [-0.5, 0.5] (relative error
-// 8e-5, well inside the bf16 rounding of P), the integer added into the exponent field.
-__device__ __forceinline__ float exp2_fma(float x) {
-    x = fmaxf(x, -126.f);
-    const float z = x + 12582912.f;
-    const float f = x - (z - 12582912.f);
-    float p = fmaf(f, 0.055088684f, 0.24260405f);
-    p = fmaf(p, f, 0.69327623f);
-    p = fmaf(p, f, 0.99992895f);
-    return __int_as_float(__float_as_int(p) + (__float_as_int(z) << 23));
-}
 
 // PAGED instantiations carry the paged producer; the others are compiled without it (its call sites cost the
 // contiguous kernels registers they do not have to spare).
@@ -757,9 +746,15 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                         float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
                         for (int c = 0; c < NC / 2; ++c) {
-                            const float e0 = exp2f(fmaf(__uint_as_float(sraw[2 * c]), p.scale_log2, -m_use));
+                            const float x0 = fmaf(__uint_as_float(sraw[2 * c]), p.scale_log2, -m_use);
                             const float x1 = fmaf(__uint_as_float(sraw[2 * c + 1]), p.scale_log2, -m_use);
-                            const float e1 = (c % kPolyEvery == kPolyEvery - 1) ? exp2_fma(x1) : exp2f(x1);
+                            float e0, e1;
+                            if (PAIR && c % (2 * kPolyEvery) == 2 * kPolyEvery - 1) {
+                                exp2_fma_pair(x0, x1, e0, e1);
+                            } else {
+                                e0 = exp2f(x0);
+                                e1 = (!PAIR && c % kPolyEvery == kPolyEvery - 1) ? exp2_fma(x1) : exp2f(x1);
+                            }
                             sum0 += e0; sum1 += e1;
                             pd[c] = pack_bf16(e0, e1);
                         }

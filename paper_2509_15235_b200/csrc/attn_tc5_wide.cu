@@ -2,15 +2,15 @@
 // unit is (sequence, kv head, block of 256 query rows), two accumulator tiles of 128 rows that share every K/V stage.
 //
 // What bounds it: the tensor pipe (2048 cycles per 128-token step: two score products and two PV products of
-// 128 x 128 x 128) and beside it the exponentials (2 x 1024 cycles on the special-function pipe, an eighth of them moved to the
-// FMA pipe); over a long call the power cap.  The one-tile kernel spends 2670 cycles on half of that: its eight softmax
+// 128 x 128 x 128) and beside it the exponentials (2 x 1024 cycles on the special-function pipe; at head size 64, where the
+// products are half as long, an eighth of them is moved to the FMA pipe); over a long call the power cap.  The one-tile kernel spends 2670 cycles on half of that: its eight softmax
 // warps move in lock-step (two threads per row exchange the row's maximum), so the special-function pipe idles while they
 // wait, load and take maxima.  Here each tile has four softmax warps of its own, one thread per row (nothing to exchange),
 // and the tiles run out of phase: while one is in its exponentials, the tensor pipe works for the other: 3150 cycles per
 // step of both.  Each stage serves twice the rows, so L2 delivers half the bytes per product.
 // qwen3b_S32768_N128_B8: 345-363 -> 273-281 us per layer (1.0 PFLOP/s, at 1530 MHz under the power cap; 252 in a burst).
-// Tried: eight softmax warps per tile, two threads per row (282-286 against 273-277); 1/2, 1/3, 1/4 of the exponentials
-// on the FMA pipe (292, 283, 277 against 276).
+// Tried: eight softmax warps per tile, two threads per row (282-286 against 273-277); 1/2, 1/3, 1/4, 1/8 of the exponentials
+// on the FMA pipe (292, 283, 277, 276 with a cubic that was dropped for its error; none is as fast as 1/8, see kPolyEvery).
 //
 //   warp 0     TMA producer of the K ring (2 x 32 KB; head size 64: 4 x 16 KB)
 //   warp 1     issuer (one thread) of all products, in the order S_A S_B | PV_A S_A' PV_B S_B' | ...: they complete in the
@@ -62,35 +62,10 @@ constexpr int SMEM_TABRING = SMEM_SCHED + ((int)sizeof(Sched) + 15) / 16 * 16;
 constexpr int SMEM_ALLOC = SMEM_TABRING + 256;
 static_assert(SMEM_ALLOC <= 232448, "over the 227 KB a CTA may have");
 
-// ---- two fp32 lanes per instruction
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-    uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r;
-}
-__device__ __forceinline__ void up2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r; asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r; asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
-}
-// 2^x for a pair on the FMA pipe (the one-tile kernel's exp2_fma: nearest integer by the 1.5 * 2^23 trick, a cubic on the
-// remainder, relative error 8e-5).
-__device__ __forceinline__ void exp2_fma_pair(float x0, float x1, float& e0, float& e1) {
-    const uint64_t x = pk2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
-    const uint64_t z = add2(x, pk2(12582912.f, 12582912.f));
-    const uint64_t f = fma2(add2(z, pk2(-12582912.f, -12582912.f)), pk2(-1.f, -1.f), x);
-    uint64_t p = fma2(f, pk2(0.055088684f, 0.055088684f), pk2(0.24260405f, 0.24260405f));
-    p = fma2(p, f, pk2(0.69327623f, 0.69327623f));
-    p = fma2(p, f, pk2(0.99992895f, 0.99992895f));
-    float p0, p1, z0, z1;
-    up2(p, p0, p1); up2(z, z0, z1);
-    e0 = __int_as_float(__float_as_int(p0) + (__float_as_int(z0) << 23));
-    e1 = __int_as_float(__float_as_int(p1) + (__float_as_int(z1) << 23));
-}
-constexpr int kPolyEvery = 8;                  // one pair of exponentials in this many goes to the FMA pipe
+// Head size 64: one pair of exponentials in this many goes to the FMA pipe (6 x 16 heads (4 kv) x 128 nodes on 3000, 16 layers:
+// 469.1 us per pass, none 475.5).  At head size 128 none does: the steps are the tensor pipe's, and the power cap's (the
+// benchmark's 8 x 128 nodes on 32768: none 4453, one in eight 4506; 28/4 heads, 8 x 60 on 8192 355.5 / 358.9).
+constexpr int kPolyEvery = 8;
 
 template <bool CL, bool PAGED, int HD>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -433,7 +408,7 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
                         for (int c = 0; c < 32; ++c) {
                             float x0, x1, e0, e1;
                             up2(fma2(pk2(__uint_as_float(s[2 * c]), __uint_as_float(s[2 * c + 1])), sc2, mm2), x0, x1);
-                            if (c % kPolyEvery == kPolyEvery - 1) exp2_fma_pair(x0, x1, e0, e1);
+                            if (HD == 64 && c % kPolyEvery == kPolyEvery - 1) exp2_fma_pair(x0, x1, e0, e1);
                             else { e0 = exp2f(x0); e1 = exp2f(x1); }
                             if (c & 1) sum2b = add2(sum2b, pk2(e0, e1)); else sum2 = add2(sum2, pk2(e0, e1));
                             pd[c] = pack_bf16(e0, e1);

@@ -231,6 +231,52 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// ---- two fp32 lanes per instruction
+__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
+    uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r;
+}
+__device__ __forceinline__ void up2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r; asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r; asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
+}
+// 2^x on the FMA pipe (x <= 120; anything at or below -126 comes out as a denormal, which the flush-to-zero arithmetic that
+// follows reads as 0): nearest integer by the 1.5 * 2^23 trick, a polynomial of degree 5 on the remainder f in [-0.5, 0.5], the
+// integer added into the exponent field.  The polynomial is 1 + C1 f + ... + C5 f^5 with the largest relative error made
+// smallest: 9.2e-8, 1.7e-7 with the roundings of its fp32 evaluation, which is within exp2f's own 2 ulp, so that a row's sum
+// and its lse do not depend on which columns come through here (a cubic, 7.5e-5, showed in lse).
+constexpr float kExp2C1 = 0.693147f, kExp2C2 = 0.24022242f, kExp2C3 = 0.055507336f, kExp2C4 = 0.009671513f, kExp2C5 = 0.0013264727f;
+__device__ __forceinline__ float exp2_fma(float x) {
+    x = fmaxf(x, -126.f);
+    const float z = x + 12582912.f;
+    const float f = x - (z - 12582912.f);
+    float p = fmaf(f, kExp2C5, kExp2C4);
+    p = fmaf(p, f, kExp2C3);
+    p = fmaf(p, f, kExp2C2);
+    p = fmaf(p, f, kExp2C1);
+    p = fmaf(p, f, 1.f);
+    return __int_as_float(__float_as_int(p) + (__float_as_int(z) << 23));
+}
+__device__ __forceinline__ void exp2_fma_pair(float x0, float x1, float& e0, float& e1) {
+    const uint64_t x = pk2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    const uint64_t z = add2(x, pk2(12582912.f, 12582912.f));
+    const uint64_t f = fma2(add2(z, pk2(-12582912.f, -12582912.f)), pk2(-1.f, -1.f), x);
+    uint64_t p = fma2(f, pk2(kExp2C5, kExp2C5), pk2(kExp2C4, kExp2C4));
+    p = fma2(p, f, pk2(kExp2C3, kExp2C3));
+    p = fma2(p, f, pk2(kExp2C2, kExp2C2));
+    p = fma2(p, f, pk2(kExp2C1, kExp2C1));
+    p = fma2(p, f, pk2(1.f, 1.f));
+    float p0, p1, z0, z1;
+    up2(p, p0, p1); up2(z, z0, z1);
+    e0 = __int_as_float(__float_as_int(p0) + (__float_as_int(z0) << 23));
+    e1 = __int_as_float(__float_as_int(p1) + (__float_as_int(z1) << 23));
+}
+
 struct Tc5Params {
     const __nv_bfloat16* q; const int32_t* kv_len; const uint64_t* mask;
     __nv_bfloat16* out; float* lse;

@@ -114,6 +114,39 @@ def test_two_tile_units(gu, Hq, Hkv, D, N, kv_len, S_max, split_form):
     _check(gu, q, k, v, np.array(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=split_form)
 
 
+# Nodes that see one key (their own slot; kv_len 0) or two (the one committed key and their own): a row's sum is then one or
+# two exponentials, and every column of a step has a node whose weight is formed there.  Small integers in q and k make the
+# scores exact, so lse carries the roundings of the scaling, of two exponentials (2 ulp each) and of one logarithm: below
+# 2^-22 * (2 + |score|) each, 2e-6 in all for scores up to 4.
+@pytest.mark.parametrize("static", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,D,N,S_max", [(4, 4, 64, 60, 256), (4, 1, 64, 100, 256), (4, 4, 128, 60, 256), (4, 1, 128, 100, 256),
+                                              (16, 2, 64, 128, 40000), (16, 2, 128, 128, 40000)])
+def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
+    from paper_2509_15235_b200 import binding
+    rng = np.random.Generator(np.random.Philox(Hq * 1000 + N + D))
+    B, scale = 2, 1 / 16
+    small = lambda *shape: synth.f32_to_bf16_bits(rng.integers(-2, 3, size=shape).astype(np.float32))
+    q, k = small(B, N, Hq, D), np.zeros((B, Hkv, S_max, D), dtype=np.uint16)
+    k[:, :, :N + 1] = small(B, Hkv, N + 1, D)
+    v = np.zeros_like(k)
+    v[:, :, :N + 1] = synth.normal_bf16((B, Hkv, N + 1, D), 5 + N)
+    kv_len = np.array([0, 1], dtype=np.int32)
+    mask = np.zeros((B, N, (N + 63) // 64), dtype=np.uint64)
+    for i in range(N):
+        mask[:, i, i // 64] = np.uint64(1 << (i % 64))
+    if static:
+        out = torch.zeros((B, N, Hq, D), dtype=torch.bfloat16, device="cuda")
+        lse = torch.zeros((B, Hq, N), dtype=torch.float32, device="cuda")
+        binding.tree_verify_attn_static(gu.bf16_dev(q), gu.bf16_dev(k), gu.bf16_dev(v), gu.i32_dev(kv_len), gu.u64_dev(mask), scale, out, lse)
+        out, lse = out.float().cpu().numpy(), lse.cpu().numpy()
+    else:
+        out, lse, status = gu.run_attn(q, k, v, kv_len, mask, scale)
+        assert status == 0
+    want, want_lse = oracle.tree_attn(q, k[:, :, :N + 1], v[:, :, :N + 1], kv_len, mask, scale)
+    assert np.abs(out - want).max() <= TOL
+    assert np.abs(lse - want_lse).max() <= 2e-6
+
+
 def test_arbitrary_mask_bits_all_ones_and_zero_rows(gu):
     B, N, Hq, Hkv, D, S_max = 2, 20, 4, 2, 128, 256
     q = synth.normal_bf16((B, N, Hq, D), 21); k = synth.normal_bf16((B, Hkv, S_max, D), 22)
