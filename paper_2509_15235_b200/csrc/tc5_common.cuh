@@ -653,8 +653,8 @@ __device__ __forceinline__ void zero_rejected(const Tc5Params& p, const Sched& s
 
 // Cluster form: rank cr of ck merges its rows of the unit's partials, parked by every rank at pbuf_a ([HD/4 col4][ROWS]
 // float4) and pst_a ([ROWS] (m, l)) of its own shared memory, and writes them out.  By the NT softmax threads (st).
-// Contains the meeting of the cluster (meet(), false: nothing is merged) and this thread's arrival at the closing one: the
-// indices of the first round are formed before the meeting, and the thread arrives as soon as its last loads from the peers
+// Contains the meeting of the cluster (meet(), false: nothing is merged) and this warp's arrival at the closing one: the
+// indices of the first round are formed before the meeting, and a warp arrives as soon as its last loads from the peers
 // are back, so that neither the divisions nor the output's arithmetic and stores lie between the two barriers.
 template <int ROWS, int HD, int NT = 256, class Meet>
 __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st, Meet meet) {
@@ -687,7 +687,10 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
                         pv[e][j] = dsmem_ld4(dsmem_addr(pbuf_a + (c4s[e] * ROWS + lrs[e]) * 16, (uint32_t)j));
                     }
                 }
-            const bool last = item0 + NT * IT >= total;
+            // (the last round of the warp, not of the thread: at head size 64 `total` need not be a multiple of 32 - 688 items in
+            // rounds of 512 with three CTAs per unit of 128 rows - and a warp arrives with all its lanes at once; a lane past the
+            // end has outs < 0)
+            const bool last = (item0 & ~31) + NT * IT >= total;
             if (last) cluster_arrive_release();
 #pragma unroll
             for (int e = 0; e < IT; ++e) {

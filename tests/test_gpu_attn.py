@@ -114,6 +114,23 @@ def test_two_tile_units(gu, Hq, Hkv, D, N, kv_len, S_max, split_form):
     _check(gu, q, k, v, np.array(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=split_form)
 
 
+# The merge of a cluster's partials at head size 64 over every cluster size that 4 to 96 units lead to (15 units or fewer: eight
+# CTAs each, 16 to 22: six, ... 34 to 45: three), with units of 128 and of 256 rows: the share of a rank is then often no whole
+# number of warps (43 rows x 16 column quads in rounds of 512 or 256).
+@pytest.mark.parametrize("N", [31, 128])
+@pytest.mark.parametrize("B", [1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12])
+def test_head_size_64_cluster_merge_shares(gu, B, N):
+    rng = np.random.Generator(np.random.Philox(6400 + B))
+    Hq, Hkv, D, S_max = 16, 4, 64, 640
+    q = synth.normal_bf16((B, N, Hq, D), 25 + B)
+    k = synth.normal_bf16((B, Hkv, S_max, D), 26 + B)
+    v = synth.normal_bf16((B, Hkv, S_max, D), 27 + B)
+    kv_len = rng.integers(0, S_max - N + 1, size=B).astype(np.int32)
+    parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
+    mask, _, _ = oracle.tree_mask(parents)
+    _check(gu, q, k, v, kv_len, mask, 1 / math.sqrt(D), split_form=2)
+
+
 # Nodes that see one key (their own slot; kv_len 0) or two (the one committed key and their own): a row's sum is then one or
 # two exponentials, and every column of a step has a node whose weight is formed there.  Small integers in q and k make the
 # scores exact, so lse carries the roundings of the scaling, of two exponentials (2 ulp each) and of one logarithm: below
