@@ -20,7 +20,8 @@
 // sequence 25.3 -> 18.6, four 28.3 -> 21.6; V = 32000, one sequence 17.3 -> 14.1.
 //
 // Every CTA takes the same decisions from the same numbers: a CTA's sum is pushed into every peer's shared memory ahead
-// of a hardware cluster barrier and summed by everyone in the same order, so S is bit-identical in the cluster.  Sums
+// of a hardware cluster barrier and summed by everyone in the same order, so S is bit-identical in the cluster.  (The first
+// push follows a barrier phase that every CTA arrives at when it starts: nothing is written into a CTA that does not run yet.)  Sums
 // and comparisons are fp64 (the inputs are fp32): the decisions then differ from a sequential fp64 evaluation only
 // where a uniform falls within ~1e-15 of a threshold.
 #include "launch.cuh"
@@ -50,6 +51,10 @@ __device__ __forceinline__ uint32_t cl_size() {
 __device__ __forceinline__ void cl_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The barrier in two halves (each taken by whole warps): what a CTA writes into a peer's shared memory comes after its wait
+// for the phase in which every CTA, the peer too, has arrived.
+__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cl_st_f64(const double* local, uint32_t rank, double v) {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(local);
     uint32_t ra;
@@ -175,6 +180,8 @@ accept_sampled_kernel(const int32_t* __restrict__ draft_ids, const int32_t* __re
     if (tid == 0) { sh_bad = 0; sh_stop = 0; }
     if (tid < VISPEC_MAX_TREE_NODES * 4) (&kids[0][0])[tid] = 0u;
     __syncthreads();
+    cl_arrive();                                 // this CTA runs; waited for ahead of the first push, behind the first loads
+    bool peers_run = false;
     pdl_wait();
     int pr = 0, id = 0;
     if (tid < N) { pr = parents[nb + tid]; id = draft_ids[nb + tid]; ua[tid] = u_accept[nb + tid]; }
@@ -206,6 +213,8 @@ accept_sampled_kernel(const int32_t* __restrict__ draft_ids, const int32_t* __re
                 record_status_as(status, (sh_bad & 1) ? VISPEC_E_BAD_TREE : VISPEC_E_RANGE);
             }
         }
+        __syncwarp();
+        cl_wait();
         return;
     }
 
@@ -264,6 +273,7 @@ accept_sampled_kernel(const int32_t* __restrict__ draft_ids, const int32_t* __re
         const double sum = slice_sum<VEC>(rows, sh_c, slice, lane);
         if (lane == 0) seg[w] = sum;
         __syncthreads();
+        if (!peers_run) { cl_wait(); peers_run = true; }
         const int parity = iter & 1;
         if (w == 0) {
             double t = seg[lane];
@@ -369,6 +379,8 @@ accept_sampled_kernel(const int32_t* __restrict__ draft_ids, const int32_t* __re
         }
     }
     copy_wait();
+    __syncwarp();
+    if (!peers_run) cl_wait();                   // (no pass was made)
     cl_sync();                                   // nobody leaves while a peer may still push its sum here
 }
 

@@ -103,6 +103,34 @@ def test_sampled_acceptance_flags_malformed_sequences():
     assert list(got[1][1:]) == [0, 0, 0]
 
 
+@pytest.mark.parametrize("B,V", [(40, 8196), (9, 8193), (3, 20000)])
+def test_sampled_acceptance_clusters_that_start_at_different_times(B, V):
+    """More clusters than the GPU holds at once (40 sequences of 8 CTAs), calls queued one behind the other so that each starts
+    while its predecessor ends, and malformed sequences among the others, whose clusters leave without a pass: every CTA must
+    have started before a peer writes its sum there."""
+    from paper_2509_15235_b200 import binding
+    import gpu_util as gu
+    rng = np.random.Generator(np.random.Philox(B))
+    N, calls = 6, 12
+    parents = np.stack([synth.draw_tree(N, 3, 0, rng) for _ in range(B)])
+    s = synth.make_sampled_inputs(parents, V, 300 + B, sharpness=1.0, disagreement=1.5)
+    ids = s["draft_ids"].copy()
+    ids[1::5, 2] = V                                                # token out of range
+    want = oracle.accept_sampled(ids, parents, s["p_target"], s["p_draft"], s["u_accept"], s["u_bonus"])
+    f32 = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+    args = [gu.i32_dev(ids), gu.i32_dev(parents)] + [f32(s[k]) for k in ("p_target", "p_draft", "u_accept", "u_bonus")]
+    ctx = binding.VerifyContext(B, N, 4, 4, 64, 256, 1)
+    outs = [[torch.full(shape, -9, dtype=torch.int32, device="cuda") for shape in ((B, N), (B,), (B,))] for _ in range(calls)]
+    for o in outs:
+        ctx.accept_sampled(*args, *o)
+    torch.cuda.synchronize()
+    assert ctx.status_poll() == -4                                  # VISPEC_E_RANGE of the malformed ones
+    for o in outs:
+        for got, w in zip(o, want[:3]):
+            assert np.array_equal(got.cpu().numpy(), w)
+    ctx.close()
+
+
 def test_sampled_acceptance_host_errors_and_empty_batch():
     from paper_2509_15235_b200 import binding
     ctx = binding.VerifyContext(2, 4, 4, 4, 64, 256, 1)
