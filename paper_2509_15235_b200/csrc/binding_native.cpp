@@ -11,6 +11,7 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <c10/util/Exception.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "vispec.h"
@@ -87,16 +88,40 @@ struct Args {
 
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// The interpreter lock is given up for as long as this lives.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
 // The call itself, without the interpreter lock.
 template <typename F>
 PyObject* finish(const Args& g, F&& call) {
     if (!g.ok) return nullptr;
-    int rc;
     void* const st = stream();
-    Py_BEGIN_ALLOW_THREADS
-    rc = call(st);
-    Py_END_ALLOW_THREADS
+    int rc;
+    {
+        Unlocked unlocked;
+        rc = call(st);
+    }
     return PyLong_FromLong(rc);
+}
+
+// What the interpreter calls: an exception that torch throws on the way - a tensor without storage (a fake or wrapped one) has
+// no data pointer, a process without a usable device has no current stream - becomes a RuntimeError; past this frame it would
+// end the process.
+template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
+    try {
+        return F(self, args, nargs);
+    } catch (const c10::Error& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {
+        PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
+    }
+    return nullptr;
 }
 
 int size(const at::Tensor* t, int d) { return t ? static_cast<int>(t->size(d)) : 0; }
@@ -282,7 +307,7 @@ NATIVE(tree_rerank) {  // handle, cand_parent, cand_token, cand_score, K, parent
     return finish(g, [&](void* st) { return vispec_tree_rerank(c, cp, ct, cs, B, M, K, parents, ids, sel, st); });
 }
 
-#define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+#define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef kMethods[] = {
     ENTRY(tree_mask_build), ENTRY(tree_verify_attn), ENTRY(tree_verify_attn_rope), ENTRY(tree_verify_attn_paged),
     ENTRY(tree_verify_attn_static), ENTRY(rope_table_build), ENTRY(rope_tree_rows), ENTRY(rope_tree_rows_paged),

@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -48,6 +50,28 @@ def test_shape_validation_precedes_any_cuda_call(lib):
                 VispecShape(1, 8, 4, 4, 96, 512, 1), VispecShape(0, 8, 4, 4, 64, 512, 1),
                 VispecShape(1, 8, 4, 4, 64, 4, 1)):
         assert lib.vispec_ctx_create(ctypes.byref(h), ctypes.byref(bad), 0) == -3   # VISPEC_E_SHAPE
+
+
+@pytest.mark.parametrize("call", ["tree_mask_build(0, t, t, None)", "accept(0, t, t, t, t, t, t)",
+                                  "tree_rerank(0, t, t, t, 1, t, t, None)"])
+def test_a_tensor_without_storage_raises_in_python(lib, call):
+    """A fake CUDA tensor has no data pointer: torch throws inside the native module, which must come out as an exception
+    and not end the process (hence the child)."""
+    code = f"""
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+from paper_2509_15235_b200 import binding
+binding.load()
+with FakeTensorMode():
+    t = torch.empty(1, 4, device="cuda", dtype=torch.int32)
+assert t.is_cuda
+try:
+    binding._native.{call}
+except RuntimeError as e:
+    print("raised", type(e).__name__)
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=300)
+    assert r.returncode == 0 and "raised RuntimeError" in r.stdout, (r.returncode, r.stderr[-500:])
 
 
 def test_product_package_does_not_import_the_oracle():
