@@ -1042,6 +1042,9 @@ stream_probe_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_cons
         }
     }
     __syncthreads();
+    // nothing to stream (every sequence out of range), or none of the last tiles in this CTA's range: the probe must still not
+    // end before its predecessor, because what follows it on the stream waits for the probe only
+    if (tid == 0) pdl_wait();
     if (tid == 0 && *abort_flag) atomicCAS(p.status, 0, (int)VISPEC_E_TIMEOUT);
 }
 

@@ -381,6 +381,29 @@ def test_stream_probe_runs_and_validates_its_arguments(gu):
     assert e.value.code == -5                                   # D = 64: no TMA maps
 
 
+def test_stream_probe_with_nothing_to_read_keeps_the_stream_order(gu):
+    """A kernel that starts early (the commit) waits for the kernel before it, here a probe whose sequences are all out of range;
+    the probe must not end ahead of the rotary placement before it, whose rows the commit moves."""
+    from paper_2509_15235_b200 import binding
+    B, N, Hq, Hkv, D, S_max = 8, 128, 32, 32, 128, 512
+    ctx = binding.VerifyContext(B, N, Hq, Hkv, D, S_max, 1)
+    rows = lambda seed: torch.randn((B, N, Hkv, D), generator=torch.Generator("cuda").manual_seed(seed), device="cuda", dtype=torch.bfloat16)
+    kv_len, none = gu.i32_dev([100] * B), gu.i32_dev([S_max] * B)
+    path = gu.i32_dev([[0, 127] + [-1] * (N - 2)] * B)                # the last row of the tree moves to slot 101
+    alen, pos = gu.i32_dev([2] * B), gu.i32_dev(np.zeros((B, N)))
+    k, v = (torch.zeros((B, Hkv, S_max, D), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    ctx.cache_register(0, k, v)
+    for rep in range(10):
+        kn, vn, q = rows(2 * rep), rows(2 * rep + 1), rows(99)
+        ctx.rope_tree_rows(0, q, kn, vn, pos, kv_len, 10000.0)
+        ctx.stream_probe(0, none, N)
+        ctx.kv_compact(0, 1, path, alen, kv_len)
+        torch.cuda.synchronize()
+        assert torch.equal(k[:, :, 101], kn[:, 127]) and torch.equal(v[:, :, 101], vn[:, 127])   # (position 0: no rotation)
+    assert ctx.status_poll() == 0
+    ctx.close()
+
+
 def test_seeded_random_shapes_against_the_oracle(gu):
     """Sixty seeded draws of (batch, heads, group size, tree size, lengths, split form): every output element
     against the oracle.  Lengths straddle tile boundaries; some sequences are empty."""
