@@ -245,14 +245,15 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 __device__ __forceinline__ float max3(float a, float b, float c) {
     float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
 }
-// 2^x on the FMA pipe (x <= 120; anything at or below -126 comes out as a denormal, which the flush-to-zero arithmetic that
-// follows reads as 0): nearest integer by the 1.5 * 2^23 trick, a polynomial of degree 5 on the remainder f in [-0.5, 0.5], the
-// integer added into the exponent field.  The polynomial is 1 + C1 f + ... + C5 f^5 with the largest relative error made
-// smallest: 9.2e-8, 1.7e-7 with the roundings of its fp32 evaluation, which is within exp2f's own 2 ulp, so that a row's sum
-// and its lse do not depend on which columns come through here (a cubic, 7.5e-5, showed in lse).
+// 2^x on the FMA pipe (x <= 120; -inf gives exactly 0, below -126 a denormal or 0 comes out): nearest integer by the
+// 1.5 * 2^23 trick, a polynomial of degree 5 on the remainder f in [-0.5, 0.5], the integer added into the exponent field (at the
+// clamp the remainder is not negative, so 2^-127 p(f) >= 2^-127 stays a positive pattern, and 0 at f = 0).  The polynomial is
+// 1 + C1 f + ... + C5 f^5 with the largest relative error made smallest: 9.2e-8, 1.7e-7 with the roundings of its fp32
+// evaluation, which is within exp2f's own 2 ulp, so that a row's sum and its lse do not depend on which columns come through
+// here (a cubic, 7.5e-5, showed in lse).
 constexpr float kExp2C1 = 0.693147f, kExp2C2 = 0.24022242f, kExp2C3 = 0.055507336f, kExp2C4 = 0.009671513f, kExp2C5 = 0.0013264727f;
 __device__ __forceinline__ float exp2_fma(float x) {
-    x = fmaxf(x, -126.f);
+    x = fmaxf(x, -127.f);
     const float z = x + 12582912.f;
     const float f = x - (z - 12582912.f);
     float p = fmaf(f, kExp2C5, kExp2C4);
@@ -263,7 +264,7 @@ __device__ __forceinline__ float exp2_fma(float x) {
     return __int_as_float(__float_as_int(p) + (__float_as_int(z) << 23));
 }
 __device__ __forceinline__ void exp2_fma_pair(float x0, float x1, float& e0, float& e1) {
-    const uint64_t x = pk2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    const uint64_t x = pk2(fmaxf(x0, -127.f), fmaxf(x1, -127.f));
     const uint64_t z = add2(x, pk2(12582912.f, 12582912.f));
     const uint64_t f = fma2(add2(z, pk2(-12582912.f, -12582912.f)), pk2(-1.f, -1.f), x);
     uint64_t p = fma2(f, pk2(kExp2C5, kExp2C5), pk2(kExp2C4, kExp2C4));

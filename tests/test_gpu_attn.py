@@ -164,6 +164,30 @@ def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
     assert np.abs(lse - want_lse).max() <= 2e-6
 
 
+# Hidden tree rows have weight exactly 0 in every column of a step: rows that see nothing are zeros (also where one CTA has the
+# whole unit and writes the output itself), and the largest finite v in rows that nobody sees changes nothing.
+@pytest.mark.parametrize("Hq,Hkv,D,N,S_max", [(2, 2, 64, 40, 64), (8, 1, 64, 40, 64), (2, 2, 128, 40, 64), (8, 1, 128, 40, 64),
+                                              (16, 2, 64, 40, 40000), (16, 2, 128, 40, 40000)])
+@pytest.mark.parametrize("split_form", [0, 1, 2, 3])
+def test_hidden_rows_have_no_weight_in_any_column(gu, Hq, Hkv, D, N, S_max, split_form):
+    B = 2
+    q = synth.normal_bf16((B, N, Hq, D), 61)
+    k = np.zeros((B, Hkv, S_max, D), dtype=np.uint16)
+    v = np.zeros_like(k)
+    k[:, :, :64] = synth.normal_bf16((B, Hkv, 64, D), 62)
+    v[:, :, :64] = synth.normal_bf16((B, Hkv, 64, D), 63)
+    v[:, :, 8:40] = 0x7F7F                                           # 3.4e38, seen by nobody
+    mask = np.zeros((B, N, 1), dtype=np.uint64)
+    mask[:, 1::2] = np.uint64(0b10100010)                            # every other node sees slots 1, 5 and 7, the rest nothing
+    kv_len = np.zeros(B, dtype=np.int32)
+    out, lse, status = gu.run_attn(q, k, v, kv_len, mask, 0.1, split_form=split_form)
+    want, want_lse = oracle.tree_attn(q, k[:, :, :64], v[:, :, :64], kv_len, mask, 0.1)
+    assert status == 0
+    assert (out[:, 0::2] == 0).all() and np.isneginf(lse[:, :, 0::2]).all()
+    assert np.abs(out - want).max() <= TOL
+    assert np.abs(lse[:, :, 1::2] - want_lse[:, :, 1::2]).max() <= LSE_TOL
+
+
 def test_arbitrary_mask_bits_all_ones_and_zero_rows(gu):
     B, N, Hq, Hkv, D, S_max = 2, 20, 4, 2, 128, 256
     q = synth.normal_bf16((B, N, Hq, D), 21); k = synth.normal_bf16((B, Hkv, S_max, D), 22)
