@@ -704,14 +704,14 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
 #pragma unroll
                         for (int c = 0; c < 8; ++c) mx[c] = __uint_as_float(sraw[c]);
 #pragma unroll
-                        for (int c = 8; c < NC; ++c) mx[c & 7] = fmaxf(mx[c & 7], __uint_as_float(sraw[c]));
+                        for (int c = 8; c < NC; ++c) mx[c & 7] = max_nan(mx[c & 7], __uint_as_float(sraw[c]));
                         // the scale is positive, so it commutes with the maximum
-                        lmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7]))) * p.scale_log2;
+                        lmax = max_nan(max_nan(max_nan(mx[0], mx[1]), max_nan(mx[2], mx[3])), max_nan(max_nan(mx[4], mx[5]), max_nan(mx[6], mx[7]))) * p.scale_log2;
                     }
                     // the row's maximum over the tile: the other thread of the row has the other columns
                     xm[(it & 1) * 256 + ch * 128 + tl] = lmax;
                     if (!pair_sync()) { ok = false; break; }
-                    const float tmax = fmaxf(lmax, xm[(it & 1) * 256 + (ch ^ 1) * 128 + tl]);
+                    const float tmax = max_nan(lmax, xm[(it & 1) * 256 + (ch ^ 1) * 128 + tl]);
                     // move the reference maximum only when the tile exceeds it by more than the gap
                     float alpha = 1.f;
                     bool rescale = false;
@@ -721,6 +721,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                         l_run *= alpha;
                         rescale = has_o;
                     }
+                    if (!(tmax < INFINITY)) l_run = tmax - tmax;             // a NaN or an infinite score: the row is NaN (see inv_sum)
                     if (__any_sync(0xffffffffu, rescale)) {
                         // O was last written by the PV product of step it-1 (same segment: has_o is set); this thread
                         // rescales its half of the row's columns
@@ -843,7 +844,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 float2* pst = reinterpret_cast<float2*>(sm + SMEM_K + (D / 4) * ROWS * 16);  //               [ROWS] (m, l)
                 if (half == 0) {
                     const bool final_out = !CL && sg.slot < 0;
-                    const float inv = final_out ? (l_all > 0.f ? 1.f / l_all : 0.f) : 1.f;
+                    const float inv = final_out ? inv_sum(l_all) : 1.f;
                     __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * D + ch * (D / 2);
                     float4* prow = (CL ? pbuf : p.part_o + (size_t)(final_out ? 0 : sg.slot) * (D / 4) * ROWS) + (size_t)ch * (D / 8) * ROWS + lrow;
 #pragma unroll

@@ -357,9 +357,9 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
 #pragma unroll
                         for (int c = 0; c < 64; c += 16)
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) mx[e] = max3(mx[e], __uint_as_float(s[c + e]), __uint_as_float(s[c + 8 + e]));
+                            for (int e = 0; e < 8; ++e) mx[e] = max3_nan(mx[e], __uint_as_float(s[c + e]), __uint_as_float(s[c + 8 + e]));
                     }
-                    const float tmax = fmaxf(max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), mx[6]), mx[7]) * p.scale_log2;
+                    const float tmax = max_nan(max3_nan(max3_nan(mx[0], mx[1], mx[2]), max3_nan(mx[3], mx[4], mx[5]), mx[6]), mx[7]) * p.scale_log2;
                     // move the reference maximum only when the tile exceeds it by more than the gap
                     float alpha = 1.f;
                     bool rescale = false;
@@ -369,6 +369,7 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
                         l_run *= alpha;
                         rescale = has_o;
                     }
+                    if (!(tmax < INFINITY)) l_run = tmax - tmax;          // a NaN or an infinite score: the row is NaN (see inv_sum)
                     if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll
                         for (int c = 0; c < HD / 16; ++c) {
@@ -432,7 +433,7 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
                 if (!ok) break;
                 tc_fence_after();
                 const bool final_out = !CL && sg.slot < 0;
-                const float inv = final_out ? (l_run > 0.f ? 1.f / l_run : 0.f) : 1.f;
+                const float inv = final_out ? inv_sum(l_run) : 1.f;
                 __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * HD;
                 float4* prow = (CL ? reinterpret_cast<float4*>(sm + R::OFF_K) : p.part_o + (size_t)(final_out ? 0 : sg.slot) * (HD / 4) * kRows) + lrow;
 #pragma unroll

@@ -242,10 +242,17 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     uint64_t r; asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r;
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
+// The largest, NaN if any of them is (fmaxf drops it).
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r;
 }
-// 2^x on the FMA pipe (x <= 120; -inf gives exactly 0, below -126 a denormal or 0 comes out): nearest integer by the
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+    float r; asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
+}
+// 1 / l for a row's sum l >= 0; a row that saw nothing (l = 0) is scaled to zeros, one that saw a NaN or an infinite score
+// (the softmax makes its l NaN, whatever the exponentials gave) to NaN.
+__device__ __forceinline__ float inv_sum(float l) { return l > 0.f ? 1.f / l : l; }
+// 2^x on the FMA pipe (x <= 120, not NaN; -inf gives exactly 0, below -126 a denormal or 0 comes out): nearest integer by the
 // 1.5 * 2^23 trick, a polynomial of degree 5 on the remainder f in [-0.5, 0.5], the integer added into the exponent field (at the
 // clamp the remainder is not negative, so 2^-127 p(f) >= 2^-127 stays a positive pattern, and 0 at f = 0).  The polynomial is
 // 1 + C1 f + ... + C5 f^5 with the largest relative error made smallest: 9.2e-8, 1.7e-7 with the roundings of its fp32
@@ -446,7 +453,7 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
         }
         m_all = m_new;
     }
-    const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+    const float inv = inv_sum(l_all);
     __nv_bfloat16* orow = out + (((size_t)b * N + node) * Hq + head) * HD + cw * 16;
 #pragma unroll
     for (int k = 0; k < 2; ++k)
@@ -513,7 +520,7 @@ __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, 
         m_all = m_new;
     }
     if (!row_ok || part != 0) return;
-    const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+    const float inv = inv_sum(l_all);
     *reinterpret_cast<uint2*>(out + (((size_t)b * N + node) * Hq + head) * HD + c4 * 4) =
         make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
     if (lse && c4 == 0)
@@ -708,7 +715,7 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
                     ll += ml[e][j].y * w;
                     a4.x += w * pv[e][j].x; a4.y += w * pv[e][j].y; a4.z += w * pv[e][j].z; a4.w += w * pv[e][j].w;
                 }
-                const float inv2 = ll > 0.f ? 1.f / ll : 0.f;
+                const float inv2 = inv_sum(ll);
                 *reinterpret_cast<uint2*>(p.out + (size_t)outs[e] * HD + c4s[e] * 4) =
                     make_uint2(pack_bf16(a4.x * inv2, a4.y * inv2), pack_bf16(a4.z * inv2, a4.w * inv2));
                 if (c4s[e] == 0 && p.lse) {

@@ -164,6 +164,40 @@ def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
     assert np.abs(lse - want_lse).max() <= 2e-6
 
 
+# A NaN in a key (or an infinite score) makes every row that sees it NaN, whatever column of a step the key falls on.  One
+# sequence per step column modulo 16, one whose second 64 tokens are all such keys (the duplicated-row layout keeps a state of
+# its own for those), one without any.
+@pytest.mark.parametrize("static", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,D,N,S_max", [(2, 2, 64, 20, 256), (8, 1, 64, 20, 256), (2, 2, 128, 20, 256), (8, 1, 128, 20, 256),
+                                              (32, 2, 64, 20, 40000), (32, 2, 128, 20, 40000)])
+def test_nan_and_infinite_scores_reach_the_rows_that_see_them(gu, Hq, Hkv, D, N, S_max, static):
+    from paper_2509_15235_b200 import binding
+    B, S, used = 18, 192, 256
+    q = synth.normal_bf16((B, N, Hq, D), 91)
+    k = np.zeros((B, Hkv, S_max, D), dtype=np.uint16)
+    v = np.zeros_like(k)
+    k[:, :, :used] = synth.normal_bf16((B, Hkv, used, D), 92)
+    v[:, :, :used] = synth.normal_bf16((B, Hkv, used, D), 93)
+    mask, _, _ = oracle.tree_mask(np.tile(np.array([-1, 0, 0] + [1] * (N - 3), dtype=np.int32), (B, 1)))
+    kv_len = np.full(B, S, dtype=np.int32)
+    for special in (0x7FC0, 0x7F80):                                 # NaN, +inf in one element of the key
+        for b in range(16):
+            k[b, :, 2 + 16 * (b % 8) + b, 3] = special
+        k[16, :, 64:128, 3] = special
+        if static:
+            out = torch.zeros((B, N, Hq, D), dtype=torch.bfloat16, device="cuda")
+            binding.tree_verify_attn_static(gu.bf16_dev(q), gu.bf16_dev(k), gu.bf16_dev(v), gu.i32_dev(kv_len), gu.u64_dev(mask), 0.1, out)
+            out = out.float().cpu().numpy()
+        else:
+            out, _, status = gu.run_attn(q, k, v, kv_len, mask, 0.1)
+            assert status == 0
+        # an infinite element of the key: the score is +inf where q > 0 there, else -inf and the key has no weight
+        want = np.ones((B, N, Hq), dtype=bool) if special == 0x7FC0 else synth.bf16_bits_to_f32(q)[..., 3] > 0
+        want[17] = False
+        assert np.isnan(out[want]).all()
+        assert np.isfinite(out[~want]).all()
+
+
 # Hidden tree rows have weight exactly 0 in every column of a step: rows that see nothing are zeros (also where one CTA has the
 # whole unit and writes the output itself), and the largest finite v in rows that nobody sees changes nothing.
 @pytest.mark.parametrize("Hq,Hkv,D,N,S_max", [(2, 2, 64, 40, 64), (8, 1, 64, 40, 64), (2, 2, 128, 40, 64), (8, 1, 128, 40, 64),
