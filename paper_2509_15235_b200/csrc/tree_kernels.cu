@@ -312,16 +312,25 @@ accept_commit_kernel(void* const* __restrict__ cache_ptrs, int layer_begin, cons
     if (kv_len_out && writer && threadIdx.x == 0) kv_len_out[b] = S + L;
 }
 
+// Blocks of that kernel an SM holds at once; found once per device.
+static int g_commit_blocks_per_sm = 1;
+cudaError_t init_accept_commit() {
+    int n = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, accept_commit_kernel, 256, 0);
+    if (e == cudaSuccess && n > 0) g_commit_blocks_per_sm = n;
+    return e;
+}
+
 cudaError_t launch_accept_commit(void* const* cache_ptrs, int layer_begin, int layer_end, const int32_t* draft,
                                  const int32_t* target, const int32_t* parents, const int32_t* kv_len,
                                  int32_t* path, int32_t* accept_len, int32_t* bonus, int32_t* kv_len_out, int B, int N,
-                                 int Hkv, int D, int S_max, int* status, cudaStream_t st, const int32_t* block_table,
+                                 int Hkv, int D, int S_max, int sm_count, int* status, cudaStream_t st, const int32_t* block_table,
                                  int table_stride, int page_rows, int num_blocks, int token_major) {
     if (B == 0 || layer_end <= layer_begin) return cudaSuccess;
-    // Every block repeats its sequence's acceptance (2.5 us of dependent loads), so all blocks should be resident at once: 8 per
-    // SM.  Beyond that a block serves several layers, whose moves cost it 1 us each, instead of a wave that costs it all
-    // (4 x 40 heads x 8 layers 7.9 -> 5.4 us, 8 x 40 x 12 14.9 -> 7.7).
-    const int layers = layer_end - layer_begin, room = 8 * 148;
+    // Every block repeats its sequence's acceptance (2.5 us of dependent loads), so all blocks should be resident at once.  Beyond
+    // that a block serves several layers, whose moves cost it 1 us each, instead of a wave that costs it all (4 x 40 heads x 8
+    // layers 7.9 -> 5.4 us, 8 x 40 x 12 14.9 -> 7.7).
+    const int layers = layer_end - layer_begin, room = g_commit_blocks_per_sm * sm_count;
     const long long blocks = (long long)Hkv * B * layers;
     const int lpb = (int)((blocks + room - 1) / room);
     dim3 grid(Hkv, B, (layers + lpb - 1) / lpb);

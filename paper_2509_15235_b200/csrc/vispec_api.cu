@@ -67,8 +67,8 @@ bool init_device(int device) {
     static bool done[64];
     std::lock_guard<std::mutex> lock(mu);
     if (device < 64 && done[device]) return true;
-    const bool ok = init_attn_generic() == cudaSuccess && init_attn_tc5() == cudaSuccess && init_attn_tc5_wide() == cudaSuccess && init_stream_probe() == cudaSuccess &&
-                    init_accept_sampled(device) == cudaSuccess;
+    const bool ok = init_attn_generic() == cudaSuccess && init_attn_tc5() == cudaSuccess && init_attn_tc5_wide() == cudaSuccess &&
+                    init_stream_probe() == cudaSuccess && init_accept_sampled(device) == cudaSuccess && init_accept_commit() == cudaSuccess;
     if (device < 64) done[device] = ok;
     return ok;
 }
@@ -448,7 +448,7 @@ int vispec_accept_commit_paged(vispec_ctx* c, int layer_begin, int layer_end, co
     if (rc != VISPEC_OK) return rc;
     const int pr = c->page_rows[layer_begin];
     if (launch_accept_commit(c->d_cache_ptrs, layer_begin, layer_end, draft_ids, target_ids, parents, kv_len, path,
-                             accept_len, bonus, kv_len_out, B, N, s.Hkv, s.D, table_stride * pr, c->d_status,
+                             accept_len, bonus, kv_len_out, B, N, s.Hkv, s.D, table_stride * pr, c->sm_count, c->d_status,
                              (cudaStream_t)stream, block_table, table_stride, pr, c->num_blocks[layer_begin],
                              c->token_major[layer_begin]) != cudaSuccess)
         return VISPEC_E_CUDA;
@@ -592,7 +592,7 @@ int vispec_accept_commit(vispec_ctx* c, int layer_begin, int layer_end, const in
                           (cudaStream_t)stream) != cudaSuccess)
             return VISPEC_E_CUDA;
     } else if (launch_accept_commit(c->d_cache_ptrs, layer_begin, layer_end, draft_ids, target_ids, parents, kv_len,
-                                    path, accept_len, bonus, kv_len_out, B, N, s.Hkv, s.D, s.S_max, c->d_status,
+                                    path, accept_len, bonus, kv_len_out, B, N, s.Hkv, s.D, s.S_max, c->sm_count, c->d_status,
                                     (cudaStream_t)stream) != cudaSuccess) {
         return VISPEC_E_CUDA;
     }

@@ -52,10 +52,11 @@ cudaError_t launch_kv_compact(void* const* cache_ptrs, int layer_begin, int laye
                               cudaStream_t st, const int32_t* block_table = nullptr, int table_stride = 0,
                               int page_rows = 0, int num_blocks = 0, int token_major = 0);
 
+cudaError_t init_accept_commit();              // once per device, with that device current
 cudaError_t launch_accept_commit(void* const* cache_ptrs, int layer_begin, int layer_end, const int32_t* draft,
                                  const int32_t* target, const int32_t* parents, const int32_t* kv_len,
                                  int32_t* path, int32_t* accept_len, int32_t* bonus, int32_t* kv_len_out, int B, int N,
-                                 int Hkv, int D, int S_max, int* status, cudaStream_t st,
+                                 int Hkv, int D, int S_max, int sm_count, int* status, cudaStream_t st,
                                  const int32_t* block_table = nullptr, int table_stride = 0, int page_rows = 0,
                                  int num_blocks = 0, int token_major = 0);
 
