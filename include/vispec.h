@@ -110,10 +110,11 @@ typedef enum vispec_option {
      * their successor start as soon as they have started themselves, so through a run of back-to-back attention
      * calls the early reads of a later call may overlap the kernel that preceded the first of them.  The rule:
      * a kernel that writes kv_len or committed cache slots (vispec_kv_compact, vispec_accept_commit) must be
-     * followed by at least one kernel that does not start early - vispec_tree_mask_build, vispec_rope_tree_rows
-     * (it waits for its predecessor before it lets its successor in) or any ordinary kernel - before the next
-     * attention call with this option on; the decoding cycle (commit, mask build, attention x layers) satisfies
-     * it.  Otherwise set 0 for the attention calls in between: then nothing is read early. */
+     * followed by at least one kernel that waits for its predecessor before it lets its successor in - any ordinary
+     * kernel, or any call of this library other than the attention calls and the stream probe (they are all launched
+     * early, but wait first: vispec_tree_mask_build, vispec_rope_tree_rows, vispec_rope_table_build,
+     * vispec_tree_rerank, the acceptances, the commits) - before the next attention call with this option on; the
+     * decoding cycle (commit, mask build, attention x layers) satisfies it.  Otherwise set 0 for the attention calls in between: then nothing is read early. */
     VISPEC_OPT_EARLY_PREFETCH = 1,
     /* Default 0 (1 if the environment has VISPEC_FORCE_GENERIC=1 at context creation).  Route attention
      * through the shape-generic warp-level kernel even where the TMA/tcgen05 kernel applies. */

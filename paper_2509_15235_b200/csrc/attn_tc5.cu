@@ -20,13 +20,14 @@
 //
 // Inside a CTA the 12 warps are specialised:
 //   warp 0     TMA producer: K ring and V ring of 128-token stages (3 x 32 KB each, 128-byte swizzle, evict-first
-//              in L2); it runs ahead across segment boundaries
-//   warp 1     issuer (one thread) of S = Q K^T as 128x128x16 tcgen05.mma; owns the TMEM allocation
-//   warp 2     issuer (one thread) of O += P V; the two chains wait on different barriers, so each has its own
-//              thread and neither's waits delay the other's instructions
-//   warp 3     derives the schedule from kv_len; with at most 64 rows per unit (its lane 0; the whole warp on a paged
-//              cache) and on pools of 16-row blocks it then produces the V ring, so that warp 0's K copies never
-//              queue behind a wait for a V stage
+//              in L2; head size 64: 6 x 16 KB); it runs ahead across segment boundaries
+//   warp 1     issuer of S = Q K^T as 128x128x16 tcgen05.mma (the warp walks the steps and waits, one elected lane
+//              issues); owns the TMEM allocation
+//   warp 2     issuer of O += P V, likewise; the two chains wait on different barriers, so each has its own warp and
+//              neither's waits delay the other's instructions
+//   warp 3     derives the schedule from kv_len; with at most 64 rows per unit (its lane 0 in the cluster form of a
+//              contiguous cache, else the whole warp) and on pools of 16-row blocks it then produces the V ring, so that
+//              warp 0's K copies never queue behind a wait for a V stage
 //   warps 4-11 softmax: thread <-> TMEM lane; warps w and w+4 share the same 32 accumulator rows and each takes
 //              half of a step's columns (the row maximum is exchanged through shared memory), so a row costs
 //              no shuffles; they also load Q at the start of every segment and run the segment epilogue
@@ -392,18 +393,18 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     const int sk = it % NSK;
                     if (!prod_wait(bar(B_KEMPTY + sk), ((it / NSK) & 1) ^ 1)) { ok = false; break; }
                     if (leader) {
-                    mbar_expect_tx(bar(B_KFULL + sk), STAGE_BYTES);
-                    tma_load_3d(base + SMEM_K + sk * STAGE_BYTES, &k_map, bar(B_KFULL + sk), 0, tok, bh, pol);
-                    if constexpr (NH == 2) tma_load_3d(base + SMEM_K + sk * STAGE_BYTES + HALF_BYTES, &k_map, bar(B_KFULL + sk), 64, tok, bh, pol);
+                        mbar_expect_tx(bar(B_KFULL + sk), STAGE_BYTES);
+                        tma_load_3d(base + SMEM_K + sk * STAGE_BYTES, &k_map, bar(B_KFULL + sk), 0, tok, bh, pol);
+                        if constexpr (NH == 2) tma_load_3d(base + SMEM_K + sk * STAGE_BYTES + HALF_BYTES, &k_map, bar(B_KFULL + sk), 64, tok, bh, pol);
                     }
                     ++nk;
                     if constexpr (!SPLIT_V) {
                         const int sv = it % NSV;
                         if (!prod_wait(bar(B_VEMPTY + sv), ((it / NSV) & 1) ^ 1)) { ok = false; break; }
                         if (leader) {
-                        mbar_expect_tx(bar(B_VFULL + sv), STAGE_BYTES);
-                        tma_load_3d(base + SMEM_V + sv * STAGE_BYTES, &v_map, bar(B_VFULL + sv), 0, tok, bh, pol);
-                        if constexpr (NH == 2) tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
+                            mbar_expect_tx(bar(B_VFULL + sv), STAGE_BYTES);
+                            tma_load_3d(base + SMEM_V + sv * STAGE_BYTES, &v_map, bar(B_VFULL + sv), 0, tok, bh, pol);
+                            if constexpr (NH == 2) tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
                         }
                         ++nv;
                     }
@@ -463,9 +464,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     const int sv = it % NSV;
                     if (!prod_wait(bar(B_VEMPTY + sv), ((it / NSV) & 1) ^ 1)) { ok = false; break; }
                     if (leader) {
-                    mbar_expect_tx(bar(B_VFULL + sv), STAGE_BYTES);
-                    tma_load_3d(base + SMEM_V + sv * STAGE_BYTES, &v_map, bar(B_VFULL + sv), 0, tok, bh, pol);
-                    if constexpr (NH == 2) tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
+                        mbar_expect_tx(bar(B_VFULL + sv), STAGE_BYTES);
+                        tma_load_3d(base + SMEM_V + sv * STAGE_BYTES, &v_map, bar(B_VFULL + sv), 0, tok, bh, pol);
+                        if constexpr (NH == 2) tma_load_3d(base + SMEM_V + sv * STAGE_BYTES + HALF_BYTES, &v_map, bar(B_VFULL + sv), 64, tok, bh, pol);
                     }
                 }
             }

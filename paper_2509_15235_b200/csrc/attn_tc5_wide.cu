@@ -13,7 +13,7 @@
 // on the FMA pipe (292, 283, 277, 276 with a cubic that was dropped for its error; none is as fast as 1/8, see kPolyEvery).
 //
 //   warp 0     TMA producer of the K ring (2 x 32 KB; head size 64: 4 x 16 KB)
-//   warp 1     issuer (one thread) of all products, in the order S_A S_B | PV_A S_A' PV_B S_B' | ...: they complete in the
+//   warp 1     issuer (one elected lane) of all products, in the order S_A S_B | PV_A S_A' PV_B S_B' | ...: they complete in the
 //              order of issue, so S of a step may overwrite P of the step before, which frees half of the tensor memory, and
 //              the completion of S tells that O and P are free; a PV product starts when the first half of its P is there.
 //              (An issuer per tile was slower: the tiles' products interleave, both end together, and the tiles fall into

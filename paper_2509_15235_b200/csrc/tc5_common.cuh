@@ -1,5 +1,5 @@
-// Device helpers of the TMA + tcgen05 attention kernel: PTX wrappers, the work schedule every CTA derives from kv_len,
-// the merge of split-KV partials, and the launch helper.  Included by the kernel's translation unit only.
+// What the two TMA + tcgen05 attention kernels (attn_tc5.cu, attn_tc5_wide.cu) share: PTX wrappers, the exponential on the FMA
+// pipe, the work schedule every CTA derives from kv_len, the paged producer, and the merge of split-KV partials.
 #pragma once
 #include <cuda_bf16.h>
 #include <cstdint>
@@ -736,7 +736,7 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
 // for units cut into a few pieces.  Q = 1, 2, 4, 8, fine: grid (unit, group of 32/Q rows x group of 16 columns), Q lanes share
 // a row, a warp sums 4 output columns - for units cut over many CTAs (few sequences, long caches), where the rounds of
 // loads are what the merge takes: qwen3b_S32768_N16_B1 (2 units over 148 CTAs, 74 partials each) 42.7 us per layer coarse,
-// 28.1 with Q = 1, MERGE_FIG with Q = 8; with many units of two partials the coarse shape is 3 % faster.
+// 28.1 with Q = 1, 19.7 with Q = 8; with many units of two partials the coarse shape is 3 % faster.
 // The blocks are small: they are launched early (programmatic dependent launch) and must not keep the next layer's
 // attention CTAs off the SMs.
 template <int ROWS, int Q, int HD>

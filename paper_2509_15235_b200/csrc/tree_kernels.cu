@@ -1,11 +1,12 @@
-// Integer kernels of the verification step: ancestor mask, greedy acceptance, KV commit.
-// All three are latency-bound (a few KB of traffic); each is a single launch.
+// The small kernels around the attention: ancestor mask, greedy acceptance, KV commit (alone and with the acceptance), rotary
+// placement of the tree's rows and its angle table, tree rerank.  All are latency-bound (a few KB of traffic, the rotary
+// placement up to 15 MB); each is a single launch.
 //
 // What bounds them is the chain launch -> first load -> dependent load -> store, so (a) every kernel is launched with
 // programmatic stream serialisation (its blocks are resident and past their set-up when the predecessor ends; every
 // read and write comes after griddepcontrol.wait), and (b) loads that do not depend on one another go out together.
-// Only a kernel that has waited for its predecessor lets its successor in early (tree_mask_kernel, rope_rows_kernel,
-// rope_table_kernel): an attention call that follows reads kv_len and committed rows before its own wait.  The commits
+// Only a kernel that has waited for its predecessor lets its successor in early (tree_mask_kernel, tree_rerank_kernel,
+// rope_rows_kernel, rope_table_kernel): an attention call that follows reads kv_len and committed rows before its own wait.  The commits
 // never do: what follows them starts when they have ended.
 #include <cuda_bf16.h>
 

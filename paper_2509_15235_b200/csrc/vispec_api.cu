@@ -15,7 +15,8 @@ size_t workspace_bytes(const vispec_shape& s, int sm_count) {
     const size_t units64 = (size_t)s.B_max * s.Hkv * ((G * s.N_max + 63) / 64);
     const size_t slot = slot_bytes(s.D);
     // generic kernel: at most 4*SMs + units partials of 64 rows (half slots);
-    // persistent kernel: at most two partials of 128 rows per CTA, one CTA per SM.
+    // even split: at most two partials per CTA, one CTA per SM, of 128 rows, or of 256 in the two-tile kernel (which uses the
+    // generic kernel's share as well: 512 rows per SM in all).
     return kCounterBytes + (4 * (size_t)sm_count + units64) * (slot / 2) + 2 * (size_t)sm_count * slot + q_scratch_bytes(s);
 }
 
