@@ -50,3 +50,12 @@ def run_attn(q, k, v, kv_len, mask, scale, want_lse=True, B_max=None, N_max=None
     res = out.float().cpu().numpy(), (lse.cpu().numpy() if want_lse else None), status
     ctx.close()
     return res
+
+
+def kernels_of(fn):
+    """(fn(), the names of the kernels it launched)."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        res = fn()
+        torch.cuda.synchronize()
+    return res, {e.key for e in prof.key_averages()}

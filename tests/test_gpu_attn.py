@@ -111,7 +111,8 @@ def test_two_tile_units(gu, Hq, Hkv, D, N, kv_len, S_max, split_form):
         v[b, :, kv_len[b] + N:] = 0x7FC0
     parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
     mask, _, _ = oracle.tree_mask(parents)
-    _check(gu, q, k, v, np.array(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=split_form)
+    _, kernels = gu.kernels_of(lambda: _check(gu, q, k, v, np.array(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=split_form))
+    assert any("attn_tc5_wide_kernel" in n for n in kernels), kernels      # the estimates choose it: a change there must not go unseen
 
 
 # The merge of a cluster's partials at head size 64 over every cluster size that 4 to 96 units lead to (15 units or fewer: eight

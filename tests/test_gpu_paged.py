@@ -105,7 +105,9 @@ def test_paged_attention_two_tile_units(page_rows):
     for b in range(2):
         used = -(-(int(kv_len[b]) + 60) // page_rows)
         wide[b, :used] = table[b, :used]
-    out, lse, status = _run_paged(q, pools, wide, kv_len, mask, scale)
+    import gpu_util as gu
+    (out, lse, status), kernels = gu.kernels_of(lambda: _run_paged(q, pools, wide, kv_len, mask, scale))
+    assert any("attn_tc5_wide_kernel" in n for n in kernels), kernels
     want, want_lse = oracle.tree_attn(q, k, v, kv_len, mask, scale)
     assert status == 0 and not np.isnan(out).any()
     assert np.abs(out - want).max() <= TOL and np.abs(lse - want_lse).max() <= LSE_TOL

@@ -64,6 +64,23 @@ def test_sampled_acceptance_vocabulary_sizes_ragged_slices_and_many_rounds(V):
         assert (alen > 1).any() and (alen == 1).any()
 
 
+# Slices longer than the shared memory that keeps them (25600 elements of each row per CTA): clusters of 16 for few sequences, of 8
+# for many; vector and scalar loads.  Most of the weight lies on the elements that are not kept, and the star's children are
+# rejected often, so passes repeat over both parts and the bonus token comes from the unkept one.
+@pytest.mark.parametrize("B,V,ctas", [(2, 409604, 16), (2, 409605, 16), (20, 204804, 8), (20, 204805, 8)])
+def test_sampled_acceptance_slices_beyond_shared_memory(B, V, ctas):
+    N, per = 4, -(-(-(-V // ctas)) // 4) * 4
+    parents = np.tile(np.array([-1, 0, 0, 0], dtype=np.int32), (B, 1))
+    s = synth.make_sampled_inputs(parents, V, 900 + B, sharpness=1.0, disagreement=1.5)
+    unkept = (np.arange(ctas)[:, None] * per + np.arange(25600, per)).ravel()
+    unkept = unkept[unkept < V]
+    assert 0 < len(unkept) <= 4 * ctas
+    p = s["p_target"] * np.float32(0.1)
+    p[:, :, unkept] += np.float32(0.9 / len(unkept))
+    path, alen, bonus, bad = _check(parents, s["draft_ids"], p, s["p_draft"], s["u_accept"], s["u_bonus"])
+    assert bad == 0 and np.isin(bonus, unkept).any()
+
+
 def test_sampled_acceptance_degenerate_rows():
     """Zero entries, one-hot rows, an unnormalised target row whose residual is empty after the first rejection
     (the bonus token then comes from the target row), a target row without any weight (bonus -1), a star and a
