@@ -1075,6 +1075,9 @@ static int query_max_clusters(bool pair, int k) {
 // per step over 7 TB/s; the row blocks of a kv head read the same tiles, so one in n_mblocks comes from HBM; a
 // step's bytes follow the head size, its softmax does not).  The host knows only the capacity S_max, not kv_len: the
 // estimate is for full caches unless the caller has given the length it expects (VISPEC_OPT_KV_LEN_HINT).
+// Both sides of the line between the forms, clusters / even split, us per layer: 16 query and 2 kv heads, 1 x 16 nodes on 2048 10.4 /
+// 13.8, on 8192 16.9 / 15.0, on 32768 42.7 / 20.0, 4 x 60 on 8192 28.5 / 34.2; 32 heads, 1 x 60 on 3904 15.7 / 20.3, 4 x 60 on
+// 2000 30.0 / 32.3; 40 heads, 1 x 30 on 8000 30.4 / 33.4, 2 x 30 on 4000 38.7 / 36.7.
 static double tc5_step_us(const AttnArgs& a, bool pair, int n_mblocks, double ctas) {
     const double busy = ctas / a.sm_count, compute = pair ? 0.8 + 0.25 * busy : 1.05 + 0.15 * busy;
     return fmax(a.D == 64 ? 0.9 * compute : compute, ctas * 0.0093 * (a.D / 128.0) / n_mblocks);
@@ -1115,6 +1118,8 @@ static int tc5_max_cluster(const AttnArgs& a, bool pair, int n_mblocks) {
 // rows in the duplicated layout make twice the units, and a step of such a unit costs its softmax threads half the
 // columns, at the price of every K/V tile crossing from L2 twice as often and half of each product computed for nothing.
 // (As an even split the smaller blocks gain nothing.)  The best estimate decides, a form that options ask for first.
+// Clusters with 64-row units / with 128: 16 query and 2 kv heads, 1 x 16 nodes on 2048 8.9 / 10.4, 4 x 16 on 8192 17.6 / 18.2, 1 x 60 on
+// 8192 17.0 / 17.7, 8 x 60 on 2048 23.4 / 19.9, 4 x 60 on 8192 33.8 / 28.5; 28 / 4 heads, 1 x 60 on 3344 13.4 / 14.8, 4 x 60 30.7 / 25.1.
 struct Tc5Layout { bool pair; int rows, n_mblocks, ck; double est_us; };
 static Tc5Layout tc5_layout(const AttnArgs& a) {
     const int rows_total = (a.Hq / a.Hkv) * a.N;
