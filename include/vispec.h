@@ -166,7 +166,8 @@ int vispec_tree_mask_build(vispec_ctx* ctx, const int32_t* parents, int B, int N
  *   out[b][i][h] = sum_{j in A} softmax_j(scale * <q[b][i][h], k[b][h/G][j]>) * v[b][h/G][j]
  * computed with fp32 accumulation from bf16 inputs, rounded once to bf16 (nearest even).
  * lse [B,Hq,N] fp32 (optional, may be NULL) receives log sum_{j in A} exp(score_j).
- * An empty A gives out = 0 and lse = -inf.  tree_mask is an INPUT (any bit pattern is honoured,
+ * An empty A gives out = 0 and lse = -inf; a NaN or +infinite score of a key in A gives out = NaN and lse = -inf for that
+ * row.  tree_mask is an INPUT (any bit pattern is honoured,
  * it is never re-derived from parents).  Cache slots at or beyond S + N are never interpreted
  * (they may hold NaN patterns); tree rows that a node's mask hides get weight exactly 0 and must
  * hold finite values, as rows written by the K/V projection do.  `positions` [B,N] (kv_len + depth) may be
