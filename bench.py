@@ -40,11 +40,11 @@ FALLBACK_HBM_GBS = 6650.0
 # (dram__bytes_read.sum + dram__bytes_write.sum, two launches averaged).  A figure is only valid for the kernel it was
 # taken on: set an entry to None when the attention kernel changes and take the counters again.
 NCU_TRAFFIC_BYTES_PER_LAUNCH = {
-    "llava7b": 66_180_000,                # 65.58 MB read + 0.61 MB written
-    "llava13b_b4": 335_860_000,           # 330.23 MB read + 5.63 MB written
-    "qwen3b_S32768_N16_B8": 274_060_000,  # attention launch only (270.09 + 3.97 MB); the merge kernel is its own launch
-    "qwen3b_S8192_N60_B4": 35_150_000,    # four row blocks per kv head share their tiles through L2
-    "qwen7b": 7_580_000,                  # seven row blocks per kv head share their tiles through L2
+    "llava7b": 65_950_000,                # 65.58 MB read + 0.37 MB written
+    "llava13b_b4": 334_820_000,           # attention launch only (330.22 MB read + 4.59 MB written); the merge kernel is its own launch
+    "qwen3b_S32768_N16_B8": 273_330_000,  # attention launch only (270.07 + 3.25 MB); the merge kernel is its own launch
+    "qwen3b_S8192_N60_B4": 35_140_000,    # four row blocks per kv head share their tiles through L2
+    "qwen7b": 7_590_000,                  # seven row blocks per kv head share their tiles through L2
 }
 FALLBACK_BF16_TFLOPS = 1400.0             # sustained figure of the fallback measurement
 EXP_PER_CLK_PER_SM = 16                   # special-function lanes of one SM (4 per scheduler)
