@@ -301,7 +301,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         }
         for (int i = 0; i < 4; ++i) mbar_init(bar(B_PAIRX + i), 64);
         mbar_init(bar(B_QFULL), kSmx);
-        mbar_init(bar(B_XCH), 128); mbar_init(bar(B_XFREE), 128);
+        mbar_init(bar(B_XCH), kSmx); mbar_init(bar(B_XFREE), kSmx);
         mbar_init(bar(B_SEGSYNC), kSmx);
         if (ROPE) mbar_init(bar(B_ROWS), cluster_size());
         *abort_flag = 0;
@@ -801,100 +801,99 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 if (!ok) break;
 
                 // ---- segment epilogue: wait for the last product, add up the row statistics, (PAIR) merge the two
-                // halves, write out.  A thread owns columns [D/2 ch, D/2 ch + D/2) of its lane's accumulator row. ----
+                // halves, write out.  FULL: a thread owns columns [D/2 ch, D/2 ch + D/2) of its lane's accumulator row.  PAIR:
+                // the two lanes with copies of a row each take half of those columns and hand the other half over. ----
                 if (sg.n > 0) ok = mbar_wait_warp(bar(B_PVDONE + ((it - 1) & 1)), ((it - 1) >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
+                constexpr int KC = PAIR ? D / 4 : D / 2;             // output columns of a thread, from col0 on
+                const int col0 = ch * (D / 2) + (PAIR ? half * KC : 0);
+                uint32_t o[KC];
+                auto o_load = [&](int col) {
+#pragma unroll
+                    for (int c = 0; c < KC; c += KC < 32 ? 16 : 32) {
+                        if constexpr (KC < 32) tmem_ld16(lane_addr + COL_O + col + c, o + c);
+                        else tmem_ld32(lane_addr + COL_O + col + c, o + c);
+                    }
+                    tmem_wait_ld();
+                };
                 // (the tile-maximum slots are idle: the other thread of the row read its last one before it arrived
                 // for the last PV product)
                 xm[ch * 128 + tl] = l_run;
                 if (ch == 0) xm[256 + tl] = has_o ? m_ref : -INFINITY;
-                if (!pair_sync()) { ok = false; break; }
-                const float l_lane = xm[tl] + xm[128 + tl];                  // l of this lane's row copy
-                float w_me = has_o ? 1.f : 0.f, w_other = 0.f, m_all = has_o ? m_ref : -INFINITY, l_all = l_lane;
+                float w_me = has_o ? 1.f : 0.f, w_other = 0.f, m_all = has_o ? m_ref : -INFINITY, l_all;
                 if (PAIR) {
-                    if (half == 1) {
-                        // hand the raw accumulator to the lane that owns the row (the Q tile is idle: every S product
-                        // of the segment has completed); the statistics are in place already
+                    // hand the raw accumulator of the other lane's columns to it (the Q tile is idle: every S product of the
+                    // segment has completed)
+                    const int give = ch * (D / 2) + (half ^ 1) * KC;
+                    o_load(give);
 #pragma unroll
-                        for (int c = 0; c < NH; ++c) {
-                            uint32_t o[32];
-                            tmem_ld32(lane_addr + COL_O + ch * (D / 2) + c * 32, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int c4 = 0; c4 < 8; ++c4)
-                                xch[(ch * (D / 8) + c * 8 + c4) * 64 + lrow] = make_float4(__uint_as_float(o[4 * c4]), __uint_as_float(o[4 * c4 + 1]),
-                                                                                     __uint_as_float(o[4 * c4 + 2]), __uint_as_float(o[4 * c4 + 3]));
-                        }
-                        tc_fence_before();
-                        mbar_arrive(bar(B_XCH));
-                    } else {
-                        ok = mbar_wait_warp(bar(B_XCH), seg & 1, abort_flag);
-                        if (!ok) break;
-                        const float m_o = xm[256 + 64 + tl], l_o = xm[64 + tl] + xm[128 + 64 + tl];
-                        m_all = fmaxf(m_all, m_o);
-                        const float m_fin = (m_all == -INFINITY) ? 0.f : m_all;
-                        w_me = has_o ? exp2f(m_ref - m_fin) : 0.f;
-                        w_other = exp2f(m_o - m_fin);                   // 0 when the other half saw nothing
-                        l_all = l_lane * w_me + l_o * w_other;
-                    }
+                    for (int c4 = 0; c4 < KC / 4; ++c4)
+                        xch[(give / 4 + c4) * 64 + lrow] = make_float4(__uint_as_float(o[4 * c4]), __uint_as_float(o[4 * c4 + 1]),
+                                                                       __uint_as_float(o[4 * c4 + 2]), __uint_as_float(o[4 * c4 + 3]));
+                    mbar_arrive(bar(B_XCH));
+                    o_load(col0);
+                    tc_fence_before();
+                    if (!mbar_wait_warp(bar(B_XCH), seg & 1, abort_flag)) { ok = false; break; }
+                    const float m_o = xm[256 + (tl ^ 64)], l_o = xm[tl ^ 64] + xm[128 + (tl ^ 64)];
+                    m_all = fmaxf(m_all, m_o);
+                    const float m_fin = (m_all == -INFINITY) ? 0.f : m_all;
+                    w_me = has_o ? exp2f(m_ref - m_fin) : 0.f;
+                    w_other = exp2f(m_o - m_fin);                   // 0 when the other half saw nothing
+                    l_all = (xm[tl] + xm[128 + tl]) * w_me + l_o * w_other;
+                } else {
+                    mbar_arrive(bar(B_PAIRX + sp));
+                    o_load(col0);
+                    tc_fence_before();
+                    if (!mbar_wait_warp(bar(B_PAIRX + sp), px & 1, abort_flag)) { ok = false; break; }
+                    ++px;
+                    l_all = xm[tl] + xm[128 + tl];
                 }
                 // O is only defined once a product has run (an empty cluster part never ran one): select, never
                 // multiply, where the weight is zero
-                float4* pbuf = reinterpret_cast<float4*>(sm + SMEM_K);                       // cluster form: [D/4 col4][ROWS]
-                float2* pst = reinterpret_cast<float2*>(sm + SMEM_K + (D / 4) * ROWS * 16);  //               [ROWS] (m, l)
-                if (half == 0) {
-                    const bool final_out = !CL && sg.slot < 0;
-                    const float inv = final_out ? inv_sum(l_all) : 1.f;
-                    __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * D + ch * (D / 2);
-                    float4* prow = (CL ? pbuf : p.part_o + (size_t)(final_out ? 0 : sg.slot) * (D / 4) * ROWS) + (size_t)ch * (D / 8) * ROWS + lrow;
+                const bool final_out = !CL && sg.slot < 0;
+                const float inv = final_out ? inv_sum(l_all) : 1.f;
+                float v[KC];
 #pragma unroll
-                    for (int c = 0; c < NH; ++c) {
-                        uint32_t o[32];
-                        tmem_ld32(lane_addr + COL_O + ch * (D / 2) + c * 32, o);
-                        tmem_wait_ld();
-                        float v[32];
+                for (int e = 0; e < KC; ++e) v[e] = has_o ? __uint_as_float(o[e]) * w_me : 0.f;
+                if (PAIR) {
+                    if (w_other > 0.f) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = has_o ? __uint_as_float(o[e]) * w_me : 0.f;
-                        if (PAIR) {
-                            if (w_other > 0.f) {
-#pragma unroll
-                                for (int c4 = 0; c4 < 8; ++c4) {
-                                    const float4 w = xch[(ch * (D / 8) + c * 8 + c4) * 64 + lrow];
-                                    v[4 * c4] += w.x * w_other; v[4 * c4 + 1] += w.y * w_other;
-                                    v[4 * c4 + 2] += w.z * w_other; v[4 * c4 + 3] += w.w * w_other;
-                                }
-                            }
-                        }
-                        if (final_out) {
-                            if (row_ok) {
-#pragma unroll
-                                for (int c8 = 0; c8 < 4; ++c8)
-                                    *reinterpret_cast<uint4*>(orow + c * 32 + c8 * 8) =
-                                        make_uint4(pack_bf16(v[8 * c8] * inv, v[8 * c8 + 1] * inv), pack_bf16(v[8 * c8 + 2] * inv, v[8 * c8 + 3] * inv),
-                                                   pack_bf16(v[8 * c8 + 4] * inv, v[8 * c8 + 5] * inv), pack_bf16(v[8 * c8 + 6] * inv, v[8 * c8 + 7] * inv));
-                            }
-                        } else if (CL || row_ok) {
-#pragma unroll
-                            for (int c4 = 0; c4 < 8; ++c4)
-                                prow[(size_t)(c * 8 + c4) * ROWS] = make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+                        for (int c4 = 0; c4 < KC / 4; ++c4) {
+                            const float4 w = xch[(col0 / 4 + c4) * 64 + lrow];
+                            v[4 * c4] += w.x * w_other; v[4 * c4 + 1] += w.y * w_other;
+                            v[4 * c4 + 2] += w.z * w_other; v[4 * c4 + 3] += w.w * w_other;
                         }
                     }
-                    if (ch == 0) {
-                        const float2 stat = make_float2(l_all > 0.f ? m_all : -INFINITY, l_all);
-                        if (CL) {
-                            pst[lrow] = stat;
-                        } else if (row_ok) {
-                            if (final_out) {
-                                if (p.lse) p.lse[((size_t)sg.b * p.Hq + head) * N + node] =
-                                    l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
-                            } else {
-                                p.part_ml[(size_t)sg.slot * ROWS + lrow] = stat;
-                            }
-                        }
-                    }
-                    if (PAIR) mbar_arrive(bar(B_XFREE));
                 }
+                if (final_out) {
+                    if (row_ok) {
+                        __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * D + col0;
+#pragma unroll
+                        for (int c8 = 0; c8 < KC / 8; ++c8)
+                            *reinterpret_cast<uint4*>(orow + c8 * 8) =
+                                make_uint4(pack_bf16(v[8 * c8] * inv, v[8 * c8 + 1] * inv), pack_bf16(v[8 * c8 + 2] * inv, v[8 * c8 + 3] * inv),
+                                           pack_bf16(v[8 * c8 + 4] * inv, v[8 * c8 + 5] * inv), pack_bf16(v[8 * c8 + 6] * inv, v[8 * c8 + 7] * inv));
+                    }
+                } else if (row_ok) {
+                    // cluster form: parked in this CTA's shared memory, [D/4 col4][ROWS] over the K ring
+                    float4* prow = (CL ? reinterpret_cast<float4*>(sm + SMEM_K) : p.part_o + (size_t)sg.slot * (D / 4) * ROWS) + (size_t)(col0 / 4) * ROWS + lrow;
+#pragma unroll
+                    for (int c4 = 0; c4 < KC / 4; ++c4)
+                        prow[(size_t)c4 * ROWS] = make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+                }
+                if (ch == 0 && half == 0 && row_ok) {
+                    const float2 stat = make_float2(l_all > 0.f ? m_all : -INFINITY, l_all);
+                    if (CL) {
+                        reinterpret_cast<float2*>(sm + SMEM_K + (D / 4) * ROWS * 16)[lrow] = stat;      // [ROWS] (m, l)
+                    } else if (final_out) {
+                        if (p.lse) p.lse[((size_t)sg.b * p.Hq + head) * N + node] =
+                            l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+                    } else {
+                        p.part_ml[(size_t)sg.slot * ROWS + lrow] = stat;
+                    }
+                }
+                if (PAIR) mbar_arrive(bar(B_XFREE));
                 if (PAIR && !CL && pa.unit_counters && sg.slot >= 0) {
                     // ---- even split without a merge kernel (rows <= 64 only: with 128 rows the merge kernel is faster): the CTA that delivers a unit's last partial merges the
                     // unit.  Nobody waits for another CTA: a fence, one atomic per segment, and the last arrival

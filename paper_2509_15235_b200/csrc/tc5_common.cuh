@@ -115,6 +115,12 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t local, uint32_t rank) {
 __device__ __forceinline__ float4 dsmem_ld4(uint32_t a) {
     float4 v; asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory"); return v;
 }
+__device__ __forceinline__ float4 smem_ld4(uint32_t a) {
+    float4 v; asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory"); return v;
+}
+__device__ __forceinline__ float2 smem_ld2(uint32_t a) {
+    float2 v; asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory"); return v;
+}
 __device__ __forceinline__ float2 dsmem_ld2(uint32_t a) {
     float2 v; asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory"); return v;
 }
@@ -662,73 +668,81 @@ __device__ __forceinline__ void zero_rejected(const Tc5Params& p, const Sched& s
 // Cluster form: rank cr of ck merges its rows of the unit's partials, parked by every rank at pbuf_a ([HD/4 col4][ROWS]
 // float4) and pst_a ([ROWS] (m, l)) of its own shared memory, and writes them out.  By the NT softmax threads (st).
 // Contains the meeting of the cluster (meet(), false: nothing is merged) and this warp's arrival at the closing one: the
-// indices of the first round are formed before the meeting, and a warp arrives as soon as its last loads from the peers
-// are back, so that neither the divisions nor the output's arithmetic and stores lie between the two barriers.
+// indices are formed before the meeting, and a warp arrives as soon as its last loads from the peers are back, so that
+// neither the divisions nor the output's arithmetic and stores lie between the two barriers.
+// What bounds it is the bytes that cross between the SMs: 16 per cycle and SM, whatever instruction moves them (32 KB in
+// 2170 cycles by loads, bulk copies and asynchronous stores alike; by way of L2 3400).  So a rank's own partial does not
+// cross, only rows that exist are dealt out to the ranks, a thread keeps to one row and fetches its (m, l) once, and each
+// rank goes on from its own partial to the next rank's, so that the ranks do not all read from the same one.
 template <int ROWS, int HD, int NT = 256, class Meet>
 __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st, Meet meet) {
-    const int N = p.N, G = p.Hq / p.Hkv, rows_total = G * N;
-    const int rp = (ROWS + ck - 1) / ck;
-    const int row0 = cr * rp;
-    const int nrows = min(rp, ROWS - row0), total = nrows * (HD / 4);
-    // IT items (row, column quad) at a time per thread, all loads of all KM pieces issued before the first use
-    auto merge_items = [&](auto km_tag, auto it_tag) {
+    constexpr int C4 = HD / 4;                                          // column quads of a row
+    const int N = p.N, G = p.Hq / p.Hkv;
+    const int rows = min(ROWS, G * N - sg.mblock * ROWS);               // of this unit
+    const int rp = (rows + ck - 1) / ck, row0 = cr * rp, nrows = max(1, min(rp, rows - row0));
+    const bool any = row0 < rows;                                       // (fewer rows than ranks: the last ranks have none)
+    const int part = st / nrows, r = st - part * nrows, tpr = min(NT / nrows, C4);   // threads st < tpr * nrows, tpr to a row
+    const bool mine = any && part < tpr;
+    const int grow = sg.mblock * ROWS + row0 + r, node = grow / G, head = sg.kvh * G + (grow - node * G);
+    __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * HD;
+    if (!meet()) { cluster_arrive_release(); return; }
+    const uint32_t prow = pbuf_a + (uint32_t)((part * ROWS + row0 + r) * 16), prow_ml = pst_a + (uint32_t)((row0 + r) * 8);
+    auto peer = [&](int j) { const int x = cr + j; return (uint32_t)(x >= ck ? x - ck : x); };
+    // IT column quads at a time per thread, all loads of all KM pieces issued before the first use
+    auto merge_rows = [&](auto km_tag, auto it_tag) {
         constexpr int KM = decltype(km_tag)::value, IT = decltype(it_tag)::value;
-        for (int item0 = st;; item0 += NT * IT) {
-            float2 ml[IT][KM];
-            float4 pv[IT][KM];
-            int c4s[IT], lrs[IT], outs[IT];                            // outs: (sequence, node, head) row of the output, -1: none
+        float w[KM], mm, ll;
+        for (int e0 = 0;; e0 += IT) {
+            float2 ml[KM];
+            if (e0 == 0) {
 #pragma unroll
-            for (int e = 0; e < IT; ++e) {
-                const int item = item0 + e * NT, c4 = item / nrows, lr = row0 + (item - c4 * nrows), grow = sg.mblock * ROWS + lr;
-                c4s[e] = c4; lrs[e] = lr; outs[e] = -1;
-                if (item < total && grow < rows_total) outs[e] = (sg.b * N + grow / G) * p.Hq + sg.kvh * G + grow % G;
+                for (int j = 0; j < KM; ++j) {
+                    ml[j] = make_float2(-INFINITY, 0.f);
+                    if (j < ck && mine) ml[j] = j == 0 ? smem_ld2(prow_ml) : dsmem_ld2(dsmem_addr(prow_ml, peer(j)));
+                }
             }
-            if (item0 == st && !meet()) { cluster_arrive_release(); return; }
+            float4 pv[IT][KM];
 #pragma unroll
             for (int e = 0; e < IT; ++e)
 #pragma unroll
                 for (int j = 0; j < KM; ++j) {
-                    ml[e][j] = make_float2(-INFINITY, 0.f);
                     pv[e][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (j < ck && outs[e] >= 0) {
-                        ml[e][j] = dsmem_ld2(dsmem_addr(pst_a + lrs[e] * 8, (uint32_t)j));
-                        pv[e][j] = dsmem_ld4(dsmem_addr(pbuf_a + (c4s[e] * ROWS + lrs[e]) * 16, (uint32_t)j));
-                    }
+                    if (j < ck && mine && part + tpr * (e0 + e) < C4)
+                        pv[e][j] = j == 0 ? smem_ld4(prow + (uint32_t)(tpr * (e0 + e) * ROWS * 16))
+                                          : dsmem_ld4(dsmem_addr(prow + (uint32_t)(tpr * (e0 + e) * ROWS * 16), peer(j)));
                 }
-            // (the last round of the warp, not of the thread: at head size 64 `total` need not be a multiple of 32 - 688 items in
-            // rounds of 512 with three CTAs per unit of 128 rows - and a warp arrives with all its lanes at once; a lane past the
-            // end has outs < 0)
-            const bool last = (item0 & ~31) + NT * IT >= total;
+            const bool last = tpr * (e0 + IT) >= C4;
             if (last) cluster_arrive_release();
+            if (e0 == 0) {
+                mm = -INFINITY; ll = 0.f;
+#pragma unroll
+                for (int j = 0; j < KM; ++j) mm = fmaxf(mm, ml[j].x);
+                const float m_fin = (mm == -INFINITY) ? 0.f : mm;
+#pragma unroll
+                for (int j = 0; j < KM; ++j) { w[j] = exp2f(ml[j].x - m_fin); ll += ml[j].y * w[j]; }   // 0 for an empty or absent part
+                const float inv = inv_sum(ll);
+#pragma unroll
+                for (int j = 0; j < KM; ++j) w[j] *= inv;
+            }
 #pragma unroll
             for (int e = 0; e < IT; ++e) {
-                if (outs[e] < 0) continue;
-                float mm = -INFINITY;
-#pragma unroll
-                for (int j = 0; j < KM; ++j) mm = fmaxf(mm, ml[e][j].x);
-                const float m_fin = (mm == -INFINITY) ? 0.f : mm;
-                float ll = 0.f;
+                const int c4 = part + tpr * (e0 + e);
+                if (!mine || c4 >= C4) continue;
                 float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int j = 0; j < KM; ++j) {
-                    const float w = exp2f(ml[e][j].x - m_fin);          // 0 for an empty or absent part
-                    ll += ml[e][j].y * w;
-                    a4.x += w * pv[e][j].x; a4.y += w * pv[e][j].y; a4.z += w * pv[e][j].z; a4.w += w * pv[e][j].w;
+                    a4.x += w[j] * pv[e][j].x; a4.y += w[j] * pv[e][j].y; a4.z += w[j] * pv[e][j].z; a4.w += w[j] * pv[e][j].w;
                 }
-                const float inv2 = inv_sum(ll);
-                *reinterpret_cast<uint2*>(p.out + (size_t)outs[e] * HD + c4s[e] * 4) =
-                    make_uint2(pack_bf16(a4.x * inv2, a4.y * inv2), pack_bf16(a4.z * inv2, a4.w * inv2));
-                if (c4s[e] == 0 && p.lse) {
-                    const int bn = outs[e] / p.Hq, hd = outs[e] - bn * p.Hq;
-                    p.lse[((size_t)sg.b * p.Hq + hd) * N + (bn - sg.b * N)] = ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
-                }
+                *reinterpret_cast<uint2*>(orow + c4 * 4) = make_uint2(pack_bf16(a4.x, a4.y), pack_bf16(a4.z, a4.w));
             }
             if (last) break;
         }
+        if (p.lse && mine && part == 0)
+            p.lse[((size_t)sg.b * p.Hq + head) * N + node] = ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
     };
-    if (ck <= 2) merge_items(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
-    else if (ck <= 4) merge_items(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
-    else merge_items(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
+    if (ck <= 2) merge_rows(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
+    else if (ck <= 4) merge_rows(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
+    else merge_rows(std::integral_constant<int, 8>{}, std::integral_constant<int, 2>{});
 }
 
 // Merge of the partials of every unit that more than one CTA worked on, 4 warps per block.  Q = 0, coarse: grid (unit, group
