@@ -572,7 +572,21 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 qrow[k] = row < rows_total ? (sg.b * N + row / G) * p.Hq + sg.kvh * G + row % G : -1;
             }
         };
-        if (CL && !ROPE) q_rows(cl_seg);
+        // The ancestor bits of this thread's row, fetched beside the Q rows; where they are, -1 past the last row.
+        int mrow = -1;
+        uint64_t mk0 = 0, mk1 = 0;
+        auto mask_row = [&](const Seg& sg) {
+            const int row = sg.mblock * ROWS + lrow;
+            mrow = row < rows_total ? (sg.b * N + row / G) * W : -1;
+        };
+        auto mask_fetch = [&]() {
+            mk0 = mk1 = 0;
+            if (mrow >= 0) {
+                mk0 = p.mask[mrow];
+                if (W > 1) mk1 = p.mask[mrow + 1];
+            }
+        };
+        if (CL) { if (!ROPE) q_rows(cl_seg); mask_row(cl_seg); }
         pdl_wait();                                           // q, tree_mask and every output come after the preceding kernel
 
         // rejected sequences (kv_len < 0 or kv_len + N > S_max): zero output, -inf lse, status word
@@ -586,6 +600,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 if (!mbar_wait_warp(bar(B_XFREE), (seg - 1) & 1, abort_flag)) return false;
             }
             if constexpr (ROPE) {
+                mask_fetch();
                 // the Q tile and, beside it, this rank's share of the unit's tree rows into the cache (a rejected
                 // sequence, steps == 0, has no slots to write to: an empty share)
                 const int t_lo = (cr * N) / ck;
@@ -595,13 +610,14 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 mbar_arrive(bar(B_QFULL));
                 return true;
             }
-            if (!CL) q_rows(sg);
+            if (!CL) { q_rows(sg); mask_row(sg); }
             uint4 v[ITEMS];
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
                 v[k] = make_uint4(0, 0, 0, 0);
                 if (qrow[k] >= 0) v[k] = *(reinterpret_cast<const uint4*>(p.q + (size_t)qrow[k] * D) + qc);
             }
+            mask_fetch();
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
                 const int r = st / QC + QR * k;
@@ -661,15 +677,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 const bool row_ok = row < rows_total;
                 const int node = row_ok ? row / G : 0, head = sg.kvh * G + (row_ok ? row % G : 0);
                 const int S = sg.S, total = S + N;
-                uint64_t mk0 = 0, mk1 = 0;
-                if (row_ok) {
-                    const uint64_t* mrow = p.mask + ((size_t)sg.b * N + node) * W;
-                    mk0 = mrow[0];
-                    if (W > 1) mk1 = mrow[1];
-                    // bits at or beyond N are not tree nodes
-                    if (N < 64) mk0 &= (1ull << N) - 1;
-                    if (N < 128) mk1 &= N > 64 ? (1ull << (N - 64)) - 1 : 0ull;
-                }
+                // bits at or beyond N are not tree nodes
+                if (N < 64) mk0 &= (1ull << N) - 1;
+                if (N < 128) mk1 &= N > 64 ? (1ull << (N - 64)) - 1 : 0ull;
                 // m_ref and has_o are the same in both threads of a row; l_run covers this thread's columns only
                 float m_ref = -INFINITY, l_run = 0.f;
                 bool has_o = false;
