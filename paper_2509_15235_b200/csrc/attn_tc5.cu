@@ -523,6 +523,25 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             const bool leader = elect_one();
             const uint32_t v0 = desc_lo(base + SMEM_V, HALF_BYTES);
             bool ok = true;
+            if constexpr (ROPE) {
+                // Each rank of the cluster puts its share of the unit's N tree rows into the cache (its softmax threads, beside
+                // their Q tile).  The ranks whose steps contain the rows (the last, at most the last two) hold those tiles back
+                // until every rank has said that its share is in global memory: meeting of this CTA's softmax threads, fence,
+                // then one arrival per rank on that rank's barrier.  By this warp, which waits for the first P anyway: the fence
+                // (it covers what the meeting has made visible to this thread) and the signals held the softmax threads back
+                // ahead of their first step.
+                cluster_wait();                                           // the peers' barriers exist
+                cl_waited = true;
+                if (lane < ck) {
+                    ok = mbar_wait(bar(B_SEGSYNC), 0, abort_flag);
+                    if (ok) {
+                        __threadfence();                                          // the rows are in global memory ...
+                        asm volatile("fence.proxy.async.global;" ::: "memory");   // ... and ordered before bulk copies that read them
+                        mbar_arrive_peer(dsmem_addr(bar(B_ROWS), (uint32_t)lane));
+                    }
+                }
+                ok = __all_sync(0xffffffffu, ok);
+            }
             uint32_t sv = 0, pv = 0, u = 0;
             SegIter si = make_iter();
             Seg sg;
@@ -656,22 +675,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             while (ok && si.next(sg)) {
                 // every S product of the previous segment has been consumed by now, so Q may be replaced
                 if (!load_q(sg, seg)) { ok = false; break; }
-                if constexpr (ROPE) {
-                    // Each rank of the cluster has just put its share of the unit's N tree rows into the cache (beside its Q
-                    // tile).  The ranks whose steps contain the rows (the last, at most the last two) hold those tiles back
-                    // until every rank has said that its share is in global memory: fence, meeting of this CTA's softmax
-                    // threads, then one arrival per rank on that rank's barrier.
-                    __threadfence();                                          // the rows are in global memory ...
-                    asm volatile("fence.proxy.async.global;" ::: "memory");   // ... and ordered before bulk copies that read them
-                    mbar_arrive(bar(B_SEGSYNC));
-                    if (!cl_waited) { cluster_wait(); cl_waited = true; }     // the peers' barriers exist
-                    if (st < ck) {
-                        if (!mbar_wait(bar(B_SEGSYNC), sx & 1, abort_flag)) { ok = false; }
-                        else mbar_arrive_peer(dsmem_addr(bar(B_ROWS), (uint32_t)st));
-                    }
-                    ++sx;
-                    if (__any_sync(0xffffffffu, !ok)) { ok = false; break; }
-                }
+                // (fused rotary embedding: this rank's share of the tree rows is stored; warp 2 tells the other ranks)
+                if (ROPE) mbar_arrive(bar(B_SEGSYNC));
 
                 const int row = sg.mblock * ROWS + lrow;         // query row within the kv head's G*N rows
                 const bool row_ok = row < rows_total;
