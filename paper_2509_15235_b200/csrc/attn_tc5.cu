@@ -108,13 +108,13 @@ constexpr int SMEM_ALLOC = SMEM_TOTAL;                         // the base must 
 static_assert(SMEM_ALLOC <= 232448, "over the 227 KB a CTA may have");
 
 // ---- fused rotary embedding ---------------------------------------------------------------------------
-// Eight pairs (x = element j of the lower half, y = element j + D/2) rotated by their angles: fp64 with one rounding
-// to bf16 for the k rows that go to the cache, fp32 for q rows (consumed by the product, never stored).
-__device__ __forceinline__ void rope8_f64(uint4& lo, uint4& hi, const double2* cs) {
+// Pairs (x = element j of the lower half, y = element j + D/2) rotated by their angles: fp64 with one rounding to bf16 for
+// the k rows that go to the cache (two pairs), fp32 for q rows (eight pairs; consumed by the product, never stored).
+__device__ __forceinline__ void rope2_f64(uint32_t& lo, uint32_t& hi, const double2* cs) {
     __nv_bfloat16* a = reinterpret_cast<__nv_bfloat16*>(&lo);
     __nv_bfloat16* b = reinterpret_cast<__nv_bfloat16*>(&hi);
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
+    for (int t = 0; t < 2; ++t) {
         const double x = (double)__bfloat162float(a[t]), y = (double)__bfloat162float(b[t]);
         a[t] = __double2bfloat16(x * cs[t].x - y * cs[t].y);
         b[t] = __double2bfloat16(y * cs[t].x + x * cs[t].y);
@@ -132,12 +132,14 @@ __device__ __forceinline__ void rope8_f32(uint4& lo, uint4& hi, const float2* cs
 }
 // Prologue of a CTA with the fused rotary embedding (one function, so that both memory round trips overlap): the upper
 // half of the softmax threads fetches this rank's share of the tree rows, tree index in [t_lo, t_hi), of (sequence b,
-// kv head kvh): one item = (k row, pair of 16-byte chunks c and c + 8) with its eight fp64 (cos, sin) pairs, plus two
-// 16-byte chunks of v rows; then every thread fetches its part of the Q tile (chunk pair (c, c + 8) of rows st/8,
-// st/8 + 32, ... with eight fp32 pairs each); only then the k rows are rotated (fp64, one rounding: bit-compatible with the
-// rotation kernel) and written to slots S + t of the cache with the v rows, and the Q rows are rotated (fp32: they feed
+// kv head kvh), and every thread its part of the Q tile; then the k rows are rotated (fp64, one rounding: bit-compatible with
+// the rotation kernel) and written to slots S + t of the cache with the v rows, and the Q rows are rotated (fp32: they feed
 // the score product only) into the swizzled tile.  Shares of more than 16 rows take further passes after that.  Not
 // inlined: its registers stay out of the step loop's budget and its code out of the step loop's way.
+// What bounds it is the load path's lines per instruction and the registers of what is in flight, most of it angles (16 bytes
+// per k pair, 8 per q pair, against 4 of data).  So the eight threads of a k row take pairs 2c + 16u, 2c + 1 + 16u of it (neighbours
+// read neighbouring angles), and a thread's Q rows follow one another, so that they belong to one node or two and share its angles:
+// everything is in flight at once also with 128 rows per unit.
 template <bool PAIR, int ROWS>
 __device__ __noinline__ void rope_prologue(unsigned char* sm, const __nv_bfloat16* __restrict__ q, const RopeArgs p, int N_, int Hq,
                                            int Hkv_, int S_max_, int G, int rows_total, int b, int kvh, int mblock, int S,
@@ -146,98 +148,102 @@ __device__ __noinline__ void rope_prologue(unsigned char* sm, const __nv_bfloat1
     const int ps = st - HALF;                     // >= 0: this thread places rows
     const size_t cache_row0 = ((size_t)b * Hkv_ + kvh) * S_max_ + S;
     const int nk = (t_hi - t_lo) * 8, nv = (t_hi - t_lo) * 16;
-    auto k_src = [&](int i) { return reinterpret_cast<const uint4*>(p.k_new + (((size_t)b * N_ + t_lo + (i >> 3)) * Hkv_ + kvh) * D); };
-    auto k_tab = [&](int i) { return p.rope_k + ((size_t)b * N_ + t_lo + (i >> 3)) * (D / 2) + 8 * (i & 7); };
-    auto v_src = [&](int i) { return reinterpret_cast<const uint4*>(p.v_new + (((size_t)b * N_ + t_lo + (i >> 4)) * Hkv_ + kvh) * D) + (i & 15); };
-    auto k_store = [&](int i, uint4& lo, uint4& hi, const double2* cs) {
-        rope8_f64(lo, hi, cs);
-        uint4* dst = reinterpret_cast<uint4*>(p.k_cache + (cache_row0 + t_lo + (i >> 3)) * D);
-        dst[i & 7] = lo; dst[(i & 7) + 8] = hi;
+    uint32_t klo[4], khi[4];                      // pairs 2c + 16u, 2c + 1 + 16u of row t_lo + i / 8, c = i % 8
+    double2 cs[4][2];
+    uint4 vx[2];
+    auto k_load = [&](int i) {
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(p.k_new + (((size_t)b * N_ + t_lo + (i >> 3)) * Hkv_ + kvh) * D) + (i & 7);
+        const double2* tab = p.rope_k + ((size_t)b * N_ + t_lo + (i >> 3)) * (D / 2) + 2 * (i & 7);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            klo[u] = src[8 * u]; khi[u] = src[8 * u + D / 4];
+            cs[u][0] = tab[16 * u]; cs[u][1] = tab[16 * u + 1];
+        }
     };
+    auto k_store = [&](int i) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(p.k_cache + (cache_row0 + t_lo + (i >> 3)) * D) + (i & 7);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            rope2_f64(klo[u], khi[u], cs[u]);
+            dst[8 * u] = klo[u]; dst[8 * u + D / 4] = khi[u];
+        }
+    };
+    auto v_load = [&](int i) { return reinterpret_cast<const uint4*>(p.v_new + (((size_t)b * N_ + t_lo + (i >> 4)) * Hkv_ + kvh) * D)[i & 15]; };
     auto v_store = [&](int i, const uint4& x) { reinterpret_cast<uint4*>(p.v_cache + (cache_row0 + t_lo + (i >> 4)) * D)[i & 15] = x; };
-
-    // ---- tree rows, first pass (16 rows): loads
-    uint4 klo = make_uint4(0, 0, 0, 0), khi = klo, vx[2];
-    double2 cs[8];
-    const bool has_k = ps >= 0 && ps < nk;
-    if (has_k) {
-        const uint4* src = k_src(ps);
-        klo = src[ps & 7]; khi = src[(ps & 7) + 8];
-        const double2* tab = k_tab(ps);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) cs[j] = tab[j];
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-        if (ps >= 0 && ps + HALF * u < nv) vx[u] = *v_src(ps + HALF * u);
-    // (with 128 rows per unit the Q tile alone takes 96 registers per thread: there the rows are finished first; timed in
-    // one call on qwen7b: 18.7 against 20.1 us per layer of a step with both sets of loads in flight)
-    auto finish_rows = [&]() {
-        if (has_k) k_store(ps, klo, khi, cs);
+    auto rows_load = [&](int i, int j) {
+        if (i < nk) k_load(i);
 #pragma unroll
         for (int u = 0; u < 2; ++u)
-            if (ps >= 0 && ps + HALF * u < nv) v_store(ps + HALF * u, vx[u]);
+            if (j + HALF * u < nv) vx[u] = v_load(j + HALF * u);
     };
-    if (!PAIR) finish_rows();
+    auto rows_store = [&](int i, int j) {
+        if (i < nk) k_store(i);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (j + HALF * u < nv) v_store(j + HALF * u, vx[u]);
+    };
 
-    // ---- Q tile: loads
-    constexpr int PITEMS = ROWS * 8 / kSmx;
+    // K rows of the Q tile from row r0 on, one or two nodes' worth: chunk pair (c, c + 8) of each.
     const int c = st & 7;
-    uint4 lo[PITEMS], hi[PITEMS];
-    float4 tab[PITEMS][4];
+    auto q_rows = [&](auto k_tag, int r0, auto between) {
+        constexpr int K = decltype(k_tag)::value;
+        uint4 lo[K], hi[K];
+        float4 tab[2][4];
+        const int row0 = mblock * ROWS + r0, n0 = row0 / G, n1 = min(row0 + K - 1, rows_total - 1) / G;
 #pragma unroll
-    for (int k = 0; k < PITEMS; ++k) {
-        const int row = mblock * ROWS + (st >> 3) + 32 * k;
-        lo[k] = make_uint4(0, 0, 0, 0); hi[k] = lo[k];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) tab[k][j] = make_float4(1.f, 0.f, 1.f, 0.f);
-        if (row < rows_total) {
-            const int node = row / G, head = kvh * G + row % G;
-            const uint4* src = reinterpret_cast<const uint4*>(q + (((size_t)b * N_ + node) * Hq + head) * D);
-            lo[k] = src[c]; hi[k] = src[c + 8];
-            const float4* t4 = reinterpret_cast<const float4*>(p.rope_q + ((size_t)b * N_ + node) * (D / 2) + 8 * c);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) tab[k][j] = t4[j];
-        }
-    }
-
-    // ---- tree rows, first pass: rotate and store
-    if (PAIR) finish_rows();
-
-    // ---- Q tile: rotate into shared memory
-#pragma unroll
-    for (int k = 0; k < PITEMS; ++k) {
-        const int r = (st >> 3) + 32 * k;
-        rope8_f32(lo[k], hi[k], reinterpret_cast<const float2*>(tab[k]));
-        unsigned char* dst = sm + SMEM_Q + r * 128 + ((c ^ (r & 7)) << 4);
-        *reinterpret_cast<uint4*>(dst) = lo[k];
-        *reinterpret_cast<uint4*>(dst + HALF_BYTES) = hi[k];
-        if (PAIR) {
-            *reinterpret_cast<uint4*>(dst + 64 * 128) = lo[k];
-            *reinterpret_cast<uint4*>(dst + HALF_BYTES + 64 * 128) = hi[k];
-        }
-    }
-
-    // ---- tree rows beyond the first 16 of the share
-    if (ps >= 0) {
-        for (int i = ps + HALF, j = ps + 2 * HALF; i < nk || j < nv; i += HALF, j += 2 * HALF) {
-            const bool more_k = i < nk;
-            if (more_k) {
-                const uint4* src = k_src(i);
-                klo = src[i & 7]; khi = src[(i & 7) + 8];
-                const double2* tb = k_tab(i);
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) cs[jj] = tb[jj];
+        for (int k = 0; k < K; ++k) {
+            const int row = row0 + k;
+            lo[k] = make_uint4(0, 0, 0, 0); hi[k] = lo[k];
+            if (row < rows_total) {
+                const int node = row / G;
+                const uint4* src = reinterpret_cast<const uint4*>(q + (((size_t)b * N_ + node) * Hq + kvh * G + (row - node * G)) * D);
+                lo[k] = src[c]; hi[k] = src[c + 8];
             }
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (j + HALF * u < nv) vx[u] = *v_src(j + HALF * u);
-            if (more_k) k_store(i, klo, khi, cs);
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (j + HALF * u < nv) v_store(j + HALF * u, vx[u]);
         }
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const float4* t4 = reinterpret_cast<const float4*>(p.rope_q + ((size_t)b * N_ + (x ? n1 : n0)) * (D / 2) + 8 * c);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) tab[x][j] = make_float4(1.f, 0.f, 1.f, 0.f);
+            if (row0 < rows_total && (x == 0 || n1 != n0)) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) tab[x][j] = t4[j];
+            }
+        }
+        between();
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const bool second = row0 + k >= (n0 + 1) * G;
+            float4 t[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                t[j] = second ? tab[1][j] : tab[0][j];
+            rope8_f32(lo[k], hi[k], reinterpret_cast<const float2*>(t));
+            const int r = r0 + k;
+            unsigned char* dst = sm + SMEM_Q + r * 128 + ((c ^ (r & 7)) << 4);
+            *reinterpret_cast<uint4*>(dst) = lo[k];
+            *reinterpret_cast<uint4*>(dst + HALF_BYTES) = hi[k];
+            if (PAIR) {
+                *reinterpret_cast<uint4*>(dst + 64 * 128) = lo[k];
+                *reinterpret_cast<uint4*>(dst + HALF_BYTES + 64 * 128) = hi[k];
+            }
+        }
+    };
+    constexpr int K = ROWS * 8 / kSmx;            // Q rows of a thread: (st / 8) * K ...
+    if (ps >= 0) rows_load(ps, ps);
+    auto finish_rows = [&]() { if (ps >= 0) rows_store(ps, ps); };
+    if (K <= 2 || G >= K - 1) {                   // K rows in a row touch at most two nodes
+        q_rows(std::integral_constant<int, K>{}, (st >> 3) * K, finish_rows);
+    } else {
+        q_rows(std::integral_constant<int, 2>{}, (st >> 3) * K, finish_rows);
+        q_rows(std::integral_constant<int, 2>{}, (st >> 3) * K + 2, []() {});
     }
+    // tree rows beyond the first 16 of the share
+    if (ps >= 0)
+        for (int i = ps + HALF, j = ps + 2 * HALF; i < nk || j < nv; i += HALF, j += 2 * HALF) {
+            rows_load(i, j);
+            rows_store(i, j);
+        }
 }
 
 // The softmax's exponentials are what the special-function pipe (16 lanes per SM) spends a step on; one in eight of them is

@@ -205,6 +205,17 @@ def test_fused_rope_attention_matches_rope_then_attention_of_the_oracle(B, N, Hq
     ctx.close()
 
 
+@pytest.mark.parametrize("B,N,Hq,Hkv,kv_len,S_max", [
+    (1, 128, 2, 2, [300], 512),             # one head per kv head: four nodes in a thread's rows; shares of 64 tree rows and more
+    (1, 67, 4, 2, [300], 512),              # two: up to three nodes; the last row block holds 6 rows
+    (1, 43, 6, 2, [300], 512),              # three: two nodes; 129 rows, the last block holds one
+    (2, 40, 14, 2, [290, 511], 640),        # seven: row blocks start inside a node
+])
+def test_fused_rope_attention_with_128_rows_per_unit(B, N, Hq, Hkv, kv_len, S_max):
+    """Cluster form with units of 128 rows, where a thread of the prologue rotates four consecutive query rows."""
+    test_fused_rope_attention_matches_rope_then_attention_of_the_oracle(B, N, Hq, Hkv, kv_len, S_max, 2)
+
+
 @pytest.mark.parametrize("split_form", [0, 1])
 def test_fused_rope_attention_leaves_a_sequence_that_does_not_fit_alone(split_form):
     """kv_len + N > S_max for one sequence: its cache rows stay as they were (nothing is written past its slots), its
