@@ -956,8 +956,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         __syncwarp();
         if (!cl_waited) { cluster_wait(); cl_waited = true; }     // (fused rotary embedding: the start-up phase, warps 0-3)
         if (warp >= 4) {
-            cluster_merge<ROWS, D>(p, cl_seg, ck, cr, base + SMEM_K, base + SMEM_K + (D / 4) * ROWS * 16, tid - 128,
-                                   [&]() { cluster_sync_all(); return *abort_flag == 0; });
+            cluster_merge<ROWS, D>(p, cl_seg, ck, cr, base + SMEM_K, base + SMEM_K + (D / 4) * ROWS * 16, tid - 128, abort_flag);
         } else {
             cluster_sync_all();
             if (warp == 1) {

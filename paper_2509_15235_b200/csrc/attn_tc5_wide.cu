@@ -476,8 +476,7 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
         }
         if (CL) {
             __syncwarp();
-            cluster_merge<kRows, HD>(p, cl_seg, ck, cr, base + R::OFF_K, base + R::OFF_K + (HD / 4) * kRows * 16, tid - 128,
-                                     [&]() { cluster_sync_all(); return *abort_flag == 0; });   // every CTA of the unit has parked its partial
+            cluster_merge<kRows, HD>(p, cl_seg, ck, cr, base + R::OFF_K, base + R::OFF_K + (HD / 4) * kRows * 16, tid - 128, abort_flag);
         }
     }
     tc_fence_before();

@@ -667,15 +667,16 @@ __device__ __forceinline__ void zero_rejected(const Tc5Params& p, const Sched& s
 
 // Cluster form: rank cr of ck merges its rows of the unit's partials, parked by every rank at pbuf_a ([HD/4 col4][ROWS]
 // float4) and pst_a ([ROWS] (m, l)) of its own shared memory, and writes them out.  By the NT softmax threads (st).
-// Contains the meeting of the cluster (meet(), false: nothing is merged) and this warp's arrival at the closing one: the
-// indices are formed before the meeting, and a warp arrives as soon as its last loads from the peers are back, so that
-// neither the divisions nor the output's arithmetic and stores lie between the two barriers.
+// Contains the meeting of the cluster and this warp's arrival at the closing one: the indices (a chain of divisions) are formed
+// between the arrival at the meeting and the wait, and a warp arrives at the closing barrier as soon as its last loads from
+// the peers are back, so that neither the divisions nor the output's arithmetic and stores lie on the way.
 // What bounds it is the bytes that cross between the SMs: 16 per cycle and SM, whatever instruction moves them (32 KB in
 // 2170 cycles by loads, bulk copies and asynchronous stores alike; by way of L2 3400).  So a rank's own partial does not
 // cross, only rows that exist are dealt out to the ranks, a thread keeps to one row and fetches its (m, l) once, and each
 // rank goes on from its own partial to the next rank's, so that the ranks do not all read from the same one.
-template <int ROWS, int HD, int NT = 256, class Meet>
-__device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st, Meet meet) {
+template <int ROWS, int HD, int NT = 256>
+__device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg, int ck, int cr, uint32_t pbuf_a, uint32_t pst_a, int st, volatile int* abort_flag) {
+    cluster_arrive_release();
     constexpr int C4 = HD / 4;                                          // column quads of a row
     const int N = p.N, G = p.Hq / p.Hkv;
     const int rows = min(ROWS, G * N - sg.mblock * ROWS);               // of this unit
@@ -685,9 +686,24 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
     const bool mine = any && part < tpr;
     const int grow = sg.mblock * ROWS + row0 + r, node = grow / G, head = sg.kvh * G + (grow - node * G);
     __nv_bfloat16* orow = p.out + (((size_t)sg.b * N + node) * p.Hq + head) * HD;
-    if (!meet()) { cluster_arrive_release(); return; }
-    const uint32_t prow = pbuf_a + (uint32_t)((part * ROWS + row0 + r) * 16), prow_ml = pst_a + (uint32_t)((row0 + r) * 8);
     auto peer = [&](int j) { const int x = cr + j; return (uint32_t)(x >= ck ? x - ck : x); };
+    // bit j of parts: rank peer(j) had steps.  (In short calls some have none: rank x's share [ceil(x s / ck), ceil((x + 1) s / ck)) of
+    // s < ck steps is empty unless x s % ck is 0 or above ck - s.)
+    unsigned parts = (1u << ck) - 1;
+    if (sg.steps < ck) {
+        unsigned has = 0;
+        for (int x = 0, m = 0; x < ck; ++x) {
+            if (m == 0 || m + sg.steps > ck) has |= 1u << x;
+            m += sg.steps;
+            if (m >= ck) m -= ck;
+        }
+        if (sg.steps == 0) has = 0;
+        parts &= (has >> cr) | (has << (ck - cr));
+    }
+    if (!mine) parts = 0;
+    cluster_wait();
+    if (*abort_flag) { cluster_arrive_release(); return; }
+    const uint32_t prow = pbuf_a + (uint32_t)((part * ROWS + row0 + r) * 16), prow_ml = pst_a + (uint32_t)((row0 + r) * 8);
     // IT column quads at a time per thread, all loads of all KM pieces issued before the first use
     auto merge_rows = [&](auto km_tag, auto it_tag) {
         constexpr int KM = decltype(km_tag)::value, IT = decltype(it_tag)::value;
@@ -698,7 +714,7 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
 #pragma unroll
                 for (int j = 0; j < KM; ++j) {
                     ml[j] = make_float2(-INFINITY, 0.f);
-                    if (j < ck && mine) ml[j] = j == 0 ? smem_ld2(prow_ml) : dsmem_ld2(dsmem_addr(prow_ml, peer(j)));
+                    if ((parts >> j) & 1) ml[j] = j == 0 ? smem_ld2(prow_ml) : dsmem_ld2(dsmem_addr(prow_ml, peer(j)));
                 }
             }
             float4 pv[IT][KM];
@@ -707,7 +723,7 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
 #pragma unroll
                 for (int j = 0; j < KM; ++j) {
                     pv[e][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (j < ck && mine && part + tpr * (e0 + e) < C4)
+                    if (((parts >> j) & 1) && part + tpr * (e0 + e) < C4)
                         pv[e][j] = j == 0 ? smem_ld4(prow + (uint32_t)(tpr * (e0 + e) * ROWS * 16))
                                           : dsmem_ld4(dsmem_addr(prow + (uint32_t)(tpr * (e0 + e) * ROWS * 16), peer(j)));
                 }
@@ -742,6 +758,7 @@ __device__ __forceinline__ void cluster_merge(const Tc5Params& p, const Seg& sg,
     };
     if (ck <= 2) merge_rows(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
     else if (ck <= 4) merge_rows(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
+    else if (tpr >= C4) merge_rows(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{});
     else merge_rows(std::integral_constant<int, 8>{}, std::integral_constant<int, 2>{});
 }
 
