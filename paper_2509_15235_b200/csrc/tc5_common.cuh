@@ -411,7 +411,7 @@ struct SegIter {
 
 // One (row, 16 output columns) of a unit: the partials of CTAs c0..c1 (slot 2c if the unit starts CTA c's range,
 // else 2c + 1) folded into the final output.  Shared by the merge kernel and by the attention kernel's own merge.
-template <int ROWS, int HD>
+template <int ROWS, int HD, bool WAIT = false>      // WAIT: for the kernel that writes the partials, ahead of the first load
 __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o, const float2* __restrict__ part_ml,
                                                __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int geff,
                                                int ub, int c0, int c1, int b, int node, int head, int Hq, int N,
@@ -423,9 +423,14 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
     float4 acc[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (WAIT && c1 < c0) pdl_wait();                  // (a lane without a row)
     for (int cb = c0; cb <= c1; cb += 4) {
         float2 ml[4];
         float4 v[4][4];
+        int slot[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) slot[j] = slot_of(min(cb + j, c1));
+        if (WAIT && cb == c0) pdl_wait();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int c = cb + j;
@@ -433,9 +438,8 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
 #pragma unroll
             for (int k = 0; k < 4; ++k) v[j][k] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (c <= c1) {
-                const int slot = slot_of(c);
-                ml[j] = __ldcg(&part_ml[(size_t)slot * ROWS + lrow]);
-                const float4* src = part_o + ((size_t)slot * (HD / 4) + cw * 4) * ROWS + lrow;
+                ml[j] = __ldcg(&part_ml[(size_t)slot[j] * ROWS + lrow]);
+                const float4* src = part_o + ((size_t)slot[j] * (HD / 4) + cw * 4) * ROWS + lrow;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) v[j][k] = __ldcg(src + (size_t)k * ROWS);
             }
@@ -459,6 +463,7 @@ __device__ __forceinline__ void merge_row_cols(const float4* __restrict__ part_o
         }
         m_all = m_new;
     }
+    if (WAIT && c1 < c0) return;
     const float inv = inv_sum(l_all);
     __nv_bfloat16* orow = out + (((size_t)b * N + node) * Hq + head) * HD + cw * 16;
 #pragma unroll
@@ -487,15 +492,18 @@ __device__ __forceinline__ void merge_row_c4(const float4* __restrict__ part_o, 
     for (int cb = c0; cb <= c1; cb += Q * U) {
         float2 ml[U];
         float4 v[U];
+        int slot[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) slot[j] = slot_of(min(cb + part + j * Q, c1));
+        if (cb == c0) pdl_wait();                         // the partials are complete
 #pragma unroll
         for (int j = 0; j < U; ++j) {
             const int c = cb + part + j * Q;
             ml[j] = make_float2(-INFINITY, 0.f);
             v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (c <= c1 && row_ok) {
-                const int slot = slot_of(c);
-                ml[j] = __ldcg(&part_ml[(size_t)slot * ROWS + lrow]);
-                v[j] = __ldcg(part_o + ((size_t)slot * (HD / 4) + c4) * ROWS + lrow);
+                ml[j] = __ldcg(&part_ml[(size_t)slot[j] * ROWS + lrow]);
+                v[j] = __ldcg(part_o + ((size_t)slot[j] * (HD / 4) + c4) * ROWS + lrow);
             }
         }
         float m_new = m_all;
@@ -788,12 +796,13 @@ attn_tc5_merge_kernel(const Tc5Params p) {
         T += st * spb;
         live += st > 0 ? spb : 0;
     }
-    pdl_wait();                                        // the partials are complete
-    if (steps == 0) return;
+    // Everything that does not hang on the partials comes ahead of the dependency, down to the first group's addresses (each
+    // behind a division); every block waits, also one with nothing to do: what follows on the stream waits for this kernel only.
+    if (steps == 0) { pdl_wait(); return; }
     const int geff = sched_ctas(T, live, LOCK ? p.grid_attn / p.n_mblocks : p.grid_attn, p.min_steps, sched_round_steps(p));
     const int ub = base_b + (LOCK ? uib / p.n_mblocks : uib) * steps, ue = ub + steps;
     const int c0 = cta_of(ub, T, geff), c1 = cta_of(ue - 1, T, geff);
-    if (c0 == c1) return;                              // one CTA had the whole unit and wrote the output itself
+    if (c0 == c1) { pdl_wait(); return; }              // one CTA had the whole unit and wrote the output itself
     const int G = p.Hq / p.Hkv, N = p.N;
     const int kvh = uib / p.n_mblocks, mblock = uib - kvh * p.n_mblocks;
     constexpr int CB = Q > 0 ? HD / 16 : HD / 64, RW = Q > 0 ? 32 / Q : 32;     // blocks and rows per group of rows
@@ -806,8 +815,8 @@ attn_tc5_merge_kernel(const Tc5Params p) {
     const int smul = LOCK ? p.n_mblocks : 1, sadd = LOCK ? mblock : 0;
     if constexpr (Q > 0)
         merge_row_c4<ROWS, HD, Q>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, lane / RW, row_ok, smul, sadd);
-    else if (row_ok)
-        merge_row_cols<ROWS, HD>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, c1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
+    else
+        merge_row_cols<ROWS, HD, true>(p.part_o, p.part_ml, p.out, p.lse, T, geff, ub, c0, row_ok ? c1 : c0 - 1, b, node, head, p.Hq, N, lrow, cw, smul, sadd);
 }
 
 // Host side: the merge of `units` units written by `ctas` CTAs; as many lanes share a row as keep the grid within what
