@@ -372,20 +372,40 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             const bool leader = (CL && !PAGED) || elect_one();
             const uint64_t pol = l2_evict_first_policy();
             bool waited = !p.early;
-            int it = 0, nk = 0, nv = 0;          // steps started; K / V stages issued
+            int it = 0, nk = 0, nv = 0;          // steps started; K stages used (one per step, one per later segment's Q), V stages issued
             bool ok = true;
             SegIter si = make_iter();
             Seg sg;
+            // Even split: the Q rows of a CTA's later segments come through the K ring, one stage ahead of the segment's first K tile,
+            // so that they are there when the segment before ends (a round trip to memory behind a saturated HBM is 3.5 us; a
+            // CTA's every further segment cost 7 us with it, for which its rings stood still: llava13b_b4's CTAs ended after 41, 49
+            // or 56 us by the number of their segments).  The softmax threads copy them on into the Q tile.
+            auto q_stage = [&]() -> bool {
+                const int sk = nk % NSK, r_n = min(ROWS, rows_total - sg.mblock * ROWS);
+                if (!waited) { pdl_wait(); waited = true; }
+                if (!prod_wait(bar(B_KEMPTY + sk), ((nk / NSK) & 1) ^ 1)) return false;
+                if (leader) mbar_expect_tx(bar(B_KFULL + sk), (uint32_t)r_n * D * 2);
+                __syncwarp();
+                for (int r = lane; r < r_n; r += 32) {
+                    const int row = sg.mblock * ROWS + r;
+                    bulk_load(base + SMEM_K + sk * STAGE_BYTES + r * (D * 2), p.q + (((size_t)sg.b * N + row / G) * p.Hq + sg.kvh * G + row % G) * D,
+                              D * 2, bar(B_KFULL + sk));
+                }
+                ++nk;
+                return true;
+            };
             if constexpr (PAGED) {
-                while (ok && si.next(sg)) {
-                    const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING, abort_flag, pol, it, waited, lane, split_v ? 1 : 0);
+                for (int seg = 0; ok && si.next(sg); ++seg) {
+                    if (!CL && seg > 0 && !q_stage()) { ok = false; break; }
+                    const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING, abort_flag, pol, it, waited, lane, split_v ? 1 : 0, nk - it);
                     const int done = (int)(r & 0x0fffffffu);
                     it += done; nv += split_v ? 0 : done; nk += done + (int)((r >> 28) & 1u);
                     ok = !((r >> 29) & 1u);
                     waited = (r >> 30) & 1u;
                 }
             }
-            while (!PAGED && ok && si.next(sg)) {
+            for (int seg = 0; !PAGED && ok && si.next(sg); ++seg) {
+                if (!CL && seg > 0 && !q_stage()) { ok = false; break; }
                 const int bh = sg.b * p.Hkv + sg.kvh;
                 const int n = CL ? sg.n : __shfl_sync(0xffffffffu, sg.n, 0);
                 for (int t = 0; t < n; ++t, ++it) {
@@ -396,8 +416,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                         if (!mbar_wait_cluster(bar(B_ROWS), 0, abort_flag)) { ok = false; break; }
                         asm volatile("fence.proxy.async.global;" ::: "memory");
                     }
-                    const int sk = it % NSK;
-                    if (!prod_wait(bar(B_KEMPTY + sk), ((it / NSK) & 1) ^ 1)) { ok = false; break; }
+                    const int sk = nk % NSK;
+                    if (!prod_wait(bar(B_KEMPTY + sk), ((nk / NSK) & 1) ^ 1)) { ok = false; break; }
                     if (leader) {
                         mbar_expect_tx(bar(B_KFULL + sk), STAGE_BYTES);
                         tma_load_3d(base + SMEM_K + sk * STAGE_BYTES, &k_map, bar(B_KFULL + sk), 0, tok, bh, pol);
@@ -499,6 +519,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             while (ok && si.next(sg)) {
                 const int n = __shfl_sync(0xffffffffu, sg.n, 0);
                 if (!mbar_wait_warp(bar(B_QFULL), seg & 1, abort_flag)) { ok = false; break; }
+                if (!CL && seg > 0) {                                  // the stage that the Q rows came in has been read
+                    if (leader) mbar_arrive(bar(B_KEMPTY) + 8u * sk);
+                    if (++sk == NSK) { sk = 0; pk ^= 1; }
+                }
                 for (int t = 0; t < n; ++t, ++it) {
                     const uint32_t bs = it & 1;
                     if (!mbar_wait_warp(bar(B_KFULL) + 8u * sk, pk, abort_flag)) { ok = false; break; }
@@ -619,7 +643,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
 
         // Q of a segment -> shared memory, rows in the swizzled K-major layout of a K stage (PAIR: rows 64-127
         // repeat rows 0-63).  Thread t moves 16-byte chunk t%16 of rows t/16, t/16 + 16, ... (head size 64: t%8 of t/8, t/8 + 32, ...)
-        auto load_q = [&](const Seg& sg, int seg) -> bool {
+        auto load_q = [&](const Seg& sg, int seg, int it) -> bool {
             if (PAIR && seg > 0) {
                 // the tile doubles as the exchange area of the previous segment's epilogue
                 if (!mbar_wait_warp(bar(B_XFREE), (seg - 1) & 1, abort_flag)) return false;
@@ -635,14 +659,25 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 mbar_arrive(bar(B_QFULL));
                 return true;
             }
-            if (!CL) { q_rows(sg); mask_row(sg); }
             uint4 v[ITEMS];
+            if (CL || seg == 0) {
+                if (!CL) { q_rows(sg); mask_row(sg); }
 #pragma unroll
-            for (int k = 0; k < ITEMS; ++k) {
-                v[k] = make_uint4(0, 0, 0, 0);
-                if (qrow[k] >= 0) v[k] = *(reinterpret_cast<const uint4*>(p.q + (size_t)qrow[k] * D) + qc);
+                for (int k = 0; k < ITEMS; ++k) {
+                    v[k] = make_uint4(0, 0, 0, 0);
+                    if (qrow[k] >= 0) v[k] = *(reinterpret_cast<const uint4*>(p.q + (size_t)qrow[k] * D) + qc);
+                }
+                mask_fetch();
+            } else {
+                const int ik = it + seg - 1, sk = ik % NSK;          // the producer's stage for it
+                if (!mbar_wait_warp(bar(B_KFULL + sk), (ik / NSK) & 1, abort_flag)) return false;
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) {
+                    const int r = st / QC + QR * k;
+                    v[k] = make_uint4(0, 0, 0, 0);
+                    if (sg.mblock * ROWS + r < rows_total) v[k] = *reinterpret_cast<const uint4*>(sm + SMEM_K + sk * STAGE_BYTES + r * (D * 2) + qc * 16);
+                }
             }
-            mask_fetch();
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
                 const int r = st / QC + QR * k;
@@ -680,7 +715,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             float4* xch = reinterpret_cast<float4*>(sm + SMEM_Q);
             while (ok && si.next(sg)) {
                 // every S product of the previous segment has been consumed by now, so Q may be replaced
-                if (!load_q(sg, seg)) { ok = false; break; }
+                if (!load_q(sg, seg, it)) { ok = false; break; }
                 // (fused rotary embedding: this rank's share of the tree rows is stored; warp 2 tells the other ranks)
                 if (ROPE) mbar_arrive(bar(B_SEGSYNC));
 
@@ -820,6 +855,12 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     mbar_arrive(bar(B_PFULL + bs));
                 }
                 if (!ok) break;
+                // (the next segment's mask row is on its way from here on)
+                if constexpr (!CL) {
+                    SegIter ahead = si;
+                    Seg nx;
+                    if (ahead.next(nx)) { mask_row(nx); mask_fetch(); }
+                }
 
                 // ---- segment epilogue: wait for the last product, add up the row statistics, (PAIR) merge the two
                 // halves, write out.  FULL: a thread owns columns [D/2 ch, D/2 ch + D/2) of its lane's accumulator row.  PAIR:

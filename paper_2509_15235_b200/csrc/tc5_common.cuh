@@ -96,6 +96,11 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(pol) : "memory");
 }
+// Untiled copy of `bytes` (a multiple of 16, both addresses on 16 bytes) from global to shared memory.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -590,7 +595,8 @@ template <class R>   // ring geometry: stages, bytes, offsets in shared memory, 
 __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensorMap* k_map, const CUtensorMap* v_map,
                                                int b, int kvh, int st0, int n, int S, uint32_t base, uint32_t bars,
                                                uint32_t ring, volatile int* abort_flag, uint64_t pol, int it,
-                                               bool waited, int lane, int which /* 0: K and V, 1: K only, 2: V only */) {
+                                               bool waited, int lane, int which /* 0: K and V, 1: K only, 2: V only */,
+                                               int koff = 0 /* stages of the K ring used beyond one per step */) {
     auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
     const int nsub = STEP / p.page_rows;
     const uint32_t sub_bytes = (uint32_t)p.page_rows * 128u;
@@ -624,11 +630,11 @@ __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensor
             }
         }
         const uint32_t tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, load)) * sub_bytes * 2u;
-        const int sk = it % R::NSK, sv = it % R::NSV;
+        const int ik = it + koff, sk = ik % R::NSK, sv = it % R::NSV;
         bool w = true;
         if (which != 2) {
             if (lane == 0) {
-                w = mbar_wait(bar(R::KEMPTY + sk), ((it / R::NSK) & 1) ^ 1, abort_flag);
+                w = mbar_wait(bar(R::KEMPTY + sk), ((ik / R::NSK) & 1) ^ 1, abort_flag);
                 if (w) mbar_expect_tx(bar(R::KFULL + sk), tx);
             }
             w = __shfl_sync(0xffffffffu, w, 0);                          // the byte count is posted before any lane copies
