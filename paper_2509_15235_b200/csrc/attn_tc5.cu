@@ -353,8 +353,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         cl_seg.n = ((cr + 1) * cl_seg.steps + ck - 1) / ck - cl_seg.st0;
         cl_seg.slot = -1;
     }
+    using Iter = SegIter<PAIR && !CL>;
     auto make_iter = [&]() {
-        SegIter it; it.s = &sched; it.B = p.B; it.n_mblocks = p.n_mblocks; it.g = lo; it.lo = lo; it.hi = hi; it.cta = cta;
+        Iter it; it.s = &sched; it.B = p.B; it.n_mblocks = p.n_mblocks; it.seg_cost_ = p.seg_cost; it.g = lo; it.lo = lo; it.hi = hi; it.cta = cta;
         it.cl = CL; it.cl_done = false; it.cl_seg = cl_seg;
         return it;
     };
@@ -374,7 +375,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             bool waited = !p.early;
             int it = 0, nk = 0, nv = 0;          // steps started; K stages used (one per step, one per later segment's Q), V stages issued
             bool ok = true;
-            SegIter si = make_iter();
+            Iter si = make_iter();
             Seg sg;
             // Even split: the Q rows of a CTA's later segments come through the K ring, one stage ahead of the segment's first K tile,
             // so that they are there when the segment before ends (a round trip to memory behind a saturated HBM is 3.5 us; a
@@ -456,7 +457,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 const uint64_t pol = l2_evict_first_policy();
                 bool waited = !p.early, ok = true;
                 int it = 0;
-                SegIter si = make_iter();
+                Iter si = make_iter();
                 Seg sg;
                 while (ok && si.next(sg)) {
                     const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING + 128, abort_flag, pol, it, waited, lane, 2);
@@ -475,7 +476,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             bool waited = !p.early;
             int it = 0;
             bool ok = true;
-            SegIter si = make_iter();
+            Iter si = make_iter();
             Seg sg;
             while (ok && si.next(sg)) {
                 const int bh = sg.b * p.Hkv + sg.kvh;
@@ -514,7 +515,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             const uint32_t k0 = desc_lo(base + SMEM_K, 16), qb = desc_lo(base + SMEM_Q, 16);
             bool ok = true;
             uint32_t sk = 0, pk = 0, it = 0, seg = 0;              // ring position with its phase, steps, segments
-            SegIter si = make_iter();
+            Iter si = make_iter();
             Seg sg;
             while (ok && si.next(sg)) {
                 const int n = __shfl_sync(0xffffffffu, sg.n, 0);
@@ -573,7 +574,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 ok = __all_sync(0xffffffffu, ok);
             }
             uint32_t sv = 0, pv = 0, u = 0;
-            SegIter si = make_iter();
+            Iter si = make_iter();
             Seg sg;
             while (ok && si.next(sg)) {
                 const int n = __shfl_sync(0xffffffffu, sg.n, 0);
@@ -708,7 +709,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             tmem_wait_st();
         }
         if (active) {
-            SegIter si = make_iter();
+            Iter si = make_iter();
             Seg sg;
             int it = 0, seg = 0;
             bool ok = true;
@@ -857,7 +858,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 if (!ok) break;
                 // (the next segment's mask row is on its way from here on)
                 if constexpr (!CL) {
-                    SegIter ahead = si;
+                    Iter ahead = si;
                     Seg nx;
                     if (ahead.next(nx)) { mask_row(nx); mask_fetch(); }
                 }
@@ -965,8 +966,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     if (!mbar_wait_warp(bar(B_SEGSYNC), sx & 1, abort_flag)) { ok = false; break; }
                     ++sx;
                     const int uib = sg.kvh * p.n_mblocks + sg.mblock;
-                    const int ub = sched.base[sg.b] + uib * sg.steps;
-                    const int c0 = cta_of(ub, T, geff), c1 = cta_of(ub + sg.steps - 1, T, geff);
+                    const int ub = sched.base[sg.b] + uib * (sg.steps + p.seg_cost), u0 = ub + p.seg_cost;
+                    const int c0 = cta_of(u0, T, geff), c1 = cta_of(u0 + sg.steps - 1, T, geff);
                     if (st == 0) {
                         int* cnt = pa.unit_counters + (sg.b * p.Hkv * p.n_mblocks + uib);
                         const bool last = atomicAdd(cnt, 1) == c1 - c0;
@@ -1069,7 +1070,7 @@ stream_probe_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_cons
     const int cta = blockIdx.x;
     if (cta < geff && lane == 0) {
         const int lo = cta_lo(cta, T, geff), hi = cta_lo(cta + 1, T, geff);
-        SegIter si; si.s = &sched; si.B = p.B; si.n_mblocks = p.n_mblocks; si.g = lo; si.lo = lo; si.hi = hi; si.cta = cta;
+        SegIter<false> si; si.s = &sched; si.B = p.B; si.n_mblocks = p.n_mblocks; si.seg_cost_ = 0; si.g = lo; si.lo = lo; si.hi = hi; si.cta = cta;
         si.cl = false; si.cl_done = false;
         Seg sg;
         int n = 0;                                             // stages handled so far
@@ -1180,6 +1181,7 @@ static int tc5_max_cluster(const AttnArgs& a, bool pair, int n_mblocks) {
 // (As an even split the smaller blocks gain nothing.)  The best estimate decides, a form that options ask for first.
 // Clusters with 64-row units / with 128: 16 query and 2 kv heads, 1 x 16 nodes on 2048 8.9 / 10.4, 4 x 16 on 8192 17.6 / 18.2, 1 x 60 on
 // 8192 17.0 / 17.7, 8 x 60 on 2048 23.4 / 19.9, 4 x 60 on 8192 33.8 / 28.5; 28 / 4 heads, 1 x 60 on 3344 13.4 / 14.8, 4 x 60 30.7 / 25.1.
+constexpr int kSegCost = 4;                     // see SegIter; in steps
 struct Tc5Layout { bool pair; int rows, n_mblocks, ck; double est_us; };
 static Tc5Layout tc5_layout(const AttnArgs& a) {
     const int rows_total = (a.Hq / a.Hkv) * a.N;
@@ -1205,7 +1207,7 @@ bool attn_tc5_supports(const AttnArgs& a) {
     const int rows_total = (a.Hq / a.Hkv) * a.N;
     const int rows = rows_total <= 64 ? 64 : 128;
     const long long n_mblocks = (rows_total + 63) / 64;          // the most either layout makes
-    const long long t_max = (long long)a.B * a.Hkv * n_mblocks * ((a.S_max + STEP - 1) / STEP);
+    const long long t_max = (long long)a.B * a.Hkv * n_mblocks * ((a.S_max + STEP - 1) / STEP + kSegCost);
     if (t_max * a.sm_count >= (1ll << 31)) return false;
     if (!(a.scale > 0.f)) return false;       // the kernel takes the maximum before scaling
     return kCounterBytes + tc5_partial_bytes(a.sm_count, rows, a.D) <= a.ws_bytes;
@@ -1262,6 +1264,8 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     const int rows = lay.rows, n_mblocks = lay.n_mblocks, ck = lay.ck;
     const int units = a.B * a.Hkv * n_mblocks;
     const long long t_max = (long long)units * ((a.S_max + STEP - 1) / STEP);
+    // (more units than CTAs, so ranges do not begin and end with units: only there does the number of segments differ)
+    const int seg_cost = pair && ck == 0 && units > a.sm_count ? kSegCost : 0;
     const int grid = ck > 0 ? units * ck : (int)(t_max < a.sm_count ? t_max : a.sm_count);
 
     Tc5Params p = {};
@@ -1271,7 +1275,7 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     p.part_o = (float4*)ws;
     p.part_ml = (float2*)(ws + (size_t)2 * grid * rows * a.D * 4);
     p.B = a.B; p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.S_max = a.S_max; p.n_mblocks = n_mblocks;
-    p.grid_attn = grid; p.min_steps = 2; p.early = a.early_prefetch ? 1 : 0; p.step = STEP;
+    p.grid_attn = grid; p.min_steps = 2; p.early = a.early_prefetch ? 1 : 0; p.step = STEP; p.seg_cost = seg_cost;
     p.scale_log2 = a.scale * 1.4426950408889634f;
     p.status = a.status;
     cudaError_t err;

@@ -142,7 +142,7 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
         cl_seg.slot = -1;
     }
     struct Iter {
-        SegIter it; int n_mblocks, mblock;
+        SegIter<false> it; int n_mblocks, mblock;
         __device__ __forceinline__ bool next(Seg& o) {
             if (!it.next(o)) return false;
             if (!it.cl) { o.mblock = mblock; if (o.slot >= 0) o.slot = o.slot * n_mblocks + mblock; }
@@ -150,7 +150,7 @@ attn_tc5_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_con
         }
     };
     auto make_iter = [&]() {
-        Iter x; x.it.s = &sched; x.it.B = p.B; x.it.n_mblocks = 1; x.it.g = lo; x.it.lo = lo; x.it.hi = hi; x.it.cta = group;
+        Iter x; x.it.s = &sched; x.it.B = p.B; x.it.n_mblocks = 1; x.it.seg_cost_ = 0; x.it.g = lo; x.it.lo = lo; x.it.hi = hi; x.it.cta = group;
         x.it.cl = CL; x.it.cl_done = false; x.it.cl_seg = cl_seg; x.n_mblocks = p.n_mblocks; x.mblock = my_block;
         return x;
     };

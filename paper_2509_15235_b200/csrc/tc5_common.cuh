@@ -308,12 +308,13 @@ struct Tc5Params {
     float scale_log2;
     int* status;
     int step;                  // cached tokens per pipeline step (rows of one K or V stage)
+    int seg_cost;              // even split: steps that a segment's start is counted as when the line is cut (see SegIter)
     int lock;                  // even split by groups of n_mblocks CTAs: CTA c works for group c / n_mblocks on row block c % n_mblocks
 };
 
 // The schedule every CTA (and the merge kernel) derives from kv_len.
 struct Sched {
-    int base[kMaxB + 1];   // first global step of sequence b; base[B] = T
+    int base[kMaxB + 1];   // where sequence b starts on the line (see SegIter); base[B] = T
     int steps[kMaxB];      // steps of one unit of sequence b (0: sequence rejected or empty)
     int len[kMaxB];        // committed length S of sequence b
     int units;             // units with at least one step
@@ -335,13 +336,14 @@ static __device__ void sched_build(Sched& s, const Tc5Params& p, int lane, int k
             s.steps[b] = st;
             s.len[b] = S;
         }
-        int x = st * upb;
+        const int len = st > 0 ? (st + p.seg_cost) * upb : 0;
+        int x = len;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        if (b < p.B) s.base[b] = carry + x - st * upb;
+        if (b < p.B) s.base[b] = carry + x - len;
         carry += __shfl_sync(0xffffffffu, x, 31);
     }
     if (lane == 0) s.base[p.B] = carry;
@@ -371,7 +373,7 @@ __device__ __forceinline__ int sched_ctas(int T, int units, int grid, int min_st
 }
 // (T * grid < 2^31 is checked on the host, so 32-bit arithmetic suffices)
 __device__ __forceinline__ int cta_lo(int c, int T, int geff) { return (int)(((unsigned)c * (unsigned)T) / (unsigned)geff); }
-// The CTA whose range holds global step g.
+// The CTA whose range holds place g of the line.
 __device__ __forceinline__ int cta_of(int g, int T, int geff) {
     int c = (int)((((unsigned)g + 1u) * (unsigned)geff - 1u) / (unsigned)T);
     c = c > geff - 1 ? geff - 1 : c;
@@ -383,9 +385,14 @@ __device__ __forceinline__ int cta_of(int g, int T, int geff) {
 struct Seg {
     int b, kvh, mblock, st0, n, steps, S, slot;    // slot < 0: the segment is a whole unit
 };
+// The line that the even split cuts: every unit is seg_cost places without work, then its steps.  A CTA whose range takes in the
+// start of a unit pays for one more segment (a Q tile, an empty pipeline and an epilogue: 5 us with rows <= 64, as long as 4
+// steps), and so gets as many steps less; without it llava13b_b4's CTAs ended after 44, 49 or 54 us by the number of their segments.
+// COST: seg_cost may be other than 0 (rows <= 64; elsewhere the register that it takes costs more).
+template <bool COST>
 struct SegIter {
     const Sched* s;
-    int B, n_mblocks, g, lo, hi, cta;
+    int B, n_mblocks, seg_cost_, g, lo, hi, cta;
     bool cl, cl_done;          // cluster schedule: exactly one segment (possibly empty), given in cl_seg
     Seg cl_seg;
     __device__ __forceinline__ bool next(Seg& o) {
@@ -395,22 +402,25 @@ struct SegIter {
             o = cl_seg;
             return true;
         }
-        if (g >= hi) return false;
-        int l = 0, r = B;                               // first b with base[b] > g, minus one
-        while (l < r) { const int m = (l + r) >> 1; if (s->base[m] <= g) l = m + 1; else r = m; }
-        o.b = l - 1;
-        o.steps = s->steps[o.b];
-        o.S = s->len[o.b];
-        const int rel = g - s->base[o.b];
-        const int uib = rel / o.steps;
-        o.st0 = rel - uib * o.steps;
-        o.n = min(hi - g, o.steps - o.st0);
-        o.kvh = uib / n_mblocks;
-        o.mblock = uib - o.kvh * n_mblocks;
-        const bool whole = (o.st0 == 0 && o.n == o.steps);
-        o.slot = whole ? -1 : (g == lo ? 2 * cta : 2 * cta + 1);
-        g += o.n;
-        return true;
+        const int seg_cost = COST ? seg_cost_ : 0;
+        for (;;) {
+            if (g >= hi) return false;
+            int l = 0, r = B;                               // first b with base[b] > g, minus one
+            while (l < r) { const int m = (l + r) >> 1; if (s->base[m] <= g) l = m + 1; else r = m; }
+            o.b = l - 1;
+            o.steps = s->steps[o.b];
+            o.S = s->len[o.b];
+            const int rel = g - s->base[o.b], len = o.steps + seg_cost;
+            const int uib = rel / len, off = rel - uib * len, end = min(len, off + hi - g);   // of this unit, places [off, end)
+            o.st0 = COST ? max(off - seg_cost, 0) : off;
+            o.n = end - seg_cost - o.st0;
+            o.kvh = uib / n_mblocks;
+            o.mblock = uib - o.kvh * n_mblocks;
+            const bool whole = (o.st0 == 0 && o.n == o.steps);
+            o.slot = whole ? -1 : (g == lo ? 2 * cta : 2 * cta + 1);
+            g += end - off;
+            if (!COST || o.n > 0) return true;
+        }
     }
 };
 
@@ -799,15 +809,15 @@ attn_tc5_merge_kernel(const Tc5Params p) {
         const int S = p.kv_len[bb];
         const int st = (S >= 0 && S + p.N <= p.S_max) ? (S + p.N + p.step - 1) / p.step : 0;
         if (bb == b) { base_b = T; steps = st; }
-        T += st * spb;
+        T += st > 0 ? (st + p.seg_cost) * spb : 0;
         live += st > 0 ? spb : 0;
     }
     // Everything that does not hang on the partials comes ahead of the dependency, down to the first group's addresses (each
     // behind a division); every block waits, also one with nothing to do: what follows on the stream waits for this kernel only.
     if (steps == 0) { pdl_wait(); return; }
     const int geff = sched_ctas(T, live, LOCK ? p.grid_attn / p.n_mblocks : p.grid_attn, p.min_steps, sched_round_steps(p));
-    const int ub = base_b + (LOCK ? uib / p.n_mblocks : uib) * steps, ue = ub + steps;
-    const int c0 = cta_of(ub, T, geff), c1 = cta_of(ue - 1, T, geff);
+    const int ub = base_b + (LOCK ? uib / p.n_mblocks : uib) * (steps + p.seg_cost), u0 = ub + p.seg_cost;   // where the unit starts, its first step
+    const int c0 = cta_of(u0, T, geff), c1 = cta_of(u0 + steps - 1, T, geff);
     if (c0 == c1) { pdl_wait(); return; }              // one CTA had the whole unit and wrote the output itself
     const int G = p.Hq / p.Hkv, N = p.N;
     const int kvh = uib / p.n_mblocks, mblock = uib - kvh * p.n_mblocks;

@@ -132,6 +132,25 @@ def test_head_size_64_cluster_merge_shares(gu, B, N):
     _check(gu, q, k, v, kv_len, mask, 1 / math.sqrt(D), split_form=2)
 
 
+@pytest.mark.parametrize("split_form", [1, 3])
+@pytest.mark.parametrize("Hkv,D,N,kv_len,S_max", [
+    (48, 128, 60, [0, 5, 70, 900], 1024),     # units of 1, 1, 2 and 8 steps: ranges that begin or end where a unit has no work
+    (80, 128, 3, [1300, 125], 1408),          # units of 11 and 1 steps, three rows each
+    (52, 64, 33, [700, 300, 1], 768),
+])
+def test_more_units_than_ctas(gu, Hkv, D, N, kv_len, S_max, split_form):
+    """The even split with several segments per CTA: their starts count as steps when the line is cut, and the q rows of later
+    segments come through the K ring."""
+    B = len(kv_len)
+    rng = np.random.Generator(np.random.Philox(4000 + N))
+    q = synth.normal_bf16((B, N, Hkv, D), 4001)
+    k = synth.normal_bf16((B, Hkv, S_max, D), 4002)
+    v = synth.normal_bf16((B, Hkv, S_max, D), 4003)
+    parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
+    mask, _, _ = oracle.tree_mask(parents)
+    _check(gu, q, k, v, np.asarray(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=split_form)
+
+
 # Nodes that see one key (their own slot; kv_len 0) or two (the one committed key and their own): a row's sum is then one or
 # two exponentials, and every column of a step has a node whose weight is formed there.  Small integers in q and k make the
 # scores exact, so lse carries the roundings of the scaling, of two exponentials (2 ulp each) and of one logarithm: below
