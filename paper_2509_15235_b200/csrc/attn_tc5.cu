@@ -253,6 +253,242 @@ __device__ __noinline__ void rope_prologue(unsigned char* sm, const __nv_bfloat1
 // 455.3 / 454.8 / 451.8; 1 in 6 moves nothing, 1 in 4 and 1 in 2 are slower (issue slots).
 constexpr int kPolyEvery = 4;
 
+// ---- 128 rows per unit in the cluster form: two groups of softmax warps on alternate steps ----------------------
+// With two threads per row (below) all eight warps move in lock-step: they wait, load and exchange maxima together, and meanwhile
+// neither the special-function pipe nor the tensor pipe has work (2240 cycles per step, of which the exponentials are 1024 and the
+// products 1024).  Here a row belongs to one thread of each group of four warps; group x takes the steps of parity x whole, with a
+// reference maximum, a sum and an accumulator of its own (added up at the end), so nothing is exchanged, and while one group is in
+// its exponentials the products of the other run.  P overwrites S, which makes room for the second accumulator; one warp issues all
+// products, S(0) S(1) | PV(0) S(2) | PV(1) S(3) | ...: they complete in the order of issue, so S(t + 2) may overwrite P(t), and its
+// completion tells that PV(t) is complete.  1880 cycles per step (qwen3b_S8192_N60_B4 485 -> 465 us per pass); what bounds it now is
+// shared memory, whose 128 bytes per cycle feed both operands of S (512 cycles), V (256) and the copies coming in (512).  In the even
+// split, whose CTAs have fewer steps here, the longer first step costs more than the loop gains (qwen3b_S32768_N16_B1 324 -> 329),
+// and rows <= 64, where a thread has half the columns, gain 0.5 % and lose 2.5 % in the smallest calls: both keep two threads per row.
+// TMEM: S_0 0..127, S_1 128..255 (P of the step in the first 64 columns of its S), O_0 256, O_1 384.
+enum { B_PHALF0 = B_PFULL, B_PHALF1 = B_SFREE };     // halves of P, by accumulator (128 arrivals)
+
+template <int HD>
+__device__ __forceinline__ void alternate_issue(uint32_t base, uint32_t bars, uint32_t tmem, int n_, volatile int* abort_flag) {
+    constexpr int NH = HD / 64, STAGE = NH * HALF_BYTES, NSK = kMaxRing / NH, NSV = kMaxRing / NH;
+    constexpr uint32_t IDESC_S = instr_desc(0), IDESC_O = instr_desc(1, HD);   // B = K stage, K-major; V stage, MN-major
+    constexpr uint32_t DESC_HI = desc_hi(1024);
+    auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
+    const bool leader = elect_one();
+    const int n = __shfl_sync(0xffffffffu, n_, 0);
+    const uint32_t k0 = desc_lo(base + SMEM_K, 16), v0 = desc_lo(base + SMEM_V, HALF_BYTES), qb = desc_lo(base + SMEM_Q, 16);
+    uint32_t sk = 0, pk = 0, sv = 0, pv = 0;                    // ring positions with their phases
+    // A wait costs 150 cycles also where the answer is there.  So what a step needs is asked for ahead, without blocking, between
+    // the last step's PV and S products, whose issue takes long enough for the answers to come; only where the answer was no it is
+    // waited for.
+    bool k_ok = false, v_ok = false, p_ok[2] = {false, false};
+    auto have = [&](bool asked, uint32_t b, uint32_t phase) {
+        return __all_sync(0xffffffffu, asked) || mbar_wait_warp(b, phase, abort_flag);
+    };
+    auto score = [&](uint32_t x) {                             // S_x = Q K^T
+        if (!have(k_ok, bar(B_KFULL) + 8u * sk, pk)) return false;
+        k_ok = false;
+        tc_fence_after();
+        if (leader) {
+            const uint32_t kb = k0 + sk * (STAGE >> 4), d = tmem + COL_S + x * 128;
+#pragma unroll
+            for (int ks = 0; ks < HD / 16; ++ks) {             // 16 d-columns per instruction: 32 B of each Q and K row
+                const uint32_t koff = ((ks >> 2) * HALF_BYTES + (ks & 3) * 32) >> 4;
+                tc_mma_ss(d, qb + koff, DESC_HI, kb + koff, DESC_HI, IDESC_S, ks > 0 ? 1u : 0u);
+            }
+            tc_commit(bar(B_SFULL) + 8u * x);
+            tc_commit(bar(B_KEMPTY) + 8u * sk);
+        }
+        if (++sk == NSK) { sk = 0; pk ^= 1; }
+        return true;
+    };
+    if (!mbar_wait_warp(bar(B_QFULL), 0, abort_flag)) return;
+    if (n > 0 && !score(0)) return;
+    if (n > 1 && !score(1)) return;
+    for (int t = 0; t < n; ++t) {
+        const uint32_t x = t & 1;
+        if (t + 2 < n) k_ok = mbar_test(bar(B_KFULL) + 8u * sk, pk);
+        if (!have(v_ok, bar(B_VFULL) + 8u * sv, pv)) return;
+        const uint32_t vb = v0 + sv * (STAGE >> 4), pb = tmem + COL_S + x * 128, d = tmem + COL_O + x * 128;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {                          // O_x += P_x V(step), each half of the tokens as soon as its P is there
+            if (!have(p_ok[h], bar(h ? B_PHALF1 : B_PHALF0) + 8u * x, (t >> 1) & 1)) return;
+            tc_fence_after();
+            if (leader) {
+#pragma unroll
+                for (int ks = 4 * h; ks < 4 * h + 4; ++ks)     // 16 tokens per instruction: 8 P columns, 16 V rows (2 KB)
+                    tc_mma_ts(d, pb + ks * 8, vb + ks * 128, DESC_HI, IDESC_O, (t > 1 || ks > 0) ? 1u : 0u);
+            }
+        }
+        if (leader) {
+            tc_commit(bar(B_VEMPTY) + 8u * sv);
+            tc_commit(bar(B_PVDONE) + 8u * x);
+        }
+        if (++sv == NSV) { sv = 0; pv ^= 1; }
+        v_ok = p_ok[0] = p_ok[1] = false;
+        if (t + 1 < n) {
+            v_ok = mbar_test(bar(B_VFULL) + 8u * sv, pv);
+            p_ok[0] = mbar_test(bar(B_PHALF0) + 8u * (x ^ 1), ((t + 1) >> 1) & 1);
+            p_ok[1] = mbar_test(bar(B_PHALF1) + 8u * (x ^ 1), ((t + 1) >> 1) & 1);
+        }
+        if (t + 2 < n && !score(x)) return;
+    }
+}
+
+// One softmax thread's row of the segment (lane tl, group x), down to the partial parked in shared memory.  False: a wait gave up.
+template <int HD>
+__device__ __forceinline__ bool alternate_softmax(unsigned char* sm, uint32_t bars, uint32_t tmem, const Seg& sg, int N, float scale_log2,
+                                                  uint64_t mk0, uint64_t mk1, bool row_ok, int x, int tl, volatile int* abort_flag) {
+    constexpr int NH = HD / 64, STAGE = NH * HALF_BYTES, NSV = kMaxRing / NH, ROWS = 128;
+    auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
+    const uint32_t lane_addr = tmem + ((uint32_t)(tl & ~31) << 16), s_addr = lane_addr + COL_S + x * 128, o_addr = lane_addr + COL_O + x * 128;
+    const int S = sg.S, total = S + N;
+    float m_ref = -INFINITY, l_run = 0.f;
+    bool has_o = false;
+    for (int t = x; t < sg.n; t += 2) {
+        const int tok0 = (sg.st0 + t) * STEP;
+        // (this product was issued after this group's last PV product, so that one is complete too: O_x and P are free)
+        if (!mbar_wait_warp(bar(B_SFULL + x), (t >> 1) & 1, abort_flag)) return false;
+        tc_fence_after();
+        const bool tail = tok0 + STEP > S;                     // reaches past the committed prefix: ancestor bits
+        uint64_t a0 = 0, a1 = 0;                               // bit c: column c may be attended to (prefix column, or visible tree node)
+        if (tail) {
+            const int t0 = tok0 - S;                           // tree index of column 0 (may be negative)
+            if (t0 >= 0) shr128(mk0, mk1, t0, a0, a1); else shl128_fill(mk0, mk1, -t0, a0, a1);
+        }
+        // The row is read in halves of 64 columns, the upper half twice (held whole it would take the registers of both).
+        uint32_t s[64];
+        auto load_half = [&](int h) {
+            tmem_ld32(s_addr + h * 64, s);
+            tmem_ld32(s_addr + h * 64 + 32, s + 32);
+            tmem_wait_ld();
+            if (tail) {
+                const uint64_t a = h ? a1 : a0;
+#pragma unroll
+                for (int c = 0; c < 64; ++c)
+                    if (!((a >> c) & 1ull)) s[c] = 0xff800000u;   // -inf
+            }
+        };
+        float mx[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) mx[e] = -INFINITY;
+#pragma unroll 1
+        for (int h = 1; h >= 0; --h) {
+            load_half(h);
+#pragma unroll
+            for (int c = 0; c < 64; c += 16)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) mx[e] = max3_nan(mx[e], __uint_as_float(s[c + e]), __uint_as_float(s[c + 8 + e]));
+        }
+        // the scale is positive, so it commutes with the maximum
+        const float tmax = max_nan(max3_nan(max3_nan(mx[0], mx[1], mx[2]), max3_nan(mx[3], mx[4], mx[5]), mx[6]), mx[7]) * scale_log2;
+        // move the reference maximum only when the tile exceeds it by more than the gap
+        float alpha = 1.f;
+        bool rescale = false;
+        if (tmax > m_ref + kRescaleGap) {                      // also true on the first finite tile (m_ref = -inf)
+            alpha = exp2f(m_ref - tmax);                       // 0 when m_ref = -inf
+            m_ref = tmax;
+            l_run *= alpha;
+            rescale = has_o;
+        }
+        if (!(tmax < INFINITY)) l_run = tmax - tmax;            // a NaN or an infinite score: the row is NaN (see inv_sum)
+        if (__any_sync(0xffffffffu, rescale)) {
+#pragma unroll
+            for (int c = 0; c < HD / 16; ++c) {
+                uint32_t o[16];
+                tmem_ld16(o_addr + c * 16, o);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                tmem_st16(o_addr + c * 16, o);
+            }
+        }
+        bool fail = false;
+        if (tok0 + STEP > total) {
+            // last step of the sequence: V rows past the last key may hold anything, and they meet weight-0 columns of P in the
+            // product: clear them (lane r clears row r)
+            const int sv = t % NSV;
+            fail = !mbar_wait(bar(B_VFULL + sv), (t / NSV) & 1, abort_flag);
+            if (!fail && tok0 + tl >= total) {
+                unsigned char* vrow = sm + SMEM_V + sv * STAGE + tl * 128;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
+                    if (NH == 2) *reinterpret_cast<uint4*>(vrow + HALF_BYTES + c * 16) = make_uint4(0, 0, 0, 0);
+                }
+            }
+            fence_async_smem();
+        }
+        if (__any_sync(0xffffffffu, fail)) return false;
+        // P = exp2(scale * s - m_ref) as bf16 pairs (column c of P holds tokens 2c, 2c+1), handed on by halves
+        const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
+        const uint64_t sc2 = pk2(scale_log2, scale_log2), mm2 = pk2(-m_use, -m_use);
+        uint64_t sum2 = pk2(0.f, 0.f), sum2b = sum2;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1) load_half(1);                          // (P of the first half lies in columns 0..31)
+            uint32_t pd[32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) {
+                float x0, x1, e0, e1;
+                up2(fma2(pk2(__uint_as_float(s[2 * c]), __uint_as_float(s[2 * c + 1])), sc2, mm2), x0, x1);
+                if (c % 8 == 7) exp2_fma_pair(x0, x1, e0, e1);  // (see kPolyEvery)
+                else { e0 = exp2f(x0); e1 = exp2f(x1); }
+                if (c & 1) sum2b = add2(sum2b, pk2(e0, e1)); else sum2 = add2(sum2, pk2(e0, e1));
+                pd[c] = pack_bf16(e0, e1);
+            }
+            tmem_st32(s_addr + h * 32, pd);
+            tmem_wait_st();
+            tc_fence_before();
+            mbar_arrive(bar(h ? B_PHALF1 : B_PHALF0) + 8u * x);
+        }
+        float l0, l1;
+        up2(add2(sum2, sum2b), l0, l1);
+        l_run += l0 + l1;
+        has_o = true;
+    }
+
+    // The row's statistics, of both groups, go round while the last products run; then this thread adds up columns
+    // [HD/2 x, HD/2 x + HD/2) of the lane's two accumulators and parks them over the K ring, [HD/4 col4][ROWS].
+    float* xm = reinterpret_cast<float*>(sm + SMEM_XM);       // [group][lane] l, then the same of m
+    xm[x * 128 + tl] = l_run;
+    xm[256 + x * 128 + tl] = has_o ? m_ref : -INFINITY;
+    mbar_arrive(bar(B_XCH));
+    // (everybody past its last step: every product but each accumulator's last PV is complete, and a wait can tell the phase it
+    // waits for from the one before)
+    if (!mbar_wait_warp(bar(B_XCH), 0, abort_flag)) return false;
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+        const int t = sg.n - 1 - ((sg.n - 1 - y) & 1);         // the accumulator's last step
+        if (t >= 0 && !mbar_wait_warp(bar(B_PVDONE + y), (t >> 1) & 1, abort_flag)) return false;
+    }
+    tc_fence_after();
+    const float m0 = xm[256 + tl], m1 = xm[384 + tl], m_all = fmaxf(m0, m1), m_fin = (m_all == -INFINITY) ? 0.f : m_all;
+    const float w0 = exp2f(m0 - m_fin), w1 = exp2f(m1 - m_fin);   // 0 where nothing was seen
+    const float l_all = xm[tl] * w0 + xm[128 + tl] * w1;
+    float4* prow = reinterpret_cast<float4*>(sm + SMEM_K) + (size_t)x * (HD / 8) * ROWS + tl;
+#pragma unroll
+    for (int cc = 0; cc < HD / 2; cc += 32) {
+        uint32_t o0[32], o1[32];
+        tmem_ld32(lane_addr + COL_O + x * (HD / 2) + cc, o0);
+        tmem_ld32(lane_addr + COL_O + 128 + x * (HD / 2) + cc, o1);
+        tmem_wait_ld();
+        float v[32];
+        // (an accumulator is only defined once a product has run: select, never multiply, where the weight is zero)
+#pragma unroll
+        for (int e = 0; e < 32; ++e)
+            v[e] = (w0 > 0.f ? __uint_as_float(o0[e]) * w0 : 0.f) + (w1 > 0.f ? __uint_as_float(o1[e]) * w1 : 0.f);
+        if (row_ok) {
+#pragma unroll
+            for (int c4 = 0; c4 < 8; ++c4)
+                prow[(size_t)(cc / 4 + c4) * ROWS] = make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+        }
+    }
+    tc_fence_before();
+    if (x == 0 && row_ok)
+        reinterpret_cast<float2*>(sm + SMEM_K + (HD / 4) * ROWS * 16)[tl] = make_float2(l_all > 0.f ? m_all : -INFINITY, l_all);
+    return true;
+}
+
 // PAGED instantiations carry the paged producer; the others are compiled without it (its call sites cost the
 // contiguous kernels registers they do not have to spare).
 template <bool PAIR, bool CL, bool PAGED, bool ROPE = false, int HD = 128>
@@ -269,6 +505,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     constexpr int D = HD, NH = HD / 64, STAGE_BYTES = NH * HALF_BYTES, NSK = kMaxRing / NH, NSV = kMaxRing / NH;
     constexpr int ROWS = PAIR ? 64 : 128;      // distinct query rows per CTA
     constexpr int NC = PAIR ? 32 : 64;         // tokens of a step one softmax thread handles (two threads per row)
+    constexpr bool ALT = CL && !PAIR;          // alternate steps instead (alternate_softmax)
     // The V ring can have a producer of its own, the spare warp (its lane 0; paged: all of it).  With at most 64 rows per
     // unit it always has; with 128 only for pools of 16-row blocks, where one warp issuing a step's 32 copies is what
     // holds the call back (larger blocks lose 1 % with two producers, like the contiguous cache).
@@ -302,8 +539,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         for (int i = 0; i < NSK; ++i) { mbar_init(bar(B_KFULL + i), 1); mbar_init(bar(B_KEMPTY + i), 1); }
         for (int i = 0; i < NSV; ++i) { mbar_init(bar(B_VFULL + i), 1); mbar_init(bar(B_VEMPTY + i), 1); }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SFREE + i), kSmx);
-            mbar_init(bar(B_PFULL + i), kSmx); mbar_init(bar(B_PVDONE + i), 1);
+            mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SFREE + i), ALT ? 128 : kSmx);
+            mbar_init(bar(B_PFULL + i), ALT ? 128 : kSmx); mbar_init(bar(B_PVDONE + i), 1);
         }
         for (int i = 0; i < 4; ++i) mbar_init(bar(B_PAIRX + i), 64);
         mbar_init(bar(B_QFULL), kSmx);
@@ -508,7 +745,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         // The whole warp walks through the steps and waits, one elected lane issues: with uniform control flow the
         // descriptors live in uniform registers, where the instructions take them from.  Against one lane doing it all:
         // llava7b 16.7 -> 16.2 us per layer, qwen7b 15.2 -> 14.5, qwen3b_S8192_N60_B4 31.3 -> 29.7, qwen3b_S32768_N16_B1 29.2 -> 28.9.
-        if (active) {
+        if constexpr (ALT) {
+            alternate_issue<HD>(base, bars, tmem, cl_seg.n, abort_flag);
+        } else if (active) {
             constexpr uint32_t IDESC_S = instr_desc(0);            // B = K stage, K-major
             constexpr uint32_t DESC_HI = desc_hi(1024);            // 8 rows x 128 B between row groups, everywhere
             const bool leader = elect_one();
@@ -573,6 +812,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 }
                 ok = __all_sync(0xffffffffu, ok);
             }
+            if constexpr (ALT) ok = false;                                // (warp 1 issues these products too)
             uint32_t sv = 0, pv = 0, u = 0;
             Iter si = make_iter();
             Seg sg;
@@ -727,6 +967,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 // bits at or beyond N are not tree nodes
                 if (N < 64) mk0 &= (1ull << N) - 1;
                 if (N < 128) mk1 &= N > 64 ? (1ull << (N - 64)) - 1 : 0ull;
+                if constexpr (ALT) {
+                    ok = alternate_softmax<HD>(sm, bars, tmem, sg, N, p.scale_log2, mk0, mk1, row_ok, ch, tl, abort_flag);
+                    break;
+                }
                 // m_ref and has_o are the same in both threads of a row; l_run covers this thread's columns only
                 float m_ref = -INFINITY, l_run = 0.f;
                 bool has_o = false;

@@ -132,6 +132,24 @@ def test_head_size_64_cluster_merge_shares(gu, B, N):
     _check(gu, q, k, v, kv_len, mask, 1 / math.sqrt(D), split_form=2)
 
 
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("N,kv_len,S_max", [
+    (16, [3, 40, 240], 256),                  # one and two steps: most ranks of a cluster have none
+    (16, [1400, 900, 2100], 2176),            # one to three steps per rank
+    (17, [4400, 3300, 2900], 4480),           # three to five; two row blocks, the last of 8 rows
+])
+def test_units_of_128_rows_in_clusters(gu, D, N, kv_len, S_max):
+    """The cluster form whose two groups of softmax warps take alternate steps: none, one, odd and even numbers of them."""
+    B, Hq, Hkv = len(kv_len), 16, 2
+    rng = np.random.Generator(np.random.Philox(4100 + N))
+    q = synth.normal_bf16((B, N, Hq, D), 4101)
+    k = synth.normal_bf16((B, Hkv, S_max, D), 4102)
+    v = synth.normal_bf16((B, Hkv, S_max, D), 4103)
+    parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
+    mask, _, _ = oracle.tree_mask(parents)
+    _check(gu, q, k, v, np.asarray(kv_len, dtype=np.int32), mask, 1 / math.sqrt(D), split_form=2)
+
+
 @pytest.mark.parametrize("split_form", [1, 3])
 @pytest.mark.parametrize("Hkv,D,N,kv_len,S_max", [
     (48, 128, 60, [0, 5, 70, 900], 1024),     # units of 1, 1, 2 and 8 steps: ranges that begin or end where a unit has no work
