@@ -1383,8 +1383,15 @@ static int query_max_clusters(bool pair, int k) {
 // Both sides of the line between the forms, clusters / even split, us per layer: 16 query and 2 kv heads, 1 x 16 nodes on 2048 10.4 /
 // 13.8, on 8192 16.9 / 15.0, on 32768 42.7 / 20.0, 4 x 60 on 8192 28.5 / 34.2; 32 heads, 1 x 60 on 3904 15.7 / 20.3, 4 x 60 on
 // 2000 30.0 / 32.3; 40 heads, 1 x 30 on 8000 30.4 / 33.4, 2 x 30 on 4000 38.7 / 36.7.
-static double tc5_step_us(const AttnArgs& a, bool pair, int n_mblocks, double ctas) {
-    const double busy = ctas / a.sm_count, compute = pair ? 0.8 + 0.25 * busy : 1.05 + 0.15 * busy;
+// (alternate: units of 128 rows in clusters, whose softmax groups take alternate steps: 0.92 us per step where two threads per row take
+// 1.18.  Where many row blocks share few heads in large clusters a step takes a quarter longer - 16 query and 2 kv heads, 128 nodes: one
+// sequence of 32768 in clusters of eight 1.16, four of 8192 in clusters of two 0.90 -, beyond four ranks the merge grows, and in long
+// calls the power cap weighs more on it than on the two-tile kernel, whose rows share their K/V tiles.  One-tile clusters / two-tile
+// kernel, us per layer in runs of seconds: 8 x 60 nodes on 8192 44.6 / 45.6, 4 x 60 on 16384 44.6 / 47.8, on 32768 81.1 / 79.8, 8 x 128 on
+// 8192 77.6 / 82.1, 2 x 128 on 40000 92.1 / 89.4; in short ones 39.5 / 43.4, 39.5 / 44.8, 72.3 / 70.9, 70.1 / 74.9; 1 x 128 on 32768
+// 49.0 / 42.0; 28 / 4 heads, 2 x 92 on 40000 142 / 125; 16 / 4 heads of size 64, 6 x 60 on 3000 17.7 / 21.7, 6 x 128 30.1 / 27.0.)
+static double tc5_step_us(const AttnArgs& a, bool pair, int n_mblocks, double ctas, bool alternate) {
+    const double busy = ctas / a.sm_count, compute = pair ? 0.8 + 0.25 * busy : alternate ? 0.80 + 0.14 * busy : 1.05 + 0.15 * busy;
     return fmax(a.D == 64 ? 0.9 * compute : compute, ctas * 0.0093 * (a.D / 128.0) / n_mblocks);
 }
 static int tc5_steps(const AttnArgs& a) {
@@ -1392,7 +1399,10 @@ static int tc5_steps(const AttnArgs& a) {
     return (slots + STEP - 1) / STEP;
 }
 static double tc5_cluster_us(const AttnArgs& a, bool pair, int n_mblocks, int k) {
-    return (pair ? 6.9 : 9.6) + (double)((tc5_steps(a) + k - 1) / k) * tc5_step_us(a, pair, n_mblocks, (double)a.B * a.Hkv * n_mblocks * k);
+    const double ctas = (double)a.B * a.Hkv * n_mblocks * k, steps = (double)((tc5_steps(a) + k - 1) / k);
+    const double us = steps * tc5_step_us(a, pair, n_mblocks, ctas, !pair);
+    if (pair) return 6.9 + us;
+    return 9.4 + us + 0.35 * (k > 4 ? k - 4 : 0) + (n_mblocks > 4 && k > 4 ? 0.24 * steps : 0.0) + 0.22 * (ctas / a.sm_count) * fmax(0.0, steps - 32.0);
 }
 // (even split: the CTAs as sched_ctas counts them; partials of 128 rows cost 34 ns per CTA, written and merged, those of 64
 // rows go in the fixed part; where there are more units than CTAs every further segment of a CTA costs a Q tile, a
@@ -1405,7 +1415,7 @@ static double tc5_even_us(const AttnArgs& a, bool pair, int n_mblocks) {
         const double r = floor(n / units) * units;
         if (n_mblocks > 1 || ceil(T / r) - ceil(T / n) <= 3.0) n = r;
     }
-    return (pair ? 9.5 : 10.4 + 0.034 * n) + ceil(T / n) * tc5_step_us(a, pair, n_mblocks, n) + (units > n && n_mblocks > 1 ? 11.0 * units / n : 0.0);
+    return (pair ? 9.5 : 10.4 + 0.034 * n) + ceil(T / n) * tc5_step_us(a, pair, n_mblocks, n, false) + (units > n && n_mblocks > 1 ? 11.0 * units / n : 0.0);
 }
 
 // Cluster size of the cluster form: one cluster per unit, as large as all clusters fit at once (0: they do not).

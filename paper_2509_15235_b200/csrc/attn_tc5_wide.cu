@@ -544,11 +544,13 @@ WidePlan attn_tc5_wide_plan(const AttnArgs& a) {
     const int heads = a.B * a.Hkv;
     const double T = steps * heads;
     double n = fmin((double)groups, fmax(1.0, floor(T / 2.0)));
+    double uneven = 0.0;                       // ranges that cross heads: two segments in some groups
     if (heads <= n) {                          // as sched_ctas counts the groups
         const double r = floor(n / heads) * heads;
         if (ceil(T / r) - ceil(T / n) <= 3.0) n = r;
+        else uneven = 3.0;
     }
-    const double est = (a.D == 64 ? 13.7 : 15.5) + ceil(T / n) * fmax(a.D == 64 ? 1.6 : 2.0, n * 0.0093 * hbm) + (heads > n ? 11.0 * heads / n : 0.0);
+    const double est = uneven + (a.D == 64 ? 13.7 : 15.5) + ceil(T / n) * fmax(a.D == 64 ? 1.6 : 2.0, n * 0.0093 * hbm) + (heads > n ? 11.0 * heads / n : 0.0);
     if (est < w.est_us) { w.ck = 0; w.grid = groups * nmb; w.est_us = est; }
     return w;
 }
