@@ -1534,14 +1534,14 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     p.status = a.status;
     cudaError_t err;
     const bool paged = a.page_rows != 0;
-    // Even split, at most 64 rows per unit: short calls and those with many units merge in the attention kernel (the last
-    // arrival at a unit, by the counters at the head of the workspace), the others with the merge kernel, which runs beside
-    // the next call's start.  Measured, in the kernel / with the merge kernel, us per layer (13B heads): 4 x 60 nodes on
-    // 1000 tokens 28.2 / 29.1, 8 x 16 on 1000 39.4 / 41.0, 8 x 16 on 3000 91.1 / 91.7; 4 x 60 on 4000 66.5 / 65.3, 4 x 31 on
-    // 2000 36.4 / 34.1, 2 x 30 on 4000 37.6 / 34.3.  Blocks of 128 rows, a grid with more units than counters and split form
-    // 3 always get the merge kernel.
+    // Even split, at most 64 rows per unit: short calls and those of more units than CTAs merge in the attention kernel (the last
+    // arrival at a unit, by the counters at the head of the workspace; the ranges then end at different units, and most merges lie
+    // within the call), the others with the merge kernel.  Measured, in the kernel / with the merge kernel, us per layer (13B
+    // heads): 4 x 60 nodes on 1000 tokens 28.2 / 29.1, 8 x 16 on 3000 91.1 / 91.7, 4 x 60 on 3000-5000 62.9 / 64.2 (70.2 / 72.2 with the
+    // rotation kernel between the calls), 6 x 16 on 1000-4000 64.9 / 67.0, 4 x 31 on 2000 33.8 / 33.9; 2 x 30 on 4000 37.6 / 34.3.
+    // Blocks of 128 rows, a grid with more units than counters and split form 3 always get the merge kernel.
     const bool own_merge = pair && ck == 0 && a.tc5_path != 3 && !a.no_counters && (size_t)units * sizeof(int) <= kCounterBytes &&
-                           (a.tc5_path == 1 || tc5_steps(a) < 12 || units > 2 * a.sm_count);
+                           (a.tc5_path == 1 || tc5_steps(a) < 12 || units > a.sm_count);
     const PagedArgs pa = {a.block_table, a.table_stride, a.page_rows, a.num_blocks, a.Hkv, a.N, a.token_major, a.status,
                           own_merge ? (int*)a.ws : nullptr};
     auto launch_attn = [&](auto kernel, int cluster) {
