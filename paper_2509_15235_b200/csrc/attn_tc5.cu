@@ -24,13 +24,16 @@
 //   warp 1     issuer of S = Q K^T as 128x128x16 tcgen05.mma (the warp walks the steps and waits, one elected lane
 //              issues); owns the TMEM allocation
 //   warp 2     issuer of O += P V, likewise; the two chains wait on different barriers, so each has its own warp and
-//              neither's waits delay the other's instructions
+//              neither's waits delay the other's instructions.  With the fused rotary embedding it also tells the ranks of the
+//              cluster that this one's tree rows are placed
 //   warp 3     derives the schedule from kv_len; with at most 64 rows per unit (its lane 0 in the cluster form of a
 //              contiguous cache, else the whole warp) and on pools of 16-row blocks it then produces the V ring, so that
 //              warp 0's K copies never queue behind a wait for a V stage
 //   warps 4-11 softmax: thread <-> TMEM lane; warps w and w+4 share the same 32 accumulator rows and each takes
 //              half of a step's columns (the row maximum is exchanged through shared memory), so a row costs
-//              no shuffles; they also load Q at the start of every segment and run the segment epilogue
+//              no shuffles; they also load Q at the start of every segment (a later segment's comes through the K ring) and run
+//              the segment epilogue.  Units of 128 rows in the cluster form: the two groups take alternate steps instead, and warp 1
+//              issues all products (alternate_softmax, alternate_issue)
 // TMEM map (512 columns x 128 lanes): S[0] 0..127, S[1] 128..255, O 256..383, P[0] 384..447, P[1] 448..511.
 // P (bf16, packed two per column) is the A operand of the PV product and never touches shared memory; Q
 // sits in shared memory in the same swizzled K-major layout as a K stage.  S and P are double-buffered: S
@@ -260,8 +263,9 @@ constexpr int kPolyEvery = 4;
 // reference maximum, a sum and an accumulator of its own (added up at the end), so nothing is exchanged, and while one group is in
 // its exponentials the products of the other run.  P overwrites S, which makes room for the second accumulator; one warp issues all
 // products, S(0) S(1) | PV(0) S(2) | PV(1) S(3) | ...: they complete in the order of issue, so S(t + 2) may overwrite P(t), and its
-// completion tells that PV(t) is complete.  1880 cycles per step (qwen3b_S8192_N60_B4 485 -> 465 us per pass); what bounds it now is
-// shared memory, whose 128 bytes per cycle feed both operands of S (512 cycles), V (256) and the copies coming in (512).  In the even
+// completion tells that PV(t) is complete.  1880 cycles per step (qwen3b_S8192_N60_B4 485 -> 465 us per pass; tensor pipe active 35 %
+// of a launch against 31 %).  What is left is a group's chain, products of its own step and of the other group's among it, and beside
+// it shared memory, whose 128 bytes per cycle feed both operands of S (512 cycles), V (256) and the copies coming in (512).  In the even
 // split, whose CTAs have fewer steps here, the longer first step costs more than the loop gains (qwen3b_S32768_N16_B1 324 -> 329),
 // and rows <= 64, where a thread has half the columns, gain 0.5 % and lose 2.5 % in the smallest calls: both keep two threads per row.
 // TMEM: S_0 0..127, S_1 128..255 (P of the step in the first 64 columns of its S), O_0 256, O_1 384.
@@ -1380,9 +1384,9 @@ static int query_max_clusters(bool pair, int k) {
 // per step over 7 TB/s; the row blocks of a kv head read the same tiles, so one in n_mblocks comes from HBM; a
 // step's bytes follow the head size, its softmax does not).  The host knows only the capacity S_max, not kv_len: the
 // estimate is for full caches unless the caller has given the length it expects (VISPEC_OPT_KV_LEN_HINT).
-// Both sides of the line between the forms, clusters / even split, us per layer: 16 query and 2 kv heads, 1 x 16 nodes on 2048 10.4 /
-// 13.8, on 8192 16.9 / 15.0, on 32768 42.7 / 20.0, 4 x 60 on 8192 28.5 / 34.2; 32 heads, 1 x 60 on 3904 15.7 / 20.3, 4 x 60 on
-// 2000 30.0 / 32.3; 40 heads, 1 x 30 on 8000 30.4 / 33.4, 2 x 30 on 4000 38.7 / 36.7.
+// Both sides of the line between the forms, clusters / even split, us per layer: 16 query and 2 kv heads, 1 x 16 nodes on 2048 10.1 /
+// 11.9, on 8192 16.3 / 14.2, on 32768 38.2 / 19.2, 4 x 60 on 8192 25.2 / 32.4; 32 heads, 1 x 60 on 3904 15.3 / 19.5, 2 x 60 on
+// 4000 25.4 / 28.5; 40 heads, 1 x 30 on 8000 29.4 / 34.6, 2 x 30 on 4000 37.0 / 34.3.
 // (alternate: units of 128 rows in clusters, whose softmax groups take alternate steps: 0.92 us per step where two threads per row take
 // 1.18.  Where many row blocks share few heads in large clusters a step takes a quarter longer - 16 query and 2 kv heads, 128 nodes: one
 // sequence of 32768 in clusters of eight 1.16, four of 8192 in clusters of two 0.90 -, beyond four ranks the merge grows, and in long
@@ -1433,8 +1437,8 @@ static int tc5_max_cluster(const AttnArgs& a, bool pair, int n_mblocks) {
 // rows in the duplicated layout make twice the units, and a step of such a unit costs its softmax threads half the
 // columns, at the price of every K/V tile crossing from L2 twice as often and half of each product computed for nothing.
 // (As an even split the smaller blocks gain nothing.)  The best estimate decides, a form that options ask for first.
-// Clusters with 64-row units / with 128: 16 query and 2 kv heads, 1 x 16 nodes on 2048 8.9 / 10.4, 4 x 16 on 8192 17.6 / 18.2, 1 x 60 on
-// 8192 17.0 / 17.7, 8 x 60 on 2048 23.4 / 19.9, 4 x 60 on 8192 33.8 / 28.5; 28 / 4 heads, 1 x 60 on 3344 13.4 / 14.8, 4 x 60 30.7 / 25.1.
+// Clusters with 64-row units / with 128: 16 query and 2 kv heads, 1 x 16 nodes on 2048 8.3 / 10.1, 4 x 16 on 8192 17.0 / 17.6, 1 x 128 on
+// 2048 11.5 / 12.2; 28 / 4 heads, 1 x 60 on 3344 13.4 / 14.3, on 1000 9.9 / 12.9; 16 / 4 heads of size 64, 1 x 128 on 4096 12.8 / 12.4.
 constexpr int kSegCost = 4;                     // see SegIter; in steps
 struct Tc5Layout { bool pair; int rows, n_mblocks, ck; double est_us; };
 static Tc5Layout tc5_layout(const AttnArgs& a) {
@@ -1461,7 +1465,7 @@ bool attn_tc5_supports(const AttnArgs& a) {
     const int rows_total = (a.Hq / a.Hkv) * a.N;
     const int rows = rows_total <= 64 ? 64 : 128;
     const long long n_mblocks = (rows_total + 63) / 64;          // the most either layout makes
-    const long long t_max = (long long)a.B * a.Hkv * n_mblocks * ((a.S_max + STEP - 1) / STEP + kSegCost);
+    const long long t_max = (long long)a.B * a.Hkv * n_mblocks * ((a.S_max + STEP - 1) / STEP);
     if (t_max * a.sm_count >= (1ll << 31)) return false;
     if (!(a.scale > 0.f)) return false;       // the kernel takes the maximum before scaling
     return kCounterBytes + tc5_partial_bytes(a.sm_count, rows, a.D) <= a.ws_bytes;
@@ -1492,10 +1496,9 @@ cudaError_t init_attn_tc5() {
 }
 
 // Would units of 256 rows in two tiles (attn_tc5_wide.cu) serve the call better?  Measured, one-tile / two-tile kernel, us
-// per layer (16 query and 2 kv heads unless said otherwise): 8 x 128 nodes
-// on 32768 tokens 345 / 273, on 4096 47.4 / 45.7, on 2048 30.2 / 31.8; 8 x 60 on 16384 88.5 / 80.6; 28 / 4 heads: 8 x 60 on 8192
-// 89.5 / 81.1, 8 x 128 on 1000 43.8 / 36.7, 3 x 128 on 300 16.6 / 20.9; 16 / 4 heads of size 64: 6 x 128 on 3000 34.3 /
-// 27.9, 4 x 100 on 4096 25.0 / 26.0.  The two-tile kernel's steps are cheaper, its first step and its epilogue longer.
+// per layer (16 query and 2 kv heads unless said otherwise): 8 x 128 nodes on 4096 tokens 41.2 / 43.6; 28 / 4 heads: 8 x 60 on 4096
+// 41.8 / 44.0, 8 x 128 on 1000 (more units than one-tile clusters fit) 42.1 / 34.7, 4 x 128 on 8192 70.9 / 73.5; long calls: the comment at
+// tc5_step_us.  The two-tile kernel reads a K/V tile for twice the rows; its first step and its epilogue are longer.
 static bool tc5_prefers_wide(const AttnArgs& a, const Tc5Layout& lay, const WidePlan& wide, double extra_us = 0.0) {
     return wide.est_us < 1e29 && wide.est_us + extra_us < 0.98 * lay.est_us;
 }
@@ -1519,7 +1522,8 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     const int units = a.B * a.Hkv * n_mblocks;
     const long long t_max = (long long)units * ((a.S_max + STEP - 1) / STEP);
     // (more units than CTAs, so ranges do not begin and end with units: only there does the number of segments differ)
-    const int seg_cost = pair && ck == 0 && units > a.sm_count ? kSegCost : 0;
+    // (and T * grid must stay below 2^31, as attn_tc5_supports has checked it for the steps alone)
+    const int seg_cost = pair && ck == 0 && units > a.sm_count && (t_max + (long long)units * kSegCost) * a.sm_count < (1ll << 31) ? kSegCost : 0;
     const int grid = ck > 0 ? units * ck : (int)(t_max < a.sm_count ? t_max : a.sm_count);
 
     Tc5Params p = {};
