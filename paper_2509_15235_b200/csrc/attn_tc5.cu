@@ -1543,9 +1543,11 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     // within the call), the others with the merge kernel.  Measured, in the kernel / with the merge kernel, us per layer (13B
     // heads): 4 x 60 nodes on 1000 tokens 28.2 / 29.1, 8 x 16 on 3000 91.1 / 91.7, 4 x 60 on 3000-5000 62.9 / 64.2 (70.2 / 72.2 with the
     // rotation kernel between the calls), 6 x 16 on 1000-4000 64.9 / 67.0, 4 x 31 on 2000 33.8 / 33.9; 2 x 30 on 4000 37.6 / 34.3.
+    // Pools of 16-row blocks, whose producers are the slower part, gain from twice as many units on (4 x 60 on 3000-5000 with the
+    // rotation kernel between, 16-row blocks 72.9 / 71.7, 128-row blocks 71.3 / 72.0).
     // Blocks of 128 rows, a grid with more units than counters and split form 3 always get the merge kernel.
     const bool own_merge = pair && ck == 0 && a.tc5_path != 3 && !a.no_counters && (size_t)units * sizeof(int) <= kCounterBytes &&
-                           (a.tc5_path == 1 || tc5_steps(a) < 12 || units > a.sm_count);
+                           (a.tc5_path == 1 || tc5_steps(a) < 12 || units > (a.page_rows == 16 ? 2 : 1) * a.sm_count);
     const PagedArgs pa = {a.block_table, a.table_stride, a.page_rows, a.num_blocks, a.Hkv, a.N, a.token_major, a.status,
                           own_merge ? (int*)a.ws : nullptr};
     auto launch_attn = [&](auto kernel, int cluster) {
