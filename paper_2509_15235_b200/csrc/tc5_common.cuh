@@ -308,9 +308,13 @@ struct Tc5Params {
     float scale_log2;
     int* status;
     int step;                  // cached tokens per pipeline step (rows of one K or V stage)
-    int seg_cost;              // even split: steps that a segment's start is counted as when the line is cut (see SegIter)
-    int lock;                  // even split by groups of n_mblocks CTAs: CTA c works for group c / n_mblocks on row block c % n_mblocks
+    short seg_cost;            // even split: steps that a segment's start is counted as when the line is cut (see SegIter)
+    short lock;                // even split by groups of n_mblocks CTAs: CTA c works for group c / n_mblocks on row block c % n_mblocks
 };
+// Two descriptors, this and PagedArgs are 416 bytes of kernel parameters.  With more of them a launch takes 0.35 us of host time longer
+// (424 or 488 bytes: 7.65 and 7.8 us a call of vispec_tree_verify_attn_static on 4 heads of size 64, 1 x 8 nodes on 256 tokens, against
+// 7.3), and that is what bounds the shortest calls.
+static_assert(sizeof(Tc5Params) <= 112, "a larger parameter block makes every launch slower");
 
 // The schedule every CTA (and the merge kernel) derives from kv_len.
 struct Sched {
