@@ -1205,7 +1205,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     }
                 }
                 if (PAIR) mbar_arrive(bar(B_XFREE));
-                if (PAIR && !CL && pa.unit_counters && sg.slot >= 0) {
+                if constexpr (PAIR && !CL) if (pa.unit_counters && sg.slot >= 0) {
                     // ---- even split without a merge kernel (rows <= 64 only: with 128 rows the merge kernel is faster): the CTA that delivers a unit's last partial merges the
                     // unit.  Nobody waits for another CTA: a fence, one atomic per segment, and the last arrival
                     // reads the others' partials (written before their fences) from L2. ----
@@ -1557,8 +1557,7 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
         // fused rotary embedding (contiguous caches): the table holds B*N*D/2 fp64 (cos, sin) pairs, then the same in fp32
         const size_t n = (size_t)a.B * a.N * (D / 2);
         const RopeArgs ra = {(const double2*)a.rope_table, (const float2*)((const double2*)a.rope_table + n),
-                             (const __nv_bfloat16*)a.k_new, (const __nv_bfloat16*)a.v_new, (__nv_bfloat16*)a.k, (__nv_bfloat16*)a.v,
-                             own_merge ? (int*)a.ws : nullptr};
+                             (const __nv_bfloat16*)a.k_new, (const __nv_bfloat16*)a.v_new, (__nv_bfloat16*)a.k, (__nv_bfloat16*)a.v};
         auto launch_rope = [&](auto kernel, int cluster) {
             return launch_pdl(kernel, dim3(grid), dim3(kThreads), SMEM_ALLOC, st, cluster, *a.k_map, *a.v_map, p, ra);
         };

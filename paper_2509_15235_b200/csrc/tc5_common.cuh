@@ -585,10 +585,10 @@ struct RopeArgs {
     const float2* rope_q;      // the same angles in fp32: the q rows' rotation (q is only consumed, never written back)
     const __nv_bfloat16* k_new; const __nv_bfloat16* v_new;   // [B][N][Hkv][D] rows of the tree, to be placed at slots S + i
     __nv_bfloat16* k_cache; __nv_bfloat16* v_cache;            // [B][Hkv][S_max][D]
-    int* unit_counters;        // as in PagedArgs
 };
 struct PagedArgs { const int32_t* block_table; int table_stride, page_rows, num_blocks, Hkv, N, token_major; int* status;
                    int* unit_counters; };   // even split: arrivals per unit (all zero between calls); nullptr: a merge kernel follows
+static_assert(sizeof(RopeArgs) <= 48 && sizeof(PagedArgs) <= 48, "a larger parameter block makes every launch slower (see Tc5Params)");
 
 // ---- producer of a paged segment ---------------------------------------------------------------------
 // Paged cache: a step's 128 slots are 128 / page_rows pool blocks, each its own box.  Run by the whole producer
