@@ -622,7 +622,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             // so that they are there when the segment before ends (a round trip to memory behind a saturated HBM is 3.5 us; a
             // CTA's every further segment cost 7 us with it, for which its rings stood still: llava13b_b4's CTAs ended after 41, 49
             // or 56 us by the number of their segments).  The softmax threads copy them on into the Q tile.
-            auto q_stage = [&]() -> bool {
+            auto q_stage = [&](const Seg& sg) -> bool {
                 const int sk = nk % NSK, r_n = min(ROWS, rows_total - sg.mblock * ROWS);
                 if (!waited) { pdl_wait(); waited = true; }
                 if (!prod_wait(bar(B_KEMPTY + sk), ((nk / NSK) & 1) ^ 1)) return false;
@@ -638,16 +638,16 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             };
             if constexpr (PAGED) {
                 for (int seg = 0; ok && si.next(sg); ++seg) {
-                    if (!CL && seg > 0 && !q_stage()) { ok = false; break; }
-                    const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING, abort_flag, pol, it, waited, lane, split_v ? 1 : 0, nk - it);
+                    const QStage qs = {p.q, p.Hq, G, sg.mblock * ROWS, !CL && seg > 0 ? min(ROWS, rows_total - sg.mblock * ROWS) : 0};
+                    const uint32_t r = produce_paged<Ring128>(pa, &k_map, &v_map, sg.b, sg.kvh, sg.st0, sg.n, sg.S, base, bars, base + SMEM_TABRING, abort_flag, pol, it, waited, lane, split_v ? 1 : 0, nk - it, qs);
                     const int done = (int)(r & 0x0fffffffu);
-                    it += done; nv += split_v ? 0 : done; nk += done + (int)((r >> 28) & 1u);
+                    it += done; nv += split_v ? 0 : done; nk += done + (int)((r >> 28) & 1u) + (int)(r >> 31);
                     ok = !((r >> 29) & 1u);
                     waited = (r >> 30) & 1u;
                 }
             }
             for (int seg = 0; !PAGED && ok && si.next(sg); ++seg) {
-                if (!CL && seg > 0 && !q_stage()) { ok = false; break; }
+                if (!CL && seg > 0 && !q_stage(sg)) { ok = false; break; }
                 const int bh = sg.b * p.Hkv + sg.kvh;
                 const int n = CL ? sg.n : __shfl_sync(0xffffffffu, sg.n, 0);
                 for (int t = 0; t < n; ++t, ++it) {

@@ -600,18 +600,37 @@ static_assert(sizeof(RopeArgs) <= 48 && sizeof(PagedArgs) <= 48, "a larger param
 // at or past kv_len + N are not fetched: their table entries need not exist, and the rows they would fill are
 // masked like any slot past the end.  Not inlined, so that it stays out of the kernel's register budget, and
 // everything by value, so that the caller's counters stay in registers.  Returns steps issued in full | K-only
-// step << 28 | a wait gave up << 29 | has waited for the preceding kernel << 30 (the same in every lane).
+// step << 28 | a wait gave up << 29 | has waited for the preceding kernel << 30 | Q rows sent << 31 (the same in every lane).
 constexpr int STEP = 128;                      // tokens per pipeline step = rows of one K or V stage
 constexpr int HALF_BYTES = STEP * 128;         // one d-half (64 columns) of a stage: 128 rows x 128 B
 constexpr int kTabRing = 4, kTabAhead = 3;     // steps held in a ring / steps a copy is issued ahead (two rings of
                                                // 128 bytes: the K producer's and, where V has its own warp, the V producer's)
+// The Q rows of a unit that come through the K ring ahead of its first step (n == 0: they do not): row r of the n is that of
+// node (row0 + r) / G, the (row0 + r) % G-th head of the kv head.  Here and not in a call of its own: what lived across both calls did
+// not fit the registers that a call preserves (44 bytes of spills in the kernel with 128 rows per unit).
+struct QStage { const __nv_bfloat16* q; int Hq, G, row0, n; };
 template <class R>   // ring geometry: stages, bytes, offsets in shared memory, barrier indices
 __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensorMap* k_map, const CUtensorMap* v_map,
                                                int b, int kvh, int st0, int n, int S, uint32_t base, uint32_t bars,
                                                uint32_t ring, volatile int* abort_flag, uint64_t pol, int it,
                                                bool waited, int lane, int which /* 0: K and V, 1: K only, 2: V only */,
-                                               int koff = 0 /* stages of the K ring used beyond one per step */) {
+                                               int koff = 0 /* stages of the K ring used beyond one per step */, QStage qs = {}) {
     auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
+    uint32_t told = 0;                                                   // the upper bits of the answer
+    if (qs.n > 0) {
+        const int ik = it + koff, sk = ik % R::NSK;
+        if (!waited) { pdl_wait(); waited = true; }
+        if (!__all_sync(0xffffffffu, mbar_wait(bar(R::KEMPTY + sk), ((ik / R::NSK) & 1) ^ 1, abort_flag))) return 2u << 28 | 1u << 30;
+        if (lane == 0) mbar_expect_tx(bar(R::KFULL + sk), (uint32_t)qs.n * (R::STAGE / STEP));
+        __syncwarp();                                                    // the byte count is posted before any lane copies
+        for (int r = lane; r < qs.n; r += 32) {
+            const int row = qs.row0 + r;
+            bulk_load(base + R::OFF_K + sk * R::STAGE + r * (R::STAGE / STEP),
+                      qs.q + (((size_t)b * p.N + row / qs.G) * qs.Hq + kvh * qs.G + row % qs.G) * (R::STAGE / STEP / 2), R::STAGE / STEP, bar(R::KFULL + sk));
+        }
+        ++koff;
+        told = 1u << 31;
+    }
     const int nsub = STEP / p.page_rows;
     const uint32_t sub_bytes = (uint32_t)p.page_rows * 128u;
     const int32_t* trow = p.block_table + (size_t)b * p.table_stride;
@@ -624,7 +643,6 @@ __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensor
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     for (int t = 0; t < kTabAhead; ++t) issue(t);
-    uint32_t fail = 0;
     int t = 0;
     for (; t < n; ++t, ++it) {
         issue(t + kTabAhead);
@@ -652,7 +670,7 @@ __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensor
                 if (w) mbar_expect_tx(bar(R::KFULL + sk), tx);
             }
             w = __shfl_sync(0xffffffffu, w, 0);                          // the byte count is posted before any lane copies
-            if (!w) { fail = 2u << 28; break; }
+            if (!w) { told |= 2u << 28; break; }
             if (load) {
                 tma_load_3d(base + R::OFF_K + sk * R::STAGE + lane * sub_bytes, k_map, bar(R::KFULL + sk), 0, c1, c2, pol);
                 tma_load_3d(base + R::OFF_K + sk * R::STAGE + HALF_BYTES + lane * sub_bytes, k_map, bar(R::KFULL + sk), 64, c1, c2, pol);
@@ -664,7 +682,7 @@ __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensor
                 if (w) mbar_expect_tx(bar(R::VFULL + sv), tx);
             }
             w = __shfl_sync(0xffffffffu, w, 0);
-            if (!w) { fail = (which == 2 ? 2u : 3u) << 28; break; }      // (V only: nothing of this step was issued)
+            if (!w) { told |= (which == 2 ? 2u : 3u) << 28; break; }      // (V only: nothing of this step was issued)
             if (load) {
                 tma_load_3d(base + R::OFF_V + sv * R::STAGE + lane * sub_bytes, v_map, bar(R::VFULL + sv), 0, c1, c2, pol);
                 tma_load_3d(base + R::OFF_V + sv * R::STAGE + HALF_BYTES + lane * sub_bytes, v_map, bar(R::VFULL + sv), 64, c1, c2, pol);
@@ -672,7 +690,7 @@ __device__ __noinline__ uint32_t produce_paged(const PagedArgs p, const CUtensor
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");                     // nothing of this segment stays in flight
-    return (uint32_t)t | fail | (waited ? 1u << 30 : 0u);
+    return (uint32_t)t | told | (waited ? 1u << 30 : 0u);
 }
 
 // Rejected sequences (kv_len < 0 or kv_len + N > S_max): zero output, -inf lse, status word.  By the NT softmax threads.

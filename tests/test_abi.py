@@ -85,3 +85,18 @@ def test_product_package_does_not_import_the_oracle():
         if f.endswith((".py", ".c")):
             src = open(os.path.join(ROOT, "oracle", f)).read()
             assert "paper_2509_15235_b200" not in src and "vispec.h" not in src
+
+
+@pytest.mark.parametrize("source", ["attn_tc5.cu", "attn_tc5_wide.cu"])
+def test_no_attention_kernel_spills_registers(source, tmp_path):
+    """The kernels are compiled for one CTA per SM with every register in use: one value too many and the step loop goes through
+    local memory.  What the assembler reports, kernel by kernel."""
+    from paper_2509_15235_b200 import build
+    cmd = [os.environ.get("NVCC", "nvcc"), *build.NVCC_FLAGS, "-I", os.path.join(build.ROOT, "include"), "-I", build.CSRC, "-c",
+           os.path.join(build.CSRC, source), "-o", str(tmp_path / "out.o")]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
+    said = re.findall(r"Compiling entry function '(\w+)'.*?(\d+) bytes spill stores, (\d+) bytes spill loads", res.stdout + res.stderr, flags=re.S)
+    attn = [s for s in said if "attn_tc5" in s[0]]
+    assert len(attn) >= 6
+    assert [s for s in attn if s[1:] != ("0", "0")] == []

@@ -3,6 +3,7 @@
 Paging is a layout, not arithmetic: the oracle runs on the contiguous cache the pool was cut from.  The paged
 attention must agree with the oracle within the attention tolerance AND bit for bit with the contiguous GPU call
 (same tiles, same order of operations)."""
+import functools
 import math
 
 import numpy as np
@@ -93,6 +94,37 @@ def test_paged_attention_equals_contiguous_and_oracle(page_rows, split_form, tok
     assert np.abs(out - want).max() <= TOL and np.abs(lse - want_lse).max() <= LSE_TOL
     ref, ref_lse, st = gu.run_attn(q, k, v, kv_len, mask, scale, split_form=split_form)
     assert st == 0 and np.array_equal(out, ref) and np.array_equal(lse, ref_lse)
+
+
+@functools.lru_cache(maxsize=1)
+def _many_units(B, N, Hq, Hkv, S_list, S_max):
+    q, k, v, kv_len, mask, _ = _case(B, N, Hq, Hkv, list(S_list), S_max, 900 + Hkv)
+    scale = 1 / math.sqrt(128)
+    return q, k, v, kv_len, mask, scale, oracle.tree_attn(q, k, v, kv_len, mask, scale)
+
+
+@pytest.mark.parametrize("B,N,Hq,Hkv,S_list,S_max", [
+    (4, 60, 40, 40, (1500, 900, 1300, 5), 1664),      # 160 units of 8 to 13 steps and of one: several segments per CTA
+    (4, 20, 160, 80, (1100, 1030, 970, 1000), 1152),  # more than two units per SM, two heads per kv head
+    (4, 40, 80, 40, (1500, 900, 1300, 5), 1664),      # 80 rows: units of 128
+    (2, 92, 84, 28, (1400, 700), 1536),               # 276 rows: three blocks, the last of 20 rows
+])
+@pytest.mark.parametrize("page_rows,token_major", [(16, False), (16, True), (32, True), (128, False)])
+@pytest.mark.parametrize("split_form", [0, 1, 3])
+def test_paged_attention_with_more_units_than_ctas(B, N, Hq, Hkv, S_list, S_max, page_rows, token_major, split_form):
+    """The q rows of a CTA's later segments take stages of the K ring beside the pool's blocks, the starts of segments count as
+    steps when the line is cut (rows <= 64), and units merge in the kernel or after it.  The forced forms are bit for bit the contiguous
+    call's; the library's own choice may merge elsewhere on a pool."""
+    import gpu_util as gu
+    q, k, v, kv_len, mask, scale, (want, want_lse) = _many_units(B, N, Hq, Hkv, S_list, S_max)
+    rng = np.random.Generator(np.random.Philox(page_rows + token_major))
+    pools, table = _page((k, v), page_rows, rng)
+    out, lse, status = _run_paged(q, pools, table, kv_len, mask, scale, split_form, token_major=token_major)
+    assert status == 0 and not np.isnan(out).any()
+    assert np.abs(out - want).max() <= TOL and np.abs(lse - want_lse).max() <= LSE_TOL
+    if split_form:
+        ref, ref_lse, st = gu.run_attn(q, k, v, kv_len, mask, scale, split_form=split_form)
+        assert st == 0 and np.array_equal(out, ref) and np.array_equal(lse, ref_lse)
 
 
 @pytest.mark.parametrize("page_rows", [16, 64, 128])
