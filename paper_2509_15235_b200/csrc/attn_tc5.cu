@@ -1541,13 +1541,18 @@ cudaError_t launch_attn_tc5(const AttnArgs& a, cudaStream_t st, int* n_launches)
     // Even split, at most 64 rows per unit: short calls and those of more units than CTAs merge in the attention kernel (the last
     // arrival at a unit, by the counters at the head of the workspace; the ranges then end at different units, and most merges lie
     // within the call), the others with the merge kernel.  Measured, in the kernel / with the merge kernel, us per layer (13B
-    // heads): 4 x 60 nodes on 1000 tokens 28.2 / 29.1, 8 x 16 on 3000 91.1 / 91.7, 4 x 60 on 3000-5000 62.9 / 64.2 (70.2 / 72.2 with the
-    // rotation kernel between the calls), 6 x 16 on 1000-4000 64.9 / 67.0, 4 x 31 on 2000 33.8 / 33.9; 2 x 30 on 4000 37.6 / 34.3.
-    // Pools of 16-row blocks, whose producers are the slower part, gain from twice as many units on (4 x 60 on 3000-5000 with the
-    // rotation kernel between, 16-row blocks 72.9 / 71.7, 128-row blocks 71.3 / 72.0).
+    // heads): 4 x 60 nodes on 1000 tokens 28.2 / 29.1, 8 x 16 on 3000 91.1 / 91.7; 2 x 30 on 4000 37.6 / 34.3.
+    // Just above one unit per CTA little lies within the call, and what is merged late counts against the rows merged: 160 units on 1500-3000
+    // tokens with the rotation kernel between the calls (a quarter of a pass of four layers), 16 nodes 44.2 / 42.2, 31 nodes 46.2 / 44.8, 40 nodes 48.6 / 48.7, 60 nodes 49.6 / 50.1
+    // (on 3000-5000: 16 nodes 67.1 / 66.4, 60 nodes 72.4 / 74.7); 200 units 56.4 / 56.7 and 63.4 / 64.6, 280 units 69.4 / 70.9 and 78.2 / 80.3.
+    // Pools of 16-row blocks, whose producers are the slower part, gain from twice as many units as SMs on, 16 and 60 nodes: 160 units
+    // 47.4 / 43.2 and 52.5 / 51.2, 200 units 60.3 / 57.2 and 67.5 / 65.3, 240 units 65.1 / 61.4 and 79.7 / 78.6, 280 units 74.9 / 72.1 and 82.5 / 82.7, 320 units
+    // 79.2 / 78.2 and 97.1 / 97.5 (without the rotation kernel 74.6 / 75.4 and 86.9 / 87.1).  Blocks of 32 to 128 rows are within 1 % of the
+    // contiguous cache's line with 60 nodes (200 units 65.2-65.4 / 65.3-65.7) and up to 3 % on the other side of it with 16 (58.0-58.4 / 57.2-58.0).
     // Blocks of 128 rows, a grid with more units than counters and split form 3 always get the merge kernel.
+    const int crowd = a.page_rows == 16 ? 8 : (a.Hq / a.Hkv) * a.N <= 32 ? 5 : 4;      // quarters of a unit per SM
     const bool own_merge = pair && ck == 0 && a.tc5_path != 3 && !a.no_counters && (size_t)units * sizeof(int) <= kCounterBytes &&
-                           (a.tc5_path == 1 || tc5_steps(a) < 12 || units > (a.page_rows == 16 ? 2 : 1) * a.sm_count);
+                           (a.tc5_path == 1 || tc5_steps(a) < 12 || 4ll * units > (long long)crowd * a.sm_count);
     const PagedArgs pa = {a.block_table, a.table_stride, a.page_rows, a.num_blocks, a.Hkv, a.N, a.token_major, a.status,
                           own_merge ? (int*)a.ws : nullptr};
     auto launch_attn = [&](auto kernel, int cluster) {

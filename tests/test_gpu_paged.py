@@ -127,6 +127,29 @@ def test_paged_attention_with_more_units_than_ctas(B, N, Hq, Hkv, S_list, S_max,
         assert st == 0 and np.array_equal(out, ref) and np.array_equal(lse, ref_lse)
 
 
+@pytest.mark.parametrize("page_rows,N,heads,own", [
+    (16, 60, 40, False), (16, 60, 80, True),                     # blocks of 16 rows: from two units per SM on
+    (64, 60, 40, True), (64, 33, 40, True),                      # others: from one on ...
+    (64, 32, 40, False), (64, 32, 50, True),                     # ... with at most 32 rows per unit from five quarters on
+    (0, 32, 40, False), (0, 33, 40, True), (0, 32, 50, True),    # contiguous caches likewise
+])
+def test_units_of_crowded_lines_merge_in_the_kernel(page_rows, N, heads, own):
+    """Which of the two merges serves an even split of 160, 200 and 320 units (148 SMs), and that it is right."""
+    import gpu_util as gu
+    assert torch.cuda.get_device_properties(0).multi_processor_count == 148
+    q, k, v, kv_len, mask, rng = _case(4, N, heads, heads, [1500, 900, 1300, 5], 1664, 1200 + N)
+    if page_rows:
+        pools, table = _page((k, v), page_rows, rng)
+        (out, lse, status), kernels = gu.kernels_of(lambda: _run_paged(q, pools, table, kv_len, mask, 0.09))
+    else:
+        (out, lse, status), kernels = gu.kernels_of(lambda: gu.run_attn(q, k, v, kv_len, mask, 0.09))
+    assert any("attn_tc5_kernel" in n for n in kernels) and any("attn_tc5_merge_kernel" in n for n in kernels) != own
+    h = [0, heads // 2, heads - 1]
+    want, want_lse = oracle.tree_attn(q[:, :, h], k[:, h], v[:, h], kv_len, mask, 0.09)
+    assert status == 0 and not np.isnan(out).any()
+    assert np.abs(out[:, :, h] - want).max() <= TOL and np.abs(lse[:, h] - want_lse).max() <= LSE_TOL
+
+
 @pytest.mark.parametrize("page_rows", [16, 64, 128])
 def test_paged_attention_two_tile_units(page_rows):
     """Units of 256 rows, which the host chooses by the table's capacity (40960 slots, of which few are in use)."""
