@@ -262,8 +262,12 @@ constexpr int kPolyEvery = 4;
 // products 1024).  Here a row belongs to one thread of each group of four warps; group x takes the steps of parity x whole, with a
 // reference maximum, a sum and an accumulator of its own (added up at the end), so nothing is exchanged, and while one group is in
 // its exponentials the products of the other run.  P overwrites S, which makes room for the second accumulator; one warp issues all
-// products, S(0) S(1) | PV(0) S(2) | PV(1) S(3) | ...: they complete in the order of issue, so S(t + 2) may overwrite P(t), and its
-// completion tells that PV(t) is complete.  1880 cycles per step (qwen3b_S8192_N60_B4 485 -> 465 us per pass; tensor pipe active 35 %
+// products, S(0) S(1) | PV(0) S(2) | PV(1) S(3) | ...: S(t + 2) overwrites P(t) behind PV(t), which reads it, and its completion, for which
+// a commit also waits for all that was issued before, tells that PV(t) is complete.  That the overwriting product does not overtake the
+// reading one rests on how the tensor core works - one CTA's products start in the order of issue -, not on a documented guarantee, which
+// covers products of one shape on one accumulator (test_products_in_shared_tensor_memory_repeat_bit_for_bit looks; the two-tile kernel rests
+// on the same).  A wait for PV(t) ahead of S(t + 2): 16 query and 2 kv heads, 4 x 60 nodes on 8192 tokens 443.7 -> 450.5 us per pass of 16
+// layers, 8 x 128 on 4096 385.1 -> 388.8, 28 / 4 heads, 1 x 128 on 8192 408.0 -> 413.7, head size 64 no change.  1880 cycles per step (qwen3b_S8192_N60_B4 485 -> 465 us per pass; tensor pipe active 35 %
 // of a launch against 31 %).  What is left is a group's chain, products of its own step and of the other group's among it, and beside
 // it shared memory, whose 128 bytes per cycle feed both operands of S (512 cycles), V (256) and the copies coming in (512).  In the even
 // split, whose CTAs have fewer steps here, the longer first step costs more than the loop gains (qwen3b_S32768_N16_B1 324 -> 329),

@@ -202,6 +202,42 @@ def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
     assert np.abs(lse - want_lse).max() <= 2e-6
 
 
+# ---- units of 128 rows in clusters, whose two groups of softmax warps take alternate steps ----
+def _ran_alternate_steps(kernels):
+    """The one-tile kernel in its cluster form with units of 128 rows: template arguments false, true, ..."""
+    return any("attn_tc5_kernel<false, true" in n or "attn_tc5_kernelILb0ELb1E" in n for n in kernels)
+
+
+# P of a step lies in the tensor memory that the scores two steps on overwrite, and the order of the products alone keeps the two
+# apart: every repetition gives the same bits.  One-tile clusters and the two-tile kernel.
+@pytest.mark.parametrize("Hq,Hkv,D,B,N,S,S_max,split_form,kernel", [
+    (16, 2, 128, 4, 60, 4000, 4224, 2, "attn_tc5_kernel"), (16, 4, 64, 4, 60, 4000, 4224, 2, "attn_tc5_kernel"),
+    (16, 2, 128, 4, 128, 4000, 40000, 0, "attn_tc5_wide_kernel"),
+])
+def test_products_in_shared_tensor_memory_repeat_bit_for_bit(gu, Hq, Hkv, D, B, N, S, S_max, split_form, kernel):
+    from paper_2509_15235_b200 import binding
+    rng = np.random.Generator(np.random.Philox(73))
+    gen = torch.Generator("cuda").manual_seed(74)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+    q, k, v = rand(B, N, Hq, D), rand(B, Hkv, S_max, D), rand(B, Hkv, S_max, D)
+    mask, _, _ = oracle.tree_mask(np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)]))
+    mask, kv_len = gu.u64_dev(mask), gu.i32_dev([S - 37 * b for b in range(B)])
+    ctx = binding.VerifyContext(B, N, Hq, Hkv, D, S_max, 1)
+    ctx.ctx_set_option(binding.OPT_SPLIT_FORM, split_form)
+    ctx.cache_register(0, k, v)
+    outs = [torch.zeros_like(q) for _ in range(8)]
+    _, kernels = gu.kernels_of(lambda: ctx.tree_verify_attn(0, q, kv_len, mask, 0.09, outs[0]))
+    assert any(kernel in n for n in kernels) and (kernel != "attn_tc5_kernel" or _ran_alternate_steps(kernels)), kernels
+    first = outs[0].clone()
+    for rep in range(40):                                            # eight calls back to back, then the comparison
+        for o in outs:
+            ctx.tree_verify_attn(0, q, kv_len, mask, 0.09, o)
+        for o in outs:
+            assert torch.equal(o, first)
+    assert ctx.status_poll() == 0
+    ctx.close()
+
+
 # A NaN in a key (or an infinite score) makes every row that sees it NaN, whatever column of a step the key falls on.  One
 # sequence per step column modulo 16, one whose second 64 tokens are all such keys (the duplicated-row layout keeps a state of
 # its own for those), one without any.
