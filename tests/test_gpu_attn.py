@@ -177,6 +177,10 @@ def test_more_units_than_ctas(gu, Hkv, D, N, kv_len, S_max, split_form):
 @pytest.mark.parametrize("Hq,Hkv,D,N,S_max", [(4, 4, 64, 60, 256), (4, 1, 64, 100, 256), (4, 4, 128, 60, 256), (4, 1, 128, 100, 256),
                                               (16, 2, 64, 128, 40000), (16, 2, 128, 128, 40000)])
 def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
+    _one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static)
+
+
+def _one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static=False, split_form=0):
     from paper_2509_15235_b200 import binding
     rng = np.random.Generator(np.random.Philox(Hq * 1000 + N + D))
     B, scale = 2, 1 / 16
@@ -195,7 +199,7 @@ def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
         binding.tree_verify_attn_static(gu.bf16_dev(q), gu.bf16_dev(k), gu.bf16_dev(v), gu.i32_dev(kv_len), gu.u64_dev(mask), scale, out, lse)
         out, lse = out.float().cpu().numpy(), lse.cpu().numpy()
     else:
-        out, lse, status = gu.run_attn(q, k, v, kv_len, mask, scale)
+        out, lse, status = gu.run_attn(q, k, v, kv_len, mask, scale, split_form=split_form)
         assert status == 0
     want, want_lse = oracle.tree_attn(q, k[:, :, :N + 1], v[:, :, :N + 1], kv_len, mask, scale)
     assert np.abs(out - want).max() <= TOL
@@ -206,6 +210,73 @@ def test_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max, static):
 def _ran_alternate_steps(kernels):
     """The one-tile kernel in its cluster form with units of 128 rows: template arguments false, true, ..."""
     return any("attn_tc5_kernel<false, true" in n or "attn_tc5_kernelILb0ELb1E" in n for n in kernels)
+
+
+def _alternate_case(D, seed, B=24):
+    """24 sequences x 2 kv heads of 128 rows: clusters of three CTAs, four steps to each, so that both groups of a CTA have a second
+    step; lengths end in every part of the last step, and what lies past them is NaN."""
+    N, Hq, Hkv, S_max = 16, 16, 2, 1536
+    rng = np.random.Generator(np.random.Philox(seed))
+    q = synth.normal_bf16((B, N, Hq, D), seed + 1)
+    k = synth.normal_bf16((B, Hkv, S_max, D), seed + 2)
+    v = synth.normal_bf16((B, Hkv, S_max, D), seed + 3)
+    kv_len = np.array([S_max - N - 1 - 5 * b for b in range(B)], dtype=np.int32)
+    parents = np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)])
+    mask, _, _ = oracle.tree_mask(parents)
+    return q, k, v, kv_len, mask
+
+
+def _nan_past_the_end(kv_len, N, *caches):
+    for c in caches:
+        for b, S in enumerate(kv_len):
+            c[b, :, S + N:] = 0x7FC0
+
+
+@pytest.mark.parametrize("D", [128, 64])
+def test_alternate_steps_move_the_reference_maximum(gu, D):
+    """Scores that climb by 6 c (8.7 c in log2 units) per step, c by row from -2 to 2, so that rows of one warp move their reference in
+    other steps, and values that shrink by e^6 per step: with c = 1 every step has the same part in a row's output, whatever has become
+    of the reference since.  A row's output is measured against its largest element."""
+    q, k, v, kv_len, mask = _alternate_case(D, 7100)
+    B, N, Hq, _ = q.shape
+    step = np.arange(k.shape[2]) // 128
+    qf, kf, vf = (synth.bf16_bits_to_f32(x) for x in (q, k, v))
+    c = np.array([1, 2, 0.5, -1, 1, -2, 0, 1], dtype=np.float32)
+    qf[..., 0] = c[(np.arange(N)[:, None] + np.arange(Hq)) % 8]
+    kf[..., 0] = 6 * 16 * step                                       # (exact in bf16; the scale is 1/16)
+    vf *= np.exp(6.0 * (11 - step))[:, None].astype(np.float32)
+    q, k, v = (synth.f32_to_bf16_bits(x) for x in (qf, kf, vf))
+    clean = (k.copy(), v.copy())
+    _nan_past_the_end(kv_len, N, k, v)
+    (out, lse, status), kernels = gu.kernels_of(lambda: gu.run_attn(q, k, v, kv_len, mask, 1 / 16, split_form=2))
+    assert status == 0 and _ran_alternate_steps(kernels), kernels
+    want, want_lse = oracle.tree_attn(q, *clean, kv_len, mask, 1 / 16)
+    assert np.isfinite(out).all()
+    assert (np.abs(out - want) / np.abs(want).max(axis=-1, keepdims=True)).max() <= TOL
+    assert np.abs(lse - want_lse).max() <= LSE_TOL
+
+
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("special", [0x7FC0, 0x7F80])
+def test_alternate_steps_nan_and_infinite_scores(gu, D, special):
+    """One such key per sequence, in even and odd steps of every rank, in either half and every column modulo 16 of a step; the last
+    sequence has none."""
+    q, k, v, kv_len, mask = _alternate_case(D, 7200)
+    B, N, Hq, _ = q.shape
+    _nan_past_the_end(kv_len, N, k, v)
+    for b in range(B - 1):
+        k[b, :, (b % 11) * 128 + (64 if b >= 11 else 0) + (7 * b) % 64, 3] = special
+    (out, _, status), kernels = gu.kernels_of(lambda: gu.run_attn(q, k, v, kv_len, mask, 0.1, split_form=2))
+    assert status == 0 and _ran_alternate_steps(kernels), kernels
+    want = np.ones((B, N, Hq), dtype=bool) if special == 0x7FC0 else synth.bf16_bits_to_f32(q)[..., 3] > 0
+    want[B - 1] = False
+    assert np.isnan(out[want]).all() and np.isfinite(out[~want]).all()
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,N,S_max", [(4, 1, 64, 100, 256), (4, 1, 128, 100, 256), (16, 2, 128, 128, 512)])
+def test_alternate_steps_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_max):
+    _, kernels = gu.kernels_of(lambda: _one_or_two_keys(gu, Hq, Hkv, D, N, S_max, split_form=2))
+    assert _ran_alternate_steps(kernels), kernels
 
 
 # P of a step lies in the tensor memory that the scores two steps on overwrite, and the order of the products alone keeps the two
