@@ -1398,23 +1398,37 @@ static int query_max_clusters(bool pair, int k) {
 // kernel, us per layer in runs of seconds: 8 x 60 nodes on 8192 44.6 / 45.6, 4 x 60 on 16384 44.6 / 47.8, on 32768 81.1 / 79.8, 8 x 128 on
 // 8192 77.6 / 82.1, 2 x 128 on 40000 92.1 / 89.4; in short ones 39.5 / 43.4, 39.5 / 44.8, 72.3 / 70.9, 70.1 / 74.9; 1 x 128 on 32768
 // 49.0 / 42.0; 28 / 4 heads, 2 x 92 on 40000 142 / 125; 16 / 4 heads of size 64, 6 x 60 on 3000 17.7 / 21.7, 6 x 128 30.1 / 27.0.)
+static double tc5_compute_us(const AttnArgs& a, bool pair, double ctas, bool alternate) {
+    const double busy = ctas / a.sm_count, us = pair ? 0.8 + 0.25 * busy : alternate ? 0.80 + 0.14 * busy : 1.05 + 0.15 * busy;
+    return a.D == 64 ? 0.9 * us : us;
+}
 static double tc5_step_us(const AttnArgs& a, bool pair, int n_mblocks, double ctas, bool alternate) {
-    const double busy = ctas / a.sm_count, compute = pair ? 0.8 + 0.25 * busy : alternate ? 0.80 + 0.14 * busy : 1.05 + 0.15 * busy;
-    return fmax(a.D == 64 ? 0.9 * compute : compute, ctas * 0.0093 * (a.D / 128.0) / n_mblocks);
+    return fmax(tc5_compute_us(a, pair, ctas, alternate), ctas * 0.0093 * (a.D / 128.0) / n_mblocks);
 }
 static int tc5_steps(const AttnArgs& a) {
     const int slots = (a.kv_len_hint > 0 && a.kv_len_hint + a.N < a.S_max) ? a.kv_len_hint + a.N : a.S_max;
     return (slots + STEP - 1) / STEP;
 }
+// (late: 128 rows per kv head in clusters of four and more, which leave 20 to 50 SMs without work.  From about the fourteenth step of a
+// CTA on, when what its rings held at the start is used up and the clusters have drifted apart, a step takes longer by what the
+// CTAs draw on HBM, and the even split, on all SMs, is the faster form.  16 query and 2 kv heads, clusters / even split, us per
+// layer: 8 x 16 nodes on 12000 tokens 26.9 / 27.9, on 16384 35.2 / 34.4, on 20000 43.3 / 39.4, on 24000 51.6 / 46.5, on 32000 67.4 / 58.0; on
+// half to all of 20000 30.4 / 31.5, of 28000 41.6 / 38.9; 6 x 13 on 20000 31.8 / 32.4, on 24000 38.2 / 36.7, on 28000 42.7 / 39.5; 5 x 16 on
+// 24000 37.1 / 32.2.  Clusters of two have no such loss: 32 heads, 2 x 128 on 8000 53.5 / 62.7.)
 static double tc5_cluster_us(const AttnArgs& a, bool pair, int n_mblocks, int k) {
     const double ctas = (double)a.B * a.Hkv * n_mblocks * k, steps = (double)((tc5_steps(a) + k - 1) / k);
-    const double us = steps * tc5_step_us(a, pair, n_mblocks, ctas, !pair);
-    if (pair) return 6.9 + us;
-    return 9.4 + us + 0.35 * (k > 4 ? k - 4 : 0) + (n_mblocks > 4 && k > 4 ? 0.24 * steps : 0.0) + 0.22 * (ctas / a.sm_count) * fmax(0.0, steps - 32.0);
+    const double step = tc5_step_us(a, pair, n_mblocks, ctas, !pair);
+    if (pair) return 6.9 + steps * step;
+    const double over = 0.005 * ctas * (a.D / 128.0) - (step - tc5_compute_us(a, pair, ctas, !pair));
+    const double late = n_mblocks == 1 && k >= 4 ? fmax(0.0, over) * fmax(0.0, steps - 14.0) : 0.0;
+    return 9.4 + steps * step + late + 0.35 * (k > 4 ? k - 4 : 0) + (n_mblocks > 4 && k > 4 ? 0.24 * steps : 0.0) +
+           0.22 * (ctas / a.sm_count) * fmax(0.0, steps - 32.0);
 }
 // (even split: the CTAs as sched_ctas counts them; partials of 128 rows cost 34 ns per CTA, written and merged, those of 64
-// rows go in the fixed part; where there are more units than CTAs every further segment of a CTA costs a Q tile, a
-// pipeline start and an epilogue)
+// rows go in the fixed part; where there are more units than CTAs and several row blocks every further segment of a CTA costs a Q
+// tile, a pipeline start and an epilogue.  A call with the fused rotary embedding, which exists in clusters only, would need the rotation
+// kernel ahead of it: 16 / 2 heads, 5 x 16 on 16384 28.8 in clusters, 29.6 with kernel and even split, where the plain calls take
+// 27.1 and 25.6)
 static double tc5_even_us(const AttnArgs& a, bool pair, int n_mblocks) {
     const int units = a.B * a.Hkv * n_mblocks;
     const double T = (double)tc5_steps(a) * units;
@@ -1423,7 +1437,8 @@ static double tc5_even_us(const AttnArgs& a, bool pair, int n_mblocks) {
         const double r = floor(n / units) * units;
         if (n_mblocks > 1 || ceil(T / r) - ceil(T / n) <= 3.0) n = r;
     }
-    return (pair ? 9.5 : 10.4 + 0.034 * n) + ceil(T / n) * tc5_step_us(a, pair, n_mblocks, n, false) + (units > n && n_mblocks > 1 ? 11.0 * units / n : 0.0);
+    return (pair ? 9.5 : 10.4 + 0.034 * n) + ceil(T / n) * tc5_step_us(a, pair, n_mblocks, n, false) + (units > n && n_mblocks > 1 ? 11.0 * units / n : 0.0) +
+           (a.rope_table ? 3.0 : 0.0);
 }
 
 // Cluster size of the cluster form: one cluster per unit, as large as all clusters fit at once (0: they do not).

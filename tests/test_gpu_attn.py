@@ -278,6 +278,23 @@ def test_alternate_steps_lse_of_rows_with_one_or_two_keys(gu, Hq, Hkv, D, N, S_m
     _, kernels = gu.kernels_of(lambda: _one_or_two_keys(gu, Hq, Hkv, D, N, S_max, split_form=2))
     assert _ran_alternate_steps(kernels), kernels
 
+@pytest.mark.parametrize("B,N,S,clusters", [(8, 16, 12000, True), (8, 16, 24000, False), (6, 13, 20000, True), (6, 13, 28000, False)])
+def test_long_calls_of_one_row_block_leave_the_clusters(gu, B, N, S, clusters):
+    """16 and 2 heads, 104 and 128 rows per kv head: from where clusters of six and eight are the slower form, the even split and its merge
+    kernel serve the call.  Few tokens in use: the form follows the capacity."""
+    q = synth.normal_bf16((B, N, 16, 128), 8100)
+    kv_len = np.array([300 + 17 * b for b in range(B)], dtype=np.int32)
+    used = int(kv_len.max()) + N
+    k, v = (np.zeros((B, 2, S + 128, 128), dtype=np.uint16) for _ in range(2))
+    k[:, :, :used] = synth.normal_bf16((B, 2, used, 128), 8101)
+    v[:, :, :used] = synth.normal_bf16((B, 2, used, 128), 8102)
+    rng = np.random.Generator(np.random.Philox(8103))
+    mask, _, _ = oracle.tree_mask(np.stack([synth.draw_tree(N, 6, 4, rng) for _ in range(B)]))
+    (out, lse, status), kernels = gu.kernels_of(lambda: gu.run_attn(q, k, v, kv_len, mask, 0.09))
+    assert status == 0 and _ran_alternate_steps(kernels) == clusters and any("attn_tc5_merge_kernel" in n for n in kernels) != clusters
+    want, want_lse = oracle.tree_attn(q, k[:, :, :used], v[:, :, :used], kv_len, mask, 0.09)
+    assert np.abs(out - want).max() <= TOL and np.abs(lse - want_lse).max() <= LSE_TOL
+
 
 # P of a step lies in the tensor memory that the scores two steps on overwrite, and the order of the products alone keeps the two
 # apart: every repetition gives the same bits.  One-tile clusters and the two-tile kernel.
