@@ -250,9 +250,10 @@ __device__ __noinline__ void rope_prologue(unsigned char* sm, const __nv_bfloat1
 }
 
 // The softmax's exponentials are what the special-function pipe (16 lanes per SM) spends a step on; one in eight of them is
-// formed on the FMA pipe instead: in the duplicated-row layout two neighbouring columns of every sixteen by one packed
-// evaluation, with 128 rows one column of every eight (packed there: 517.6 against 507.1 us per pass on qwen3b_S8192_N60_B4).
-// None / 1 in 16 / 1 in 8, us per pass: llava7b 559.6 / 558.4 / 550.3, qwen3b_S8192_N60_B4 532.1 / 526.1 / 507.1, qwen7b fused
+// formed on the FMA pipe instead: in the duplicated-row layout and in alternate steps two neighbouring columns of every sixteen by one
+// packed evaluation, in the even split with 128 rows, where two threads share a row, one column of every eight (packed in that loop, which
+// then served clusters too: 517.6 against 507.1 us per pass on qwen3b_S8192_N60_B4).  Measured on the loop with two threads per row,
+// none / 1 in 16 / 1 in 8, us per pass: llava7b 559.6 / 558.4 / 550.3, qwen3b_S8192_N60_B4 532.1 / 526.1 / 507.1, qwen7b fused
 // 455.3 / 454.8 / 451.8; 1 in 6 moves nothing, 1 in 4 and 1 in 2 are slower (issue slots).
 constexpr int kPolyEvery = 4;
 
@@ -439,7 +440,7 @@ __device__ __forceinline__ bool alternate_softmax(unsigned char* sm, uint32_t ba
             for (int c = 0; c < 32; ++c) {
                 float x0, x1, e0, e1;
                 up2(fma2(pk2(__uint_as_float(s[2 * c]), __uint_as_float(s[2 * c + 1])), sc2, mm2), x0, x1);
-                if (c % 8 == 7) exp2_fma_pair(x0, x1, e0, e1);  // (see kPolyEvery)
+                if (c % (2 * kPolyEvery) == 2 * kPolyEvery - 1) exp2_fma_pair(x0, x1, e0, e1);
                 else { e0 = exp2f(x0); e1 = exp2f(x1); }
                 if (c & 1) sum2b = add2(sum2b, pk2(e0, e1)); else sum2 = add2(sum2, pk2(e0, e1));
                 pd[c] = pack_bf16(e0, e1);
@@ -625,7 +626,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             // Even split: the Q rows of a CTA's later segments come through the K ring, one stage ahead of the segment's first K tile,
             // so that they are there when the segment before ends (a round trip to memory behind a saturated HBM is 3.5 us; a
             // CTA's every further segment cost 7 us with it, for which its rings stood still: llava13b_b4's CTAs ended after 41, 49
-            // or 56 us by the number of their segments).  The softmax threads copy them on into the Q tile.
+            // or 56 us by the number of their segments, and with the rows sent ahead after 44, 49 or 54).  The softmax threads copy them on into the Q tile.
             auto q_stage = [&](const Seg& sg) -> bool {
                 const int sk = nk % NSK, r_n = min(ROWS, rows_total - sg.mblock * ROWS);
                 if (!waited) { pdl_wait(); waited = true; }

@@ -359,7 +359,8 @@ static __device__ void sched_build(Sched& s, const Tc5Params& p, int lane, int k
     }
     if (lane == 0) s.units = live * upb;
 }
-// Number of CTAs that get work: every CTA at least min_steps steps; a multiple of the unit count when
+// Number of CTAs that get a range: each at least min_steps places of the line (see SegIter; with segments' starts counted a range may hold
+// one step or none); a multiple of the unit count when
 // the units are fewer than the CTAs (equally long units then never share a CTA) - unless the CTAs left out cost more
 // steps than a second segment's Q tile and epilogue in every CTA (round_steps).  Unaligned ranges put the row blocks of a
 // kv head, where they are units of their own, at different places of the cache, which is then read once per row block
@@ -391,7 +392,8 @@ struct Seg {
 };
 // The line that the even split cuts: every unit is seg_cost places without work, then its steps.  A CTA whose range takes in the
 // start of a unit pays for one more segment (a Q tile, an empty pipeline and an epilogue: 5 us with rows <= 64, as long as 4
-// steps), and so gets as many steps less; without it llava13b_b4's CTAs ended after 44, 49 or 54 us by the number of their segments.
+// steps), and so gets as many steps less; without it llava13b_b4's CTAs, the Q rows sent ahead already, ended after 44, 49 or 54 us by
+// the number of their segments.
 // COST: seg_cost may be other than 0 (rows <= 64; elsewhere the register that it takes costs more).
 template <bool COST>
 struct SegIter {
@@ -874,8 +876,9 @@ cudaError_t launch_merge(const Tc5Params& p, int units, int ctas, cudaStream_t s
     if (blocks * 2 <= kMergeBlocks) return go(std::integral_constant<int, 2>{});
     return go(std::integral_constant<int, 1>{});
 }
-// Per-device set-up of those kernels: the merge blocks must be able to join an SM that an attention CTA has configured
-// for maximum shared memory.
+// Per-device set-up of those kernels: the merge blocks ask for the split of shared memory and L1 that the attention CTAs have
+// configured, so that an SM takes them as soon as its attention CTA has left, and the next call's CTA after them.  (Beside an attention
+// CTA there is room for neither a merge block nor one of the rotation: 16 bytes of shared memory and 1024 registers.)
 template <int ROWS, int HD>
 cudaError_t init_merge() {
     const void* kernels[5] = {(const void*)attn_tc5_merge_kernel<ROWS, 0, HD>, (const void*)attn_tc5_merge_kernel<ROWS, 1, HD>,
